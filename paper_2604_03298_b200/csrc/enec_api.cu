@@ -453,7 +453,7 @@ static enec_status decompress_one(const void* d_in, size_t in_size, enec_dtype d
     batch.jobs = nullptr;
     batch.prefix = nullptr;
     batch.n_jobs = 1;
-    batch.blockwise = blockwise ? 1 : 0;
+    batch.option = blockwise ? 1 : 0;
     batch.total_blocks = make_geometry(count).nblocks;
     batch.inline_jobs[0] = DecodeJob{static_cast<const uint8_t*>(d_in), static_cast<uint16_t*>(d_out), uint64_t(count),
                                      uint64_t(in_size)};
@@ -486,6 +486,13 @@ enec_status enec_decompress(const void* d_in, size_t in_size, enec_dtype dt, siz
 enec_status enec_decompress_ranked(const void* d_in, size_t in_size, enec_dtype dt, size_t count, void* d_out,
                                    int* d_status, enec_stream_t stream) {
     return decompress_one(d_in, in_size, dt, count, d_out, d_status, stream, true);
+}
+
+// Blocks per chunk of a ticketed list (see DecodeBatch): two, or one when that leaves CTAs (three per SM) without a
+// second chunk.
+static uint32_t batched_chunk_blocks(uint64_t total_blocks) {
+    constexpr uint64_t kCtasOfALaunch = 148 * 3;
+    return total_blocks < 4 * kCtasOfALaunch ? 1u : 2u;
 }
 
 enec_status enec_decompress_batched(const enec_batch_item* h_items, int n_items, enec_dtype dt, int* d_status,
@@ -524,7 +531,7 @@ enec_status enec_decompress_batched(const enec_batch_item* h_items, int n_items,
             part.jobs = nullptr;
             part.prefix = nullptr;
             part.n_jobs = uint32_t(n);
-            part.blockwise = 0;
+            part.option = 0;
             part.total_blocks = prefix[first + n] - prefix[first];
             for (int i = 0; i < n; ++i) part.inline_jobs[i] = jobs[first + i];
             for (int i = 0; i <= n; ++i) part.inline_prefix[i] = prefix[first + i] - prefix[first];
@@ -535,7 +542,7 @@ enec_status enec_decompress_batched(const enec_batch_item* h_items, int n_items,
     }
     DecodeBatch batch;
     batch.n_jobs = uint32_t(n_items);
-    batch.blockwise = 0;
+    batch.option = 0;
     batch.total_blocks = uint32_t(total);
     bool ticketed = false;
     // A short list travels in the launch parameters: no copy, no scratch. Unless it has so many blocks that the
@@ -550,14 +557,16 @@ enec_status enec_decompress_batched(const enec_batch_item* h_items, int n_items,
         // the blocks of a long list are handed out in chunks: a zeroed ticket word and the tensor of every chunk's
         // first block travel with the descriptors
         const size_t ticket_at = host.size();
-        const size_t n_chunks = size_t((total + kTicketChunk - 1) / kTicketChunk);
+        const uint32_t chunk = batched_chunk_blocks(total);
+        batch.option = chunk;
+        const size_t n_chunks = size_t((total + chunk - 1) / chunk);
         host.resize(ticket_at + 16 + n_chunks * sizeof(uint32_t), 0);
         {
             const uint32_t* pre = reinterpret_cast<const uint32_t*>(host.data() + jobs_bytes);
             uint32_t* chunk_job = reinterpret_cast<uint32_t*>(host.data() + ticket_at + 16);
             uint32_t j = 0;
             for (size_t c = 0; c < n_chunks; ++c) {
-                const uint64_t first = uint64_t(c) * kTicketChunk;
+                const uint64_t first = uint64_t(c) * chunk;
                 while (pre[j + 1] <= first) ++j;  // tensors without blocks are skipped
                 chunk_job[c] = j;
             }

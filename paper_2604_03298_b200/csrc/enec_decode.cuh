@@ -666,11 +666,15 @@ constexpr uint32_t kInlineJobs = 16;  // tensors of a short batch that fit the k
 
 // A launch decodes the blocks of one tensor or of a list of tensors. Blocks of all tensors form one
 // index space; a CTA takes a contiguous range of it, so it changes tensor rarely. Long lists (the kernel instance
-// with TICKET) hand the index space out in chunks of kTicketChunk consecutive blocks instead: the CTAs of an SM
+// with TICKET) hand the index space out in chunks of a few consecutive blocks instead: the CTAs of an SM
 // progress unequally, and with a fixed share each the launch ends when the slowest has finished. Such a list's
 // device arrays are laid out as [jobs | prefix, padded to 16 bytes | ticket word, 16 bytes, zero at launch | the
 // tensor of every chunk's first block], so the kernel finds the last two behind the prefix.
-constexpr uint32_t kTicketChunk = 8;
+//
+// Blocks per chunk: two, and one when the list has fewer than two chunks per CTA. A launch's last round is a chunk
+// long, so long chunks leave CTAs idle: chunks of 8 / 4 / 2 / 1 blocks took 66 / 53 / 49 / 48 us for a list of 4352
+// blocks (139 MB of bf16), 757 / 744 / 727 / 785 us for one of 84992, 27 / 18 / 12 / 10 us for one of 212; single
+// blocks lose on long lists because the loader then looks up tensor and table entries for every block.
 constexpr uint32_t kSingleTicketChunk = 2;  // one large tensor: its blocks all cost the same, and a launch has few per CTA
 __host__ __device__ inline uint64_t ticket_offset_behind_prefix(uint32_t n_jobs) {
     return align16((uint64_t(n_jobs) + 1) * sizeof(uint32_t));
@@ -680,7 +684,7 @@ struct DecodeBatch {
     const uint32_t* prefix;   // device array [n_jobs + 1]: blocks before each tensor (null with jobs)
     uint32_t n_jobs;
     uint32_t total_blocks;
-    uint32_t blockwise;       // the streams are of the block-wise variant (one tensor only)
+    uint32_t option;          // one tensor: 1 = its stream is of the block-wise variant; TICKET = 1: blocks per chunk
     DecodeJob inline_jobs[kInlineJobs];          // used when jobs is null (one tensor, or a short list)
     uint32_t inline_prefix[kInlineJobs + 1];
 };
@@ -784,7 +788,7 @@ enec_decode_kernel(const __grid_constant__ DecodeBatch batch, int* status) {
         for (uint32_t q = threadIdx.x; q < batch.n_jobs; q += blockDim.x) {
             if (all_jobs[q].count == 0) {
                 JobCtx jc;
-                const int err = load_job<DT, MAPPED>(all_jobs[q], jc, batch.blockwise != 0);
+                const int err = load_job<DT, MAPPED>(all_jobs[q], jc, TICKET != 1 && batch.option != 0);
                 if (err) report(status, err);
             }
         }
@@ -806,7 +810,7 @@ enec_decode_kernel(const __grid_constant__ DecodeBatch batch, int* status) {
         // and the blocks of the chunk in hand that are issued
         [[maybe_unused]] uint32_t chunk = 0, next_chunk = 0, in_chunk = 0;
         [[maybe_unused]] uint32_t next_j = 0, next_first = 0, next_end = 0;  // the next chunk's tensor and its range of blocks
-        constexpr uint32_t kChunk = TICKET == 2 ? kSingleTicketChunk : kTicketChunk;
+        const uint32_t kChunk = TICKET == 2 ? kSingleTicketChunk : batch.option;
         [[maybe_unused]] const uint32_t n_chunks = TICKET ? (batch.total_blocks + kChunk - 1) / kChunk : 0;
         [[maybe_unused]] uint32_t* const ticket =
             TICKET == 1 ? reinterpret_cast<uint32_t*>(reinterpret_cast<uintptr_t>(batch.prefix) + ticket_offset_behind_prefix(batch.n_jobs))
@@ -899,7 +903,7 @@ enec_decode_kernel(const __grid_constant__ DecodeBatch batch, int* status) {
                     e0 = tb[k];
                     e1 = tb[k + 1];
                 }
-                const int err = early ? load_job<DT, MAPPED>(job, jc, batch.blockwise != 0) : ENEC_ERR_BAD_STREAM;
+                const int err = early ? load_job<DT, MAPPED>(job, jc, TICKET != 1 && batch.option != 0) : ENEC_ERR_BAD_STREAM;
                 if (err) {
                     *abort_flag = 1;
                     report(status, err);
