@@ -10,6 +10,7 @@
 #include "enec_decode.cuh"
 #include "enec_encode.cuh"
 #include "enec_blockwise.cuh"
+#include "enec_fused.cuh"
 #include "enec_launch.cuh"
 
 namespace enec {
@@ -23,6 +24,7 @@ struct DeviceInfo {
     bool batch_attr_set[3] = {false, false, false};
     bool blockwise_attr_set[3] = {false, false, false};
     bool split_attr_set[3] = {false, false, false};
+    bool fused_attr_set[3] = {false, false, false};
 };
 
 // Per-device facts, for device ordinals below kMaxDevices (null beyond: the caller fails with ENEC_ERR_CUDA).
@@ -46,11 +48,13 @@ static bool aligned16(const void* p) { return (reinterpret_cast<uintptr_t>(p) & 
 struct ScratchArea {
     uint8_t* ptr = nullptr;
     size_t bytes = 0;
+    uint64_t blocks = 0;      // one-kernel compressor: blocks the area is laid out for
+    uint32_t supers[2] = {0, 0};  // one-kernel compressor: first-level sums in use in either set
     uint32_t epoch = 0;       // compressor areas: number of the last call
     bool needs_clear = true;  // compressor areas: fresh memory, a wrapped epoch or a launch that failed
 };
 
-enum ScratchKind { kScratchCompress = 0, kScratchBatch = 1, kScratchCompressBatch = 2, kScratchBlockwise = 3, kScratchDecodeTicket = 4 };
+enum ScratchKind { kScratchCompress = 0, kScratchBatch = 1, kScratchCompressBatch = 2, kScratchBlockwise = 3, kScratchDecodeTicket = 4, kScratchFused = 5 };
 
 static std::mutex g_scratch_mu;
 static ScratchArea& scratch_area(int dev, cudaStream_t stream, ScratchKind kind) {
@@ -97,6 +101,49 @@ static enec_status lease_compress_scratch(int dev, cudaStream_t stream, size_t n
     return ENEC_OK;
 }
 
+// Scratch of the one-kernel compressor (see FusedControl), laid out for `blocks` blocks:
+// [two control sets | two sets of first-level sums for two passes | a state word per block].
+static size_t fused_scratch_bytes(uint64_t blocks) {
+    return 2 * kFusedControlBytes + (4 * (blocks / kSuperBlocks) + blocks) * sizeof(unsigned long long);
+}
+static enec_status lease_fused_scratch(int dev, cudaStream_t stream, uint32_t nblocks, FusedJob& job) {
+    std::lock_guard<std::mutex> lock(g_scratch_mu);
+    ScratchArea& a = scratch_area(dev, stream, kScratchFused);
+    uint64_t blocks = a.blocks ? a.blocks : 4096;
+    while (blocks < nblocks) blocks *= 2;
+    const enec_status st = grow(a, fused_scratch_bytes(blocks));
+    if (st != ENEC_OK) return st;
+    if (blocks != a.blocks) {   // another layout
+        a.blocks = blocks;
+        a.needs_clear = true;
+    }
+    if (a.needs_clear || a.epoch > 0xFFFFFFF0u) {
+        if (cudaMemsetAsync(a.ptr, 0, a.bytes, stream) != cudaSuccess) return ENEC_ERR_CUDA;
+        a.needs_clear = false;
+        a.epoch = 0;
+        a.supers[0] = a.supers[1] = 0;
+    }
+    a.epoch += 2;  // one for each pass of the call
+    const uint32_t set = (a.epoch >> 1) & 1, other = set ^ 1;
+    unsigned long long* sums = reinterpret_cast<unsigned long long*>(a.ptr + 2 * kFusedControlBytes);
+    job.super_stride = uint32_t(blocks / kSuperBlocks);
+    job.ctl = reinterpret_cast<FusedControl*>(a.ptr + set * kFusedControlBytes);
+    job.ctl_next = reinterpret_cast<FusedControl*>(a.ptr + other * kFusedControlBytes);
+    job.super = sums + size_t(set) * 2 * job.super_stride;
+    job.super_next = sums + size_t(other) * 2 * job.super_stride;
+    job.clear_supers = a.supers[other];
+    job.state = sums + size_t(4) * job.super_stride;
+    job.epoch = a.epoch;
+    a.supers[other] = 0;
+    a.supers[set] = (nblocks + kSuperBlocks - 1) / kSuperBlocks;
+    return ENEC_OK;
+}
+
+static void mark_scratch_unclean(int dev, cudaStream_t stream, ScratchKind kind) {
+    std::lock_guard<std::mutex> lock(g_scratch_mu);
+    scratch_area(dev, stream, kind).needs_clear = true;
+}
+
 static void mark_compress_scratch_unclean(int dev, cudaStream_t stream) {
     std::lock_guard<std::mutex> lock(g_scratch_mu);
     scratch_area(dev, stream, kScratchCompress).needs_clear = true;
@@ -110,10 +157,11 @@ static void place_job(EncodeJob& job, uint8_t* scratch, uint32_t epoch) {
     job.epoch = epoch;
 }
 
-// Tensors of split_min_blocks() .. split_max_blocks() - 1 blocks are compressed in the split form (pack kernel, then
-// the kernel that places the records). Below that range the third launch costs more than the look-back it replaces;
-// there is no upper bound by default. ENEC_SPLIT_MIN_BLOCKS and ENEC_SPLIT_MAX_BLOCKS in the environment override
-// the bounds (read once; for measurements and tests).
+// enec_compress takes the one-kernel form (enec_fused.cuh) for every tensor. With ENEC_SPLIT_MIN_BLOCKS in the environment
+// (read once; for measurements and tests) it takes the forms before that: tensors of split_min_blocks() ..
+// split_max_blocks() - 1 blocks the split form (histogram, pack kernel, then the kernel that places the records), others
+// histogram and look-back kernel. One kernel against those: 4096 values 8.4 against 11.0 us, 256 blocks 14.3 / 22.5,
+// 1024 blocks 28.5 / 35.1, 3584 blocks 58 / 87, 27000 blocks 325 / 520 (bf16, in a stream).
 static uint32_t env_blocks(const char* name, uint32_t fallback) {
     const char* e = getenv(name);
     return e && *e ? uint32_t(strtoul(e, nullptr, 10)) : fallback;
@@ -124,6 +172,11 @@ static uint32_t split_min_blocks() {
 }
 static uint32_t split_max_blocks() {
     static const uint32_t value = env_blocks("ENEC_SPLIT_MAX_BLOCKS", 0xFFFFFFFFu);
+    return value;
+}
+
+static bool earlier_forms() {
+    static const bool value = getenv("ENEC_SPLIT_MIN_BLOCKS") != nullptr;
     return value;
 }
 
@@ -257,6 +310,18 @@ static enec_status compress_common(const void* d_in, enec_dtype dt, size_t count
     cudaStreamCaptureStatus capturing = cudaStreamCaptureStatusNone;
     if (cudaStreamIsCapturing(stream, &capturing) != cudaSuccess) return ENEC_ERR_CUDA;
     if (capturing != cudaStreamCaptureStatusNone) return ENEC_ERR_INVALID_ARG;
+    if (!with_params && !ranked && !earlier_forms()) {
+        FusedJob fused;
+        enec_status fst = lease_fused_scratch(dev, stream, g.nblocks, fused);
+        if (fst != ENEC_OK) return fst;
+        fused.in = static_cast<const uint8_t*>(d_in);
+        fused.out = static_cast<uint8_t*>(d_out);
+        fused.count = count;
+        fused.out_size = out_size;
+        fst = launch_fused(int(dt), fused, g.nblocks, info.sms, info.fused_attr_set, d_status, stream);
+        if (fst != ENEC_OK) mark_scratch_unclean(dev, stream, kScratchFused);
+        return fst;
+    }
     uint8_t* scratch = nullptr;
     uint32_t epoch = 0;
     enec_status st = lease_compress_scratch(dev, stream, need, &scratch, &epoch);

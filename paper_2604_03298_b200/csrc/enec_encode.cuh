@@ -1316,7 +1316,7 @@ enec_encode_kernel(const EncodeJob single, const EncodeBatch batch, int* status)
 
 // Stream of an empty tensor: header, (frequency-rank variant: an all-zero rank table) and a one-entry table
 // (16 zero bytes in every variant).
-__global__ void enec_encode_empty_kernel(uint8_t* out, int dt, int b, int n, int m, unsigned long long* out_size,
+static __global__ void enec_encode_empty_kernel(uint8_t* out, int dt, int b, int n, int m, unsigned long long* out_size,
                                          int variant = 0) {
     if (threadIdx.x != 0 || blockIdx.x != 0) return;
     const uint32_t table_at = kHeaderBytes + (variant == 1 ? kRankTableBytes : 0);

@@ -1,0 +1,1332 @@
+// enec_compress in one kernel (Sec. 5.1 compression flow with the parameter choice of Sec. 5.5).
+//
+// enec_fused_kernel, four CTAs of 256 threads per SM, blocks of 16384 elements handed out by tickets:
+//   1. Sample stage: the histogram of a sample of the tensor's blocks, spread over it (every block of a small tensor). When
+//      the last sampled block is counted, its CTA runs the search of Sec. 5.5 and publishes (b, n, m).
+//   2. Pack stage: split, transform (Sec. 5.3), group widths (Sec. 5.2), Algorithm 2, and the histogram of every block.
+//      The input is read once, apart from the sample.
+//   3. The CTA that ends last runs the search again, on the histogram of the whole tensor. When it gives the parameters
+//      that were used, the stream is the one that the search on the whole tensor leads to. When it does not, the CTAs pack
+//      the tensor again; a value that the sampled parameters cannot represent ends the pack stage at once, and the blocks
+//      not packed yet are counted first.
+// A tensor whose sample needs n > 6 exponent bits (bf16, fp32) takes the histogram of the whole tensor before it packs:
+// the table kept beside the packing has 64 rows, and rare outliers of such a tensor are what a sample misses.
+//
+// Block offsets (the prefix sum of Sec. 5.1 / 5.4): every block's count of wide groups goes to a state word and is added
+// to a sum per 128 blocks and a sum per 16384 blocks. A CTA keeps a block's packed records in shared memory while it
+// packs its next block; by then all blocks handed out before have been counted as a rule, so one warp finds the block's
+// offset with one round of loads and copies the records to their place.
+//
+// A wait concerns only work whose tickets were handed out before, hence running CTAs, and in the pack stage only blocks
+// with smaller numbers: the CTA with the smallest block that is not counted yet waits for nobody. Every wait is bounded
+// all the same and ends in ENEC_ERR_TIMEOUT.
+#pragma once
+
+#include "enec_pack.cuh"
+
+namespace enec {
+
+constexpr int kFusedThreads = 256;
+constexpr int kFusedWarps = kFusedThreads / 32;
+constexpr uint32_t kSuperBlocks = 128;     // blocks per first-level sum
+constexpr uint32_t kHyperSupers = 128;     // first-level sums per second-level sum
+constexpr uint32_t kMaxHypers = 256;       // 2^36 values
+
+// Control words of a call. The sums and the pack stage's ticket are kept per pass over the tensor (the second pass happens
+// only when the sampled parameters were not the tensor's). Words that many CTAs add to lie on lines of their own: adds to
+// one line are served one after another, about 3.6 ns each.
+struct alignas(128) Counter { uint32_t value; uint32_t pad[31]; };
+struct alignas(128) FusedControl {
+    unsigned long long hist[2][256];             // of the sample, of the whole tensor but for what is in pack_hist
+    unsigned long long pack_hist[256];           // of the pack stage
+    unsigned long long hyper[2][kMaxHypers];     // bits 63..32 blocks counted, bits 31..0 their wide groups
+    Counter hist_ticket[2], hist_done[2];
+    Counter pack_ticket[2];
+    Counter pack_done;         // blocks packed by the CTAs that have left the first pass
+    uint32_t pack_target;      // blocks handed out before the first pass was ended early (0: it was not)
+    uint32_t params[2];        // published: the parameters for hist[0], hist[1]
+    uint32_t verdict;          // published: the whole tensor's parameters, when the first pass has packed every block
+};
+constexpr uint32_t kFusedControlBytes = 16384;
+static_assert(sizeof(FusedControl) <= kFusedControlBytes, "a control set fits its slot");
+constexpr uint32_t kParamsValid = 1u << 31;   // a published word: b | n << 8 | m << 12 | valid
+constexpr uint32_t kParamsRedo = 1u << 28;    // verdict: some packed blocks held values that the sampled parameters lose
+constexpr uint32_t kParamsTake = 1u << 29;    // not a published word: there is a ticket to take
+constexpr uint32_t kPassEnded = 1u << 30;     // pack_ticket: no further blocks in this pass
+
+struct FusedJob {
+    const uint8_t* in;
+    uint8_t* out;
+    uint64_t count;
+    FusedControl* ctl;             // zero when the call starts
+    FusedControl* ctl_next;        // the next call's set, zeroed by this call ...
+    unsigned long long* super;     // first-level sums, two passes of super_stride words; zero when the call starts
+    unsigned long long* super_next;
+    uint32_t super_stride;
+    uint32_t clear_supers;         // ... with so many first-level sums per pass
+    uint32_t sample;               // blocks in the sample (nblocks: all)
+    uint32_t epoch;                // tag of the first pass's state words; the second pass's is one more
+    unsigned long long* state;     // per block: bits 63..32 epoch, bits 31..0 wide groups
+    unsigned long long* out_size;  // device, may be null
+};
+
+template <int DT>
+struct FusedShape {
+    static constexpr int E = HistShape<DT>::E;
+    static constexpr int kCtasPerSm = 3;
+    static constexpr uint32_t kWork = 32768;                           // low plane | fp16 plane | the block's values
+    static constexpr uint32_t kRows = DT == ENEC_FP16 ? 32 : 64;       // rows of the pack stage's histogram
+    static constexpr uint32_t kHistAt = kWork;
+    static constexpr uint32_t kHistBytes = kRows * HistShape<DT>::kRowBytes;
+    static constexpr uint32_t kListAt = kHistAt + kHistBytes;          // the wide groups' numbers, a byte each, by warp
+    static constexpr uint32_t kPend = 4096;                            // a block's packed records waiting for their offset
+    static constexpr uint32_t kPendAt = kListAt + 1024;
+    static constexpr uint32_t kTensorAt = kPendAt + 2 * kPend;         // FusedTensor
+    static constexpr uint32_t kSharedAt = kTensorAt + 256;             // FusedShared
+    static constexpr uint32_t kBytes = kSharedAt + 256;
+    static_assert(HistShape<DT>::kBytes <= int(kHistAt + kHistBytes), "the sample stage's table fits");
+    static_assert(kCtasPerSm * (kBytes + 1024) <= 228 * 1024, "the CTAs of an SM fit its shared memory");
+};
+
+// What a block of the pack stage needs to know about its tensor, in shared memory.
+//
+// The stage works with v = y ^ 2^(n-1) = b + 2^(n-1) - x (mod 2^n), one value per byte. PLAIN: 2^n <= b + 2^(n-1) <= 255
+// (fp16: always), so that the difference of a representable exponent neither borrows nor leaves n bits, and a word
+// pair takes two multiply-adds and a byte permutation; a value that is not representable shows as a bit above n.
+struct FusedTensor {
+    const uint8_t* in;
+    uint8_t* out;
+    uint8_t *sm, *lo, *low, *smhi, *mask, *high;   // the sections' first bytes
+    uint32_t* table;
+    unsigned long long* state;
+    unsigned long long* super;
+    unsigned long long* hyper;
+    uint64_t count;
+    uint64_t smhi_bytes, sm_bytes, lo_bytes;       // the sections' lengths
+    unsigned long long* out_size;
+    uint32_t nblocks, tail_real, tail_padded, total_groups;
+    uint32_t epoch;
+    int b, n, m, hbits;
+    uint32_t c;        // the minuend: bf16 (b + 2^(n-1)) << 8 | 255 in both halves; fp16 and the general form: per byte
+    uint32_t s4;       // 2^(n-1) in every byte
+    uint32_t nmask4;   // 2^n - 1 in every byte
+    uint32_t wide4;    // bits m .. n - 1 in every byte
+    uint32_t pad;      // two 16-bit words with exponent b and nothing else: y = 0
+    uint32_t wide_ok;  // bit 0: the input is 32-byte aligned, bit 1: the sm-lo plane is
+    uint32_t plain;
+    uint32_t smhi_at, values_at;   // shared memory: where the fp16 plane and the values start
+};
+
+struct FusedShared {
+    uint32_t mask[32];
+    uint32_t next;       // the CTA's next ticket
+    uint32_t word;       // broadcasts of thread 0
+    uint32_t before;
+    uint32_t ok;
+    uint32_t part[kFusedWarps];   // each warp's share of the wide groups before the waiting block; kNotReady: some are not counted yet
+};
+constexpr uint32_t kNotReady = 0xFFFFFFFFu;   // a tensor has at most 2^32 - 2^10 groups of 16 counted before a block
+static_assert(sizeof(FusedTensor) <= 256 && sizeof(FusedShared) <= 256, "they fit their places");
+
+__device__ __forceinline__ uint8_t* fused_smem() {
+    extern __shared__ __align__(128) uint8_t smem[];
+    return smem;
+}
+template <int DT>
+__device__ __forceinline__ FusedTensor& fused_tensor() { return *reinterpret_cast<FusedTensor*>(fused_smem() + FusedShape<DT>::kTensorAt); }
+template <int DT>
+__device__ __forceinline__ FusedShared& fused_shared() { return *reinterpret_cast<FusedShared*>(fused_smem() + FusedShape<DT>::kSharedAt); }
+
+template <int DT>
+__device__ __forceinline__ bool plain_form(int b, int n) {
+    return DT == ENEC_FP16 || (b + (1 << (n - 1)) <= 255 && (1 << n) <= b + (1 << (n - 1)));
+}
+// Whether the pack stage can keep the histogram: representable exponents are told apart by their low six bits.
+template <int DT>
+__device__ __forceinline__ bool sample_will_do(uint32_t word) {
+    const int b = int(word & 0xFF), n = int((word >> 8) & 0xF);
+    return DT == ENEC_FP16 || (n <= 6 && plain_form<DT>(b, n));
+}
+
+// A tensor's context but for what follows from (b, n, m). One thread.
+template <int DT>
+__device__ inline void set_geometry(FusedTensor& t) {
+    const Geometry g = make_geometry(t.count);
+    const Sections sec = make_sections(DT, t.count, g, 1, 1, 0);
+    t.nblocks = g.nblocks; t.tail_real = g.tail_real; t.tail_padded = g.tail_padded; t.total_groups = g.total_groups;
+    t.table = reinterpret_cast<uint32_t*>(t.out + sec.table);
+    t.mask = t.out + sec.mask;
+    t.low = t.out + sec.low;
+    t.smhi_bytes = sec.sm - sec.smhi;
+    t.sm_bytes = sec.smlo - sec.sm;
+    t.lo_bytes = sec.high - sec.smlo;
+}
+// The rest. One thread.
+template <int DT>
+__device__ inline void set_parameters(FusedTensor& t, uint32_t word) {
+    const int b = int(word & 0xFF), n = int((word >> 8) & 0xF), m = int((word >> 12) & 0xF);
+    t.b = b; t.n = n; t.m = m; t.hbits = n - m;
+    const uint32_t d = uint32_t(b) + (1u << (n - 1));
+    t.plain = plain_form<DT>(b, n);
+    if (DT == ENEC_FP16) t.c = rep4(d + 64);   // the guard bit 6 keeps the bytes apart; bits 4..0 are the difference mod 32
+    else t.c = t.plain ? ((d & 0xFF) << 8 | 0xFFu) * 0x00010001u : rep4(d);
+    t.s4 = rep4(1u << (n - 1));
+    t.nmask4 = rep4((1u << n) - 1);
+    t.wide4 = rep4((0xFFu << m) & ((1u << n) - 1));
+    t.pad = (DT == ENEC_FP16 ? uint32_t(b) << 10 : uint32_t(b) << 7) * 0x00010001u;
+    t.smhi = t.low + align16((uint64_t(t.nblocks - 1) * kBlockElems + t.tail_padded) * uint32_t(m) / 8);
+    t.sm = t.smhi + t.smhi_bytes;
+    t.lo = t.sm + t.sm_bytes;
+    t.high = t.lo + t.lo_bytes;
+    t.wide_ok = ((reinterpret_cast<uintptr_t>(t.in) & 31) == 0 ? 1u : 0u) | ((reinterpret_cast<uintptr_t>(t.lo) & 31) == 0 ? 2u : 0u);
+    t.smhi_at = (kBlockElems / 8) * uint32_t(m);
+    t.values_at = t.smhi_at + (DT == ENEC_FP16 ? kBlockElems * 3 / 8 : 0);
+}
+
+// Eq. 1 as width_eq1, the bit widths by counting leading zeros.
+__device__ __forceinline__ int width_of_range(int b, int l, int h, int E) {
+    const int pos = 32 - __clz(b - l);
+    const int neg = h - b <= 1 ? 0 : 32 - __clz(h - b - 1);
+    return min(max(pos, neg) + 1, E);
+}
+
+// ---- parameter search by one warp ------------------------------------------------------------------
+// Sec. 5.5 phases 2 and 3 on a finished histogram. With C(x) = number of values with exponents up to x, N = all of them,
+// S = sum of the exponents: for a candidate b of width n (Eq. 1) the values stored are b - x for x <= b and 2^n + b - x
+// above, so Eq. 3's cost times N is N b - S + 2^n (N - C(b)), and the values below 2^m number
+// C(b) - C(b - 2^m) + N - C(b + 2^n - 2^m): every candidate is a few table look-ups.
+// `count_of(x)` gives the histogram; `table`: 256 words of shared memory. Returns b | n << 8 | m << 12 in every lane.
+template <int DT, class CountOf>
+__device__ __forceinline__ uint32_t search_by_warp(CountOf count_of, unsigned long long* table) {
+    constexpr int E = HistShape<DT>::E;
+    constexpr int kPer = (1 << E) / 32;
+    constexpr uint32_t kAll = 0xFFFFFFFFu;
+    const int lane = int(threadIdx.x & 31);
+    unsigned long long c[kPer];
+    unsigned long long sum = 0, weighted = 0;
+    int lo = 1 << E, hi = -1;
+#pragma unroll
+    for (int i = 0; i < kPer; ++i) c[i] = count_of(lane * kPer + i);
+#pragma unroll
+    for (int i = 0; i < kPer; ++i) {
+        const int x = lane * kPer + i;
+        if (c[i]) { lo = min(lo, x); hi = x; }
+        sum += c[i];
+        weighted += c[i] * (unsigned long long)x;
+    }
+    const int l = __reduce_min_sync(kAll, lo), h = __reduce_max_sync(kAll, hi);
+    // 44 bits at most: the sum of 32 words in two halves
+    const unsigned long long S = __reduce_add_sync(kAll, uint32_t(weighted & 0x3FFFFFFu)) +
+                                 ((unsigned long long)__reduce_add_sync(kAll, uint32_t(weighted >> 26)) << 26);
+    unsigned long long incl = sum;
+#pragma unroll
+    for (int d = 1; d < 32; d <<= 1) {
+        const unsigned long long t = __shfl_up_sync(kAll, incl, d);
+        if (lane >= d) incl += t;
+    }
+    unsigned long long run = incl - sum;
+#pragma unroll
+    for (int i = 0; i < kPer; ++i) {
+        run += c[i];
+        table[lane * kPer + i] = run;
+    }
+    const unsigned long long total = __shfl_sync(kAll, incl, 31);
+    __syncwarp();
+    // the smallest of the lanes' 64-bit words, in two halves
+    auto smallest = [&](unsigned long long v) -> unsigned long long {
+        const uint32_t high = __reduce_min_sync(kAll, uint32_t(v >> 32));
+        const uint32_t low = __reduce_min_sync(kAll, uint32_t(v >> 32) == high ? uint32_t(v) : kAll);
+        return (unsigned long long)high << 32 | low;
+    };
+    unsigned long long key = ~0ull;
+    for (int b = l + lane; b <= h; b += 32) {
+        const int n = width_of_range(b, l, h, E);
+        const unsigned long long cost = total * (unsigned long long)b - S + ((total - table[b]) << n);
+        const unsigned long long mine = (cost << 12) | (unsigned long long)(n << 8) | (unsigned long long)b;  // cost < 2^44
+        key = mine < key ? mine : key;
+    }
+    key = smallest(key);
+    const int b = int(key & 0xFF), n = int((key >> 8) & 0xF);
+    // Eq. 4 at L = 16, lane m - 1 evaluates m: plain IEEE double, one rounding per operation; ties go to the smaller m
+    const int m = lane < n ? lane + 1 : n;
+    auto upto = [&](int x) { return x < 0 ? 0ull : x >= (1 << E) ? total : table[x]; };
+    const unsigned long long cnt = upto(b) - upto(b - (1 << m)) + total - upto(b + (1 << n) - (1 << m));
+    const double p = __ddiv_rn(__ull2double_rn(cnt), __ull2double_rn(total));
+    const double p2 = __dmul_rn(p, p), p4 = __dmul_rn(p2, p2), p8 = __dmul_rn(p4, p4), p16 = __dmul_rn(p8, p8);
+    const double bits = __dadd_rn(__dadd_rn(double(n), 0.0625), __dmul_rn(double(m - n), p16));
+    // positive numbers: their bit patterns are ordered as they are
+    const unsigned long long pattern = (unsigned long long)__double_as_longlong(bits);
+    const uint32_t winners = __ballot_sync(kAll, pattern == smallest(pattern));
+    __syncwarp();
+    return uint32_t(b) | (uint32_t(n) << 8) | (uint32_t(__ffs(winners)) << 12);
+}
+
+// The search on the sum of one or two histograms in global memory.
+template <int DT>
+__device__ __noinline__ uint32_t search_global(const unsigned long long* hist, const unsigned long long* more, unsigned long long* table) {
+    return search_by_warp<DT>([&](int x) { return ld_relaxed_u64(&hist[x]) + (more ? ld_relaxed_u64(&more[x]) : 0ull); }, table);
+}
+
+// ---- loads -------------------------------------------------------------------------------------------
+struct Run { uint32_t w[8]; };  // sixteen 16-bit words in element order
+
+// 32 bytes at p: one access where p is 32-byte aligned (WIDE), two of 16 bytes else. (Two bodies and a branch around a batch
+// of them, not two predicated loads: a predicated load keeps its registers occupied long before it.)
+template <bool WIDE>
+__device__ __forceinline__ Run load32(const uint8_t* p) {
+    Run r;
+    if constexpr (WIDE)
+        asm volatile("ld.global.cs.v8.b32 {%0, %1, %2, %3, %4, %5, %6, %7}, [%8];"
+                     : "=r"(r.w[0]), "=r"(r.w[1]), "=r"(r.w[2]), "=r"(r.w[3]), "=r"(r.w[4]), "=r"(r.w[5]), "=r"(r.w[6]), "=r"(r.w[7])
+                     : "l"(p));
+    else
+        asm volatile("ld.global.cs.v4.b32 {%0, %1, %2, %3}, [%8];\n\tld.global.cs.v4.b32 {%4, %5, %6, %7}, [%8+16];"
+                     : "=r"(r.w[0]), "=r"(r.w[1]), "=r"(r.w[2]), "=r"(r.w[3]), "=r"(r.w[4]), "=r"(r.w[5]), "=r"(r.w[6]), "=r"(r.w[7])
+                     : "l"(p));
+    return r;
+}
+__device__ __forceinline__ void store32(uint8_t* p, const Run& r, bool wide) {
+    if (wide) {
+        asm volatile("st.global.cs.v8.b32 [%8], {%0, %1, %2, %3, %4, %5, %6, %7};" ::"r"(r.w[0]), "r"(r.w[1]), "r"(r.w[2]), "r"(r.w[3]),
+                     "r"(r.w[4]), "r"(r.w[5]), "r"(r.w[6]), "r"(r.w[7]), "l"(p)
+                     : "memory");
+    } else {
+        __stcs(reinterpret_cast<uint4*>(p), make_uint4(r.w[0], r.w[1], r.w[2], r.w[3]));
+        __stcs(reinterpret_cast<uint4*>(p) + 1, make_uint4(r.w[4], r.w[5], r.w[6], r.w[7]));
+    }
+}
+
+// fp32: the high halves of sixteen values (the first eight in a, the others in b); their low halves go to `lo` (32 bytes).
+__device__ __forceinline__ Run split_halves(const Run& a, const Run& b, uint8_t* lo, bool wide) {
+    Run h, l;
+#pragma unroll
+    for (int i = 0; i < 4; ++i) {
+        h.w[i] = prmt(a.w[2 * i], a.w[2 * i + 1], 0x7632u);
+        h.w[4 + i] = prmt(b.w[2 * i], b.w[2 * i + 1], 0x7632u);
+        l.w[i] = prmt(a.w[2 * i], a.w[2 * i + 1], 0x5410u);
+        l.w[4 + i] = prmt(b.w[2 * i], b.w[2 * i + 1], 0x5410u);
+    }
+    store32(lo, l, wide);
+    return h;
+}
+
+// The run of a tail block: values from element `real` on (counted from the run's first) are padding. fp32: zeros behind
+// the low halves up to the plane's 16-byte boundary, `lo_room` more halves.
+template <int DT>
+__device__ __forceinline__ Run load_run_tail(const uint8_t* in, uint8_t* lo, int real, int lo_room, uint32_t pad) {
+    Run r;
+#pragma unroll
+    for (int i = 0; i < 8; ++i) {
+        uint32_t half[2];
+#pragma unroll
+        for (int q = 0; q < 2; ++q) {
+            const int e = 2 * i + q;
+            half[q] = pad & 0xFFFFu;
+            if constexpr (DT == ENEC_FP32) {
+                uint32_t full = 0;
+                if (e < real) { full = reinterpret_cast<const uint32_t*>(in)[e]; half[q] = full >> 16; }
+                if (e < lo_room) reinterpret_cast<uint16_t*>(lo)[e] = uint16_t(full);
+            } else {
+                if (e < real) half[q] = reinterpret_cast<const uint16_t*>(in)[e];
+            }
+        }
+        r.w[i] = half[0] | (half[1] << 16);
+    }
+    return r;
+}
+
+// ---- one run: transform, sign/mantissa, histogram -------------------------------------------------------
+// hist: the pack stage's table; lane4: four times the lane, the lane's column.
+template <int DT>
+__device__ __forceinline__ void count_halves(uint32_t hist, uint32_t lane4, uint32_t w) {
+    if constexpr (DT == ENEC_FP16) {
+        red_add_one(hist + (((w >> 3) & 0xF80u) | lane4));
+        red_add_one(hist + (((w >> 19) & 0xF80u) | lane4));
+    } else {
+        red_add_one(hist + ((w & 0x1F80u) | lane4));
+        red_add_one(hist + (((w >> 16) & 0x1F80u) | lane4));
+    }
+}
+
+template <int DT, bool PLAIN, bool HIST>
+__device__ __forceinline__ void transform_run(const Run& r, uint32_t minuend, uint32_t nmask4, uint32_t hist, uint32_t lane4, uint4& v,
+                                              uint4& hs, uint4& sm) {
+    uint32_t vv[4], ss[4], hh[4];
+#pragma unroll
+    for (int q = 0; q < 4; ++q) {
+        const uint32_t w0 = r.w[2 * q], w1 = r.w[2 * q + 1];
+        const uint32_t lo = prmt(w0, w1, 0x6420u), hi = prmt(w0, w1, 0x7531u);
+        if constexpr (DT == ENEC_FP16) {
+            vv[q] = minuend - ((hi >> 2) & 0x1F1F1F1Fu);
+            ss[q] = lo;
+            hh[q] = (hi & 0x03030303u) | ((hi >> 5) & 0x04040404u);
+        } else {
+            ss[q] = (hi & 0x80808080u) | (lo & 0x7F7F7F7Fu);
+            hh[q] = 0;
+            if constexpr (PLAIN) {
+                vv[q] = prmt(minuend - 2 * w0, minuend - 2 * w1, 0x7531u);
+            } else {
+                const uint32_t x = prmt(2 * w0, 2 * w1, 0x7531u);
+                vv[q] = (((minuend | 0x80808080u) - (x & 0x7F7F7F7Fu)) ^ ((minuend ^ ~x) & 0x80808080u)) & nmask4;
+            }
+        }
+        if constexpr (HIST) {
+            count_halves<DT>(hist, lane4, w0);
+            count_halves<DT>(hist, lane4, w1);
+        }
+    }
+    v = make_uint4(vv[0], vv[1], vv[2], vv[3]);
+    sm = make_uint4(ss[0], ss[1], ss[2], ss[3]);
+    hs = make_uint4(hh[0], hh[1], hh[2], hh[3]);
+}
+
+__device__ __forceinline__ uint32_t or_flipped(const uint4& v, uint32_t s4) {
+    return (v.x ^ s4) | (v.y ^ s4) | (v.z ^ s4) | (v.w ^ s4);
+}
+
+// ---- Algorithm 2 on packed bytes ---------------------------------------------------------------------
+// As pack_plane_level (a thread owns eight consecutive lanes of the deepest level), for fields that need not be clean:
+// bits above a field are masked away where it is inserted.
+template <int W>
+__device__ __forceinline__ void insert_field(uint32_t& lo, uint32_t& hi, uint32_t v, int s) {
+    constexpr uint32_t kField = (1u << W) - 1;
+    if (s + W <= 8) {
+        const uint32_t mask = rep4(kField << s);
+        lo = (lo & ~mask) | ((v << s) & mask);
+    } else if (s >= 8) {
+        const uint32_t mask = rep4(kField << (s - 8));
+        hi = (hi & ~mask) | ((v << (s - 8)) & mask);
+    } else {
+        const uint32_t mask_lo = rep4(0xFFu << s), mask_hi = rep4(kField >> (8 - s));
+        lo = (lo & ~mask_lo) | ((v << s) & mask_lo);
+        hi = (hi & ~mask_hi) | ((v >> (8 - s)) & mask_hi);
+    }
+}
+
+template <int W_IN, int LOG_UNITS>
+__device__ __forceinline__ void pack_lanes_level(uint32_t S, uint32_t nb_off, uint32_t j, uint32_t n8, const uint2 (&in)[1 << LOG_UNITS]) {
+    constexpr int F = folds_for(W_IN);
+    static_assert(F <= LOG_UNITS, "lane runs must stay whole");
+    constexpr int W = W_IN << F;
+    constexpr int LOG_LANES = LOG_UNITS - F;
+    constexpr int NL = 1 << LOG_LANES;
+    constexpr int RES = W - 8;
+    uint2 R[NL];
+#pragma unroll
+    for (int c = 0; c < NL; ++c) {
+        uint2 V = make_uint2(0, 0);
+        R[c] = make_uint2(0, 0);
+#pragma unroll
+        for (int q = 0; q < (1 << F); ++q) {
+            const int e = c + q * NL;
+            const int s = W_IN * bitrev(q, F);
+            insert_field<W_IN>(V.x, R[c].x, in[e].x, s);
+            insert_field<W_IN>(V.y, R[c].y, in[e].y, s);
+        }
+        sts64(S + nb_off + j + c * n8, V);
+    }
+    if constexpr (RES > 0) pack_lanes_level<RES, LOG_LANES>(S, nb_off + NL * n8, j, n8, R);
+}
+
+template <int DT>
+__device__ __forceinline__ void pack_lanes_any(int m, uint32_t S, uint32_t j, uint32_t n8, const uint2 (&v)[8]) {
+    switch (m) {
+        case 1: pack_lanes_level<1, 3>(S, 0, j, n8, v); break;
+        case 2: pack_lanes_level<2, 3>(S, 0, j, n8, v); break;
+        case 3: pack_lanes_level<3, 3>(S, 0, j, n8, v); break;
+        case 4: pack_lanes_level<4, 3>(S, 0, j, n8, v); break;
+        case 5: pack_lanes_level<5, 3>(S, 0, j, n8, v); break;
+        case 6: if constexpr (DT != ENEC_FP16) pack_lanes_level<6, 3>(S, 0, j, n8, v); break;
+        case 7: if constexpr (DT != ENEC_FP16) pack_lanes_level<7, 3>(S, 0, j, n8, v); break;
+        default: if constexpr (DT != ENEC_FP16) pack_lanes_level<8, 3>(S, 0, j, n8, v); break;
+    }
+}
+
+// The low plane (and the fp16 plane) of a block of N >= 128 elements from its values in shared memory, in the order before
+// the final fold; all threads.
+template <int DT>
+__device__ __forceinline__ void pack_planes(const FusedTensor& t, uint32_t work, uint32_t N, uint32_t tid) {
+    const uint32_t j = 8 * tid, n8 = N >> 3;
+    if (j >= n8) return;
+    const uint32_t values = work + t.values_at, s4 = t.s4;
+    uint2 v[8];
+#pragma unroll
+    for (int c = 0; c < 8; ++c) v[c] = lds64(values + c * n8 + j);
+    if (t.hbits == 0) {   // bit n - 1, flipped in v, belongs to the low plane
+#pragma unroll
+        for (int c = 0; c < 8; ++c) v[c] = make_uint2(v[c].x ^ s4, v[c].y ^ s4);
+    }
+    pack_lanes_any<DT>(t.m, work, j, n8, v);
+    if constexpr (DT == ENEC_FP16) {
+#pragma unroll
+        for (int c = 0; c < 8; ++c) v[c] = make_uint2(v[c].x >> 5, v[c].y >> 5);
+        pack_lanes_level<3, 3>(work + t.smhi_at, 0, j, n8, v);
+    }
+}
+
+// The final fold (see fold_plane_out), all threads.
+__device__ __forceinline__ void fold_out(uint32_t S, uint32_t T, uint8_t* dst, uint32_t tid) {
+    const uint32_t thalf = T >> 1;
+    for (uint32_t u = tid; u < (thalf >> 3); u += kFusedThreads) {
+        const uint2 lo = lds64(S + 8 * u), hi = lds64(S + thalf + 8 * u);
+        uint4 w;
+        w.x = prmt(lo.x, hi.x, 0x5140u);
+        w.y = prmt(lo.x, hi.x, 0x7362u);
+        w.z = prmt(lo.y, hi.y, 0x5140u);
+        w.w = prmt(lo.y, hi.y, 0x7362u);
+        __stcs(reinterpret_cast<uint4*>(dst + 16 * u), w);
+    }
+}
+
+// A wide group's record: Algorithm 2 with N = 16 on packed bytes, four lanes per 32-bit word. in: LANES fields of W_IN bits
+// (four per word; two lanes sit in the low half of a word). The normalised bytes of the level go to nb from byte NB on.
+template <int W_IN, int LANES, int NB, int NW>
+__device__ __forceinline__ void record_level(const uint32_t (&in)[(LANES + 3) / 4], uint32_t (&nb)[NW]) {
+    constexpr int F = folds_for(W_IN);
+    constexpr int W = W_IN << F;
+    constexpr int OUT = LANES >> F;      // lanes after the folds
+    static_assert(OUT >= 2, "a record's lanes fold down to two at least");
+    constexpr int RES = W - 8;
+    constexpr int NV = (OUT + 3) / 4;
+    uint32_t V[NV], R[NV];
+#pragma unroll
+    for (int c = 0; c < NV; ++c) {
+        V[c] = R[c] = 0;
+#pragma unroll
+        for (int q = 0; q < (1 << F); ++q) {
+            // the OUT lanes from lane q * OUT on
+            const int first = q * OUT + 4 * c;
+            const uint32_t lanes = OUT >= 4 ? in[first >> 2] : (first & 2) ? in[first >> 2] >> 16 : in[first >> 2] & 0xFFFFu;
+            insert_field<W_IN>(V[c], R[c], lanes, W_IN * bitrev(q, F));
+        }
+        if (OUT == 2) V[c] &= 0xFFFFu;
+        // bytes NB + 4 c .. of the normalised bytes (NB is even)
+        if ((NB & 2) == 0) nb[(NB >> 2) + c] |= V[c];
+        else {
+            nb[NB >> 2] |= V[c] << 16;
+            if (OUT >= 4) nb[(NB >> 2) + 1] |= V[c] >> 16;
+        }
+    }
+    if constexpr (RES > 0) record_level<RES, OUT, NB + OUT, NW>(R, nb);
+}
+
+// The record of sixteen values v as H 16-bit words: word i = normalised byte i and, above it, normalised byte i + H.
+template <int H>
+__device__ __forceinline__ void record_words(const uint4& v, uint32_t s4, int m, uint32_t (&q)[H]) {
+    constexpr uint32_t kMask = ((1u << H) - 1) * 0x01010101u;
+    const uint32_t flip = s4 >> m;
+    const uint32_t in[4] = {((v.x >> m) ^ flip) & kMask, ((v.y >> m) ^ flip) & kMask, ((v.z >> m) ^ flip) & kMask, ((v.w >> m) ^ flip) & kMask};
+    uint32_t nb[(2 * H + 3) / 4 + 1];
+#pragma unroll
+    for (int i = 0; i < (2 * H + 3) / 4 + 1; ++i) nb[i] = 0;
+    record_level<H, 16, 0>(in, nb);
+#pragma unroll
+    for (int i = 0; i < H; ++i) {
+        const int j = i + H;
+        q[i] = prmt(nb[i >> 2], nb[j >> 2], uint32_t(i & 3) | (uint32_t(4 + (j & 3)) << 4));
+    }
+}
+
+// The calling warp's wide groups (the block's values at shared address `values`, the groups' numbers at `list`): records to
+// shared memory at `pend`, or, when they do not fit there, straight to `out` (2-byte aligned). mask_word, excl: see scan_mask.
+template <int H>
+__device__ __forceinline__ void pack_records(uint32_t values, uint32_t list, uint32_t count, uint32_t mask_word, uint32_t excl,
+                                             uint32_t s4, int m, uint32_t pend, uint8_t* out) {
+    const uint32_t lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    for (uint32_t base = 0; base < count; base += 32) {
+        const uint32_t i = base + lane;
+        const uint32_t number = lds8(list + (i < count ? i : 0));
+        const uint32_t word = (number >> 5) * kFusedWarps + warp;
+        const uint32_t rank = __shfl_sync(0xFFFFFFFFu, excl, word) +
+                              __popc(__shfl_sync(0xFFFFFFFFu, mask_word, word) & ((1u << (number & 31)) - 1));
+        if (i < count) {
+            uint32_t q[H];
+            record_words<H>(lds128(values + ((number >> 5) * kFusedThreads + warp * 32 + (number & 31)) * 16), s4, m, q);
+            if (out == nullptr) {
+#pragma unroll
+                for (int k = 0; k < H; ++k) sts16(pend + (rank * H + k) * 2, q[k]);
+            } else {
+#pragma unroll
+                for (int k = 0; k < H; ++k) reinterpret_cast<uint16_t*>(out)[rank * H + k] = uint16_t(q[k]);
+            }
+        }
+    }
+}
+
+template <int DT>
+__device__ __forceinline__ void pack_records_any(int h, uint32_t values, uint32_t list, uint32_t count, uint32_t mask_word, uint32_t excl,
+                                                 uint32_t s4, int m, uint32_t pend, uint8_t* out) {
+    switch (h) {
+        case 0: break;
+        case 1: pack_records<1>(values, list, count, mask_word, excl, s4, m, pend, out); break;
+        case 2: pack_records<2>(values, list, count, mask_word, excl, s4, m, pend, out); break;
+        case 3: pack_records<3>(values, list, count, mask_word, excl, s4, m, pend, out); break;
+        case 4: pack_records<4>(values, list, count, mask_word, excl, s4, m, pend, out); break;
+        case 5: if constexpr (DT != ENEC_FP16) pack_records<5>(values, list, count, mask_word, excl, s4, m, pend, out); break;
+        case 6: if constexpr (DT != ENEC_FP16) pack_records<6>(values, list, count, mask_word, excl, s4, m, pend, out); break;
+        default: if constexpr (DT != ENEC_FP16) pack_records<7>(values, list, count, mask_word, excl, s4, m, pend, out); break;
+    }
+}
+// Number of wide groups before block k, by one warp; false when the blocks before were not counted in time.
+__device__ __forceinline__ bool groups_before(const FusedTensor& t, uint32_t k, uint32_t& before) {
+    before = 0;
+    if (k == 0) return true;
+    const uint32_t lane = threadIdx.x & 31;
+    const uint32_t sb = k / kSuperBlocks, hy = sb / kHyperSupers;
+    for (uint32_t polls = 0; polls < (1u << 20); ++polls) {
+        uint32_t sum = 0;
+        bool ready = true;
+        unsigned long long st[kSuperBlocks / 32], su[kHyperSupers / 32];
+#pragma unroll
+        for (uint32_t i = 0; i < kSuperBlocks / 32; ++i) {
+            const uint32_t at = sb * kSuperBlocks + i * 32 + lane;
+            st[i] = at < k ? ld_relaxed_u64(&t.state[at]) : (unsigned long long)t.epoch << 32;
+        }
+#pragma unroll
+        for (uint32_t i = 0; i < kHyperSupers / 32; ++i) {
+            const uint32_t at = hy * kHyperSupers + i * 32 + lane;
+            su[i] = at < sb ? ld_relaxed_u64(&t.super[at]) : (unsigned long long)kSuperBlocks << 32;
+        }
+        for (uint32_t at = lane; at < hy; at += 32) {
+            const unsigned long long w = ld_relaxed_u64(&t.hyper[at]);
+            ready = ready && (w >> 32) == kSuperBlocks * kHyperSupers;
+            sum += uint32_t(w);
+        }
+#pragma unroll
+        for (uint32_t i = 0; i < kSuperBlocks / 32; ++i) {
+            ready = ready && uint32_t(st[i] >> 32) == t.epoch;
+            sum += uint32_t(st[i]);
+        }
+#pragma unroll
+        for (uint32_t i = 0; i < kHyperSupers / 32; ++i) {
+            ready = ready && uint32_t(su[i] >> 32) == kSuperBlocks;
+            sum += uint32_t(su[i]);
+        }
+        if (__all_sync(0xFFFFFFFFu, ready)) {
+            before = __reduce_add_sync(0xFFFFFFFFu, sum);
+            return true;
+        }
+        __nanosleep(polls > 2 ? 400 : 50);
+    }
+    return false;
+}
+
+// The same question put by the warps of a CTA together, without waiting: the first four ask for the state words, the others
+// for the first-level sums ...
+static_assert(kSuperBlocks == 128 && kHyperSupers == 128 && kFusedThreads == 256, "a thread asks for one word");
+__device__ __forceinline__ unsigned long long ask_before(const FusedTensor& t, uint32_t k, uint32_t tid) {
+    const uint32_t sb = k / kSuperBlocks;
+    if (tid < 128) {
+        const uint32_t at = sb * kSuperBlocks + tid;
+        return at < k ? ld_relaxed_u64(&t.state[at]) : (unsigned long long)t.epoch << 32;
+    }
+    const uint32_t at = sb / kHyperSupers * kHyperSupers + tid - 128;
+    return at < sb ? ld_relaxed_u64(&t.super[at]) : (unsigned long long)kSuperBlocks << 32;
+}
+// ... and later each warp sums up its answers: its share, or kNotReady (the same in every lane).
+__device__ __forceinline__ uint32_t share_before(const FusedTensor& t, unsigned long long answer, uint32_t k, uint32_t tid) {
+    bool ready = uint32_t(answer >> 32) == (tid < 128 ? t.epoch : kSuperBlocks);
+    uint32_t sum = uint32_t(answer);
+    if (tid < 32) {
+        for (uint32_t i = tid; i < k / (kSuperBlocks * kHyperSupers); i += 32) {   // tensors of more than 2^28 values
+            const unsigned long long w = ld_relaxed_u64(&t.hyper[i]);
+            ready = ready && uint32_t(w >> 32) == kSuperBlocks * kHyperSupers;
+            sum += uint32_t(w);
+        }
+    }
+    sum = __reduce_add_sync(0xFFFFFFFFu, sum);
+    return __all_sync(0xFFFFFFFFu, ready) ? sum : kNotReady;
+}
+
+// All threads: `halves` 16-bit words from shared memory (4-byte aligned) to global memory (2-byte aligned).
+__device__ __forceinline__ void copy_halves(uint8_t* dst, uint32_t src, uint32_t halves, uint32_t tid) {
+    const uint32_t odd = uint32_t(reinterpret_cast<uintptr_t>(dst) >> 1) & 1;   // a leading half before the first aligned word
+    const uint32_t words = halves > odd ? (halves - odd) / 2 : 0;
+    uint32_t* d32 = reinterpret_cast<uint32_t*>(dst + 2 * odd);
+    if (odd) {
+        for (uint32_t i = tid; i < words; i += kFusedThreads) d32[i] = prmt(lds32(src + 4 * i), lds32(src + 4 * i + 4), 0x5432u);
+    } else {
+        for (uint32_t i = tid; i < words; i += kFusedThreads) d32[i] = lds32(src + 4 * i);
+    }
+    if (tid == 0 && odd && halves > 0) *reinterpret_cast<uint16_t*>(dst) = uint16_t(lds16(src));
+    if (tid == 32 && halves > odd && ((halves - odd) & 1)) *reinterpret_cast<uint16_t*>(dst + 2 * (halves - 1)) = uint16_t(lds16(src + 2 * (halves - 1)));
+}
+
+// The end of a block, by a warp that knows its offset: table entry; for the last block also the header, the end of
+// the table, the padding behind the records and the stream length.
+template <int DT>
+__device__ __forceinline__ void finish_block(const FusedTensor& t, uint32_t k, uint32_t before, uint32_t wide) {
+    if ((threadIdx.x & 31) != 0) return;
+    t.table[k] = before;
+    if (k + 1 != t.nblocks) return;
+    const uint32_t a_total = before + wide;
+    const uint64_t high_bytes = uint64_t(a_total) * 2 * uint32_t(t.hbits);
+    const uint64_t total = uint64_t(t.high - t.out) + align16(high_bytes);
+    Header hd;
+    hd.magic = kMagic;
+    hd.version = kVersion;
+    hd.dtype = DT;
+    hd.variant = 0;
+    hd.count = t.count;
+    hd.block = kBlockElems;
+    hd.b = uint8_t(t.b); hd.n = uint8_t(t.n); hd.m = uint8_t(t.m); hd.L = kGroupElems;
+    hd.nblocks = t.nblocks;
+    hd.total_groups = t.total_groups;
+    hd.a_total = a_total;
+    hd.pad1 = 0;
+    hd.total_bytes = total;
+    hd.pad2[0] = hd.pad2[1] = 0;
+    *reinterpret_cast<Header*>(t.out) = hd;
+    t.table[t.nblocks] = a_total;
+    for (uint64_t i = uint64_t(t.nblocks) + 1; i < align16(4 * (uint64_t(t.nblocks) + 1)) / 4; ++i) t.table[i] = 0;
+    for (uint64_t p = high_bytes; p < align16(high_bytes); p += 2) *reinterpret_cast<uint16_t*>(t.high + p) = 0;
+    if (t.out_size) *t.out_size = total;
+}
+
+// One access of 32 bytes, or two of 16.
+__device__ __forceinline__ Run load32_any(const uint8_t* p, bool wide) {
+    if (wide) return load32<true>(p);
+    return load32<false>(p);
+}
+// One run of sixteen values of a block, group `g` of it: sign/mantissa plane, histogram, values (16 bytes per group; fp16:
+// the bits of the fp16 plane in bits 7..5 of each byte), votes for the group mask and the numbers of the warp's wide
+// groups. number: 32 x (which of the thread's groups) + lane. Returns the OR of all values.
+template <int DT, bool PLAIN, bool HIST>
+__device__ __forceinline__ uint32_t pack_run(const Run& r, uint32_t minuend, uint32_t nmask4, uint32_t s4, uint32_t wide4, uint32_t hist,
+                                             uint32_t lane, uint32_t value_at, uint32_t number, uint32_t list, uint32_t& wide,
+                                             uint32_t* mask_word, bool store, uint8_t* sm_out) {
+    uint4 v, hs, sm;
+    transform_run<DT, PLAIN, HIST>(r, minuend, nmask4, hist, lane * 4, v, hs, sm);
+    if (store) __stcs(reinterpret_cast<uint4*>(sm_out), sm);
+    const uint32_t all = v.x | v.y | v.z | v.w;
+    const bool is_wide = (or_flipped(v, s4) & wide4) != 0;
+    if constexpr (DT == ENEC_FP16)
+        v = make_uint4((v.x & 0x1F1F1F1Fu) | (hs.x << 5), (v.y & 0x1F1F1F1Fu) | (hs.y << 5), (v.z & 0x1F1F1F1Fu) | (hs.z << 5),
+                       (v.w & 0x1F1F1F1Fu) | (hs.w << 5));
+    sts128(value_at, v);
+    const uint32_t votes = __ballot_sync(0xFFFFFFFFu, is_wide);
+    if (lane == 0) *mask_word = votes;
+    if (is_wide) sts8(list + wide + __popc(votes & ((1u << lane) - 1)), number);
+    wide += __popc(votes);
+    return all;
+}
+
+// First phase of a full block, all threads: thread t takes the groups t, t + 256, .. of the block through pack_run.
+// Returns whether some value is not representable (HIST only); `wide_of_warp`: the warp's wide groups.
+// The loop over the runs is kept rolled: unrolled it exceeds what the instruction caches hold for four CTAs in four places.
+template <int DT, bool PLAIN, bool HIST>
+__device__ __forceinline__ bool pack_front_full(const FusedTensor& t, uint32_t k, uint32_t work, uint32_t* s_mask, uint32_t tid,
+                                                uint32_t& wide_of_warp) {
+    using Shape = FusedShape<DT>;
+    constexpr uint32_t kElemBytes = DT == ENEC_FP32 ? 4 : 2;
+    constexpr uint32_t kStep = 16 * kFusedThreads;   // elements between a thread's runs
+    const uint32_t lane = tid & 31, warp = tid >> 5;
+    const uint8_t* in = t.in + (uint64_t(k) * kBlockElems + 16 * tid) * kElemBytes;
+    uint8_t* sm_out = t.sm + (uint64_t(k) * kBlockElems + 16 * tid);
+    uint8_t* lo_out = t.lo + (uint64_t(k) * kBlockElems + 16 * tid) * 2;
+    const uint32_t minuend = t.c, nmask4 = t.nmask4, s4 = t.s4, wide4 = t.wide4, wide_ok = t.wide_ok;
+    const uint32_t values = work + t.values_at + tid * 16, list = work + Shape::kListAt + warp * 128;
+    uint32_t all = 0, wide = 0;
+    const bool wide_in = (wide_ok & 1) != 0;
+    auto run = [&](const Run& r, uint32_t i) {
+        all |= pack_run<DT, PLAIN, HIST>(r, minuend, nmask4, s4, wide4, work + Shape::kHistAt, lane, values + i * kStep, i * 32 + lane, list,
+                                         wide, &s_mask[i * kFusedWarps + warp], true, sm_out + i * kStep);
+    };
+    if constexpr (DT == ENEC_FP32) {   // one run's 64 bytes in flight
+        Run a = load32_any(in, wide_in), b = load32_any(in + 32, wide_in);
+#pragma unroll 1
+        for (uint32_t i = 0; i < kBlockElems / kStep; ++i) {
+            const Run r = split_halves(a, b, lo_out + i * (kStep * 2), (wide_ok & 2) != 0);
+            in += kStep * kElemBytes;
+            if (i + 1 < kBlockElems / kStep) { a = load32_any(in, wide_in); b = load32_any(in + 32, wide_in); }
+            run(r, i);
+        }
+    } else {                           // two runs' 32 bytes
+        Run a = load32_any(in, wide_in), b = load32_any(in + kStep * kElemBytes, wide_in);
+#pragma unroll 1
+        for (uint32_t i = 0; i < kBlockElems / kStep; i += 2) {
+            in += 2 * kStep * kElemBytes;
+            run(a, i);
+            if (i + 2 < kBlockElems / kStep) a = load32_any(in, wide_in);
+            run(b, i + 1);
+            if (i + 2 < kBlockElems / kStep) b = load32_any(in + kStep * kElemBytes, wide_in);
+        }
+    }
+    wide_of_warp = wide;
+    return HIST && (DT == ENEC_FP16 ? all & rep4(0x1F) & ~nmask4 : all & ~nmask4) != 0;
+}
+
+// The same for the tensor's last block when it is not full and has at least 128 padded elements.
+template <int DT, bool PLAIN, bool HIST>
+__device__ __noinline__ bool pack_front_tail(uint32_t k, uint32_t* wide_of_warp) {
+    using Shape = FusedShape<DT>;
+    const FusedTensor& t = fused_tensor<DT>();
+    FusedShared& sh = fused_shared<DT>();
+    constexpr uint32_t kElemBytes = DT == ENEC_FP32 ? 4 : 2;
+    constexpr int E = Shape::E;
+    const uint32_t tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    const uint32_t work = smem_u32(fused_smem());
+    const uint32_t N = t.tail_padded, real = t.tail_real;
+    const uint8_t* in = t.in + uint64_t(k) * kBlockElems * kElemBytes;
+    uint8_t* out_lo = t.lo + uint64_t(k) * kBlockElems * 2;
+    if (tid < 32) sh.mask[tid] = 0;
+    bool bad = false;
+    if (HIST) {   // its real elements, one by one
+        for (uint32_t e = tid; e < real; e += kFusedThreads) {
+            const uint32_t x = exponent_of_word<DT>(exponent_word<DT>(in, e));
+            red_add_one(work + Shape::kHistAt + lane * 4 + (x & (Shape::kRows - 1)) * HistShape<DT>::kRowBytes);
+            bad = bad || (((uint32_t(t.b - int(x)) + (1u << (t.n - 1))) & ((1u << E) - 1)) >> t.n) != 0;
+        }
+    }
+    __syncthreads();
+    uint32_t wide = 0;
+#pragma unroll 1
+    for (uint32_t i = 0; i < kBlockElems / (16 * kFusedThreads); ++i) {
+        const uint32_t first = i * kFusedThreads + warp * 32;   // the warp's first group of this round
+        if (first >= N / 16) break;
+        const uint32_t g = first + lane, e0 = 16 * g;
+        const int left = int(real) - int(e0);                   // groups from N / 16 on are padding too
+        Run r;
+        if (left >= 16) {
+            if constexpr (DT == ENEC_FP32)
+                r = split_halves(load32<false>(in + uint64_t(e0) * 4), load32<false>(in + uint64_t(e0) * 4 + 32), out_lo + uint64_t(e0) * 2, false);
+            else
+                r = load32<false>(in + uint64_t(e0) * 2);
+        } else {
+            r = load_run_tail<DT>(in + uint64_t(e0) * kElemBytes, out_lo + uint64_t(e0) * 2, left,
+                                  int(align16(2 * uint64_t(real)) / 2) - int(e0), t.pad);
+        }
+        // the padding's sign/mantissa bytes are zero
+        pack_run<DT, PLAIN, false>(r, t.c, t.nmask4, t.s4, t.wide4, 0, lane, work + t.values_at + g * 16, i * 32 + lane,
+                                   work + Shape::kListAt + warp * 128, wide, &sh.mask[i * kFusedWarps + warp], left > 0,
+                                   t.sm + uint64_t(k) * kBlockElems + e0);
+    }
+    *wide_of_warp = wide;
+    return bad;
+}
+
+// Every warp: the block's mask words (lane l: word l) and the wide groups before each; returns the block's wide groups.
+__device__ __forceinline__ uint32_t scan_mask(const uint32_t* s_mask, uint32_t lane, uint32_t& word, uint32_t& before) {
+    word = s_mask[lane];
+    uint32_t incl = __popc(word);
+#pragma unroll
+    for (int d = 1; d < 32; d <<= 1) {
+        const uint32_t up = __shfl_up_sync(0xFFFFFFFFu, incl, d);
+        if (lane >= uint32_t(d)) incl += up;
+    }
+    before = incl - __popc(word);
+    return __shfl_sync(0xFFFFFFFFu, incl, 31);
+}
+
+// A tail block of 16, 32 or 64 padded elements, all threads, one element per thread, bit by bit (Algorithm 2 followed for
+// every set bit).
+template <int DT>
+__device__ __noinline__ void pack_short_block(uint32_t k, int* status) {
+    const FusedTensor& t = fused_tensor<DT>();
+    constexpr uint32_t kElemBytes = DT == ENEC_FP32 ? 4 : 2;
+    const uint32_t tid = threadIdx.x;
+    const uint32_t N = t.tail_padded, real = t.tail_real;
+    const uint8_t* in = t.in + uint64_t(k) * kBlockElems * kElemBytes;
+    uint8_t* out_sm = t.sm + uint64_t(k) * kBlockElems;
+    uint8_t* out_lo = t.lo + uint64_t(k) * kBlockElems * 2;  // fp32 only
+    const uint32_t hbits = uint32_t(t.hbits);
+    uint32_t* s_low = reinterpret_cast<uint32_t*>(fused_smem());   // 64 bytes
+    uint32_t* s_hi3 = s_low + 16;                                  // 32 bytes
+    uint32_t* s_rec = s_hi3 + 16;                                  // 4 records of up to 14 bytes
+    uint32_t* s_or = s_rec + 16;                                   // OR of y per group
+    if (tid < 64) s_low[tid] = 0;
+    __syncthreads();
+    auto put = [](uint32_t* plane, uint32_t lanes, int a, uint32_t e, uint32_t value, uint32_t base) {
+        for (int q = 0; q < a; ++q)
+            if ((value >> q) & 1) {
+                uint32_t pos; int bit;
+                alg2_locate(lanes, a, e, q, pos, bit);
+                pos += base;
+                atomicOr(&plane[pos >> 2], 1u << (8 * (pos & 3) + bit));
+            }
+    };
+    uint32_t y = 0, hs = 0;
+    if (tid < N) {
+        if (tid < real) {
+            if (DT == ENEC_FP32) reinterpret_cast<uint16_t*>(out_lo)[tid] = uint16_t(reinterpret_cast<const uint32_t*>(in)[tid]);
+            const uint32_t w = exponent_word<DT>(in, tid);
+            y = uint32_t(t.b - int(exponent_of_word<DT>(w))) & ((1u << t.n) - 1);
+            if (DT != ENEC_FP16) {
+                out_sm[tid] = uint8_t(((w >> 8) & 0x80) | (w & 0x7F));
+            } else {
+                out_sm[tid] = uint8_t(w);
+                hs = ((w >> 13) & 4) | ((w >> 8) & 3);
+            }
+        } else {
+            if (tid < uint32_t(align16(real))) out_sm[tid] = 0;
+            if (DT == ENEC_FP32 && 2 * tid < uint32_t(align16(2 * uint64_t(real)))) reinterpret_cast<uint16_t*>(out_lo)[tid] = 0;
+        }
+        atomicOr(&s_or[tid >> 4], y);
+        put(s_low, N, t.m, tid, y, 0);
+        if (DT == ENEC_FP16) put(s_hi3, N, 3, tid, hs, 0);
+    }
+    __syncthreads();
+    uint32_t mask = 0;
+    for (uint32_t g = 0; g < (N >> 4); ++g) mask |= (s_or[g] >> t.m) != 0 ? 1u << g : 0u;
+    if (tid < N && hbits > 0 && ((mask >> (tid >> 4)) & 1))
+        put(s_rec, 16, int(hbits), tid & 15, y >> t.m, __popc(mask & ((1u << (tid >> 4)) - 1)) * 2 * hbits);
+    __syncthreads();
+    // planes out, padded to 16 bytes with zeros
+    uint32_t* out_low = reinterpret_cast<uint32_t*>(t.low + uint64_t(k) * (kBlockElems / 8) * uint32_t(t.m));
+    uint32_t* out_mask = reinterpret_cast<uint32_t*>(t.mask + uint64_t(k) * (kGroupsPerBlock / 8));
+    if (tid < uint32_t(align16(uint64_t(N) * t.m / 8)) / 4) out_low[tid] = s_low[tid];
+    if (tid < 4) out_mask[tid] = tid == 0 ? mask : 0;
+    if (DT == ENEC_FP16 && tid < uint32_t(align16(uint64_t(N) * 3 / 8)) / 4)
+        reinterpret_cast<uint32_t*>(t.smhi + uint64_t(k) * (kBlockElems / 8) * 3)[tid] = s_hi3[tid];
+    const uint32_t wide = __popc(mask);
+    if (tid < 32) {
+        uint32_t before = 0;
+        const bool ok = groups_before(t, k, before);
+        if (ok) {
+            uint16_t* out_rec = reinterpret_cast<uint16_t*>(t.high + uint64_t(before) * 2 * hbits);
+            if (tid < wide * hbits) out_rec[tid] = reinterpret_cast<const uint16_t*>(s_rec)[tid];   // at most 28
+            finish_block<DT>(t, k, before, wide);
+        } else if (tid == 0) {
+            report(status, ENEC_ERR_TIMEOUT);
+        }
+    }
+    __syncthreads();
+}
+
+// ---- histogram stages ----------------------------------------------------------------------------------
+// The exponents of one block into the stage's table (column: the lane's copy), all threads.
+template <int DT>
+__device__ __forceinline__ void count_block(const uint8_t* in, uint32_t real, uint32_t column, uint32_t tid) {
+    constexpr uint32_t kPer = HistShape<DT>::kPerLoad;
+    const uint4* in4 = reinterpret_cast<const uint4*>(in);
+    const uint32_t chunks = real / kPer;
+    uint32_t at = tid;
+    for (; at + 7 * kFusedThreads < chunks; at += 8 * kFusedThreads) {
+        uint4 v[8];
+#pragma unroll
+        for (uint32_t q = 0; q < 8; ++q) v[q] = in4[at + q * kFusedThreads];
+#pragma unroll
+        for (uint32_t q = 0; q < 8; ++q) {
+            count_word_pair<DT>(column, v[q].x);
+            count_word_pair<DT>(column, v[q].y);
+            count_word_pair<DT>(column, v[q].z);
+            count_word_pair<DT>(column, v[q].w);
+        }
+    }
+    for (; at < chunks; at += kFusedThreads) {
+        const uint4 v = in4[at];
+        count_word_pair<DT>(column, v.x);
+        count_word_pair<DT>(column, v.y);
+        count_word_pair<DT>(column, v.z);
+        count_word_pair<DT>(column, v.w);
+    }
+    for (uint32_t e = chunks * kPer + tid; e < real; e += kFusedThreads)
+        red_add_one(column + exponent_of_word<DT>(exponent_word<DT>(in, e)) * HistShape<DT>::kRowBytes);
+}
+
+__device__ __forceinline__ void publish(uint32_t* where, uint32_t word) {
+    asm volatile("st.release.gpu.global.u32 [%0], %1;" ::"l"(where), "r"(word) : "memory");
+}
+// One thread: a published word; 0 when it does not come within about two seconds. When it has not come after some 20 us
+// and `ticket` says that some of `total` tickets have not been taken: kParamsTake.
+__device__ __forceinline__ uint32_t await_published(const uint32_t* where, const uint32_t* ticket = nullptr, uint32_t total = 0) {
+    for (uint32_t polls = 0; polls < (1u << 22); ++polls) {
+        uint32_t w;
+        asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(w) : "l"(where) : "memory");
+        if (w) return w;
+        if (polls > 64 && ticket && ld_relaxed_u32(ticket) < total) return kParamsTake;
+        __nanosleep(polls > 64 ? 500 : 100);
+    }
+    return 0;
+}
+
+// One thread: block k towards L2.
+template <int DT>
+__device__ __forceinline__ void fetch_block(const FusedTensor& t, uint32_t k) {
+    constexpr uint32_t kElemBytes = DT == ENEC_FP32 ? 4 : 2;
+    if (k < t.nblocks) {
+        const uint32_t bytes = ((k + 1 == t.nblocks ? t.tail_real : kBlockElems) * kElemBytes) & ~15u;
+        if (bytes) bulk_prefetch_l2(t.in + uint64_t(k) * kBlockElems * kElemBytes, bytes);
+    }
+}
+
+// All threads: `mine` more blocks are in hist[which] (or in pack_hist); the CTA that brings them to `complete` runs the search.
+template <int DT>
+__device__ __forceinline__ void count_done(FusedControl* ctl, uint32_t which, uint32_t mine, uint32_t complete) {
+    FusedShared& sh = fused_shared<DT>();
+    const uint32_t tid = threadIdx.x;
+    __threadfence();
+    __syncthreads();
+    if (tid == 0) sh.word = atomicAdd(&ctl->hist_done[which].value, mine) + mine == complete;
+    __syncthreads();
+    if (sh.word && tid < 32) {
+        __threadfence();
+        const uint32_t found = search_global<DT>(ctl->hist[which], which == 1 ? ctl->pack_hist : nullptr,
+                                                 reinterpret_cast<unsigned long long*>(fused_smem())) | kParamsValid;
+        if (tid == 0) publish(&ctl->params[which], found);
+    }
+}
+
+// The histogram of `total` blocks, every `stride`-th from `base` on, all CTAs together, and the parameters that the search
+// finds for it (0: a wait ran out). which: 0 the sample, 1 what the pack stage's histogram lacks of the whole tensor; it is
+// complete when `complete` blocks are counted here or there.
+template <int DT>
+__device__ __noinline__ uint32_t histogram_stage(FusedControl* ctl, uint32_t which, uint32_t base, uint32_t total, uint32_t stride,
+                                            uint32_t complete) {
+    const FusedTensor& t = fused_tensor<DT>();
+    FusedShared& sh = fused_shared<DT>();
+    constexpr uint32_t kElemBytes = DT == ENEC_FP32 ? 4 : 2;
+    const uint32_t tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    const uint32_t work = smem_u32(fused_smem());
+    const bool ahead = total > gridDim.x;   // tickets are asked for ahead; else a CTA has one block as a rule
+    uint32_t* const ticket = &ctl->hist_ticket[which].value;
+    bool first = true;
+    uint32_t word;
+    for (;;) {
+        __syncthreads();
+        for (uint32_t i = tid; i < uint32_t(HistShape<DT>::kBytes / 16); i += kFusedThreads) sts128(work + 16 * i, make_uint4(0, 0, 0, 0));
+        if (tid == 0) sh.word = atomicAdd(ticket, 1u);
+        __syncthreads();
+        uint32_t mine = 0;
+        for (uint32_t i = sh.word; i < total; ++mine) {
+            uint32_t asked = total;
+            if (ahead && tid == 0) {
+                asked = atomicAdd(ticket, 1u);
+                if (asked < total) fetch_block<DT>(t, base + asked * stride);
+            }
+            const uint32_t k = base + i * stride;
+            const uint32_t real = k + 1 == t.nblocks ? t.tail_real : kBlockElems;
+            count_block<DT>(t.in + uint64_t(k) * kBlockElems * kElemBytes, real, work + lane * 4, tid);
+            __syncthreads();
+            if (tid == 0) sh.word = asked;
+            __syncthreads();
+            i = sh.word;
+        }
+        if (mine) {
+            if (tid < uint32_t(HistShape<DT>::kBins)) {
+                const uint32_t n = fold_hist_row<false>(work + tid * HistShape<DT>::kRowBytes, tid);
+                if (n) atomicAdd(&ctl->hist[which][tid], (unsigned long long)n);
+            }
+            count_done<DT>(ctl, which, mine, complete);
+        }
+        __syncthreads();   // sh.word has been read by everybody
+        if (tid == 0) {
+            if (which == 0 && first) {   // the CTA's first block of the pack stage is asked for, and brought towards L2, meanwhile
+                sh.next = atomicAdd(&ctl->pack_ticket[0].value, 1u);
+                if (!mine) __nanosleep(3000);   // behind the loads of the blocks that are being counted
+                fetch_block<DT>(t, sh.next);
+            }
+            // a CTA of the grid that has not started (other work holds its SM) leaves its block to one that waits
+            sh.word = await_published(&ctl->params[which], ticket, total);
+        }
+        first = false;
+        __syncthreads();
+        word = sh.word;
+        __syncthreads();
+        if (word != kParamsTake) return word;
+    }
+}
+
+// A block with a value that the sampled parameters cannot represent: its counts are taken out of the CTA's table of the pack
+// stage, whose rows cannot tell all exponents apart, and added to the whole tensor's histogram. All threads; the shared
+// memory of the block's planes and values is used.
+template <int DT>
+__device__ __noinline__ void recount_block(FusedControl* ctl, uint32_t k) {
+    using Shape = FusedShape<DT>;
+    const FusedTensor& t = fused_tensor<DT>();
+    constexpr uint32_t kElemBytes = DT == ENEC_FP32 ? 4 : 2;
+    constexpr uint32_t kBins = HistShape<DT>::kBins, kColumns = 16;
+    const uint32_t tid = threadIdx.x, lane = tid & 31;
+    const uint32_t work = smem_u32(fused_smem());
+    const uint8_t* in = t.in + uint64_t(k) * kBlockElems * kElemBytes;
+    const uint32_t real = k + 1 == t.nblocks ? t.tail_real : kBlockElems;
+    __syncthreads();
+    for (uint32_t i = tid; i < kBins * kColumns / 4; i += kFusedThreads) sts128(work + 16 * i, make_uint4(0, 0, 0, 0));
+    __syncthreads();
+    auto move = [&](uint32_t w) {   // one value's 16-bit word
+        const uint32_t x = exponent_of_word<DT>(w);
+        asm volatile("red.shared.add.u32 [%0], %1;" ::"r"(work + Shape::kHistAt + lane * 4 + (x & (Shape::kRows - 1)) * HistShape<DT>::kRowBytes), "r"(~0u)
+                     : "memory");
+        red_add_one(work + (x * kColumns + (lane & (kColumns - 1))) * 4);
+    };
+    constexpr uint32_t kPer = HistShape<DT>::kPerLoad;
+    for (uint32_t i = tid; i < real / kPer; i += kFusedThreads) {
+        const uint4 v = reinterpret_cast<const uint4*>(in)[i];
+        const uint32_t w[4] = {v.x, v.y, v.z, v.w};
+#pragma unroll
+        for (int q = 0; q < 4; ++q) {
+            move(w[q] >> 16);
+            if (DT != ENEC_FP32) move(w[q]);
+        }
+    }
+    for (uint32_t e = real / kPer * kPer + tid; e < real; e += kFusedThreads) move(exponent_word<DT>(in, e));
+    __syncthreads();
+    if (tid < kBins) {
+        uint32_t n = 0;
+        for (uint32_t c = 0; c < kColumns; ++c) n += lds32(work + (tid * kColumns + c) * 4);
+        if (n) atomicAdd(&ctl->hist[1][tid], (unsigned long long)n);
+    }
+    __syncthreads();
+}
+
+// The pack stage's blocks, ticket after ticket, starting with the one in sh.next; all threads. HIST: the parameters come
+// from a sample. Returns the number of blocks packed, and kPassEnded where a ticket said so. (A function of its own per form, so that each has its own registers.)
+//
+// Two barriers per block: A after the first phase (values, mask and lists are complete), B after the second (planes and
+// records are complete). What follows B reads only what is not written before the next A.
+template <int DT, bool PLAIN, bool HIST>
+__device__ __noinline__ uint32_t pack_pass(FusedControl* ctl, uint32_t pass, int* status) {
+    using Shape = FusedShape<DT>;
+    constexpr uint32_t kElemBytes = DT == ENEC_FP32 ? 4 : 2;
+    constexpr int E = Shape::E;
+    const FusedTensor& t = fused_tensor<DT>();
+    FusedShared& sh = fused_shared<DT>();
+    const uint32_t tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    const uint32_t work = smem_u32(fused_smem());
+    uint32_t pend_block = 0xFFFFFFFFu, pend_wide = 0, pend_at = 0;   // the block whose records wait in shared memory
+    uint32_t iter = 0, mine = 0;
+    bool stop = false;       // a wait ran out
+    // All threads: the waiting block's records to their place. Its offset is in sh.part, if the look-up begun during the
+    // block after it (`asked_for`) found all blocks before it counted; else the first warp waits for them.
+    auto place_waiting = [&](bool asked_for) {
+        uint32_t before = 0;
+        bool ready = asked_for;
+        for (uint32_t w = 0; w < kFusedWarps; ++w) {
+            ready = ready && sh.part[w] != kNotReady;
+            before += sh.part[w];
+        }
+        if (!ready) {
+            if (warp == 0) {
+                const bool ok = groups_before(t, pend_block, before);
+                if (lane == 0) {
+                    sh.before = before;
+                    sh.ok = ok;
+                    if (!ok) report(status, ENEC_ERR_TIMEOUT);
+                }
+            }
+            __syncthreads();
+            before = sh.before;
+            if (!sh.ok) { stop = true; return; }
+        }
+        copy_halves(t.high + uint64_t(before) * 2 * uint32_t(t.hbits), pend_at, pend_wide * uint32_t(t.hbits), tid);
+        if (warp == 0) finish_block<DT>(t, pend_block, before, pend_wide);
+    };
+    // one thread: no further block is handed out; those handed out already are packed, so that nobody waits for them in vain
+    auto end_pass = [&]() {
+        const uint32_t handed = atomicOr(&ctl->pack_ticket[pass].value, kPassEnded);
+        if ((handed & kPassEnded) == 0) publish(&ctl->pack_target, handed < t.nblocks ? handed : t.nblocks);
+    };
+    uint32_t k = sh.next;
+    __syncthreads();   // before thread 0 writes the next ticket there
+    for (; k < t.nblocks; ++iter) {
+        uint32_t asked = 0;
+        if (tid == 0) asked = t.nblocks == 1 ? 1u : atomicAdd(&ctl->pack_ticket[pass].value, 1u);
+        ++mine;
+        const bool last = k + 1 == t.nblocks && t.tail_real != kBlockElems;   // the tensor's last block, not full
+        const uint32_t N = last ? t.tail_padded : kBlockElems;
+        uint32_t wide_of_warp = 0;
+        bool bad = false;
+        if (!last) {
+            bad = pack_front_full<DT, PLAIN, HIST>(t, k, work, sh.mask, tid, wide_of_warp);
+        } else if (N >= 128) {
+            bad = pack_front_tail<DT, PLAIN, HIST>(k, &wide_of_warp);
+        } else if (HIST && tid < t.tail_real) {
+            const uint32_t x = exponent_of_word<DT>(exponent_word<DT>(t.in + uint64_t(k) * kBlockElems * kElemBytes, tid));
+            red_add_one(work + Shape::kHistAt + lane * 4 + (x & (Shape::kRows - 1)) * HistShape<DT>::kRowBytes);
+            bad = (((uint32_t(t.b - int(x)) + (1u << (t.n - 1))) & ((1u << E) - 1)) >> t.n) != 0;
+        }
+        if (tid == 0) {
+            sh.next = asked;
+            fetch_block<DT>(t, asked);
+        }
+        const bool lossy = __syncthreads_or(bad) != 0;   // barrier A
+        if ((lossy || stop) && tid == 0) end_pass();
+        const bool waiting = pend_block != 0xFFFFFFFFu;
+        if (N < 128) {
+            if (waiting) place_waiting(false);
+            pend_block = 0xFFFFFFFFu;
+            if (HIST && lossy) recount_block<DT>(ctl, k);
+            __syncthreads();
+            pack_short_block<DT>(k, status);
+            k = sh.next;
+            break;   // no block comes after this one
+        }
+        unsigned long long answer = 0;
+        if (waiting) answer = ask_before(t, pend_block, tid);   // it comes while the block is packed
+        uint32_t mask_word, excl;
+        const uint32_t wide = scan_mask(sh.mask, lane, mask_word, excl);
+        if (tid == 0 && t.nblocks != 1) {
+            st_relaxed_u64(&t.state[k], ((unsigned long long)t.epoch << 32) | wide);
+            atomicAdd(&t.super[k / kSuperBlocks], (1ull << 32) | wide);
+            if (t.nblocks > kSuperBlocks * kHyperSupers) atomicAdd(&t.hyper[k / (kSuperBlocks * kHyperSupers)], (1ull << 32) | wide);
+        }
+        if (HIST && sh.next >= kPassEnded) {   // what is packed now will be packed again: the block has been counted, that is all
+            if (lossy) recount_block<DT>(ctl, k);
+            pend_block = 0xFFFFFFFFu;
+            k = sh.next;
+            break;
+        }
+        const uint32_t hbits = uint32_t(t.hbits), m = uint32_t(t.m);
+        const bool direct = wide * 2 * hbits > Shape::kPend;   // the records do not fit the waiting area
+        if (tid < uint32_t(align16(((N >> 4) + 7) / 8)) / 16)
+            reinterpret_cast<uint4*>(t.mask + uint64_t(k) * (kGroupsPerBlock / 8))[tid] = reinterpret_cast<const uint4*>(sh.mask)[tid];
+        pack_planes<DT>(t, work, N, tid);
+        if (direct) {
+            if (warp == 0) {
+                uint32_t before = 0;
+                const bool ok = groups_before(t, k, before);
+                if (ok) finish_block<DT>(t, k, before, wide);
+                else if (lane == 0) report(status, ENEC_ERR_TIMEOUT);
+                if (lane == 0) { sh.before = before; sh.ok = ok; }
+            }
+            __syncthreads();
+            if (!sh.ok) stop = true;
+        }
+        if (!direct || sh.ok)
+            pack_records_any<DT>(int(hbits), work + t.values_at, work + Shape::kListAt + warp * 128, wide_of_warp, mask_word, excl, t.s4, int(m),
+                                 work + Shape::kPendAt + (iter & 1) * Shape::kPend,
+                                 direct ? t.high + uint64_t(sh.before) * 2 * hbits : nullptr);
+        if (waiting) {
+            const uint32_t share = share_before(t, answer, pend_block, tid);
+            if (lane == 0) sh.part[warp] = share;
+        }
+        const uint32_t next = sh.next;
+        __syncthreads();                                      // barrier B
+        fold_out(work, N * m / 8, t.low + uint64_t(k) * (kBlockElems / 8) * m, tid);   // N >= 128: whole pieces of 16 bytes
+        if (DT == ENEC_FP16) fold_out(work + t.smhi_at, N * 3 / 8, t.smhi + uint64_t(k) * (kBlockElems / 8) * 3, tid);
+        if (waiting) place_waiting(true);
+        pend_block = direct ? 0xFFFFFFFFu : k;
+        pend_wide = wide;
+        pend_at = work + Shape::kPendAt + (iter & 1) * Shape::kPend;
+        if (HIST && lossy) recount_block<DT>(ctl, k);
+        k = next;
+    }
+    __syncthreads();
+    if (HIST && mine) {   // under way while the last block's offset is looked up
+        if (tid < Shape::kRows) {
+            // row r of the table holds the exponent x of that remainder that the parameters can represent
+            const uint32_t n = fold_hist_row<false>(work + Shape::kHistAt + tid * HistShape<DT>::kRowBytes, tid);
+            const uint32_t d = uint32_t(t.b) + (1u << (t.n - 1));
+            const uint32_t x = (d - ((d - tid) & (Shape::kRows - 1))) & ((1u << E) - 1);
+            if (n) atomicAdd(&ctl->pack_hist[x], (unsigned long long)n);
+        }
+    }
+    if (HIST && k >= kPassEnded) return mine | kPassEnded;
+    if (pend_block != 0xFFFFFFFFu) place_waiting(false);
+    return mine;
+}
+
+template <int DT>
+__global__ void __launch_bounds__(kFusedThreads, FusedShape<DT>::kCtasPerSm)
+enec_fused_kernel(const FusedJob job, int* status) {
+    uint8_t* const smem = fused_smem();
+    FusedTensor& t = fused_tensor<DT>();
+    FusedShared& sh = fused_shared<DT>();
+    using Shape = FusedShape<DT>;
+    const uint32_t tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    const uint32_t work = smem_u32(smem);
+    unsigned long long* const search_table = reinterpret_cast<unsigned long long*>(smem);
+    FusedControl* const ctl = job.ctl;
+    const uint32_t nblocks = uint32_t((job.count + kBlockElems - 1) / kBlockElems);
+    pdl_launch_dependents();
+    if (gridDim.x == 1)
+        for (uint32_t i = tid; i < uint32_t(HistShape<DT>::kBytes / 16); i += kFusedThreads) sts128(work + 16 * i, make_uint4(0, 0, 0, 0));
+    if (tid == 0) {
+        t.in = job.in; t.out = job.out; t.count = job.count; t.out_size = job.out_size;
+        set_geometry<DT>(t);
+    }
+    __syncthreads();
+    pdl_wait();  // nothing above touches global memory
+    {
+        // the next call on this scratch area finds its control set and sums zeroed
+        const uint32_t at = blockIdx.x * kFusedThreads + tid, all = gridDim.x * kFusedThreads;
+        for (uint32_t i = at; i < sizeof(FusedControl) / 16; i += all) reinterpret_cast<uint4*>(job.ctl_next)[i] = make_uint4(0, 0, 0, 0);
+        for (uint32_t i = at; i < job.clear_supers; i += all) job.super_next[i] = job.super_next[job.super_stride + i] = 0;
+    }
+
+    // ---- sample stage ----
+    uint32_t word = 0;                              // the parameters
+    bool exact = job.sample == nblocks;             // they are the whole tensor's
+    if (gridDim.x == 1) {  // one block: nothing to hand out, nobody to tell
+        count_block<DT>(job.in, t.tail_real, work + lane * 4, tid);
+        __syncthreads();
+        uint32_t* counts = reinterpret_cast<uint32_t*>(smem + Shape::kPendAt);
+        if (tid < uint32_t(HistShape<DT>::kBins)) counts[tid] = fold_hist_row<false>(work + tid * HistShape<DT>::kRowBytes, tid);
+        __syncthreads();
+        if (warp == 0) {
+            const uint32_t found = search_by_warp<DT>([&](int x) { return (unsigned long long)counts[x]; }, search_table);
+            if (lane == 0) { sh.word = found | kParamsValid; sh.next = 0; }
+        }
+        __syncthreads();
+        word = sh.word;
+    } else {
+        word = histogram_stage<DT>(ctl, 0, 0, job.sample, nblocks / job.sample, job.sample);
+        if (!exact && word != 0 && !sample_will_do<DT>(word)) {
+            exact = true;
+            word = histogram_stage<DT>(ctl, 1, 0, nblocks, 1, nblocks);
+        }
+    }
+
+    // ---- pack stage ----
+    for (uint32_t pass = 0;; ++pass) {
+        if (word == 0) {
+            if (tid == 0) report(status, ENEC_ERR_TIMEOUT);
+            return;
+        }
+        __syncthreads();
+        if (tid == 0) {
+            set_parameters<DT>(t, word);
+            t.state = job.state;
+            t.super = job.super + pass * job.super_stride;
+            t.hyper = ctl->hyper[pass];
+            t.epoch = job.epoch + pass;
+        }
+        if (!exact) {
+            for (uint32_t i = tid; i < Shape::kHistBytes / 16; i += kFusedThreads) sts128(work + Shape::kHistAt + 16 * i, make_uint4(0, 0, 0, 0));
+        }
+        __syncthreads();
+        const uint32_t left = !exact                       ? pack_pass<DT, true, true>(ctl, pass, status)
+                              : t.plain || DT == ENEC_FP16 ? pack_pass<DT, true, false>(ctl, pass, status)
+                                                           : pack_pass<DT, false, false>(ctl, pass, status);
+        if (exact) return;
+        exact = true;
+        const uint32_t mine = left & ~kPassEnded;
+
+        if (left & kPassEnded) {
+            // some block does not bear the sampled parameters: how many blocks had been handed out?
+            __syncthreads();
+            if (tid == 0) sh.word = await_published(&ctl->pack_target);
+            __syncthreads();
+            const uint32_t target = sh.word;
+            __syncthreads();
+            if (target != nblocks) {   // the rest of the tensor is counted, then everything packed again
+                if (mine) count_done<DT>(ctl, 1, mine, nblocks);
+                word = target ? histogram_stage<DT>(ctl, 1, target, nblocks - target, 1, nblocks) : 0u;
+                if (tid == 0) sh.next = atomicAdd(&ctl->pack_ticket[1].value, 1u);
+                continue;
+            }
+        }
+
+        // ---- the sampled parameters against the whole tensor's ----
+        __threadfence();
+        __syncthreads();
+        if (tid == 0) sh.word = mine && atomicAdd(&ctl->pack_done.value, mine) + mine == nblocks;
+        __syncthreads();
+        if (sh.word && warp == 0) {   // the last CTA to leave
+            __threadfence();
+            const uint32_t found = search_global<DT>(ctl->pack_hist, ctl->hist[1], search_table) | kParamsValid |
+                                   (ld_relaxed_u32(&ctl->pack_target) ? kParamsRedo : 0u);
+            if (lane == 0) publish(&ctl->verdict, found);
+        }
+        __syncthreads();
+        if (tid == 0) {
+            sh.word = await_published(&ctl->verdict);
+            sh.next = sh.word == word || sh.word == 0 ? 0u : atomicAdd(&ctl->pack_ticket[1].value, 1u);
+        }
+        __syncthreads();
+        if (sh.word == word) return;
+        word = sh.word & ~kParamsRedo;
+    }
+}
+
+}  // namespace enec

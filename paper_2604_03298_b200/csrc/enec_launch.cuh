@@ -19,6 +19,10 @@ struct DecodeBatch;
 enec_status launch_decode_any(int dt, const DecodeBatch& batch, int* d_status, cudaStream_t stream, bool ranked,
                               int ticketed = 0);
 
+struct FusedJob;
+// The one-kernel compressor on one tensor (see enec_fused.cuh).
+enec_status launch_fused(int dt, const FusedJob& job, uint32_t nblocks, int sms, bool* attr_set, int* d_status, cudaStream_t stream);
+
 // Launch with programmatic stream serialisation: the kernel may be scheduled while its predecessor in the
 // stream drains; it waits for the predecessor's completion itself (pdl_wait) before touching memory.
 template <class... KernelArgs, class... Args>

@@ -32,3 +32,72 @@ def test_batched_decompress_chunk_lengths(total_blocks):
         for s, o in zip(srcs, outs):
             assert torch.equal(s.view(torch.int16), o.view(torch.int16))
             o.zero_()
+
+
+def _compress_twice(enec, t, dt):
+    """Two calls in a row (the second finds the scratch as the first left it); the stream, checked to be the same twice."""
+    n = t.numel()
+    cap = enec.enec_max_compressed_size(dt, n)
+    got = []
+    for _ in range(2):
+        buf = torch.full((cap + 64,), 0xA5, dtype=torch.uint8, device="cuda")
+        size, status = torch.zeros(1, dtype=torch.int64, device="cuda"), status_tensor()
+        assert enec.enec_compress(t, dt, n, buf, cap, size, status) == 0
+        assert int(status.item()) == 0
+        assert bool((buf[cap:] == 0xA5).all()), "wrote behind the capacity"
+        got.append(buf[:int(size.item())].cpu().numpy())
+    assert np.array_equal(got[0], got[1])
+    return got[0]
+
+
+def _words(t, dt):
+    return t.view(torch.int32).cpu().numpy().view(np.uint32) if dt == 2 else words_of(t)
+
+
+@pytest.mark.parametrize("dt", [0, 1, 2])
+@pytest.mark.parametrize("blocks", [1, 2, 127, 128, 129, 443, 444, 445, 704, 705, 1408, 1409])
+@pytest.mark.parametrize("tail", [0, 37, 5003])
+def test_compress_around_the_size_where_a_sample_is_taken(oracle, dt, blocks, tail):
+    """Blocks of the tensor around 128 (the first-level sums), around the number of CTAs (444) and around 44 MB (704 blocks of
+    fp32, 1408 of the others), from where on the parameters come from a sample, with a full, a short and an ordinary last
+    block."""
+    import paper_2604_03298_b200 as enec
+    t = _weights(blocks * 16384 + tail, dt, blocks + tail)
+    assert np.array_equal(_compress_twice(enec, t, dt), oracle.compress(_words(t, dt), dt))
+
+
+@pytest.mark.parametrize("dt", [0, 1, 2])
+@pytest.mark.parametrize("what", ["one zero", "one huge", "zero in the tail", "wider rest", "narrower rest", "sample too wide",
+                                  "all wide", "constant"])
+def test_compress_when_the_sample_misleads(oracle, dt, what):
+    """2961 blocks, of which every twentieth is sampled. The stream has to be the one that the search on the whole tensor
+    leads to."""
+    import paper_2604_03298_b200 as enec
+    blocks = 2961
+    t = _weights(blocks * 16384 + 4000, dt, 7, 0.0002 if what == "one huge" else 0.02)
+    t = torch.where(t == 0, torch.full_like(t, 0.001), t)
+    if dt == 1:
+        t = torch.where(t.abs() < 2e-3, torch.full_like(t, 2e-3), t)   # fp16: a narrow range of exponents otherwise
+    body = t[:blocks * 16384].view(blocks, 16384)
+    if what == "one zero":
+        body[2641, 77] = 0
+    elif what == "one huge":
+        body[1, 16000] = 60000.0
+    elif what == "zero in the tail":
+        t[-3] = 0
+    elif what == "wider rest":
+        body[1::2] *= 3.0
+        body[2::4] *= 0.4
+    elif what == "narrower rest":
+        body[1::20] = 0.02
+        body[2::20] = 0.02
+        body[3::4] = 0.02
+    elif what == "sample too wide":
+        body[0, 5] = 0
+        body[2000, 6] = 3e4
+    elif what == "all wide":
+        bits = torch.randint(0, 1 << 15, (t.numel(),), device="cuda", generator=torch.Generator(device="cuda").manual_seed(3))
+        t = (bits.to(torch.int32) << 16 if dt == 2 else bits.to(torch.int16)).view(DTYPES[dt])
+    else:
+        t = torch.full_like(t, 0.75)
+    assert np.array_equal(_compress_twice(enec, t, dt), oracle.compress(_words(t, dt), dt))
