@@ -244,12 +244,15 @@ __device__ inline int load_job(const DecodeJob& job, JobCtx& c, bool blockwise =
 // cap = records per block that fit; records beyond it are read from global memory by the consumers.
 // nibble: the expanded records take eight bytes each (n - m <= 4: byte j of a record's two words holds element j in
 // its low and element j + 4 in its high half), which lets full blocks with many wide groups still fit.
+// plain (n - m = 2): the records are used as they are staged, four bytes each; the only expanded slot is the one that narrow
+// groups point to. Every group of a block fits.
 struct StageLayout {
     uint32_t mask, rank, low, smhi, sm, raw, expanded, cap, bytes;
 };
 constexpr uint32_t kStageRankTable = kStageBytes - kRankTableBytes;  // where a stage keeps a stream's rank table
 // mapped: the stage also holds the stream's rank -> exponent table (its last 256 bytes).
-__host__ __device__ inline StageLayout make_stage_layout(int dt, int m, int hbits, bool mapped = false, bool nibble = false) {
+__host__ __device__ inline StageLayout make_stage_layout(int dt, int m, int hbits, bool mapped = false, bool nibble = false,
+                                                              bool plain = false) {
     StageLayout L;
     const uint32_t usable = mapped ? kStageRankTable : kStageBytes;
     L.mask = kStageMetaBytes;
@@ -258,12 +261,12 @@ __host__ __device__ inline StageLayout make_stage_layout(int dt, int m, int hbit
     L.smhi = L.low + kBlockElems * uint32_t(m) / 8;
     L.sm = L.smhi + (dt == ENEC_FP16 ? kBlockElems * 3 / 8 : 0);
     L.raw = L.sm + kBlockElems;  // at most 35072 (m = 8, or fp16 with m = 5), so a stage always has room
-    const uint32_t expanded_size = nibble ? 8 : 16;
+    const uint32_t expanded_size = plain ? 0 : nibble ? 8 : 16;
     uint32_t cap = hbits > 0 ? (usable - L.raw - 64) / (uint32_t(2 * hbits) + expanded_size) : 0;
     if (cap > kGroupsPerBlock) cap = kGroupsPerBlock;
     L.cap = cap;
     L.expanded = L.raw + uint32_t(align16(uint64_t(cap) * 2 * hbits + 32));
-    L.bytes = L.expanded + (cap + 1) * expanded_size;
+    L.bytes = L.expanded + (plain ? 16 : (cap + 1) * expanded_size);
     return L;
 }
 static_assert(kStageMetaBytes + kGroupsPerBlock / 8 + kGroupsPerBlock * 2 + 2 * kBlockElems + 64 + kRankTableBytes <= kStageBytes,
@@ -283,10 +286,11 @@ struct RunCtx {
     int n;
 };
 
-// The eight-byte form of the expanded records exists in the fp16 kernel only: fp16 weights have five exponent
-// bits and (n, m) = (5, 3), so half of their groups can be wide, more than a stage holds in the sixteen-byte form;
-// the bf16 and fp32 kernels, whose blocks fit, carry none of its code (measured: with it their one-stream rate
+// The other forms of the records exist in the fp16 kernel only: fp16 weights have five exponent
+// bits and (n, m) = (5, 3), so half of their groups and more can be wide, more than a stage holds in the sixteen-byte form;
+// the bf16 and fp32 kernels, whose blocks fit, carry none of their code (measured: with it their one-stream rate
 // fell by 1.5 to 4 %, from code layout alone).
+enum RecordForm : int { kSixteenBytes = 0, kEightBytes = 1, kStaged = 2 };   // bits 8..7 of BlockDesc::code
 template <int DT, bool MAPPED>
 constexpr bool kNibbleForm = DT == ENEC_FP16 && !MAPPED;
 
@@ -448,13 +452,18 @@ __device__ __forceinline__ void decode_block(const RunCtx& r, uint32_t s_low, ui
 // The frequency-rank variant (MAPPED) has no sign position: nothing is flipped, the slot of narrow groups holds
 // zeros, and the exponent comes from the stage's rank table (shared address in r.c4) instead of the subtraction.
 // tid = 0..255; thread tid owns the runs c * 2048 + 8 tid (c < 8).
-// NIBBLE: the expanded records are in the eight-byte form (see StageLayout).
-template <int DT, int M, int HB, bool MAPPED = false, bool NIBBLE = false>
+// FORM: how the records are kept (see StageLayout). kStaged: a record of two-bit values is one word whose bytes 0, 2, 1, 3 are
+// the four lanes of Algorithm 2; the bits of elements 0..3, 4..7, 8..11, 12..15 sit at 0, 4, 2, 6 of each byte. Unpacking it
+// where it is used costs no more than reading an expanded one, every group of a block has room, and there is nothing to
+// expand: 4099 x 4093 heavy-tailed fp16 with 650 wide groups per block (the eight-byte form holds 608) 21.7 -> 17.9 us,
+// 4096 x 4096 with 490 15.6 -> 14.4 us.
+template <int DT, int M, int HB, bool MAPPED = false, int FORM = kSixteenBytes>
 __device__ __forceinline__ void decode_full_block(const RunCtx& r, uint32_t s_low, uint32_t s_smhi, uint32_t tid) {
     constexpr int n = M + HB;
     constexpr uint32_t Hm = 0x80808080u;
     const uint32_t rank_addr = r.rank + (tid >> 1) * 2;
-    const uint32_t exp_addr = r.expanded + (tid & 1) * (NIBBLE ? 4 : 8);
+    const uint32_t exp_addr = FORM == kStaged ? r.expanded : r.expanded + (tid & 1) * (FORM == kEightBytes ? 4 : 8);
+    [[maybe_unused]] const uint32_t half_shift = 2 * (tid & 1);
     const uint32_t sm_addr = r.sm + 8 * tid;
     uint4* out = reinterpret_cast<uint4*>(r.out + 8 * tid);
     [[maybe_unused]] uint32_t* out32 = reinterpret_cast<uint32_t*>(r.out) + 8 * tid;
@@ -483,7 +492,10 @@ __device__ __forceinline__ void decode_full_block(const RunCtx& r, uint32_t s_lo
         if constexpr (HB > 0) {
 #pragma unroll
             for (int q = 0; q < 4; ++q) {
-                if constexpr (NIBBLE) {
+                if constexpr (FORM == kStaged) {
+                    const uint32_t w = (prmt(lds32(exp_addr + rk[4 * h + q] * 4), 0u, 0x3120u) ^ 0xAAAAAAAAu) >> half_shift;
+                    hi[q] = make_uint2(w & 0x03030303u, (w >> 4) & 0x03030303u);
+                } else if constexpr (FORM == kEightBytes) {
                     const uint32_t w = lds32(exp_addr + rk[4 * h + q] * 8);
                     hi[q] = make_uint2(w & 0x0F0F0F0Fu, (w >> 4) & 0x0F0F0F0Fu);
                 } else {
@@ -653,7 +665,7 @@ struct BlockDesc {
     uint32_t expect;    // wide groups of the block according to the prefix table
     uint32_t N;         // padded block length
     uint32_t real;      // real elements
-    uint32_t code;      // m * 8 + (n - m); bit 7: the expanded records take the eight-byte form
+    uint32_t code;      // m * 8 + (n - m); bits 8..7: RecordForm
     uint32_t b, n;
     StageLayout L;
     uint16_t* out;        // global: first element of the block
@@ -969,14 +981,20 @@ enec_decode_kernel(const __grid_constant__ DecodeBatch batch, int* status) {
                 failed = true;
                 break;
             }
-            // a full block with more wide groups than the stage holds in the sixteen-byte form takes the eight-byte
-            // form when that holds them all (and its consumers will take the branch-free body)
+            // fp16: a full block whose records have two bits per value is used as it is staged; one with more wide groups than
+            // the stage holds in the sixteen-byte form takes the eight-byte form when that holds them all (its
+            // consumers take the branch-free body either way)
             StageLayout Lb = L;
-            bool nibble = false;
-            if (kNibbleForm<DT, MAPPED> && hbits >= 1 && hbits <= 4 && expect > L.cap && real == kBlockElems &&
+            uint32_t form = kSixteenBytes;
+            if (kNibbleForm<DT, MAPPED> && hbits >= 1 && hbits <= 4 && real == kBlockElems &&
                 plain_subtraction<DT>(uint32_t(blk_b), uint32_t(blk_n))) {
-                const StageLayout L8 = make_stage_layout(DT, blk_m, hbits, false, true);
-                if (expect <= L8.cap) { Lb = L8; nibble = true; }
+                if (hbits == 2 && (h0 & 3) == 0) {   // (with parameters per block a block's records may start between words)
+                    Lb = make_stage_layout(DT, blk_m, hbits, false, false, true);
+                    form = kStaged;
+                } else if (expect > L.cap) {
+                    const StageLayout L8 = make_stage_layout(DT, blk_m, hbits, false, true);
+                    if (expect <= L8.cap) { Lb = L8; form = kEightBytes; }
+                }
             }
             const uint64_t w0 = h0 & ~uint64_t(15);
             uint32_t staged = expect < Lb.cap ? expect : Lb.cap;  // records staged in shared memory
@@ -994,7 +1012,7 @@ enec_decode_kernel(const __grid_constant__ DecodeBatch batch, int* status) {
             d->expect = expect;
             d->N = N;
             d->real = real;
-            d->code = uint32_t(blk_m * 8 + hbits) | (nibble ? 128u : 0u);
+            d->code = uint32_t(blk_m * 8 + hbits) | (form << 7);
             d->b = uint32_t(blk_b);
             d->n = uint32_t(blk_n);
             d->L = Lb;
@@ -1057,7 +1075,8 @@ enec_decode_kernel(const __grid_constant__ DecodeBatch batch, int* status) {
         const BlockDesc* d = reinterpret_cast<const BlockDesc*>(smem + sizeof(DecodeShared) + size_t(s) * kStageBytes);
         if (TICKET && d->N == 0) break;  // the loader's end mark
         const uint32_t N = d->N, expect = d->expect, code = kNibbleForm<DT, MAPPED> ? d->code & 127u : d->code;
-        const bool nibble = kNibbleForm<DT, MAPPED> && (d->code & 128u) != 0;  // only set for blocks that take the branch-free body
+        const uint32_t form = kNibbleForm<DT, MAPPED> ? d->code >> 7 : uint32_t(kSixteenBytes);  // others only for blocks that take the branch-free body
+        const bool nibble = form == kEightBytes;
         const uint32_t b = d->b, n = d->n;
         const uint32_t hbits = code & 7;
         const uint32_t cap = d->L.cap;
@@ -1071,15 +1090,18 @@ enec_decode_kernel(const __grid_constant__ DecodeBatch batch, int* status) {
             // the branch-free body wants narrow groups to point at the flip slot and flipped records
             const uint32_t flip4 = MAPPED ? 0u : rep4(1u << (hbits - 1));
             if (tid == 0) {
-                if (nibble) sts64(st + o_exp + cap * 8, make_uint2(flip4 | (flip4 << 4), flip4 | (flip4 << 4)));
+                if (form == kStaged) sts32(st + o_exp, 0);
+                else if (nibble) sts64(st + o_exp + cap * 8, make_uint2(flip4 | (flip4 << 4), flip4 | (flip4 << 4)));
                 else sts128(st + o_exp + cap * 16, make_uint4(flip4, flip4, flip4, flip4));
             }
-            const uint32_t wide = build_rank_array(st + d->L.mask, st + o_rank, N, tid, full_block ? cap : kNotWide);
+            // staged records are counted in words from the block's first one on, the slot of narrow groups too
+            const uint32_t narrow = form == kStaged ? (o_exp - o_raw - d->first) / 4 : cap;
+            const uint32_t wide = build_rank_array(st + d->L.mask, st + o_rank, N, tid, full_block ? narrow : kNotWide);
             if (wide != expect && lane == 0) {  // the prefix table must agree with the mask
                 *abort_flag = 1;
                 report(status, ENEC_ERR_BAD_STREAM);
             }
-            expand_records_any(int(hbits), st + o_raw + d->first, st + o_exp, d->staged, tid, full_block ? flip4 : 0, nibble);
+            if (form != kStaged) expand_records_any(int(hbits), st + o_raw + d->first, st + o_exp, d->staged, tid, full_block ? flip4 : 0, nibble);
         }
         RunCtx r;
         {
@@ -1093,7 +1115,7 @@ enec_decode_kernel(const __grid_constant__ DecodeBatch batch, int* status) {
             r.cap = cap;
             r.sm = st + o_sm;
             r.rank = st + o_rank;
-            r.expanded = st + o_exp;
+            r.expanded = form == kStaged ? st + o_raw + d->first : st + o_exp;
             r.out = d->out;
             r.high = d->high;
             r.lo = d->lo;
@@ -1101,13 +1123,22 @@ enec_decode_kernel(const __grid_constant__ DecodeBatch batch, int* status) {
             r.real = d->real;
         }
         if (consumer_barrier_or(*abort_flag != 0)) break;
-        if (nibble) {  // a full block with more wide groups than the sixteen-byte form holds
+        if (form == kStaged) {
+            if constexpr (kNibbleForm<DT, MAPPED>) {
+                switch (code) {
+                    case 1 * 8 + 2: decode_full_block<DT, 1, 2, false, kStaged>(r, st + o_low, st + o_smhi, tid); break;
+                    case 2 * 8 + 2: decode_full_block<DT, 2, 2, false, kStaged>(r, st + o_low, st + o_smhi, tid); break;
+                    case 3 * 8 + 2: decode_full_block<DT, 3, 2, false, kStaged>(r, st + o_low, st + o_smhi, tid); break;
+                    default: break;
+                }
+            }
+        } else if (nibble) {  // a full block with more wide groups than the sixteen-byte form holds
             if constexpr (kNibbleForm<DT, MAPPED>) {
                 switch (code) {
 #define ENEC_CASE(DTV, MV, HV)                                                               \
     case MV * 8 + HV:                                                                        \
-        if constexpr (HV >= 1 && HV <= 4 && (DTV != ENEC_FP16 || MV + HV <= 5))               \
-            decode_full_block<DTV, MV, HV, false, true>(r, st + o_low, st + o_smhi, tid);    \
+        if constexpr (HV >= 1 && HV <= 4 && HV != 2 && (DTV != ENEC_FP16 || MV + HV <= 5))    \
+            decode_full_block<DTV, MV, HV, false, kEightBytes>(r, st + o_low, st + o_smhi, tid); \
         break;
                     ENEC_FOR_EACH_MH(ENEC_CASE, DT)
                     ENEC_FOR_EACH_MH_BF16_ONLY(ENEC_CASE, DT)
