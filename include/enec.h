@@ -156,8 +156,8 @@ enec_status enec_decompress_batched(const enec_batch_item* h_items, int n_items,
                                     enec_stream_t stream);
 
 /*
- * Compress n_items tensors of one dtype with two launches (the histograms and parameter searches of all
- * tensors, then the encode of all their blocks), each tensor into a stream of its own exactly as
+ * Compress n_items tensors of one dtype with one launch (histograms, parameter searches and encode of all
+ * tensors, in waves), each tensor into a stream of its own exactly as
  * enec_compress would write it. Entries in HOST memory: d_in = values, d_out = stream buffer, count =
  * elements, size = capacity of d_out (at least enec_max_compressed_size(dt, count)). d_out_sizes (device
  * array of n_items 8-byte words, may be NULL) receives the stream lengths. Meant for checkpoints made of

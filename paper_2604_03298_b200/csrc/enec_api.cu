@@ -10,7 +10,7 @@
 #include "enec_decode.cuh"
 #include "enec_encode.cuh"
 #include "enec_blockwise.cuh"
-#include "enec_fused.cuh"
+#include "enec_fused_list.cuh"
 #include "enec_launch.cuh"
 
 namespace enec {
@@ -21,10 +21,10 @@ struct DeviceInfo {
     int sms = 0;
     bool hist_attr_set[3] = {false, false, false};
     bool encode_attr_set[3] = {false, false, false};
-    bool batch_attr_set[3] = {false, false, false};
     bool blockwise_attr_set[3] = {false, false, false};
     bool split_attr_set[3] = {false, false, false};
     bool fused_attr_set[3] = {false, false, false};
+    bool fused_list_attr_set[3] = {false, false, false};
 };
 
 // Per-device facts, for device ordinals below kMaxDevices (null beyond: the caller fails with ENEC_ERR_CUDA).
@@ -232,9 +232,9 @@ static enec_status launch_encode(const EncodeJob& job, uint32_t nblocks, bool se
         if (may_split && !job.ranked && nblocks >= split_min_blocks() && nblocks < split_max_blocks()) return launch_split<DT>(job, nblocks, d_status, info, stream);
     }
     if (!info.encode_attr_set[DT]) {
-        if (cudaFuncSetAttribute(enec_encode_kernel<DT, false, false>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+        if (cudaFuncSetAttribute(enec_encode_kernel<DT, false>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                  int(EncodeSmem<DT>::kBytes)) != cudaSuccess ||
-            cudaFuncSetAttribute(enec_encode_kernel<DT, false, true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+            cudaFuncSetAttribute(enec_encode_kernel<DT, true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                  int(EncodeSmem<DT>::kBytes)) != cudaSuccess)
             return ENEC_ERR_CUDA;
         info.encode_attr_set[DT] = true;
@@ -242,39 +242,10 @@ static enec_status launch_encode(const EncodeJob& job, uint32_t nblocks, bool se
     uint32_t grid = uint32_t(info.sms) * 4;  // four resident CTAs per SM, each takes block after block
     if (grid > nblocks) grid = nblocks;
     const cudaError_t err =
-        job.ranked ? launch_pdl(enec_encode_kernel<DT, false, true>, grid, kEncodeThreads, EncodeSmem<DT>::kBytes, stream,
-                                job, EncodeBatch{}, d_status)
-                   : launch_pdl(enec_encode_kernel<DT, false, false>, grid, kEncodeThreads, EncodeSmem<DT>::kBytes, stream,
-                                job, EncodeBatch{}, d_status);
-    g_launches.fetch_add(1, std::memory_order_relaxed);
-    return err == cudaSuccess ? ENEC_OK : ENEC_ERR_CUDA;
-}
-
-// The two launches of a batched compress call: histograms and parameter search of every tensor, then the
-// encode of all their blocks.
-template <int DT>
-static enec_status launch_encode_batched(const EncodeJob* d_jobs, const HistUnit* d_units, uint32_t n_units,
-                                         const EncodeBatch& batch, int* d_status, DeviceInfo& info, cudaStream_t stream) {
-    const uint32_t hist_smem = HistShape<DT>::kBytes;
-    if (!info.batch_attr_set[DT]) {
-        if (cudaFuncSetAttribute(enec_histogram_batched_kernel<DT>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                 int(hist_smem)) != cudaSuccess ||
-            cudaFuncSetAttribute(enec_encode_kernel<DT, true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                 int(EncodeSmem<DT>::kBytes)) != cudaSuccess)
-            return ENEC_ERR_CUDA;
-        info.batch_attr_set[DT] = true;
-    }
-    uint32_t grid = uint32_t(info.sms) * 3;
-    if (grid > n_units) grid = n_units;
-    // the second word of the call's ticket area hands out the histogram units (the first one the blocks of the encode)
-    if (launch_pdl(enec_histogram_batched_kernel<DT>, grid, kHistThreads, hist_smem, stream, d_jobs, d_units, n_units,
-                   batch.ticket + 4) != cudaSuccess)
-        return ENEC_ERR_CUDA;
-    g_launches.fetch_add(1, std::memory_order_relaxed);
-    grid = uint32_t(info.sms) * 4;
-    if (grid > batch.total_blocks) grid = batch.total_blocks;
-    const cudaError_t err = launch_pdl(enec_encode_kernel<DT, true>, grid, kEncodeThreads, EncodeSmem<DT>::kBytes, stream,
-                                       EncodeJob{}, batch, d_status);
+        job.ranked ? launch_pdl(enec_encode_kernel<DT, true>, grid, kEncodeThreads, EncodeSmem<DT>::kBytes, stream,
+                                job, d_status)
+                   : launch_pdl(enec_encode_kernel<DT, false>, grid, kEncodeThreads, EncodeSmem<DT>::kBytes, stream,
+                                job, d_status);
     g_launches.fetch_add(1, std::memory_order_relaxed);
     return err == cudaSuccess ? ENEC_OK : ENEC_ERR_CUDA;
 }
@@ -707,74 +678,98 @@ enec_status enec_compress_batched(const enec_batch_item* h_items, int n_items, e
     if (cudaStreamIsCapturing(stream, &capturing) != cudaSuccess) return ENEC_ERR_CUDA;
     if (capturing != cudaStreamCaptureStatusNone) return ENEC_ERR_INVALID_ARG;
     unsigned long long* sizes = reinterpret_cast<unsigned long long*>(d_out_sizes);
-    // device scratch of the call: [ticket | control words per tensor | state word per block | jobs | prefix | units];
-    // everything in front of the tables is cleared, the tables are copied from the host
-    constexpr size_t kCtlStride = (sizeof(EncodeControl) + 63) & ~size_t(63);
-    std::vector<uint32_t> prefix(size_t(n_items) + 1);
-    std::vector<HistUnit> units;
-    uint64_t total_blocks = 0;
+    // tensors of two blocks or more first, each from a multiple of kHistBlocks on in the index space of blocks, then those of
+    // one block; tensors without elements are written by launches of their own
+    std::vector<FusedListItem> items;
+    std::vector<uint32_t> chunk_item;
+    items.reserve(size_t(n_items));
+    uint64_t index = 0, state_words = 0;
+    uint32_t n_multi = 0;
+    auto add = [&](int i, uint64_t first_block, uint32_t nblocks) {
+        items.push_back(FusedListItem{static_cast<const uint8_t*>(h_items[i].d_in), static_cast<uint8_t*>(h_items[i].d_out),
+                                      uint64_t(h_items[i].count), sizes ? sizes + i : nullptr, nullptr, nullptr, nullptr,
+                                      uint32_t(first_block), nblocks});
+    };
     for (int i = 0; i < n_items; ++i) {
-        prefix[i] = uint32_t(total_blocks);
-        const uint64_t count = h_items[i].count;
-        if (count == 0) continue;  // written by a launch of its own below
-        total_blocks += make_geometry(count).nblocks;
-        const uint64_t chunks = (count * uint64_t(elem_bytes(dt))) >> 4;
-        const uint32_t n = chunks ? uint32_t((chunks + kHistUnitChunks - 1) / kHistUnitChunks) : 1u;
-        for (uint32_t u = 0; u < n; ++u) units.push_back(HistUnit{uint32_t(i), u, n, 0u});
+        const uint32_t nblocks = make_geometry(h_items[i].count).nblocks;
+        if (nblocks < 2) continue;
+        if ((index + nblocks) >> 31) return ENEC_ERR_INVALID_ARG;  // block indices are 32-bit
+        add(i, index, nblocks);
+        const uint64_t chunks = (nblocks + kHistBlocks - 1) / kHistBlocks;
+        chunk_item.insert(chunk_item.end(), size_t(chunks), n_multi);
+        index += chunks * kHistBlocks;
+        state_words += nblocks + (nblocks + kSuperBlocks - 1) / kSuperBlocks + nblocks / (kSuperBlocks * kHyperSupers) + 1;
+        ++n_multi;
     }
-    if (total_blocks >> 32) return ENEC_ERR_INVALID_ARG;
-    prefix[n_items] = uint32_t(total_blocks);
-    const size_t off_ctl = 256;
-    const size_t off_state = (off_ctl + size_t(n_items) * kCtlStride + 255) & ~size_t(255);
-    const size_t off_jobs = (off_state + size_t(total_blocks) * sizeof(unsigned long long) + 255) & ~size_t(255);
-    const size_t off_prefix = off_jobs + size_t(n_items) * sizeof(EncodeJob);
-    const size_t off_units = (off_prefix + prefix.size() * sizeof(uint32_t) + 15) & ~size_t(15);
-    const size_t need = off_units + units.size() * sizeof(HistUnit);
-    uint8_t* scratch = nullptr;
-    const enec_status st = get_scratch(dev, stream, kScratchCompressBatch, need, &scratch);
-    if (st != ENEC_OK) return st;
-    std::vector<uint8_t> host(need - off_jobs);
-    EncodeJob* jobs = reinterpret_cast<EncodeJob*>(host.data());
+    const uint32_t multi_blocks = uint32_t(index);
     for (int i = 0; i < n_items; ++i) {
-        EncodeJob& job = jobs[i];
-        job.in = static_cast<const uint16_t*>(h_items[i].d_in);
-        job.out = static_cast<uint8_t*>(h_items[i].d_out);
-        job.count = h_items[i].count;
-        job.ctl = reinterpret_cast<EncodeControl*>(scratch + off_ctl + size_t(i) * kCtlStride);
-        job.ctl_next = nullptr;
-        job.state = reinterpret_cast<unsigned long long*>(scratch + off_state) + prefix[i];
-        job.epoch = 1;  // the area was just cleared
-        job.out_size = sizes ? sizes + i : nullptr;
-        job.b = 0; job.n = 0; job.m = 0;
-        job.from_search = 1;
-        job.check = 0;
-        job.ranked = 0;
-    }
-    memcpy(host.data() + (off_prefix - off_jobs), prefix.data(), prefix.size() * sizeof(uint32_t));
-    if (!units.empty()) memcpy(host.data() + (off_units - off_jobs), units.data(), units.size() * sizeof(HistUnit));
-    for (int i = 0; i < n_items; ++i) {
+        if (make_geometry(h_items[i].count).nblocks == 1) add(i, index++, 1u);
         if (h_items[i].count != 0) continue;
         enec_encode_empty_kernel<<<1, 32, 0, stream>>>(static_cast<uint8_t*>(h_items[i].d_out), int(dt), 0, 1, 1,
                                                       sizes ? sizes + i : nullptr);
         g_launches.fetch_add(1, std::memory_order_relaxed);
         if (cudaGetLastError() != cudaSuccess) return ENEC_ERR_CUDA;
     }
-    if (total_blocks == 0) return ENEC_OK;
-    if (cudaMemsetAsync(scratch, 0, off_jobs, stream) != cudaSuccess) return ENEC_ERR_CUDA;
+    if (items.empty()) return ENEC_OK;
+    if (index >> 31) return ENEC_ERR_INVALID_ARG;
+    // the order of the units
+    std::vector<FusedListSegment> segments;
+    uint32_t tickets = 0;
+    auto segment = [&](uint32_t kind, uint32_t first, uint32_t end) {
+        if (first == end) return;
+        segments.push_back(FusedListSegment{tickets, first, kind});
+        tickets += kind == kUnitCount ? (end - first) / kHistBlocks : end - first;
+    };
+    std::vector<uint32_t> wave{0};   // first blocks of the waves, and the end of the last
+    for (uint32_t j = 0; j < n_multi; ++j) {
+        const uint32_t end = j + 1 < n_multi ? items[j + 1].first_block : multi_blocks;
+        if (j + 1 == n_multi || uint64_t(end - wave.back()) * kBlockElems * elem_bytes(dt) >= kWaveBytes) wave.push_back(end);
+    }
+    const size_t waves = wave.size() - 1;
+    if (waves) segment(kUnitCount, wave[0], wave[1]);
+    segment(kUnitWhole, multi_blocks, uint32_t(index));
+    for (size_t w = 0; w < waves; ++w) {
+        if (w + 1 < waves) segment(kUnitCount, wave[w + 1], wave[w + 2]);
+        segment(kUnitPack, wave[w], wave[w + 1]);
+    }
+    segments.push_back(FusedListSegment{tickets, 0, kUnitEnd});
+    // device scratch of the call: [ticket | control words per tensor | state words and sums], cleared, and
+    // [tensors | tensor of every chunk | segments], copied from the host
+    const size_t off_controls = 256;
+    const size_t off_state = off_controls + size_t(n_multi) * sizeof(FusedItemControl);
+    const size_t off_items = (off_state + size_t(state_words) * sizeof(unsigned long long) + 255) & ~size_t(255);
+    const size_t off_chunks = off_items + items.size() * sizeof(FusedListItem);
+    const size_t off_segments = off_chunks + ((chunk_item.size() + 3) & ~size_t(3)) * sizeof(uint32_t);
+    const size_t need = off_segments + segments.size() * sizeof(FusedListSegment);
+    uint8_t* scratch = nullptr;
+    const enec_status st = get_scratch(dev, stream, kScratchCompressBatch, need, &scratch);
+    if (st != ENEC_OK) return st;
+    unsigned long long* words = reinterpret_cast<unsigned long long*>(scratch + off_state);
+    for (uint32_t j = 0; j < n_multi; ++j) {
+        FusedListItem& item = items[j];
+        item.state = words;
+        item.super = item.state + item.nblocks;
+        item.hyper = item.super + (item.nblocks + kSuperBlocks - 1) / kSuperBlocks;
+        words = item.hyper + item.nblocks / (kSuperBlocks * kHyperSupers) + 1;
+    }
+    std::vector<uint8_t> host(need - off_items);
+    memcpy(host.data(), items.data(), items.size() * sizeof(FusedListItem));
+    if (!chunk_item.empty()) memcpy(host.data() + (off_chunks - off_items), chunk_item.data(), chunk_item.size() * sizeof(uint32_t));
+    memcpy(host.data() + (off_segments - off_items), segments.data(), segments.size() * sizeof(FusedListSegment));
+    if (cudaMemsetAsync(scratch, 0, off_items, stream) != cudaSuccess) return ENEC_ERR_CUDA;
     // pageable source: the call returns once the bytes are staged, so `host` may go out of scope
-    if (cudaMemcpyAsync(scratch + off_jobs, host.data(), host.size(), cudaMemcpyHostToDevice, stream) != cudaSuccess)
+    if (cudaMemcpyAsync(scratch + off_items, host.data(), host.size(), cudaMemcpyHostToDevice, stream) != cudaSuccess)
         return ENEC_ERR_CUDA;
-    EncodeBatch batch;
-    batch.jobs = reinterpret_cast<const EncodeJob*>(scratch + off_jobs);
-    batch.prefix = reinterpret_cast<const uint32_t*>(scratch + off_prefix);
-    batch.n_jobs = uint32_t(n_items);
-    batch.total_blocks = uint32_t(total_blocks);
-    batch.ticket = reinterpret_cast<uint32_t*>(scratch);
-    const HistUnit* d_units = reinterpret_cast<const HistUnit*>(scratch + off_units);
-    const uint32_t n_units = uint32_t(units.size());
-    return dt == ENEC_BF16   ? launch_encode_batched<ENEC_BF16>(batch.jobs, d_units, n_units, batch, d_status, info, stream)
-           : dt == ENEC_FP16 ? launch_encode_batched<ENEC_FP16>(batch.jobs, d_units, n_units, batch, d_status, info, stream)
-                             : launch_encode_batched<ENEC_FP32>(batch.jobs, d_units, n_units, batch, d_status, info, stream);
+    FusedList list;
+    list.items = reinterpret_cast<const FusedListItem*>(scratch + off_items);
+    list.controls = reinterpret_cast<FusedItemControl*>(scratch + off_controls);
+    list.chunk_item = reinterpret_cast<const uint32_t*>(scratch + off_chunks);
+    list.segments = reinterpret_cast<const FusedListSegment*>(scratch + off_segments);
+    list.n_segments = uint32_t(segments.size() - 1);
+    list.n_multi = n_multi;
+    list.multi_blocks = multi_blocks;
+    list.ticket = reinterpret_cast<uint32_t*>(scratch);
+    return launch_fused_list(int(dt), list, tickets, info.sms, info.fused_list_attr_set, d_status, stream);
 }
 
 enec_status enec_compress_noalloc(const void* d_in, enec_dtype dt, size_t count, void* d_out, size_t out_capacity,

@@ -367,95 +367,6 @@ enec_histogram_kernel(const uint16_t* __restrict__ in, uint64_t count, EncodeCon
     else parameter_search<DT>(ctl);
 }
 
-// Histograms of a list of tensors in one launch. The tensors are cut into units of at most kHistUnitChunks
-// 16-byte loads; a CTA takes unit after unit, adds the unit's counts to its tensor's histogram, and the CTA
-// that finishes a tensor's last outstanding unit runs that tensor's parameter search.
-constexpr uint32_t kHistUnitChunks = 16384;  // 256 KB
-struct HistUnit {
-    uint32_t job;            // tensor of the unit
-    uint32_t index;          // unit number inside the tensor
-    uint32_t units_of_job;
-    uint32_t pad;
-};
-
-template <int DT>
-__global__ void __launch_bounds__(kHistThreads, 3)
-enec_histogram_batched_kernel(const EncodeJob* __restrict__ jobs, const HistUnit* __restrict__ units, uint32_t n_units,
-                              uint32_t* ticket) {
-    extern __shared__ __align__(128) uint8_t smem[];
-    __shared__ uint32_t cta_hist[256];
-    __shared__ int s_last;
-    constexpr int kPerLoad = HistShape<DT>::kPerLoad;
-    pdl_launch_dependents();
-    const uint32_t tid = threadIdx.x, lane = tid & 31;
-    const uint32_t base = smem_u32(smem) + lane * 4;
-    for (uint32_t i = tid; i < uint32_t(HistShape<DT>::kBytes / 16); i += kHistThreads)
-        reinterpret_cast<uint4*>(smem)[i] = make_uint4(0, 0, 0, 0);
-    cta_hist[tid] = 0;
-    __syncthreads();
-    pdl_wait();  // nothing above touches global memory
-    // CTA c starts on unit c; after that units are handed out by `ticket` (zero when the launch starts), asked for
-    // a unit ahead: the CTAs of an SM do not progress equally
-    __shared__ uint32_t s_next_unit;
-    for (uint32_t u = blockIdx.x; u < n_units;) {
-        uint32_t asked = 0;
-        if (tid == 0) asked = atomicAdd(ticket, 1u);
-        const HistUnit unit = units[u];
-        const uint16_t* in = jobs[unit.job].in;
-        const uint64_t count = jobs[unit.job].count;
-        EncodeControl* ctl = jobs[unit.job].ctl;
-        const uint64_t nchunks = count / kPerLoad;
-        const uint64_t first = uint64_t(unit.index) * kHistUnitChunks;
-        const uint64_t end = first + kHistUnitChunks < nchunks ? first + kHistUnitChunks : nchunks;
-        const uint4* in4 = reinterpret_cast<const uint4*>(in);
-        for (uint64_t at = first + tid; at < end; at += 4 * kHistThreads) {
-            uint4 v[4];
-#pragma unroll
-            for (uint32_t q = 0; q < 4; ++q) {
-                v[q] = make_uint4(0, 0, 0, 0);
-                if (at + q * kHistThreads < end) v[q] = in4[at + q * kHistThreads];
-            }
-#pragma unroll
-            for (uint32_t q = 0; q < 4; ++q) {
-                if (at + q * kHistThreads < end) {
-                    count_word_pair<DT>(base, v[q].x);
-                    count_word_pair<DT>(base, v[q].y);
-                    count_word_pair<DT>(base, v[q].z);
-                    count_word_pair<DT>(base, v[q].w);
-                }
-            }
-        }
-        __syncthreads();
-        // fold the row of bin `tid` and clear it for the next unit
-        if (tid < uint32_t(HistShape<DT>::kBins)) cta_hist[tid] = fold_hist_row<true>(smem_u32(smem) + tid * HistShape<DT>::kRowBytes, tid);
-        __syncthreads();
-        if (tid == 0 && unit.index + 1 == unit.units_of_job) {  // the values behind the last whole 16-byte load
-            constexpr int sh = DT == ENEC_BF16 ? 7 : 10;
-            for (uint64_t e = nchunks * kPerLoad; e < count; ++e) {
-                const uint32_t x = DT == ENEC_FP32 ? (reinterpret_cast<const uint32_t*>(in)[e] >> 23) & 0xFFu
-                                                   : (uint32_t(in[e]) >> sh) & (HistShape<DT>::kBins - 1);
-                cta_hist[x] += 1;
-            }
-        }
-        __syncthreads();
-        if (cta_hist[tid]) atomicAdd(&ctl->hist[tid], (unsigned long long)cta_hist[tid]);
-        cta_hist[tid] = 0;
-        __threadfence();
-        __syncthreads();
-        if (tid == 0) {
-            s_last = atomicAdd(&ctl->hist_done, 1u) == unit.units_of_job - 1;
-            s_next_unit = gridDim.x + asked;
-        }
-        __syncthreads();
-        u = s_next_unit;
-        if (s_last) {
-            __threadfence();
-            parameter_search<DT>(ctl);
-        }
-        __syncthreads();
-    }
-}
-
 // ---------------------------------------------------------------------------------------------------
 // Algorithm 2 on packed bytes (forward). A thread that owns the eight lanes j..j+7 of the deepest level
 // owns, at every level, whole runs of eight consecutive lanes: the 64 elements {j + c N/8 + i : c, i < 8}.
@@ -987,24 +898,6 @@ __device__ __forceinline__ void resolve_block(const EncodeJob& job, const Encode
     }
 }
 
-// A list of tensors compressed by one launch: the blocks of all tensors form one index space that the
-// CTAs' tickets run over; every tensor keeps its own control words, state words and output.
-struct EncodeBatch {
-    const EncodeJob* jobs;   // device array [n_jobs]
-    const uint32_t* prefix;  // device array [n_jobs + 1]: blocks before each tensor
-    uint32_t n_jobs;
-    uint32_t total_blocks;
-    uint32_t* ticket;        // next block of the index space (zero when the launch starts)
-};
-
-// What a block needs to know about its tensor (batched launches keep it in shared memory per block).
-struct BlockCtx {
-    EncodeJob job;
-    EncodeTensor tensor;
-    TransformCtx tc;
-    uint32_t k;  // block index inside the tensor
-};
-
 template <int DT, bool RANKED = false>
 __device__ __forceinline__ void fill_tensor_ctx(const EncodeJob& job, EncodeTensor& tensor, TransformCtx& tc) {
     constexpr int E = DT == ENEC_FP16 ? 5 : 8;
@@ -1023,12 +916,11 @@ __device__ __forceinline__ void fill_tensor_ctx(const EncodeJob& job, EncodeTens
     tc.lut = 0;
 }
 
-// BATCH = false: one tensor, described by `single`. BATCH = true: the tensors of `batch`; `single` is unused.
-// RANKED (one tensor only): the frequency-rank variant; a separate instance, so that the usual one carries
+// RANKED: the frequency-rank variant; a separate instance, so that the usual one carries
 // nothing of the table look-ups.
-template <int DT, bool BATCH, bool RANKED = false>
+template <int DT, bool RANKED = false>
 __global__ void __launch_bounds__(kEncodeThreads, 4)
-enec_encode_kernel(const EncodeJob single, const EncodeBatch batch, int* status) {
+enec_encode_kernel(const EncodeJob job, int* status) {
     // dynamic shared memory: low plane | fp16 sign/mantissa-high plane | two record buffers
     extern __shared__ __align__(16) uint8_t enc_smem[];
     uint8_t* s_low = enc_smem;                                   // normalised bytes of the low plane
@@ -1040,32 +932,21 @@ enec_encode_kernel(const EncodeJob single, const EncodeBatch batch, int* status)
     pdl_wait();  // nothing above touches global memory
     const uint32_t tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     __shared__ uint8_t s_lut[RANKED ? 256 : 1];
-    __shared__ BlockCtx s_ctx[BATCH ? 3 : 1];  // batched: this block's, the previous block's and the next block's tensor
-    EncodeTensor single_tensor{};
-    TransformCtx single_tc{};
-    if constexpr (!BATCH) {
-        if (blockIdx.x == 0) {  // the next call on this scratch area finds its control set zeroed
-            single.ctl_next->hist[tid] = 0;
-            if (tid == 0) { single.ctl_next->ticket = 0; single.ctl_next->hist_done = 0; single.ctl_next->reserved = 0; }
-        }
-        fill_tensor_ctx<DT, RANKED>(single, single_tensor, single_tc);
-        if constexpr (RANKED) {  // the exponent -> rank table of the tensor, for every block of this CTA
-            s_lut[tid] = single.ctl->lut[tid];
-            single_tc.lut = smem_u32(s_lut);
-        }
+    EncodeTensor tensor{};
+    TransformCtx tc{};
+    if (blockIdx.x == 0) {  // the next call on this scratch area finds its control set zeroed
+        job.ctl_next->hist[tid] = 0;
+        if (tid == 0) { job.ctl_next->ticket = 0; job.ctl_next->hist_done = 0; job.ctl_next->reserved = 0; }
     }
-    uint32_t* const ticket = BATCH ? batch.ticket : &single.ctl->ticket;
-    const uint32_t total_blocks = BATCH ? batch.total_blocks : single_tensor.g.nblocks;
-    // batched, thread 0 only: the tensor of a ticket (tickets of a CTA grow, so the search only moves forward)
-    uint32_t ctx_j = 0;
-    auto stage_ctx = [&](uint32_t ticket_value, uint32_t slot) {
-        if (ticket_value >= total_blocks) return;
-        while (batch.prefix[ctx_j + 1] <= ticket_value) ++ctx_j;
-        BlockCtx& cx = s_ctx[slot];
-        cx.job = batch.jobs[ctx_j];
-        fill_tensor_ctx<DT>(cx.job, cx.tensor, cx.tc);
-        cx.k = ticket_value - batch.prefix[ctx_j];
-    };
+    fill_tensor_ctx<DT, RANKED>(job, tensor, tc);
+    if constexpr (RANKED) {  // the exponent -> rank table of the tensor, for every block of this CTA
+        s_lut[tid] = job.ctl->lut[tid];
+        tc.lut = smem_u32(s_lut);
+    }
+    uint32_t* const ticket = &job.ctl->ticket;
+    const Geometry& g = tensor.g;
+    const Sections& sec = tensor.sec;
+    const int b = tensor.b, n = tensor.n, m = tensor.m, hbits = tensor.hbits;
 
     // Persistent loop over tickets. A block's look-back is put off until the CTA has done the first half of
     // its next block: by then the predecessors, which started at about the same time, have published their
@@ -1074,27 +955,14 @@ enec_encode_kernel(const EncodeJob single, const EncodeBatch batch, int* status)
     // waits end.
     uint32_t pending_block = 0xFFFFFFFFu, pending_wide = 0, cur = 0;
     bool pending_bad = false;
-    if (tid == 0) {
-        sh.next[0] = atomicAdd(ticket, 1u);
-        if constexpr (BATCH) stage_ctx(sh.next[0], 0);
-    }
+    if (tid == 0) sh.next[0] = atomicAdd(ticket, 1u);
     uint32_t iter = 0;
     for (;; ++iter) {
     __syncthreads();
-    if (sh.next[iter & 1] >= total_blocks) break;
+    if (sh.next[iter & 1] >= g.nblocks) break;
     // the ticket after this one goes to the other slot, which nobody reads before the next barrier
-    if (tid == 0) {
-        sh.next[(iter + 1) & 1] = atomicAdd(ticket, 1u);
-        if constexpr (BATCH) stage_ctx(sh.next[(iter + 1) & 1], (iter + 1) % 3);
-    }
-    const BlockCtx& cx = s_ctx[BATCH ? iter % 3 : 0];
-    const EncodeJob& job = BATCH ? cx.job : single;
-    const EncodeTensor& tensor = BATCH ? cx.tensor : single_tensor;
-    const TransformCtx& tc = BATCH ? cx.tc : single_tc;
-    const Geometry& g = tensor.g;
-    const Sections& sec = tensor.sec;
-    const int b = tensor.b, n = tensor.n, m = tensor.m, hbits = tensor.hbits;
-    const uint32_t k = BATCH ? cx.k : sh.next[iter & 1];
+    if (tid == 0) sh.next[(iter + 1) & 1] = atomicAdd(ticket, 1u);
+    const uint32_t k = sh.next[iter & 1];
     uint8_t* s_rec = s_rec_base + cur * EncodeSmem<DT>::kRecBytes;
     const bool last = k + 1 == g.nblocks;
     const uint32_t N = last ? g.tail_padded : kBlockElems;
@@ -1229,7 +1097,7 @@ enec_encode_kernel(const EncodeJob single, const EncodeBatch batch, int* status)
     {
         // the CTA's next block is known by now: pull its 32 KB towards L2 (one 128-byte line per thread, two for fp32)
         // so that the loads of the next iteration do not wait for DRAM
-        const uint32_t next_block = BATCH ? 0xFFFFFFFFu : sh.next[(iter + 1) & 1];  // batched: tensors are small
+        const uint32_t next_block = sh.next[(iter + 1) & 1];
         if (next_block < g.nblocks) {
             const uint8_t* base = reinterpret_cast<const uint8_t*>(job.in);
             const uint8_t* end = base + job.count * kElemBytes;
@@ -1298,8 +1166,7 @@ enec_encode_kernel(const EncodeJob single, const EncodeBatch batch, int* status)
 
     // the previous block of this CTA, whose records wait in the other buffer
     if (pending_block != 0xFFFFFFFFu) {
-        const BlockCtx& px = s_ctx[BATCH ? (iter + 2) % 3 : 0];
-        resolve_block<DT, RANKED>(BATCH ? px.job : single, BATCH ? px.tensor : single_tensor, pending_block, pending_wide, pending_bad,
+        resolve_block<DT, RANKED>(job, tensor, pending_block, pending_wide, pending_bad,
                           s_rec_base + (cur ^ 1) * EncodeSmem<DT>::kRecBytes, sh, status);
     }
     pending_block = k;
@@ -1308,8 +1175,7 @@ enec_encode_kernel(const EncodeJob single, const EncodeBatch batch, int* status)
     cur ^= 1;
     }
     if (pending_block != 0xFFFFFFFFu) {
-        const BlockCtx& px = s_ctx[BATCH ? (iter + 2) % 3 : 0];
-        resolve_block<DT, RANKED>(BATCH ? px.job : single, BATCH ? px.tensor : single_tensor, pending_block, pending_wide, pending_bad,
+        resolve_block<DT, RANKED>(job, tensor, pending_block, pending_wide, pending_bad,
                           s_rec_base + (cur ^ 1) * EncodeSmem<DT>::kRecBytes, sh, status);
     }
 }

@@ -81,8 +81,8 @@ struct FusedShape {
     static constexpr uint32_t kListAt = kHistAt + kHistBytes;          // the wide groups' numbers, a byte each, by warp
     static constexpr uint32_t kPend = 4096;                            // a block's packed records waiting for their offset
     static constexpr uint32_t kPendAt = kListAt + 1024;
-    static constexpr uint32_t kTensorAt = kPendAt + 2 * kPend;         // FusedTensor
-    static constexpr uint32_t kSharedAt = kTensorAt + 256;             // FusedShared
+    static constexpr uint32_t kTensorAt = kPendAt + 2 * kPend;         // two FusedTensor (lists: the block's and the waiting block's)
+    static constexpr uint32_t kSharedAt = kTensorAt + 2 * 256;         // FusedShared
     static constexpr uint32_t kBytes = kSharedAt + 256;
     static_assert(HistShape<DT>::kBytes <= int(kHistAt + kHistBytes), "the sample stage's table fits");
     static_assert(kCtasPerSm * (kBytes + 1024) <= 228 * 1024, "the CTAs of an SM fit its shared memory");
@@ -115,6 +115,7 @@ struct FusedTensor {
     uint32_t wide_ok;  // bit 0: the input is 32-byte aligned, bit 1: the sm-lo plane is
     uint32_t plain;
     uint32_t smhi_at, values_at;   // shared memory: where the fp16 plane and the values start
+    uint32_t first_block;          // lists: index of the tensor's first block in the list's index space
 };
 
 struct FusedShared {
@@ -123,6 +124,7 @@ struct FusedShared {
     uint32_t word;       // broadcasts of thread 0
     uint32_t before;
     uint32_t ok;
+    uint32_t unit[2][2];          // lists: what the CTA does now and next, see FusedListUnit
     uint32_t part[kFusedWarps];   // each warp's share of the wide groups before the waiting block; kNotReady: some are not counted yet
 };
 constexpr uint32_t kNotReady = 0xFFFFFFFFu;   // a tensor has at most 2^32 - 2^10 groups of 16 counted before a block
@@ -133,7 +135,9 @@ __device__ __forceinline__ uint8_t* fused_smem() {
     return smem;
 }
 template <int DT>
-__device__ __forceinline__ FusedTensor& fused_tensor() { return *reinterpret_cast<FusedTensor*>(fused_smem() + FusedShape<DT>::kTensorAt); }
+__device__ __forceinline__ FusedTensor& fused_tensor(uint32_t slot = 0) {
+    return *reinterpret_cast<FusedTensor*>(fused_smem() + FusedShape<DT>::kTensorAt + slot * 256);
+}
 template <int DT>
 __device__ __forceinline__ FusedShared& fused_shared() { return *reinterpret_cast<FusedShared*>(fused_smem() + FusedShape<DT>::kSharedAt); }
 
@@ -758,9 +762,9 @@ __device__ __forceinline__ bool pack_front_full(const FusedTensor& t, uint32_t k
 
 // The same for the tensor's last block when it is not full and has at least 128 padded elements.
 template <int DT, bool PLAIN, bool HIST>
-__device__ __noinline__ bool pack_front_tail(uint32_t k, uint32_t* wide_of_warp) {
+__device__ __noinline__ bool pack_front_tail(uint32_t k, uint32_t* wide_of_warp, uint32_t slot = 0) {
     using Shape = FusedShape<DT>;
-    const FusedTensor& t = fused_tensor<DT>();
+    const FusedTensor& t = fused_tensor<DT>(slot);
     FusedShared& sh = fused_shared<DT>();
     constexpr uint32_t kElemBytes = DT == ENEC_FP32 ? 4 : 2;
     constexpr int E = Shape::E;
@@ -821,8 +825,8 @@ __device__ __forceinline__ uint32_t scan_mask(const uint32_t* s_mask, uint32_t l
 // A tail block of 16, 32 or 64 padded elements, all threads, one element per thread, bit by bit (Algorithm 2 followed for
 // every set bit).
 template <int DT>
-__device__ __noinline__ void pack_short_block(uint32_t k, int* status) {
-    const FusedTensor& t = fused_tensor<DT>();
+__device__ __noinline__ void pack_short_block(uint32_t k, int* status, uint32_t slot = 0) {
+    const FusedTensor& t = fused_tensor<DT>(slot);
     constexpr uint32_t kElemBytes = DT == ENEC_FP32 ? 4 : 2;
     const uint32_t tid = threadIdx.x;
     const uint32_t N = t.tail_padded, real = t.tail_real;

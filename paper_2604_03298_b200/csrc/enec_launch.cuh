@@ -23,6 +23,10 @@ struct FusedJob;
 // The one-kernel compressor on one tensor (see enec_fused.cuh).
 enec_status launch_fused(int dt, const FusedJob& job, uint32_t nblocks, int sms, bool* attr_set, int* d_status, cudaStream_t stream);
 
+struct FusedList;
+// The one-kernel compressor on a list of tensors (see enec_fused_list.cuh).
+enec_status launch_fused_list(int dt, const FusedList& list, uint32_t tickets, int sms, bool* attr_set, int* d_status, cudaStream_t stream);
+
 // Launch with programmatic stream serialisation: the kernel may be scheduled while its predecessor in the
 // stream drains; it waits for the predecessor's completion itself (pdl_wait) before touching memory.
 template <class... KernelArgs, class... Args>

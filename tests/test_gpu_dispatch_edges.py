@@ -101,3 +101,42 @@ def test_compress_when_the_sample_misleads(oracle, dt, what):
     else:
         t = torch.full_like(t, 0.75)
     assert np.array_equal(_compress_twice(enec, t, dt), oracle.compress(_words(t, dt), dt))
+
+
+@pytest.mark.parametrize("dt", [0, 1, 2])
+def test_compress_batched_across_waves(oracle, dt):
+    """A list whose tensors are counted and packed in several waves of 24 MB (one tensor is more than a wave), with tensors
+    of one block, of a few elements, and with last blocks of every kind between them."""
+    import paper_2604_03298_b200 as enec
+    counts = [16384 * 820 + 5, 16384 * 2, 100, 16384, 16385, 0, 16384 * 5 - 1, 2048, 16384 * 129, 37, 16384 * 400, 16384 * 500 + 60,
+              16384 * 3, 5, 16384 * 7 + 8000]
+    srcs = [_weights(c, dt, 70 + i, 0.02 * (1 + i % 4)) for i, c in enumerate(counts)]
+    caps = [enec.enec_max_compressed_size(dt, c) for c in counts]
+    for _ in range(2):   # twice: the call's scratch is reused
+        bufs = [torch.full((c + 16,), 0xA5, dtype=torch.uint8, device="cuda") for c in caps]
+        sizes, status = torch.zeros(len(counts), dtype=torch.int64, device="cuda"), status_tensor()
+        assert enec.enec_compress_batched([(s, b, c, cap) for s, b, c, cap in zip(srcs, bufs, counts, caps)], dt, sizes, status) == 0
+        assert int(status.item()) == 0
+        for i, (b, n, cap) in enumerate(zip(bufs, sizes.tolist(), caps)):
+            assert bool((b[cap:] == 0xA5).all())
+            assert np.array_equal(b[:n].cpu().numpy(), oracle.compress(_words(srcs[i], dt), dt)), f"tensor {i}"
+
+
+@pytest.mark.parametrize("dt", [0, 1, 2])
+@pytest.mark.parametrize("count", [65, 127, 128, 4096, 8193, 16383, 16384 * 3 + 65, 16384 * 2 + 8192, 16384 * 2 + 16375])
+@pytest.mark.parametrize("wide", [False, True])
+def test_decompress_last_blocks(oracle, dt, count, wide):
+    """Last blocks of 128 padded elements or more take a body of their own; `wide`: with more wide groups than the sixteen-byte
+    form of the expanded records has room for."""
+    import paper_2604_03298_b200 as enec
+    t = _weights(count, dt, count, 0.02)
+    if wide:   # one value in ten far below the others
+        t = torch.where(torch.rand(count, device="cuda", generator=torch.Generator(device="cuda").manual_seed(5)) < 0.1, t / 64, t)
+    w = _words(t, dt)
+    stream = torch.from_numpy(oracle.compress(w, dt)).cuda()
+    out = torch.full((count + 64,), 1.0, dtype=DTYPES[dt], device="cuda")
+    status = status_tensor()
+    assert enec.enec_decompress(stream, stream.numel(), dt, count, out, status) == 0
+    assert int(status.item()) == 0
+    assert torch.equal(out[:count].view(BITS[dt]), t.view(BITS[dt]))
+    assert bool((out[count:] == 1.0).all()), "wrote behind the tensor"
