@@ -74,15 +74,17 @@ template <int DT>
 struct FusedShape {
     static constexpr int E = HistShape<DT>::E;
     static constexpr int kCtasPerSm = 3;
-    static constexpr uint32_t kWork = 32768;                           // low plane | fp16 plane | the block's values
+    // low plane | fp16 plane | the block's values: at the same places for every m, since a list's next block may have another
+    static constexpr uint32_t kSmhiAt = kBlockElems * 5 / 8, kValuesAt = kBlockElems, kWork = 2 * kBlockElems;
+    static_assert(kSmhiAt + kBlockElems * 3 / 8 <= kValuesAt, "the planes end before the values");
     static constexpr uint32_t kRows = DT == ENEC_FP16 ? 32 : 64;       // rows of the pack stage's histogram
     static constexpr uint32_t kHistAt = kWork;
     static constexpr uint32_t kHistBytes = kRows * HistShape<DT>::kRowBytes;
     static constexpr uint32_t kListAt = kHistAt + kHistBytes;          // the wide groups' numbers, a byte each, by warp
     static constexpr uint32_t kPend = 4096;                            // a block's packed records waiting for their offset
     static constexpr uint32_t kPendAt = kListAt + 1024;
-    static constexpr uint32_t kTensorAt = kPendAt + 2 * kPend;         // two FusedTensor (lists: the block's and the waiting block's)
-    static constexpr uint32_t kSharedAt = kTensorAt + 2 * 256;         // FusedShared
+    static constexpr uint32_t kTensorAt = kPendAt + 2 * kPend;         // FusedTensor (lists: of the block, the waiting block, the next)
+    static constexpr uint32_t kSharedAt = kTensorAt + 3 * 256;         // FusedShared
     static constexpr uint32_t kBytes = kSharedAt + 256;
     static_assert(HistShape<DT>::kBytes <= int(kHistAt + kHistBytes), "the sample stage's table fits");
     static_assert(kCtasPerSm * (kBytes + 1024) <= 228 * 1024, "the CTAs of an SM fit its shared memory");
@@ -114,7 +116,6 @@ struct FusedTensor {
     uint32_t pad;      // two 16-bit words with exponent b and nothing else: y = 0
     uint32_t wide_ok;  // bit 0: the input is 32-byte aligned, bit 1: the sm-lo plane is
     uint32_t plain;
-    uint32_t smhi_at, values_at;   // shared memory: where the fp16 plane and the values start
     uint32_t first_block;          // lists: index of the tensor's first block in the list's index space
 };
 
@@ -124,7 +125,7 @@ struct FusedShared {
     uint32_t word;       // broadcasts of thread 0
     uint32_t before;
     uint32_t ok;
-    uint32_t unit[2][2];          // lists: what the CTA does now and next, see FusedListUnit
+    uint32_t unit[2][3];          // lists: what the CTA does now and next (see enec_fused_list_kernel)
     uint32_t part[kFusedWarps];   // each warp's share of the wide groups before the waiting block; kNotReady: some are not counted yet
 };
 constexpr uint32_t kNotReady = 0xFFFFFFFFu;   // a tensor has at most 2^32 - 2^10 groups of 16 counted before a block
@@ -183,8 +184,6 @@ __device__ inline void set_parameters(FusedTensor& t, uint32_t word) {
     t.lo = t.sm + t.sm_bytes;
     t.high = t.lo + t.lo_bytes;
     t.wide_ok = ((reinterpret_cast<uintptr_t>(t.in) & 31) == 0 ? 1u : 0u) | ((reinterpret_cast<uintptr_t>(t.lo) & 31) == 0 ? 2u : 0u);
-    t.smhi_at = (kBlockElems / 8) * uint32_t(m);
-    t.values_at = t.smhi_at + (DT == ENEC_FP16 ? kBlockElems * 3 / 8 : 0);
 }
 
 // Eq. 1 as width_eq1, the bit widths by counting leading zeros.
@@ -280,7 +279,7 @@ template <bool WIDE>
 __device__ __forceinline__ Run load32(const uint8_t* p) {
     Run r;
     if constexpr (WIDE)
-        asm volatile("ld.global.cs.v8.b32 {%0, %1, %2, %3, %4, %5, %6, %7}, [%8];"
+        asm volatile("ld.global.L1::no_allocate.v8.b32 {%0, %1, %2, %3, %4, %5, %6, %7}, [%8];"
                      : "=r"(r.w[0]), "=r"(r.w[1]), "=r"(r.w[2]), "=r"(r.w[3]), "=r"(r.w[4]), "=r"(r.w[5]), "=r"(r.w[6]), "=r"(r.w[7])
                      : "l"(p));
     else
@@ -450,9 +449,10 @@ __device__ __forceinline__ void pack_lanes_any(int m, uint32_t S, uint32_t j, ui
 // the final fold; all threads.
 template <int DT>
 __device__ __forceinline__ void pack_planes(const FusedTensor& t, uint32_t work, uint32_t N, uint32_t tid) {
+    using Shape = FusedShape<DT>;
     const uint32_t j = 8 * tid, n8 = N >> 3;
     if (j >= n8) return;
-    const uint32_t values = work + t.values_at, s4 = t.s4;
+    const uint32_t values = work + Shape::kValuesAt, s4 = t.s4;
     uint2 v[8];
 #pragma unroll
     for (int c = 0; c < 8; ++c) v[c] = lds64(values + c * n8 + j);
@@ -464,7 +464,7 @@ __device__ __forceinline__ void pack_planes(const FusedTensor& t, uint32_t work,
     if constexpr (DT == ENEC_FP16) {
 #pragma unroll
         for (int c = 0; c < 8; ++c) v[c] = make_uint2(v[c].x >> 5, v[c].y >> 5);
-        pack_lanes_level<3, 3>(work + t.smhi_at, 0, j, n8, v);
+        pack_lanes_level<3, 3>(work + Shape::kSmhiAt, 0, j, n8, v);
     }
 }
 
@@ -717,44 +717,43 @@ __device__ __forceinline__ uint32_t pack_run(const Run& r, uint32_t minuend, uin
 
 // First phase of a full block, all threads: thread t takes the groups t, t + 256, .. of the block through pack_run.
 // Returns whether some value is not representable (HIST only); `wide_of_warp`: the warp's wide groups.
-// The loop over the runs is kept rolled: unrolled it exceeds what the instruction caches hold for four CTAs in four places.
+// All loads of a thread's four runs are in flight together (3584 blocks of bf16: 56.2 us; two runs, in a rolled loop, 59.6) and
+// take no room in L1, of which the shared memory of three CTAs leaves little.
 template <int DT, bool PLAIN, bool HIST>
 __device__ __forceinline__ bool pack_front_full(const FusedTensor& t, uint32_t k, uint32_t work, uint32_t* s_mask, uint32_t tid,
                                                 uint32_t& wide_of_warp) {
     using Shape = FusedShape<DT>;
     constexpr uint32_t kElemBytes = DT == ENEC_FP32 ? 4 : 2;
     constexpr uint32_t kStep = 16 * kFusedThreads;   // elements between a thread's runs
+    static_assert(kBlockElems == 4 * kStep, "a thread has four runs");
     const uint32_t lane = tid & 31, warp = tid >> 5;
     const uint8_t* in = t.in + (uint64_t(k) * kBlockElems + 16 * tid) * kElemBytes;
     uint8_t* sm_out = t.sm + (uint64_t(k) * kBlockElems + 16 * tid);
     uint8_t* lo_out = t.lo + (uint64_t(k) * kBlockElems + 16 * tid) * 2;
     const uint32_t minuend = t.c, nmask4 = t.nmask4, s4 = t.s4, wide4 = t.wide4, wide_ok = t.wide_ok;
-    const uint32_t values = work + t.values_at + tid * 16, list = work + Shape::kListAt + warp * 128;
+    const uint32_t values = work + Shape::kValuesAt + tid * 16, list = work + Shape::kListAt + warp * 128;
     uint32_t all = 0, wide = 0;
     const bool wide_in = (wide_ok & 1) != 0;
     auto run = [&](const Run& r, uint32_t i) {
         all |= pack_run<DT, PLAIN, HIST>(r, minuend, nmask4, s4, wide4, work + Shape::kHistAt, lane, values + i * kStep, i * 32 + lane, list,
                                          wide, &s_mask[i * kFusedWarps + warp], true, sm_out + i * kStep);
     };
-    if constexpr (DT == ENEC_FP32) {   // one run's 64 bytes in flight
+    if constexpr (DT == ENEC_FP32) {   // one run's 64 bytes in flight (two runs', unrolled: 1024 blocks 45.3 -> 49.6 us)
         Run a = load32_any(in, wide_in), b = load32_any(in + 32, wide_in);
 #pragma unroll 1
-        for (uint32_t i = 0; i < kBlockElems / kStep; ++i) {
+        for (uint32_t i = 0; i < 4; ++i) {
             const Run r = split_halves(a, b, lo_out + i * (kStep * 2), (wide_ok & 2) != 0);
             in += kStep * kElemBytes;
-            if (i + 1 < kBlockElems / kStep) { a = load32_any(in, wide_in); b = load32_any(in + 32, wide_in); }
+            if (i < 3) { a = load32_any(in, wide_in); b = load32_any(in + 32, wide_in); }
             run(r, i);
         }
-    } else {                           // two runs' 32 bytes
-        Run a = load32_any(in, wide_in), b = load32_any(in + kStep * kElemBytes, wide_in);
-#pragma unroll 1
-        for (uint32_t i = 0; i < kBlockElems / kStep; i += 2) {
-            in += 2 * kStep * kElemBytes;
-            run(a, i);
-            if (i + 2 < kBlockElems / kStep) a = load32_any(in, wide_in);
-            run(b, i + 1);
-            if (i + 2 < kBlockElems / kStep) b = load32_any(in + kStep * kElemBytes, wide_in);
-        }
+    } else {                           // all of the thread's runs
+        const Run a = load32_any(in, wide_in), b = load32_any(in + kStep * kElemBytes, wide_in),
+                  c = load32_any(in + 2 * kStep * kElemBytes, wide_in), d = load32_any(in + 3 * kStep * kElemBytes, wide_in);
+        run(a, 0);
+        run(b, 1);
+        run(c, 2);
+        run(d, 3);
     }
     wide_of_warp = wide;
     return HIST && (DT == ENEC_FP16 ? all & rep4(0x1F) & ~nmask4 : all & ~nmask4) != 0;
@@ -801,7 +800,7 @@ __device__ __noinline__ bool pack_front_tail(uint32_t k, uint32_t* wide_of_warp,
                                   int(align16(2 * uint64_t(real)) / 2) - int(e0), t.pad);
         }
         // the padding's sign/mantissa bytes are zero
-        pack_run<DT, PLAIN, false>(r, t.c, t.nmask4, t.s4, t.wide4, 0, lane, work + t.values_at + g * 16, i * 32 + lane,
+        pack_run<DT, PLAIN, false>(r, t.c, t.nmask4, t.s4, t.wide4, 0, lane, work + Shape::kValuesAt + g * 16, i * 32 + lane,
                                    work + Shape::kListAt + warp * 128, wide, &sh.mask[i * kFusedWarps + warp], left > 0,
                                    t.sm + uint64_t(k) * kBlockElems + e0);
     }
@@ -980,7 +979,7 @@ __device__ __noinline__ uint32_t histogram_stage(FusedControl* ctl, uint32_t whi
     const FusedTensor& t = fused_tensor<DT>();
     FusedShared& sh = fused_shared<DT>();
     constexpr uint32_t kElemBytes = DT == ENEC_FP32 ? 4 : 2;
-    const uint32_t tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    const uint32_t tid = threadIdx.x, lane = tid & 31;
     const uint32_t work = smem_u32(fused_smem());
     const bool ahead = total > gridDim.x;   // tickets are asked for ahead; else a CTA has one block as a rule
     uint32_t* const ticket = &ctl->hist_ticket[which].value;
@@ -1187,7 +1186,7 @@ __device__ __noinline__ uint32_t pack_pass(FusedControl* ctl, uint32_t pass, int
             if (!sh.ok) stop = true;
         }
         if (!direct || sh.ok)
-            pack_records_any<DT>(int(hbits), work + t.values_at, work + Shape::kListAt + warp * 128, wide_of_warp, mask_word, excl, t.s4, int(m),
+            pack_records_any<DT>(int(hbits), work + Shape::kValuesAt, work + Shape::kListAt + warp * 128, wide_of_warp, mask_word, excl, t.s4, int(m),
                                  work + Shape::kPendAt + (iter & 1) * Shape::kPend,
                                  direct ? t.high + uint64_t(sh.before) * 2 * hbits : nullptr);
         if (waiting) {
@@ -1197,7 +1196,7 @@ __device__ __noinline__ uint32_t pack_pass(FusedControl* ctl, uint32_t pass, int
         const uint32_t next = sh.next;
         __syncthreads();                                      // barrier B
         fold_out(work, N * m / 8, t.low + uint64_t(k) * (kBlockElems / 8) * m, tid);   // N >= 128: whole pieces of 16 bytes
-        if (DT == ENEC_FP16) fold_out(work + t.smhi_at, N * 3 / 8, t.smhi + uint64_t(k) * (kBlockElems / 8) * 3, tid);
+        if (DT == ENEC_FP16) fold_out(work + Shape::kSmhiAt, N * 3 / 8, t.smhi + uint64_t(k) * (kBlockElems / 8) * 3, tid);
         if (waiting) place_waiting(true);
         pend_block = direct ? 0xFFFFFFFFu : k;
         pend_wide = wide;

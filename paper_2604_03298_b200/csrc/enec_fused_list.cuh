@@ -19,7 +19,7 @@
 namespace enec {
 
 constexpr uint32_t kHistBlocks = 4;
-constexpr uint64_t kWaveBytes = uint64_t(24) << 20;
+constexpr uint64_t kWaveBytes = uint64_t(40) << 20;
 
 struct alignas(16) FusedItemControl {
     unsigned long long hist[256];
@@ -79,28 +79,63 @@ enec_fused_list_kernel(const FusedList list, int* status) {
     pdl_launch_dependents();
     pdl_wait();  // nothing above touches global memory
 
-    // thread 0: the kind and the first block of a ticket's unit (tickets of a CTA grow, so the search moves forward)
-    uint32_t segment = 0;
-    auto unit_of = [&](uint32_t ticket, uint32_t& kind, uint32_t& block) {
+    // Scout: the last warp looks ahead, so that a unit's tensor is in shared memory when the unit begins. Its first lane knows
+    // the next unit at the start of this one (the ticket was asked for a unit before), the unit's tensor index in the
+    // middle, and if that tensor's parameters are there by then, the warp brings them; all of it is written before
+    // the unit's last barrier. sh.unit[i & 1] for unit i: kind | tensor << 2, first block, whether the tensor is in its slot.
+    const bool scout = warp == kFusedWarps - 1;
+    uint32_t segment = 0, ticket_after = 0, next_kind = 0, next_block = 0, next_item = 0;
+    auto unit_of = [&](uint32_t ticket) {   // tickets of a CTA grow, so the search moves forward
         while (segment < list.n_segments && list.segments[segment + 1].first_ticket <= ticket) ++segment;
-        if (segment == list.n_segments) { kind = kUnitEnd; block = 0; return; }
+        next_kind = kUnitEnd;
+        next_block = next_item = 0;
+        if (segment == list.n_segments) return;
         const FusedListSegment s = list.segments[segment];
-        kind = s.kind;
-        block = s.first_block + (ticket - s.first_ticket) * (kind == kUnitCount ? kHistBlocks : 1);
+        next_kind = s.kind;
+        next_block = s.first_block + (ticket - s.first_ticket) * (s.kind == kUnitCount ? kHistBlocks : 1);
+        next_item = next_block >= list.multi_blocks ? list.n_multi + (next_block - list.multi_blocks) : list.chunk_item[next_block / kHistBlocks];
     };
-    auto item_of = [&](uint32_t kind, uint32_t block) -> uint32_t {
-        return kind == kUnitEnd ? 0u : block >= list.multi_blocks ? list.n_multi + (block - list.multi_blocks) : list.chunk_item[block / kHistBlocks];
+    uint32_t brought[2], brought_ready = 0;
+    auto scout_start = [&]() {
+        if (scout && lane == 0) {
+            unit_of(ticket_after);
+            ticket_after = atomicAdd(list.ticket, 1u);
+        }
     };
-    uint32_t ticket_after = 0;   // thread 0: the ticket of the unit after the next one
-    if (tid == 0) {
-        uint32_t kind, block;
-        unit_of(atomicAdd(list.ticket, 1u), kind, block);
-        sh.unit[0][0] = kind | item_of(kind, block) << 2;
-        sh.unit[0][1] = block;
+    auto scout_middle = [&]() {
+        if (!scout) return;
+        uint32_t ready = 0;
+        if (lane == 0 && next_kind == kUnitPack)
+            asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(ready) : "l"(&list.controls[next_item].ready) : "memory");
+        brought_ready = __shfl_sync(0xFFFFFFFFu, ready, 0);
+        if (brought_ready) {
+            const uint32_t* from = reinterpret_cast<const uint32_t*>(&list.controls[__shfl_sync(0xFFFFFFFFu, next_item, 0)].tensor);
+            brought[0] = ld_relaxed_u32(from + lane);
+            brought[1] = lane + 32 < sizeof(FusedTensor) / 4 ? ld_relaxed_u32(from + lane + 32) : 0u;
+        }
+    };
+    auto scout_end = [&](uint32_t iter, uint32_t next_slot) {
+        if (!scout) return;
+        if (brought_ready) {
+            uint32_t* to = reinterpret_cast<uint32_t*>(&fused_tensor<DT>(next_slot));
+            to[lane] = brought[0];
+            if (lane + 32 < sizeof(FusedTensor) / 4) to[lane + 32] = brought[1];
+        }
+        if (lane == 0) {
+            sh.unit[(iter + 1) & 1][0] = next_kind | next_item << 2;
+            sh.unit[(iter + 1) & 1][1] = next_block;
+            sh.unit[(iter + 1) & 1][2] = brought_ready;
+        }
+    };
+    if (scout && lane == 0) {
+        unit_of(atomicAdd(list.ticket, 1u));
+        sh.unit[0][0] = next_kind | next_item << 2;
+        sh.unit[0][1] = next_block;
+        sh.unit[0][2] = 0;
         ticket_after = atomicAdd(list.ticket, 1u);
-        sh.ok = 0;
     }
-    uint32_t pend_block = 0xFFFFFFFFu, pend_wide = 0, pend_at = 0, pend_slot = 0;   // the block whose records wait in shared memory
+    uint32_t pend_block = 0xFFFFFFFFu, pend_wide = 0, pend_at = 0, pend_slot = 1;   // the block whose records wait in shared memory
+    uint32_t slot = 0;                                                             // of this unit's tensor
     bool stop = false;
     auto place_waiting = [&](bool asked_for) {   // see pack_pass
         const FusedTensor& t = fused_tensor<DT>(pend_slot);
@@ -115,51 +150,52 @@ enec_fused_list_kernel(const FusedList list, int* status) {
                 const bool ok = groups_before(t, pend_block, before);
                 if (lane == 0) {
                     sh.before = before;
-                    sh.word = ok;
+                    sh.ok = ok;
                     if (!ok) report(status, ENEC_ERR_TIMEOUT);
                 }
             }
             __syncthreads();
             before = sh.before;
-            if (!sh.word) { stop = true; return; }
+            if (!sh.ok) { stop = true; return; }
         }
         copy_halves(t.high + uint64_t(before) * 2 * uint32_t(t.hbits), pend_at, pend_wide * uint32_t(t.hbits), tid);
         if (warp == 0) finish_block<DT>(t, pend_block, before, pend_wide);
     };
+    auto share_waiting = [&](unsigned long long answer) {
+        const uint32_t share = share_before(fused_tensor<DT>(pend_slot), answer, pend_block, tid);
+        if (lane == 0) sh.part[warp] = share;
+    };
+    auto clear_table = [&]() {
+        for (uint32_t i = tid; i < uint32_t(HistShape<DT>::kBytes / 16); i += kFusedThreads) sts128(work + 16 * i, make_uint4(0, 0, 0, 0));
+    };
 
+    __syncthreads();
     for (uint32_t iter = 0;; ++iter) {
-        __syncthreads();
-        const uint32_t unit = sh.unit[iter & 1][0], block = sh.unit[iter & 1][1];
-        const uint32_t kind = unit & 3, item_index = unit >> 2;
-        const bool loaded = sh.ok != 0;    // the tensor of this unit is in its slot
+        // (whatever is written before a unit's last barrier is read after it; the barriers A and B are those of pack_pass)
+        const uint32_t kind = sh.unit[iter & 1][0] & 3, item_index = sh.unit[iter & 1][0] >> 2, block = sh.unit[iter & 1][1];
+        const bool loaded = sh.unit[iter & 1][2] != 0;
         if (kind == kUnitEnd || stop) break;
-        // thread 0 looks ahead: the next unit, its tensor (needed at the end of this unit), and the ticket after that
-        uint32_t next_kind = 0, next_block = 0, next_item = 0;
-        if (tid == 0) {
-            unit_of(ticket_after, next_kind, next_block);
-            next_item = item_of(next_kind, next_block);
-            ticket_after = atomicAdd(list.ticket, 1u);
-        }
+        scout_start();
         const bool waiting = pend_block != 0xFFFFFFFFu;
-        const uint32_t slot = pend_slot ^ 1;   // this unit's tensor
+        const uint32_t next_slot = 3 - slot - pend_slot;
         unsigned long long answer = 0;
-        uint32_t wide = 0;
-        bool packed = false, direct = false;
+        uint32_t wide = 0, k = 0;
+        bool leaves_records = false;
         if (kind == kUnitCount) {
             const FusedListItem& item = list.items[item_index];
             FusedItemControl& ctl = list.controls[item_index];
             const uint32_t first = block - item.first_block;
             const uint32_t n = item.nblocks - first < kHistBlocks ? item.nblocks - first : kHistBlocks;
-            for (uint32_t i = tid; i < uint32_t(HistShape<DT>::kBytes / 16); i += kFusedThreads) sts128(work + 16 * i, make_uint4(0, 0, 0, 0));
-            if (waiting) answer = ask_before(fused_tensor<DT>(pend_slot), pend_block, tid);
-            __syncthreads();
             const uint64_t from = uint64_t(first) * kBlockElems;
             const uint64_t left = item.count - from;
-            count_block<DT>(item.in + from * kElemBytes, left < n * kBlockElems ? uint32_t(left) : n * kBlockElems, work + lane * 4, tid);
-            if (waiting) {
-                const uint32_t share = share_before(fused_tensor<DT>(pend_slot), answer, pend_block, tid);
-                if (lane == 0) sh.part[warp] = share;
-            }
+            const uint8_t* in = item.in + from * kElemBytes;
+            __syncthreads();   // the planes of the block before have been read
+            clear_table();
+            if (waiting) answer = ask_before(fused_tensor<DT>(pend_slot), pend_block, tid);
+            __syncthreads();
+            count_block<DT>(in, left < n * kBlockElems ? uint32_t(left) : n * kBlockElems, work + lane * 4, tid);
+            if (waiting) share_waiting(answer);
+            scout_middle();
             __syncthreads();
             if (tid < uint32_t(HistShape<DT>::kBins)) {
                 const uint32_t c = fold_hist_row<false>(work + tid * HistShape<DT>::kRowBytes, tid);
@@ -168,6 +204,7 @@ enec_fused_list_kernel(const FusedList list, int* status) {
             __threadfence();
             __syncthreads();
             if (tid == 0) sh.word = atomicAdd(&ctl.done, n) + n == item.nblocks;
+            scout_end(iter, next_slot);
             __syncthreads();
             if (sh.word && warp == 0) {
                 __threadfence();
@@ -177,13 +214,14 @@ enec_fused_list_kernel(const FusedList list, int* status) {
                     publish(&ctl.ready, 1u);
                 }
             }
-            if (waiting) __syncthreads();   // sh.word has been read by everybody
+            __syncthreads();
         } else {
             const FusedTensor& t = fused_tensor<DT>(slot);
             bool present = true;   // not an index between two tensors
             if (kind == kUnitWhole) {
                 const FusedListItem& item = list.items[item_index];
-                for (uint32_t i = tid; i < uint32_t(HistShape<DT>::kBytes / 16); i += kFusedThreads) sts128(work + 16 * i, make_uint4(0, 0, 0, 0));
+                __syncthreads();
+                clear_table();
                 __syncthreads();
                 count_block<DT>(item.in, uint32_t(item.count), work + lane * 4, tid);
                 __syncthreads();
@@ -196,7 +234,7 @@ enec_fused_list_kernel(const FusedList list, int* status) {
                 }
                 __syncthreads();
             } else {
-                if (!loaded) {   // its parameters were not there when this CTA looked: wait for them
+                if (!loaded) {   // its parameters were not there when the scout looked: wait for them
                     const FusedItemControl& ctl = list.controls[item_index];
                     if (tid == 0) sh.word = await_published(&ctl.ready);
                     __syncthreads();
@@ -209,97 +247,77 @@ enec_fused_list_kernel(const FusedList list, int* status) {
                     __syncthreads();
                 }
                 present = block - t.first_block < t.nblocks;
+                if (present) k = block - t.first_block;
             }
-            if (present) {
-                const uint32_t k = kind == kUnitWhole ? 0u : block - t.first_block;
-                const bool last = k + 1 == t.nblocks && t.tail_real != kBlockElems;
-                const uint32_t N = last ? t.tail_padded : kBlockElems;
-                uint32_t wide_of_warp = 0;
-                if (!last) {
-                    if (t.plain || DT == ENEC_FP16) pack_front_full<DT, true, false>(t, k, work, sh.mask, tid, wide_of_warp);
-                    else pack_front_full<DT, false, false>(t, k, work, sh.mask, tid, wide_of_warp);
-                } else if (N >= 128) {
-                    if (t.plain || DT == ENEC_FP16) pack_front_tail<DT, true, false>(k, &wide_of_warp, slot);
-                    else pack_front_tail<DT, false, false>(k, &wide_of_warp, slot);
+            const bool last = k + 1 == t.nblocks && t.tail_real != kBlockElems;
+            const uint32_t N = last ? t.tail_padded : kBlockElems;
+            uint32_t wide_of_warp = 0;
+            if (!present) {
+            } else if (!last) {
+                if (t.plain || DT == ENEC_FP16) pack_front_full<DT, true, false>(t, k, work, sh.mask, tid, wide_of_warp);
+                else pack_front_full<DT, false, false>(t, k, work, sh.mask, tid, wide_of_warp);
+            } else if (N >= 128) {
+                if (t.plain || DT == ENEC_FP16) pack_front_tail<DT, true, false>(k, &wide_of_warp, slot);
+                else pack_front_tail<DT, false, false>(k, &wide_of_warp, slot);
+            }
+            __syncthreads();                                      // barrier A
+            if (waiting) answer = ask_before(fused_tensor<DT>(pend_slot), pend_block, tid);
+            scout_middle();
+            if (present && N < 128) {
+                pack_short_block<DT>(k, status, slot);            // its records go straight to their place
+            } else if (present) {
+                uint32_t mask_word, excl;
+                wide = scan_mask(sh.mask, lane, mask_word, excl);
+                if (tid == 0 && t.nblocks != 1) {
+                    st_relaxed_u64(&t.state[k], ((unsigned long long)t.epoch << 32) | wide);
+                    atomicAdd(&t.super[k / kSuperBlocks], (1ull << 32) | wide);
+                    if (t.nblocks > kSuperBlocks * kHyperSupers) atomicAdd(&t.hyper[k / (kSuperBlocks * kHyperSupers)], (1ull << 32) | wide);
                 }
-                __syncthreads();                                      // barrier A of pack_pass
-                if (waiting) answer = ask_before(fused_tensor<DT>(pend_slot), pend_block, tid);
-                if (N < 128) {
-                    pack_short_block<DT>(k, status, slot);            // its records go straight to their place
-                    if (waiting) {
-                        const uint32_t share = share_before(fused_tensor<DT>(pend_slot), answer, pend_block, tid);
-                        if (lane == 0) sh.part[warp] = share;
+                const uint32_t hbits = uint32_t(t.hbits), m = uint32_t(t.m);
+                // records that do not fit the waiting area, or (one block) need not wait, go straight to their place
+                const bool direct = t.nblocks == 1 || wide * 2 * hbits > Shape::kPend;
+                if (tid < uint32_t(align16(((N >> 4) + 7) / 8)) / 16)
+                    reinterpret_cast<uint4*>(t.mask + uint64_t(k) * (kGroupsPerBlock / 8))[tid] = reinterpret_cast<const uint4*>(sh.mask)[tid];
+                pack_planes<DT>(t, work, N, tid);
+                if (direct) {
+                    if (warp == 0) {
+                        uint32_t before = 0;
+                        const bool ok = groups_before(t, k, before);
+                        if (ok) finish_block<DT>(t, k, before, wide);
+                        else if (lane == 0) report(status, ENEC_ERR_TIMEOUT);
+                        if (lane == 0) { sh.before = before; sh.ok = ok; }
                     }
-                    direct = true;
-                } else {
-                    uint32_t mask_word, excl;
-                    wide = scan_mask(sh.mask, lane, mask_word, excl);
-                    if (tid == 0 && t.nblocks != 1) {
-                        st_relaxed_u64(&t.state[k], ((unsigned long long)t.epoch << 32) | wide);
-                        atomicAdd(&t.super[k / kSuperBlocks], (1ull << 32) | wide);
-                        if (t.nblocks > kSuperBlocks * kHyperSupers) atomicAdd(&t.hyper[k / (kSuperBlocks * kHyperSupers)], (1ull << 32) | wide);
-                    }
-                    const uint32_t hbits = uint32_t(t.hbits), m = uint32_t(t.m);
-                    // records that do not fit the waiting area, or (one block) need not wait, go straight to their place
-                    direct = t.nblocks == 1 || wide * 2 * hbits > Shape::kPend;
-                    if (tid < uint32_t(align16(((N >> 4) + 7) / 8)) / 16)
-                        reinterpret_cast<uint4*>(t.mask + uint64_t(k) * (kGroupsPerBlock / 8))[tid] = reinterpret_cast<const uint4*>(sh.mask)[tid];
-                    pack_planes<DT>(t, work, N, tid);
-                    if (direct) {
-                        if (warp == 0) {
-                            uint32_t before = 0;
-                            const bool ok = groups_before(t, k, before);
-                            if (ok) finish_block<DT>(t, k, before, wide);
-                            else if (lane == 0) report(status, ENEC_ERR_TIMEOUT);
-                            if (lane == 0) { sh.before = before; sh.word = ok; }
-                        }
-                        __syncthreads();
-                        if (!sh.word) stop = true;
-                    }
-                    if (!stop)
-                        pack_records_any<DT>(int(hbits), work + t.values_at, work + Shape::kListAt + warp * 128, wide_of_warp, mask_word, excl,
-                                             t.s4, int(m), work + Shape::kPendAt + (iter & 1) * Shape::kPend,
-                                             direct ? t.high + uint64_t(sh.before) * 2 * hbits : nullptr);
-                    if (waiting) {
-                        const uint32_t share = share_before(fused_tensor<DT>(pend_slot), answer, pend_block, tid);
-                        if (lane == 0) sh.part[warp] = share;
-                    }
-                    __syncthreads();                                  // barrier B of pack_pass
-                    fold_out(work, N * m / 8, t.low + uint64_t(k) * (kBlockElems / 8) * m, tid);
-                    if (DT == ENEC_FP16) fold_out(work + t.smhi_at, N * 3 / 8, t.smhi + uint64_t(k) * (kBlockElems / 8) * 3, tid);
+                    __syncthreads();
+                    if (!sh.ok) stop = true;
                 }
-                packed = true;
-            } else if (waiting) {
-                const uint32_t share = share_before(fused_tensor<DT>(pend_slot), ask_before(fused_tensor<DT>(pend_slot), pend_block, tid), pend_block, tid);
-                if (lane == 0) sh.part[warp] = share;
+                if (!stop)
+                    pack_records_any<DT>(int(hbits), work + Shape::kValuesAt, work + Shape::kListAt + warp * 128, wide_of_warp, mask_word, excl,
+                                         t.s4, int(m), work + Shape::kPendAt + (iter & 1) * Shape::kPend,
+                                         direct ? t.high + uint64_t(sh.before) * 2 * hbits : nullptr);
+                leaves_records = !direct;
+            }
+            if (waiting) share_waiting(answer);
+            scout_end(iter, next_slot);
+            __syncthreads();                                      // barrier B
+            if (present && N >= 128) {
+                const uint32_t m = uint32_t(t.m);
+                fold_out(work, N * m / 8, t.low + uint64_t(k) * (kBlockElems / 8) * m, tid);
+                if (DT == ENEC_FP16) fold_out(work + Shape::kSmhiAt, N * 3 / 8, t.smhi + uint64_t(k) * (kBlockElems / 8) * 3, tid);
             }
         }
-        __syncthreads();   // sh.part is complete
         if (waiting) {
             place_waiting(true);
             pend_block = 0xFFFFFFFFu;
         }
-        if (packed && !direct) {
-            pend_block = kind == kUnitWhole ? 0u : block - fused_tensor<DT>(slot).first_block;
+        if (leaves_records) {
+            pend_block = k;
             pend_wide = wide;
             pend_at = work + Shape::kPendAt + (iter & 1) * Shape::kPend;
             pend_slot = slot;
         }
-        __syncthreads();   // the slot that the next unit's tensor goes to is free; sh.word and sh.before have been read
-        // the next unit, and its tensor if the search is through by now
-        if (tid == 0) {
-            sh.unit[(iter + 1) & 1][0] = next_kind | next_item << 2;
-            sh.unit[(iter + 1) & 1][1] = next_block;
-            uint32_t ready = 0;
-            if (next_kind == kUnitPack)
-                asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(ready) : "l"(&list.controls[next_item].ready) : "memory");
-            sh.ok = ready;
-        }
-        __syncthreads();
-        if (sh.ok && tid < sizeof(FusedTensor) / 4)
-            reinterpret_cast<uint32_t*>(&fused_tensor<DT>(pend_slot ^ 1))[tid] =
-                ld_relaxed_u32(reinterpret_cast<const uint32_t*>(&list.controls[sh.unit[(iter + 1) & 1][0] >> 2].tensor) + tid);
+        slot = next_slot;
     }
+    __syncthreads();   // sh.before has been read by everybody
     if (pend_block != 0xFFFFFFFFu && !stop) place_waiting(false);
 }
 

@@ -105,10 +105,10 @@ def test_compress_when_the_sample_misleads(oracle, dt, what):
 
 @pytest.mark.parametrize("dt", [0, 1, 2])
 def test_compress_batched_across_waves(oracle, dt):
-    """A list whose tensors are counted and packed in several waves of 24 MB (one tensor is more than a wave), with tensors
+    """A list whose tensors are counted and packed in several waves of 40 MB (one tensor is more than a wave), with tensors
     of one block, of a few elements, and with last blocks of every kind between them."""
     import paper_2604_03298_b200 as enec
-    counts = [16384 * 820 + 5, 16384 * 2, 100, 16384, 16385, 0, 16384 * 5 - 1, 2048, 16384 * 129, 37, 16384 * 400, 16384 * 500 + 60,
+    counts = [16384 * 1300 + 5, 16384 * 2, 100, 16384, 16385, 0, 16384 * 5 - 1, 2048, 16384 * 129, 37, 16384 * 400, 16384 * 500 + 60,
               16384 * 3, 5, 16384 * 7 + 8000]
     srcs = [_weights(c, dt, 70 + i, 0.02 * (1 + i % 4)) for i, c in enumerate(counts)]
     caps = [enec.enec_max_compressed_size(dt, c) for c in counts]
