@@ -1,6 +1,7 @@
 """ctypes binding of libenec.so. Argument marshalling only."""
 import ctypes as C
 import os
+import threading
 
 import torch
 
@@ -171,38 +172,66 @@ def enec_allocation_count() -> int:
 
 
 # ---- convenience wrappers (allocation with torch, status check) --------------------------------------
+class _Answer:
+    """Where a checked call's kernels leave stream length and status: 16 bytes of pinned host memory, which the GPU writes
+    itself, so that the call neither clears nor copies device memory and waits for its stream only once."""
+
+    def __init__(self):
+        self.memory = torch.zeros(2, dtype=torch.int64).pin_memory()
+        self.address = self.memory.data_ptr()
+        self.size = C.c_int64.from_address(self.address)
+        self.status = C.c_int32.from_address(self.address + 8)
+        self.stream = None   # set while kernels may still write here: a call that failed half way leaves it set
+
+
+_local = threading.local()
+
+
+def _answer():
+    """This thread's answer memory, cleared. (One per thread is enough: a checked call ends after its stream's work has.)"""
+    a = getattr(_local, "answer", None)
+    if a is None:
+        a = _local.answer = _Answer()
+    elif a.stream is not None:
+        a.stream.synchronize()
+    a.size.value = 0
+    a.status.value = 0
+    a.stream = torch.cuda.current_stream()
+    return a
+
+
+def _finish(a, st, where):
+    """Waits for the call's stream and raises on an error of the call (st) or of its kernels. (Cleared and copied device memory,
+    as before, cost 15 us more for each call: norm weights there and back took 86 us, 55 us now.)"""
+    if st != 0:
+        raise EnecError(st, where)
+    a.stream.synchronize()
+    a.stream = None
+    if a.status.value != 0:
+        raise EnecError(a.status.value, where + " (device)")
+
+
 def compress_tensor(t: torch.Tensor, params=None) -> torch.Tensor:
-    """Compresses a CUDA bf16/fp16/fp32 tensor; returns the stream as a uint8 CUDA tensor (synchronises once to
-    read the stream length)."""
+    """Compresses a CUDA bf16/fp16/fp32 tensor; returns the stream as a uint8 CUDA tensor (waits for the current stream
+    once to learn the stream length)."""
     dt = _DT[t.dtype]
     t = t.contiguous()
     count = t.numel()
     cap = enec_max_compressed_size(dt, count)
     out = torch.empty(cap, dtype=torch.uint8, device=t.device)
-    meta = torch.zeros(2, dtype=torch.int64, device=t.device)   # [0] = size, [1] = status
-    status = meta[1:].view(torch.int32)
+    a = _answer()
     if params is None:
-        st = enec_compress(t, dt, count, out, cap, meta, status)
+        st = lib().enec_compress(t.data_ptr(), dt, count, out.data_ptr(), cap, a.address, a.address + 8, a.stream.cuda_stream)
     else:
-        st = enec_compress_with_params(t, dt, count, *params, out, cap, meta, status)
-    if st != 0:
-        raise EnecError(st, "enec_compress")
-    size, dev_status = meta.tolist()
-    dev_status = dev_status & 0xFFFFFFFF
-    dev_status = dev_status - (1 << 32) if dev_status & 0x80000000 else dev_status
-    if dev_status != 0:
-        raise EnecError(dev_status, "enec_compress (device)")
-    return out[:size]
+        st = lib().enec_compress_with_params(t.data_ptr(), dt, count, *params, out.data_ptr(), cap, a.address, a.address + 8, a.stream.cuda_stream)
+    _finish(a, st, "enec_compress")
+    return out[:a.size.value]
 
 
 def decompress_tensor(stream: torch.Tensor, dtype: torch.dtype, shape) -> torch.Tensor:
     dt = _DT[dtype]
     out = torch.empty(shape, dtype=dtype, device=stream.device)
-    status = torch.zeros(1, dtype=torch.int32, device=stream.device)
-    st = enec_decompress(stream, stream.numel(), dt, out.numel(), out, status)
-    if st != 0:
-        raise EnecError(st, "enec_decompress")
-    dev_status = int(status.item())
-    if dev_status != 0:
-        raise EnecError(dev_status, "enec_decompress (device)")
+    a = _answer()
+    st = lib().enec_decompress(stream.data_ptr(), stream.numel(), dt, out.numel(), out.data_ptr(), a.address + 8, a.stream.cuda_stream)
+    _finish(a, st, "enec_decompress")
     return out

@@ -140,3 +140,40 @@ def test_decompress_last_blocks(oracle, dt, count, wide):
     assert int(status.item()) == 0
     assert torch.equal(out[:count].view(BITS[dt]), t.view(BITS[dt]))
     assert bool((out[count:] == 1.0).all()), "wrote behind the tensor"
+
+
+def test_checked_calls_report_errors_and_recover():
+    """compress_tensor / decompress_tensor read length and status from pinned host memory that the kernels write: an error is
+    raised, and the next call on the thread starts clean; threads do not share the memory."""
+    import threading
+    import paper_2604_03298_b200 as enec
+    t = _weights(16384 * 3 + 100, 0, 5)
+    for _ in range(2):
+        with pytest.raises(enec.EnecError) as err:
+            enec.compress_tensor(t, params=(100, 1, 1))   # loses exponents
+        assert err.value.status == -5
+        s = enec.compress_tensor(t)
+        assert torch.equal(enec.decompress_tensor(s, t.dtype, t.shape).view(torch.int16), t.view(torch.int16))
+        bad = s.clone()
+        bad[8] ^= 1                                      # another count in the header
+        with pytest.raises(enec.EnecError) as err:
+            enec.decompress_tensor(bad, t.dtype, t.shape)
+        assert err.value.status == -4
+    empty = enec.compress_tensor(t[:0])
+    assert empty.numel() == 80 and enec.decompress_tensor(empty, t.dtype, (0,)).numel() == 0
+
+    def work(seed, ok):
+        x = _weights(16384 * 2 + seed, 0, seed)
+        with torch.cuda.stream(torch.cuda.Stream()):
+            x.record_stream(torch.cuda.current_stream())
+            torch.cuda.current_stream().wait_stream(torch.cuda.default_stream())
+            ok[seed] = all(torch.equal(enec.decompress_tensor(enec.compress_tensor(x), x.dtype, x.shape).view(torch.int16), x.view(torch.int16))
+                           for _ in range(20))
+
+    ok = {}
+    threads = [threading.Thread(target=work, args=(i, ok)) for i in range(4)]
+    for th in threads:
+        th.start()
+    for th in threads:
+        th.join()
+    assert ok == {i: True for i in range(4)}
