@@ -13,6 +13,7 @@ static enec_status launch_fused_dt(FusedJob job, uint32_t nblocks, int sms, bool
         attr_set = true;
     }
     uint32_t grid = uint32_t(sms) * Shape::kCtasPerSm;
+    if (grid > kMaxFusedGrid) grid = kMaxFusedGrid;
     if (grid > nblocks) grid = nblocks;
     // Up to 44 MB the sample is the whole tensor: its second reading comes from L2, and the parameters need no check. Beyond,
     // one block per SM is sampled. bf16, sampled against whole: 740 blocks 24.8 / 23.1 us, 1024 28.0 / 28.8, 1500 33.9 /

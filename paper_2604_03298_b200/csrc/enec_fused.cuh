@@ -1,13 +1,13 @@
 // enec_compress in one kernel (Sec. 5.1 compression flow with the parameter choice of Sec. 5.5).
 //
-// enec_fused_kernel, four CTAs of 256 threads per SM, blocks of 16384 elements handed out by tickets:
+// enec_fused_kernel, three CTAs of 256 threads per SM, blocks of 16384 elements handed out by tickets:
 //   1. Sample stage: the histogram of a sample of the tensor's blocks, spread over it (every block of a small tensor). When
 //      the last sampled block is counted, its CTA runs the search of Sec. 5.5 and publishes (b, n, m).
 //   2. Pack stage: split, transform (Sec. 5.3), group widths (Sec. 5.2), Algorithm 2, and the histogram of every block.
 //      The input is read once, apart from the sample.
-//   3. The CTA that ends last runs the search again, on the histogram of the whole tensor. When it gives the parameters
-//      that were used, the stream is the one that the search on the whole tensor leads to. When it does not, the CTAs pack
-//      the tensor again; a value that the sampled parameters cannot represent ends the pack stage at once, and the blocks
+//   3. The CTA that counts the last block runs the search again, on the histogram of the whole tensor. When it gives the
+//      parameters that were used, the stream is the one that the search on the whole tensor leads to. When it does not, the
+//      CTAs pack the tensor again; a value that the sampled parameters cannot represent ends the pack stage at once, and the blocks
 //      not packed yet are counted first.
 // A tensor whose sample needs n > 6 exponent bits (bf16, fp32) takes the histogram of the whole tensor before it packs:
 // the table kept beside the packing has 64 rows, and rare outliers of such a tensor are what a sample misses.
@@ -35,23 +35,28 @@ constexpr uint32_t kMaxHypers = 256;       // 2^36 values
 // Control words of a call. The sums and the pack stage's ticket are kept per pass over the tensor (the second pass happens
 // only when the sampled parameters were not the tensor's). Words that many CTAs add to lie on lines of their own: adds to
 // one line are served one after another, about 3.6 ns each.
+constexpr uint32_t kClaimWords = 16;
+constexpr uint32_t kMaxFusedGrid = 32 * kClaimWords;
 struct alignas(128) Counter { uint32_t value; uint32_t pad[31]; };
 struct alignas(128) FusedControl {
     unsigned long long hist[2][256];             // of the sample, of the whole tensor but for what is in pack_hist
     unsigned long long pack_hist[256];           // of the pack stage
     unsigned long long hyper[2][kMaxHypers];     // bits 63..32 blocks counted, bits 31..0 their wide groups
     Counter hist_ticket[2], hist_done[2];
+    Counter claims[kClaimWords];   // a bit per CTA: the block it starts with in the sample stage is taken
     Counter pack_ticket[2];
-    Counter pack_done;         // blocks packed by the CTAs that have left the first pass
+    Counter pack_done;         // blocks of the first pass whose counts are in pack_hist (or hist[1])
+    Counter pack_left;         // blocks packed by the CTAs that have left the first pass, when there is a second
     uint32_t pack_target;      // blocks handed out before the first pass was ended early (0: it was not)
     uint32_t params[2];        // published: the parameters for hist[0], hist[1]
-    uint32_t verdict;          // published: the whole tensor's parameters, when the first pass has packed every block
+    uint32_t verdict;          // published: the whole tensor's parameters, when the first pass has counted every block
+    uint32_t all_left;         // published: the first pass writes no more
 };
 constexpr uint32_t kFusedControlBytes = 16384;
 static_assert(sizeof(FusedControl) <= kFusedControlBytes, "a control set fits its slot");
 constexpr uint32_t kParamsValid = 1u << 31;   // a published word: b | n << 8 | m << 12 | valid
 constexpr uint32_t kParamsRedo = 1u << 28;    // verdict: some packed blocks held values that the sampled parameters lose
-constexpr uint32_t kParamsTake = 1u << 29;    // not a published word: there is a ticket to take
+constexpr uint32_t kParamsTake = 1u << 29;    // not a published word: there is a block to take
 constexpr uint32_t kPassEnded = 1u << 30;     // pack_ticket: no further blocks in this pass
 
 struct FusedJob {
@@ -927,20 +932,35 @@ __device__ __forceinline__ void count_block(const uint8_t* in, uint32_t real, ui
         red_add_one(column + exponent_of_word<DT>(exponent_word<DT>(in, e)) * HistShape<DT>::kRowBytes);
 }
 
+// publish: with all that the thread (and, before a barrier, its CTA) has written; publish_word: the word stands for itself.
 __device__ __forceinline__ void publish(uint32_t* where, uint32_t word) {
     asm volatile("st.release.gpu.global.u32 [%0], %1;" ::"l"(where), "r"(word) : "memory");
 }
+__device__ __forceinline__ void publish_word(uint32_t* where, uint32_t word) {
+    asm volatile("st.relaxed.gpu.global.u32 [%0], %1;" ::"l"(where), "r"(word) : "memory");
+}
+// A count of finished work, by one thread after a barrier of its CTA: what the CTA has written is there for whoever sees the
+// sum, and what the others before it have written for this CTA.
+__device__ __forceinline__ uint32_t add_acq_rel(uint32_t* where, uint32_t n) {
+    uint32_t old;
+    asm volatile("atom.acq_rel.gpu.global.add.u32 %0, [%1], %2;" : "=r"(old) : "l"(where), "r"(n) : "memory");
+    return old;
+}
 // One thread: a published word; 0 when it does not come within about two seconds. When it has not come after some 20 us
-// and `ticket` says that some of `total` tickets have not been taken: kParamsTake.
-__device__ __forceinline__ uint32_t await_published(const uint32_t* where, const uint32_t* ticket = nullptr, uint32_t total = 0) {
+// and `left()` finds work that nobody has taken: kParamsTake.
+template <class Left>
+__device__ __forceinline__ uint32_t await_published(const uint32_t* where, Left left) {
     for (uint32_t polls = 0; polls < (1u << 22); ++polls) {
         uint32_t w;
         asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(w) : "l"(where) : "memory");
         if (w) return w;
-        if (polls > 64 && ticket && ld_relaxed_u32(ticket) < total) return kParamsTake;
+        if (polls > 64 && left()) return kParamsTake;
         __nanosleep(polls > 64 ? 500 : 100);
     }
     return 0;
+}
+__device__ __forceinline__ uint32_t await_published(const uint32_t* where) {
+    return await_published(where, [] { return false; });
 }
 
 // One thread: block k towards L2.
@@ -958,21 +978,22 @@ template <int DT>
 __device__ __forceinline__ void count_done(FusedControl* ctl, uint32_t which, uint32_t mine, uint32_t complete) {
     FusedShared& sh = fused_shared<DT>();
     const uint32_t tid = threadIdx.x;
-    __threadfence();
     __syncthreads();
-    if (tid == 0) sh.word = atomicAdd(&ctl->hist_done[which].value, mine) + mine == complete;
+    if (tid == 0) sh.word = add_acq_rel(&ctl->hist_done[which].value, mine) + mine == complete;
     __syncthreads();
     if (sh.word && tid < 32) {
-        __threadfence();
         const uint32_t found = search_global<DT>(ctl->hist[which], which == 1 ? ctl->pack_hist : nullptr,
                                                  reinterpret_cast<unsigned long long*>(fused_smem())) | kParamsValid;
-        if (tid == 0) publish(&ctl->params[which], found);
+        if (tid == 0) publish_word(&ctl->params[which], found);
     }
 }
 
 // The histogram of `total` blocks, every `stride`-th from `base` on, all CTAs together, and the parameters that the search
 // finds for it (0: a wait ran out). which: 0 the sample, 1 what the pack stage's histogram lacks of the whole tensor; it is
 // complete when `complete` blocks are counted here or there.
+// In the sample stage a CTA starts with the block of its own number: it loads it at once and claims it meanwhile (444 CTAs
+// that ask one ticket and wait for the answer begin up to 2 us later). The rest goes by tickets. A claim, because the block
+// of a CTA that has not started (other work holds its SM) is taken by one that waits; the CTA drops its counts then.
 template <int DT>
 __device__ __noinline__ uint32_t histogram_stage(FusedControl* ctl, uint32_t which, uint32_t base, uint32_t total, uint32_t stride,
                                             uint32_t complete) {
@@ -981,29 +1002,63 @@ __device__ __noinline__ uint32_t histogram_stage(FusedControl* ctl, uint32_t whi
     constexpr uint32_t kElemBytes = DT == ENEC_FP32 ? 4 : 2;
     const uint32_t tid = threadIdx.x, lane = tid & 31;
     const uint32_t work = smem_u32(fused_smem());
-    const bool ahead = total > gridDim.x;   // tickets are asked for ahead; else a CTA has one block as a rule
     uint32_t* const ticket = &ctl->hist_ticket[which].value;
-    bool first = true;
+    const uint32_t claimed = which != 0 ? 0 : total < gridDim.x ? total : gridDim.x;   // blocks that are claimed
+    auto claim = [&](uint32_t i) { return (atomicOr(&ctl->claims[i / 32].value, 1u << (i & 31)) >> (i & 31) & 1) == 0; };
+    auto unclaimed = [&](uint32_t w) {
+        const uint32_t bits = claimed - 32 * w < 32 ? (1u << (claimed - 32 * w)) - 1 : ~0u;
+        return bits & ~ld_relaxed_u32(&ctl->claims[w].value);
+    };
     uint32_t word;
-    for (;;) {
+    for (bool first = true;; first = false) {
         __syncthreads();
         for (uint32_t i = tid; i < uint32_t(HistShape<DT>::kBytes / 16); i += kFusedThreads) sts128(work + 16 * i, make_uint4(0, 0, 0, 0));
-        if (tid == 0) sh.word = atomicAdd(ticket, 1u);
-        __syncthreads();
-        uint32_t mine = 0;
-        for (uint32_t i = sh.word; i < total; ++mine) {
-            uint32_t asked = total;
-            if (ahead && tid == 0) {
-                asked = atomicAdd(ticket, 1u);
-                if (asked < total) fetch_block<DT>(t, base + asked * stride);
+        const bool own = first && blockIdx.x < claimed;
+        uint32_t taken = 0;   // thread 0: not zero when somebody else counts the block of this CTA's number
+        uint32_t i = blockIdx.x;
+        const uint32_t bit = own ? 1u << (i & 31) : 0;
+        if (own) {
+            if (tid == 0) taken = atomicOr(&ctl->claims[i / 32].value, bit);   // the answer comes while the block is counted
+            __syncthreads();
+        } else {
+            if (tid == 0) {
+                uint32_t got = total;
+                if (claimed == 0) {
+                    got = atomicAdd(ticket, 1u);
+                } else if (!first) {
+                    for (uint32_t w = 0; 32 * w < claimed && got == total; ++w)
+                        for (uint32_t bits = unclaimed(w); bits && got == total; bits &= bits - 1) {
+                            const uint32_t c = 32 * w + uint32_t(__ffs(bits)) - 1;
+                            if (claim(c)) got = c;
+                        }
+                }
+                sh.word = got;
             }
+            __syncthreads();
+            i = sh.word;
+        }
+        uint32_t mine = 0;
+        while (i < total) {
+            // (asked for, not waited for: fetching the next block towards L2 meanwhile, 1024 blocks 26.9 us instead of 25.5)
+            uint32_t asked = 0;
+            if (tid == 0 && claimed < total) asked = atomicAdd(ticket, 1u);
             const uint32_t k = base + i * stride;
             const uint32_t real = k + 1 == t.nblocks ? t.tail_real : kBlockElems;
             count_block<DT>(t.in + uint64_t(k) * kBlockElems * kElemBytes, real, work + lane * 4, tid);
             __syncthreads();
-            if (tid == 0) sh.word = asked;
+            if (tid == 0) {
+                sh.word = claimed < total ? claimed + asked : total;
+                sh.ok = (taken & bit) == 0;
+                taken = 0;
+            }
             __syncthreads();
             i = sh.word;
+            if (sh.ok) {
+                ++mine;
+            } else {
+                for (uint32_t j = tid; j < uint32_t(HistShape<DT>::kBytes / 16); j += kFusedThreads) sts128(work + 16 * j, make_uint4(0, 0, 0, 0));
+                __syncthreads();
+            }
         }
         if (mine) {
             if (tid < uint32_t(HistShape<DT>::kBins)) {
@@ -1016,13 +1071,16 @@ __device__ __noinline__ uint32_t histogram_stage(FusedControl* ctl, uint32_t whi
         if (tid == 0) {
             if (which == 0 && first) {   // the CTA's first block of the pack stage is asked for, and brought towards L2, meanwhile
                 sh.next = atomicAdd(&ctl->pack_ticket[0].value, 1u);
-                if (!mine) __nanosleep(3000);   // behind the loads of the blocks that are being counted
+                if (!mine) __nanosleep(2000);   // behind the loads of the blocks that are being counted
                 fetch_block<DT>(t, sh.next);
             }
-            // a CTA of the grid that has not started (other work holds its SM) leaves its block to one that waits
-            sh.word = await_published(&ctl->params[which], ticket, total);
+            sh.word = await_published(&ctl->params[which], [&] {
+                if (claimed == 0) return ld_relaxed_u32(ticket) < total;
+                for (uint32_t w = 0; 32 * w < claimed; ++w)
+                    if (unclaimed(w)) return true;
+                return false;
+            });
         }
-        first = false;
         __syncthreads();
         word = sh.word;
         __syncthreads();
@@ -1072,8 +1130,22 @@ __device__ __noinline__ void recount_block(FusedControl* ctl, uint32_t k) {
     __syncthreads();
 }
 
+// A warp, when the CTA has flushed the histogram of its blocks of the first pass: `mine` more blocks are counted. The warp
+// that completes the tensor runs the search, with the CTA's table of the pack stage as its shared memory.
+template <int DT>
+__device__ __noinline__ void first_pass_counted(FusedControl* ctl, uint32_t mine, uint32_t nblocks) {
+    uint32_t last = 0;
+    if ((threadIdx.x & 31) == 0) last = add_acq_rel(&ctl->pack_done.value, mine) + mine == nblocks;
+    if (!__shfl_sync(0xFFFFFFFFu, last, 0)) return;
+    const uint32_t found = search_global<DT>(ctl->pack_hist, ctl->hist[1],
+                                             reinterpret_cast<unsigned long long*>(fused_smem() + FusedShape<DT>::kHistAt)) |
+                           kParamsValid | (ld_relaxed_u32(&ctl->pack_target) ? kParamsRedo : 0u);
+    if ((threadIdx.x & 31) == 0) publish_word(&ctl->verdict, found);
+}
+
 // The pack stage's blocks, ticket after ticket, starting with the one in sh.next; all threads. HIST: the parameters come
-// from a sample. Returns the number of blocks packed, and kPassEnded where a ticket said so. (A function of its own per form, so that each has its own registers.)
+// from a sample. Returns the number of blocks packed, and kPassEnded where a ticket said so: those blocks have not been added
+// to pack_done yet. (A function of its own per form, so that each has its own registers.)
 //
 // Two barriers per block: A after the first phase (values, mask and lists are complete), B after the second (planes and
 // records are complete). What follows B reads only what is not written before the next A.
@@ -1117,7 +1189,7 @@ __device__ __noinline__ uint32_t pack_pass(FusedControl* ctl, uint32_t pass, int
     // one thread: no further block is handed out; those handed out already are packed, so that nobody waits for them in vain
     auto end_pass = [&]() {
         const uint32_t handed = atomicOr(&ctl->pack_ticket[pass].value, kPassEnded);
-        if ((handed & kPassEnded) == 0) publish(&ctl->pack_target, handed < t.nblocks ? handed : t.nblocks);
+        if ((handed & kPassEnded) == 0) publish_word(&ctl->pack_target, handed < t.nblocks ? handed : t.nblocks);
     };
     uint32_t k = sh.next;
     __syncthreads();   // before thread 0 writes the next ticket there
@@ -1205,14 +1277,17 @@ __device__ __noinline__ uint32_t pack_pass(FusedControl* ctl, uint32_t pass, int
         k = next;
     }
     __syncthreads();
-    if (HIST && mine) {   // under way while the last block's offset is looked up
-        if (tid < Shape::kRows) {
-            // row r of the table holds the exponent x of that remainder that the parameters can represent
-            const uint32_t n = fold_hist_row<false>(work + Shape::kHistAt + tid * HistShape<DT>::kRowBytes, tid);
+    if (HIST && mine && warp == kFusedWarps - 1) {
+        // The CTA's counts go out, and the search on the whole tensor's is run, while the first warp looks up the last block's offset.
+        // Row r of the table holds the exponent x of that remainder that the parameters can represent.
+        for (uint32_t row = lane; row < Shape::kRows; row += 32) {
+            const uint32_t n = fold_hist_row<false>(work + Shape::kHistAt + row * HistShape<DT>::kRowBytes, row);
             const uint32_t d = uint32_t(t.b) + (1u << (t.n - 1));
-            const uint32_t x = (d - ((d - tid) & (Shape::kRows - 1))) & ((1u << E) - 1);
+            const uint32_t x = (d - ((d - row) & (Shape::kRows - 1))) & ((1u << E) - 1);
             if (n) atomicAdd(&ctl->pack_hist[x], (unsigned long long)n);
         }
+        __syncwarp();
+        if (k < kPassEnded) first_pass_counted<DT>(ctl, mine, t.nblocks);
     }
     if (HIST && k >= kPassEnded) return mine | kPassEnded;
     if (pend_block != 0xFFFFFFFFu) place_waiting(false);
@@ -1311,24 +1386,21 @@ enec_fused_kernel(const FusedJob job, int* status) {
         }
 
         // ---- the sampled parameters against the whole tensor's ----
-        __threadfence();
         __syncthreads();
-        if (tid == 0) sh.word = mine && atomicAdd(&ctl->pack_done.value, mine) + mine == nblocks;
-        __syncthreads();
-        if (sh.word && warp == 0) {   // the last CTA to leave
-            __threadfence();
-            const uint32_t found = search_global<DT>(ctl->pack_hist, ctl->hist[1], search_table) | kParamsValid |
-                                   (ld_relaxed_u32(&ctl->pack_target) ? kParamsRedo : 0u);
-            if (lane == 0) publish(&ctl->verdict, found);
-        }
-        __syncthreads();
+        if (mine && (left & kPassEnded) && warp == 0) first_pass_counted<DT>(ctl, mine, nblocks);
         if (tid == 0) {
-            sh.word = await_published(&ctl->verdict);
-            sh.next = sh.word == word || sh.word == 0 ? 0u : atomicAdd(&ctl->pack_ticket[1].value, 1u);
+            const uint32_t verdict = await_published(&ctl->verdict);
+            if (verdict != word && verdict != 0) {
+                // a second pass: it begins when the first one's last bytes have been written
+                if (mine && add_acq_rel(&ctl->pack_left.value, mine) + mine == nblocks) publish(&ctl->all_left, 1u);
+                sh.ok = await_published(&ctl->all_left);
+                sh.next = atomicAdd(&ctl->pack_ticket[1].value, 1u);
+            }
+            sh.word = verdict;
         }
         __syncthreads();
         if (sh.word == word) return;
-        word = sh.word & ~kParamsRedo;
+        word = sh.ok ? sh.word & ~kParamsRedo : 0u;
     }
 }
 

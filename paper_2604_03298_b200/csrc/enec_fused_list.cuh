@@ -201,13 +201,11 @@ enec_fused_list_kernel(const FusedList list, int* status) {
                 const uint32_t c = fold_hist_row<false>(work + tid * HistShape<DT>::kRowBytes, tid);
                 if (c) atomicAdd(&ctl.hist[tid], (unsigned long long)c);
             }
-            __threadfence();
             __syncthreads();
-            if (tid == 0) sh.word = atomicAdd(&ctl.done, n) + n == item.nblocks;
+            if (tid == 0) sh.word = add_acq_rel(&ctl.done, n) + n == item.nblocks;
             scout_end(iter, next_slot);
             __syncthreads();
             if (sh.word && warp == 0) {
-                __threadfence();
                 const uint32_t found = search_global<DT>(ctl.hist, nullptr, search_table);
                 if (lane == 0) {
                     fill_tensor<DT>(ctl.tensor, item, found);
