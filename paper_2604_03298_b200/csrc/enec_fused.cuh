@@ -771,23 +771,19 @@ __device__ __noinline__ bool pack_front_tail(uint32_t k, uint32_t* wide_of_warp,
     const FusedTensor& t = fused_tensor<DT>(slot);
     FusedShared& sh = fused_shared<DT>();
     constexpr uint32_t kElemBytes = DT == ENEC_FP32 ? 4 : 2;
-    constexpr int E = Shape::E;
     const uint32_t tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const uint32_t work = smem_u32(fused_smem());
     const uint32_t N = t.tail_padded, real = t.tail_real;
     const uint8_t* in = t.in + uint64_t(k) * kBlockElems * kElemBytes;
     uint8_t* out_lo = t.lo + uint64_t(k) * kBlockElems * 2;
     if (tid < 32) sh.mask[tid] = 0;
-    bool bad = false;
-    if (HIST) {   // its real elements, one by one
-        for (uint32_t e = tid; e < real; e += kFusedThreads) {
-            const uint32_t x = exponent_of_word<DT>(exponent_word<DT>(in, e));
-            red_add_one(work + Shape::kHistAt + lane * 4 + (x & (Shape::kRows - 1)) * HistShape<DT>::kRowBytes);
-            bad = bad || (((uint32_t(t.b - int(x)) + (1u << (t.n - 1))) & ((1u << E) - 1)) >> t.n) != 0;
-        }
+    if (HIST && tid < (real & 15)) {   // the values of the one run that is part padding are counted one by one
+        const uint32_t x = exponent_of_word<DT>(exponent_word<DT>(in, (real & ~15u) + tid));
+        red_add_one(work + Shape::kHistAt + lane * 4 + (x & (Shape::kRows - 1)) * HistShape<DT>::kRowBytes);
     }
     __syncthreads();
-    uint32_t wide = 0;
+    uint32_t wide = 0, all = 0;
+    // (one run at a time: with more registers the full blocks' loop, which shares its frame with the call, loses 6 %)
 #pragma unroll 1
     for (uint32_t i = 0; i < kBlockElems / (16 * kFusedThreads); ++i) {
         const uint32_t first = i * kFusedThreads + warp * 32;   // the warp's first group of this round
@@ -800,15 +796,20 @@ __device__ __noinline__ bool pack_front_tail(uint32_t k, uint32_t* wide_of_warp,
                 r = split_halves(load32<false>(in + uint64_t(e0) * 4), load32<false>(in + uint64_t(e0) * 4 + 32), out_lo + uint64_t(e0) * 2, false);
             else
                 r = load32<false>(in + uint64_t(e0) * 2);
+            if (HIST) {
+#pragma unroll
+                for (int q = 0; q < 8; ++q) count_halves<DT>(work + Shape::kHistAt, lane * 4, r.w[q]);
+            }
         } else {
             r = load_run_tail<DT>(in + uint64_t(e0) * kElemBytes, out_lo + uint64_t(e0) * 2, left,
                                   int(align16(2 * uint64_t(real)) / 2) - int(e0), t.pad);
         }
         // the padding's sign/mantissa bytes are zero
-        pack_run<DT, PLAIN, false>(r, t.c, t.nmask4, t.s4, t.wide4, 0, lane, work + Shape::kValuesAt + g * 16, i * 32 + lane,
-                                   work + Shape::kListAt + warp * 128, wide, &sh.mask[i * kFusedWarps + warp], left > 0,
-                                   t.sm + uint64_t(k) * kBlockElems + e0);
+        all |= pack_run<DT, PLAIN, false>(r, t.c, t.nmask4, t.s4, t.wide4, 0, lane, work + Shape::kValuesAt + g * 16, i * 32 + lane,
+                                          work + Shape::kListAt + warp * 128, wide, &sh.mask[i * kFusedWarps + warp], left > 0,
+                                          t.sm + uint64_t(k) * kBlockElems + e0);
     }
+    const bool bad = HIST && (DT == ENEC_FP16 ? all & rep4(0x1F) & ~t.nmask4 : all & ~t.nmask4) != 0;
     *wide_of_warp = wide;
     return bad;
 }
@@ -1193,7 +1194,8 @@ __device__ __noinline__ uint32_t pack_pass(FusedControl* ctl, uint32_t pass, int
     };
     uint32_t k = sh.next;
     __syncthreads();   // before thread 0 writes the next ticket there
-    for (; k < t.nblocks; ++iter) {
+    const uint32_t limit = t.nblocks - (t.tail_padded < 128 ? 1 : 0);   // a last block of less than 128 elements: behind the loop
+    for (; k < limit; ++iter) {
         uint32_t asked = 0;
         if (tid == 0) asked = t.nblocks == 1 ? 1u : atomicAdd(&ctl->pack_ticket[pass].value, 1u);
         ++mine;
@@ -1203,12 +1205,8 @@ __device__ __noinline__ uint32_t pack_pass(FusedControl* ctl, uint32_t pass, int
         bool bad = false;
         if (!last) {
             bad = pack_front_full<DT, PLAIN, HIST>(t, k, work, sh.mask, tid, wide_of_warp);
-        } else if (N >= 128) {
+        } else {
             bad = pack_front_tail<DT, PLAIN, HIST>(k, &wide_of_warp);
-        } else if (HIST && tid < t.tail_real) {
-            const uint32_t x = exponent_of_word<DT>(exponent_word<DT>(t.in + uint64_t(k) * kBlockElems * kElemBytes, tid));
-            red_add_one(work + Shape::kHistAt + lane * 4 + (x & (Shape::kRows - 1)) * HistShape<DT>::kRowBytes);
-            bad = (((uint32_t(t.b - int(x)) + (1u << (t.n - 1))) & ((1u << E) - 1)) >> t.n) != 0;
         }
         if (tid == 0) {
             sh.next = asked;
@@ -1217,15 +1215,6 @@ __device__ __noinline__ uint32_t pack_pass(FusedControl* ctl, uint32_t pass, int
         const bool lossy = __syncthreads_or(bad) != 0;   // barrier A
         if ((lossy || stop) && tid == 0) end_pass();
         const bool waiting = pend_block != 0xFFFFFFFFu;
-        if (N < 128) {
-            if (waiting) place_waiting(false);
-            pend_block = 0xFFFFFFFFu;
-            if (HIST && lossy) recount_block<DT>(ctl, k);
-            __syncthreads();
-            pack_short_block<DT>(k, status);
-            k = sh.next;
-            break;   // no block comes after this one
-        }
         unsigned long long answer = 0;
         if (waiting) answer = ask_before(t, pend_block, tid);   // it comes while the block is packed
         uint32_t mask_word, excl;
@@ -1277,6 +1266,22 @@ __device__ __noinline__ uint32_t pack_pass(FusedControl* ctl, uint32_t pass, int
         k = next;
     }
     __syncthreads();
+    const bool ends_short = k < t.nblocks;   // the CTA has that block: all others have been handed out
+    if (ends_short) {
+        ++mine;
+        if (HIST) {
+            bool bad = false;
+            if (tid < t.tail_real) {
+                const uint32_t x = exponent_of_word<DT>(exponent_word<DT>(t.in + uint64_t(k) * kBlockElems * kElemBytes, tid));
+                red_add_one(work + Shape::kHistAt + lane * 4 + (x & (Shape::kRows - 1)) * HistShape<DT>::kRowBytes);
+                bad = (((uint32_t(t.b - int(x)) + (1u << (t.n - 1))) & ((1u << E) - 1)) >> t.n) != 0;
+            }
+            if (__syncthreads_or(bad)) {
+                if (tid == 0) end_pass();
+                recount_block<DT>(ctl, k);
+            }
+        }
+    }
     if (HIST && mine && warp == kFusedWarps - 1) {
         // The CTA's counts go out, and the search on the whole tensor's is run, while the first warp looks up the last block's offset.
         // Row r of the table holds the exponent x of that remainder that the parameters can represent.
@@ -1291,6 +1296,10 @@ __device__ __noinline__ uint32_t pack_pass(FusedControl* ctl, uint32_t pass, int
     }
     if (HIST && k >= kPassEnded) return mine | kPassEnded;
     if (pend_block != 0xFFFFFFFFu) place_waiting(false);
+    if (ends_short) {
+        __syncthreads();
+        pack_short_block<DT>(k, status);
+    }
     return mine;
 }
 
