@@ -697,6 +697,7 @@ struct DecodeBatch {
     uint32_t n_jobs;
     uint32_t total_blocks;
     uint32_t option;          // one tensor: 1 = its stream is of the block-wise variant; TICKET = 1: blocks per chunk
+    uint32_t apart;           // fixed shares: 1 = the last CTA has the last block and no other (see launch_decode)
     DecodeJob inline_jobs[kInlineJobs];          // used when jobs is null (one tensor, or a short list)
     uint32_t inline_prefix[kInlineJobs + 1];
 };
@@ -774,8 +775,9 @@ enec_decode_kernel(const __grid_constant__ DecodeBatch batch, int* status) {
 
     pdl_launch_dependents();
     // everything up to pdl_wait() may run while the previous kernel of the stream still does
-    const uint32_t first_block = uint32_t(uint64_t(blockIdx.x) * batch.total_blocks / gridDim.x);
-    const uint32_t end_block = uint32_t(uint64_t(blockIdx.x + 1) * batch.total_blocks / gridDim.x);
+    const uint32_t shares = gridDim.x - batch.apart, shared_blocks = batch.total_blocks - batch.apart;
+    const uint32_t first_block = uint32_t(uint64_t(blockIdx.x) * shared_blocks / shares);
+    const uint32_t end_block = blockIdx.x < shares ? uint32_t(uint64_t(blockIdx.x + 1) * shared_blocks / shares) : batch.total_blocks;
     const uint32_t n_mine = end_block - first_block;
     if (threadIdx.x == kConsumerWarps * 32) {
         if constexpr (TICKET == 2)  // the CTA's first chunk

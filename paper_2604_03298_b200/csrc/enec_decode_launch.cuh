@@ -24,7 +24,7 @@ inline DecodeDevice* decode_device(int dev) {
 }
 
 template <int DT>
-inline enec_status launch_decode(const DecodeBatch& batch, int* d_status, cudaStream_t stream, bool ranked = false,
+inline enec_status launch_decode(DecodeBatch batch, int* d_status, cudaStream_t stream, bool ranked = false,
                                  int ticketed = 0) {
     int dev = 0;
     if (cudaGetDevice(&dev) != cudaSuccess) return ENEC_ERR_CUDA;
@@ -46,6 +46,13 @@ inline enec_status launch_decode(const DecodeBatch& batch, int* d_status, cudaSt
     uint32_t grid = uint32_t(info.sms) * 3;  // three resident CTAs per SM
     if (grid > batch.total_blocks) grid = batch.total_blocks;
     if (grid == 0) grid = 1;
+    // A last block that is not full takes the general body, which is slower and whose code comes from memory when another kernel
+    // has run since: a CTA of its own begins it at once, where the other CTAs' largest share stays what it is. 1024 blocks of
+    // fp32 and one value, right after they were compressed: 46 -> 39 us; 1023 blocks of fp16 and 15335 values 16.7 -> 14.5.
+    batch.apart = 0;
+    if (ticketed == 0 && batch.jobs == nullptr && batch.n_jobs == 1 && batch.total_blocks > grid && grid > 1 &&
+        batch.inline_jobs[0].count % kBlockElems != 0)
+        batch.apart = (batch.total_blocks - 1 + grid - 2) / (grid - 1) == (batch.total_blocks + grid - 1) / grid ? 1 : 0;
     const cudaError_t err =
         ranked         ? launch_pdl(enec_decode_kernel<DT, true>, grid, kDecodeThreads, kDecodeSmemBytes, stream, batch, d_status)
         : ticketed == 1 ? launch_pdl(enec_decode_kernel<DT, false, 1>, grid, kDecodeThreads, kDecodeSmemBytes, stream, batch,

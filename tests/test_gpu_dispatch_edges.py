@@ -142,6 +142,17 @@ def test_decompress_last_blocks(oracle, dt, count, wide):
     assert bool((out[count:] == 1.0).all()), "wrote behind the tensor"
 
 
+@pytest.mark.parametrize("dt", [0, 1, 2])
+@pytest.mark.parametrize("blocks", [443, 444, 445, 887, 888, 889, 1331])
+@pytest.mark.parametrize("tail", [0, 1, 5003])
+def test_decompress_last_block_apart(dt, blocks, tail):
+    """Sizes around multiples of the number of CTAs (three per SM), where a ragged last block gets a CTA of its own or not."""
+    import paper_2604_03298_b200 as enec
+    t = _weights(blocks * 16384 + tail, dt, blocks + tail)
+    out = enec.decompress_tensor(enec.compress_tensor(t), t.dtype, t.shape)
+    assert torch.equal(out.view(BITS[dt]), t.view(BITS[dt]))
+
+
 def test_checked_calls_report_errors_and_recover():
     """compress_tensor / decompress_tensor read length and status from pinned host memory that the kernels write: an error is
     raised, and the next call on the thread starts clean; threads do not share the memory."""
