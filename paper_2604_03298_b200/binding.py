@@ -181,32 +181,39 @@ class _Answer:
         self.address = self.memory.data_ptr()
         self.size = C.c_int64.from_address(self.address)
         self.status = C.c_int32.from_address(self.address + 8)
-        self.stream = None   # set while kernels may still write here: a call that failed half way leaves it set
+        self.where = None      # (device, stream handle) of the last call, and the stream as an object
+        self.stream = None
+        self.pending = False   # kernels may still write here: a call that failed half way leaves it set
 
 
 _local = threading.local()
 
 
 def _answer():
-    """This thread's answer memory, cleared. (One per thread is enough: a checked call ends after its stream's work has.)"""
+    """This thread's answer memory, cleared, and the current stream's handle. (One per thread is enough: a checked call ends
+    after its stream's work has. Asking torch for the stream object on every call took 3 us.)"""
     a = getattr(_local, "answer", None)
     if a is None:
         a = _local.answer = _Answer()
-    elif a.stream is not None:
+    elif a.pending:
         a.stream.synchronize()
     a.size.value = 0
     a.status.value = 0
-    a.stream = torch.cuda.current_stream()
-    return a
+    device = torch.cuda.current_device()
+    handle = torch._C._cuda_getCurrentRawStream(device)
+    if a.where != (device, handle):
+        a.stream, a.where = torch.cuda.current_stream(), (device, handle)
+    a.pending = True
+    return a, handle
 
 
 def _finish(a, st, where):
     """Waits for the call's stream and raises on an error of the call (st) or of its kernels. (Cleared and copied device memory,
-    as before, cost 15 us more for each call: norm weights there and back took 86 us, 55 us now.)"""
+    as before, cost 15 us more for each call: 4 M values there and back took 97 us, 62 us now.)"""
     if st != 0:
         raise EnecError(st, where)
     a.stream.synchronize()
-    a.stream = None
+    a.pending = False
     if a.status.value != 0:
         raise EnecError(a.status.value, where + " (device)")
 
@@ -219,11 +226,11 @@ def compress_tensor(t: torch.Tensor, params=None) -> torch.Tensor:
     count = t.numel()
     cap = enec_max_compressed_size(dt, count)
     out = torch.empty(cap, dtype=torch.uint8, device=t.device)
-    a = _answer()
+    a, stream_handle = _answer()
     if params is None:
-        st = lib().enec_compress(t.data_ptr(), dt, count, out.data_ptr(), cap, a.address, a.address + 8, a.stream.cuda_stream)
+        st = lib().enec_compress(t.data_ptr(), dt, count, out.data_ptr(), cap, a.address, a.address + 8, stream_handle)
     else:
-        st = lib().enec_compress_with_params(t.data_ptr(), dt, count, *params, out.data_ptr(), cap, a.address, a.address + 8, a.stream.cuda_stream)
+        st = lib().enec_compress_with_params(t.data_ptr(), dt, count, *params, out.data_ptr(), cap, a.address, a.address + 8, stream_handle)
     _finish(a, st, "enec_compress")
     return out[:a.size.value]
 
@@ -231,7 +238,7 @@ def compress_tensor(t: torch.Tensor, params=None) -> torch.Tensor:
 def decompress_tensor(stream: torch.Tensor, dtype: torch.dtype, shape) -> torch.Tensor:
     dt = _DT[dtype]
     out = torch.empty(shape, dtype=dtype, device=stream.device)
-    a = _answer()
-    st = lib().enec_decompress(stream.data_ptr(), stream.numel(), dt, out.numel(), out.data_ptr(), a.address + 8, a.stream.cuda_stream)
+    a, stream_handle = _answer()
+    st = lib().enec_decompress(stream.data_ptr(), stream.numel(), dt, out.numel(), out.data_ptr(), a.address + 8, stream_handle)
     _finish(a, st, "enec_decompress")
     return out
