@@ -281,7 +281,7 @@ static enec_status compress_common(const void* d_in, enec_dtype dt, size_t count
     cudaStreamCaptureStatus capturing = cudaStreamCaptureStatusNone;
     if (cudaStreamIsCapturing(stream, &capturing) != cudaSuccess) return ENEC_ERR_CUDA;
     if (capturing != cudaStreamCaptureStatusNone) return ENEC_ERR_INVALID_ARG;
-    if (!with_params && !ranked && !earlier_forms()) {
+    if (!ranked && !earlier_forms()) {
         FusedJob fused;
         enec_status fst = lease_fused_scratch(dev, stream, g.nblocks, fused);
         if (fst != ENEC_OK) return fst;
@@ -289,6 +289,7 @@ static enec_status compress_common(const void* d_in, enec_dtype dt, size_t count
         fused.out = static_cast<uint8_t*>(d_out);
         fused.count = count;
         fused.out_size = out_size;
+        fused.given = with_params ? uint32_t(b) | uint32_t(n) << 8 | uint32_t(m) << 12 | kParamsValid : 0u;
         fst = launch_fused(int(dt), fused, g.nblocks, info.sms, info.fused_attr_set, d_status, stream);
         if (fst != ENEC_OK) mark_scratch_unclean(dev, stream, kScratchFused);
         return fst;

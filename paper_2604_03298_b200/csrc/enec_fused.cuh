@@ -9,6 +9,9 @@
 //      parameters that were used, the stream is the one that the search on the whole tensor leads to. When it does not, the
 //      CTAs pack the tensor again; a value that the sampled parameters cannot represent ends the pack stage at once, and the blocks
 //      not packed yet are counted first.
+// Parameters given by the caller: stage 2 alone, without the histogram, from the first block on; a value that they lose ends
+// the call without a stream. (With a look-back kernel, or two kernels from 2048 blocks up, 3584 blocks of bf16 took 54 us, now 38.7;
+// 1024 blocks 23.2 -> 15.1, fp16 4096 blocks 63.8 -> 47.5, fp32 8192 blocks 192 -> 168.)
 // A tensor whose sample needs n > 6 exponent bits (bf16, fp32) takes the histogram of the whole tensor before it packs:
 // the table kept beside the packing has 64 rows, and rare outliers of such a tensor are what a sample misses.
 //
@@ -49,6 +52,7 @@ struct alignas(128) FusedControl {
     Counter pack_left;         // blocks packed by the CTAs that have left the first pass, when there is a second
     uint32_t pack_target;      // blocks handed out before the first pass was ended early (0: it was not)
     uint32_t params[2];        // published: the parameters for hist[0], hist[1]
+    uint32_t lossy;            // given parameters: some block holds a value that they lose
     uint32_t verdict;          // published: the whole tensor's parameters, when the first pass has counted every block
     uint32_t all_left;         // published: the first pass writes no more
 };
@@ -70,6 +74,7 @@ struct FusedJob {
     uint32_t super_stride;
     uint32_t clear_supers;         // ... with so many first-level sums per pass
     uint32_t sample;               // blocks in the sample (nblocks: all)
+    uint32_t given;                // the caller's parameters, as a published word (0: search)
     uint32_t epoch;                // tag of the first pass's state words; the second pass's is one more
     unsigned long long* state;     // per block: bits 63..32 epoch, bits 31..0 wide groups
     unsigned long long* out_size;  // device, may be null
@@ -121,6 +126,7 @@ struct FusedTensor {
     uint32_t pad;      // two 16-bit words with exponent b and nothing else: y = 0
     uint32_t wide_ok;  // bit 0: the input is 32-byte aligned, bit 1: the sm-lo plane is
     uint32_t plain;
+    const uint32_t* lossy;         // given parameters: see FusedControl
     uint32_t first_block;          // lists: index of the tensor's first block in the list's index space
 };
 
@@ -358,7 +364,7 @@ __device__ __forceinline__ void count_halves(uint32_t hist, uint32_t lane4, uint
     }
 }
 
-template <int DT, bool PLAIN, bool HIST>
+template <int DT, bool PLAIN, bool HIST, bool CHECK>
 __device__ __forceinline__ void transform_run(const Run& r, uint32_t minuend, uint32_t nmask4, uint32_t hist, uint32_t lane4, uint4& v,
                                               uint4& hs, uint4& sm) {
     uint32_t vv[4], ss[4], hh[4];
@@ -377,7 +383,8 @@ __device__ __forceinline__ void transform_run(const Run& r, uint32_t minuend, ui
                 vv[q] = prmt(minuend - 2 * w0, minuend - 2 * w1, 0x7531u);
             } else {
                 const uint32_t x = prmt(2 * w0, 2 * w1, 0x7531u);
-                vv[q] = (((minuend | 0x80808080u) - (x & 0x7F7F7F7Fu)) ^ ((minuend ^ ~x) & 0x80808080u)) & nmask4;
+                vv[q] = ((minuend | 0x80808080u) - (x & 0x7F7F7F7Fu)) ^ ((minuend ^ ~x) & 0x80808080u);
+                if (!CHECK) vv[q] &= nmask4;
             }
         }
         if constexpr (HIST) {
@@ -665,11 +672,16 @@ __device__ __forceinline__ void copy_halves(uint8_t* dst, uint32_t src, uint32_t
 
 // The end of a block, by a warp that knows its offset: table entry; for the last block also the header, the end of
 // the table, the padding behind the records and the stream length.
-template <int DT>
+// CHECK (given parameters): nothing of that, when some block lost a value. Its CTA has said so before it published its count.
+template <int DT, bool CHECK = false>
 __device__ __forceinline__ void finish_block(const FusedTensor& t, uint32_t k, uint32_t before, uint32_t wide) {
     if ((threadIdx.x & 31) != 0) return;
     t.table[k] = before;
     if (k + 1 != t.nblocks) return;
+    if constexpr (CHECK) {
+        __threadfence();
+        if (ld_relaxed_u32(t.lossy)) return;
+    }
     const uint32_t a_total = before + wide;
     const uint64_t high_bytes = uint64_t(a_total) * 2 * uint32_t(t.hbits);
     const uint64_t total = uint64_t(t.high - t.out) + align16(high_bytes);
@@ -702,12 +714,12 @@ __device__ __forceinline__ Run load32_any(const uint8_t* p, bool wide) {
 // One run of sixteen values of a block, group `g` of it: sign/mantissa plane, histogram, values (16 bytes per group; fp16:
 // the bits of the fp16 plane in bits 7..5 of each byte), votes for the group mask and the numbers of the warp's wide
 // groups. number: 32 x (which of the thread's groups) + lane. Returns the OR of all values.
-template <int DT, bool PLAIN, bool HIST>
+template <int DT, bool PLAIN, bool HIST, bool CHECK = false>
 __device__ __forceinline__ uint32_t pack_run(const Run& r, uint32_t minuend, uint32_t nmask4, uint32_t s4, uint32_t wide4, uint32_t hist,
                                              uint32_t lane, uint32_t value_at, uint32_t number, uint32_t list, uint32_t& wide,
                                              uint32_t* mask_word, bool store, uint8_t* sm_out) {
     uint4 v, hs, sm;
-    transform_run<DT, PLAIN, HIST>(r, minuend, nmask4, hist, lane * 4, v, hs, sm);
+    transform_run<DT, PLAIN, HIST, CHECK>(r, minuend, nmask4, hist, lane * 4, v, hs, sm);
     if (store) __stcs(reinterpret_cast<uint4*>(sm_out), sm);
     const uint32_t all = v.x | v.y | v.z | v.w;
     const bool is_wide = (or_flipped(v, s4) & wide4) != 0;
@@ -726,7 +738,7 @@ __device__ __forceinline__ uint32_t pack_run(const Run& r, uint32_t minuend, uin
 // Returns whether some value is not representable (HIST only); `wide_of_warp`: the warp's wide groups.
 // All loads of a thread's four runs are in flight together (3584 blocks of bf16: 56.2 us; two runs, in a rolled loop, 59.6) and
 // take no room in L1, of which the shared memory of three CTAs leaves little.
-template <int DT, bool PLAIN, bool HIST>
+template <int DT, bool PLAIN, bool HIST, bool CHECK = false>
 __device__ __forceinline__ bool pack_front_full(const FusedTensor& t, uint32_t k, uint32_t work, uint32_t* s_mask, uint32_t tid,
                                                 uint32_t& wide_of_warp) {
     using Shape = FusedShape<DT>;
@@ -742,7 +754,7 @@ __device__ __forceinline__ bool pack_front_full(const FusedTensor& t, uint32_t k
     uint32_t all = 0, wide = 0;
     const bool wide_in = (wide_ok & 1) != 0;
     auto run = [&](const Run& r, uint32_t i) {
-        all |= pack_run<DT, PLAIN, HIST>(r, minuend, nmask4, s4, wide4, work + Shape::kHistAt, lane, values + i * kStep, i * 32 + lane, list,
+        all |= pack_run<DT, PLAIN, HIST, CHECK>(r, minuend, nmask4, s4, wide4, work + Shape::kHistAt, lane, values + i * kStep, i * 32 + lane, list,
                                          wide, &s_mask[i * kFusedWarps + warp], true, sm_out + i * kStep);
     };
     if constexpr (DT == ENEC_FP32) {   // one run's 64 bytes in flight (two runs', unrolled: 1024 blocks 45.3 -> 49.6 us)
@@ -763,11 +775,11 @@ __device__ __forceinline__ bool pack_front_full(const FusedTensor& t, uint32_t k
         run(d, 3);
     }
     wide_of_warp = wide;
-    return HIST && (DT == ENEC_FP16 ? all & rep4(0x1F) & ~nmask4 : all & ~nmask4) != 0;
+    return (HIST || CHECK) && (DT == ENEC_FP16 ? all & rep4(0x1F) & ~nmask4 : all & ~nmask4) != 0;
 }
 
 // The same for the tensor's last block when it is not full and has at least 128 padded elements.
-template <int DT, bool PLAIN, bool HIST>
+template <int DT, bool PLAIN, bool HIST, bool CHECK = false>
 __device__ __noinline__ bool pack_front_tail(uint32_t k, uint32_t* wide_of_warp, uint32_t slot = 0) {
     using Shape = FusedShape<DT>;
     const FusedTensor& t = fused_tensor<DT>(slot);
@@ -807,11 +819,11 @@ __device__ __noinline__ bool pack_front_tail(uint32_t k, uint32_t* wide_of_warp,
                                   int(align16(2 * uint64_t(real)) / 2) - int(e0), t.pad);
         }
         // the padding's sign/mantissa bytes are zero
-        all |= pack_run<DT, PLAIN, false>(r, t.c, t.nmask4, t.s4, t.wide4, 0, lane, work + Shape::kValuesAt + g * 16, i * 32 + lane,
+        all |= pack_run<DT, PLAIN, false, CHECK>(r, t.c, t.nmask4, t.s4, t.wide4, 0, lane, work + Shape::kValuesAt + g * 16, i * 32 + lane,
                                           work + Shape::kListAt + warp * 128, wide, &sh.mask[i * kFusedWarps + warp], left > 0,
                                           t.sm + uint64_t(k) * kBlockElems + e0);
     }
-    const bool bad = HIST && (DT == ENEC_FP16 ? all & rep4(0x1F) & ~t.nmask4 : all & ~t.nmask4) != 0;
+    const bool bad = (HIST || CHECK) && (DT == ENEC_FP16 ? all & rep4(0x1F) & ~t.nmask4 : all & ~t.nmask4) != 0;
     *wide_of_warp = wide;
     return bad;
 }
@@ -831,7 +843,7 @@ __device__ __forceinline__ uint32_t scan_mask(const uint32_t* s_mask, uint32_t l
 
 // A tail block of 16, 32 or 64 padded elements, all threads, one element per thread, bit by bit (Algorithm 2 followed for
 // every set bit).
-template <int DT>
+template <int DT, bool CHECK = false>
 __device__ __noinline__ void pack_short_block(uint32_t k, int* status, uint32_t slot = 0) {
     const FusedTensor& t = fused_tensor<DT>(slot);
     constexpr uint32_t kElemBytes = DT == ENEC_FP32 ? 4 : 2;
@@ -896,7 +908,7 @@ __device__ __noinline__ void pack_short_block(uint32_t k, int* status, uint32_t 
         if (ok) {
             uint16_t* out_rec = reinterpret_cast<uint16_t*>(t.high + uint64_t(before) * 2 * hbits);
             if (tid < wide * hbits) out_rec[tid] = reinterpret_cast<const uint16_t*>(s_rec)[tid];   // at most 28
-            finish_block<DT>(t, k, before, wide);
+            finish_block<DT, CHECK>(t, k, before, wide);
         } else if (tid == 0) {
             report(status, ENEC_ERR_TIMEOUT);
         }
@@ -1148,11 +1160,11 @@ __device__ __noinline__ void first_pass_counted(FusedControl* ctl, uint32_t mine
 
 // The pack stage's blocks, ticket after ticket, starting with the one in sh.next; all threads. HIST: the parameters come
 // from a sample. Returns the number of blocks packed, and kPassEnded where a ticket said so: those blocks have not been added
-// to pack_done yet. (A function of its own per form, so that each has its own registers.)
+// to pack_done yet. CHECK: the parameters are the caller's; a value that they lose ends the call without a stream. (A function of its own per form, so that each has its own registers.)
 //
 // Two barriers per block: A after the first phase (values, mask and lists are complete), B after the second (planes and
 // records are complete). What follows B reads only what is not written before the next A.
-template <int DT, bool PLAIN, bool HIST>
+template <int DT, bool PLAIN, bool HIST, bool CHECK = false>
 __device__ __noinline__ uint32_t pack_pass(FusedControl* ctl, uint32_t pass, int* status) {
     using Shape = FusedShape<DT>;
     constexpr uint32_t kElemBytes = DT == ENEC_FP32 ? 4 : 2;
@@ -1187,12 +1199,17 @@ __device__ __noinline__ uint32_t pack_pass(FusedControl* ctl, uint32_t pass, int
             if (!sh.ok) { stop = true; return; }
         }
         copy_halves(t.high + uint64_t(before) * 2 * uint32_t(t.hbits), pend_at, pend_wide * uint32_t(t.hbits), tid);
-        if (warp == 0) finish_block<DT>(t, pend_block, before, pend_wide);
+        if (warp == 0) finish_block<DT, CHECK>(t, pend_block, before, pend_wide);
     };
     // one thread: no further block is handed out; those handed out already are packed, so that nobody waits for them in vain
     auto end_pass = [&]() {
         const uint32_t handed = atomicOr(&ctl->pack_ticket[pass].value, kPassEnded);
         if ((handed & kPassEnded) == 0) publish_word(&ctl->pack_target, handed < t.nblocks ? handed : t.nblocks);
+    };
+    auto say_lossy = [&]() {   // one thread, before the block's count is published
+        report(status, ENEC_ERR_PARAMS_NOT_LOSSLESS);
+        atomicOr(&ctl->lossy, 1u);
+        __threadfence();
     };
     uint32_t k = sh.next;
     __syncthreads();   // before thread 0 writes the next ticket there
@@ -1206,15 +1223,16 @@ __device__ __noinline__ uint32_t pack_pass(FusedControl* ctl, uint32_t pass, int
         uint32_t wide_of_warp = 0;
         bool bad = false;
         if (!last) {
-            bad = pack_front_full<DT, PLAIN, HIST>(t, k, work, sh.mask, tid, wide_of_warp);
+            bad = pack_front_full<DT, PLAIN, HIST, CHECK>(t, k, work, sh.mask, tid, wide_of_warp);
         } else {
-            bad = pack_front_tail<DT, PLAIN, HIST>(k, &wide_of_warp);
+            bad = pack_front_tail<DT, PLAIN, HIST, CHECK>(k, &wide_of_warp);
         }
         if (tid == 0) {
             sh.next = asked;
             fetch_block<DT>(t, asked);
         }
         const bool lossy = __syncthreads_or(bad) != 0;   // barrier A
+        if (CHECK && lossy && tid == 0) say_lossy();
         if ((lossy || stop) && tid == 0) end_pass();
         const bool waiting = pend_block != 0xFFFFFFFFu;
         unsigned long long answer = 0;
@@ -1233,7 +1251,8 @@ __device__ __noinline__ uint32_t pack_pass(FusedControl* ctl, uint32_t pass, int
             break;
         }
         const uint32_t hbits = uint32_t(t.hbits), m = uint32_t(t.m);
-        const bool direct = wide * 2 * hbits > Shape::kPend;   // the records do not fit the waiting area
+        // the records do not fit the waiting area, or there is nothing to wait for (one block: 8.85 -> 8.5 us)
+        const bool direct = wide * 2 * hbits > Shape::kPend || t.nblocks == 1;
         if (tid < uint32_t(align16(((N >> 4) + 7) / 8)) / 16)
             reinterpret_cast<uint4*>(t.mask + uint64_t(k) * (kGroupsPerBlock / 8))[tid] = reinterpret_cast<const uint4*>(sh.mask)[tid];
         pack_planes<DT>(t, work, N, tid);
@@ -1241,7 +1260,7 @@ __device__ __noinline__ uint32_t pack_pass(FusedControl* ctl, uint32_t pass, int
             if (warp == 0) {
                 uint32_t before = 0;
                 const bool ok = groups_before(t, k, before);
-                if (ok) finish_block<DT>(t, k, before, wide);
+                if (ok) finish_block<DT, CHECK>(t, k, before, wide);
                 else if (lane == 0) report(status, ENEC_ERR_TIMEOUT);
                 if (lane == 0) { sh.before = before; sh.ok = ok; }
             }
@@ -1271,16 +1290,17 @@ __device__ __noinline__ uint32_t pack_pass(FusedControl* ctl, uint32_t pass, int
     const bool ends_short = k < t.nblocks;   // the CTA has that block: all others have been handed out
     if (ends_short) {
         ++mine;
-        if (HIST) {
+        if (HIST || CHECK) {
             bool bad = false;
             if (tid < t.tail_real) {
                 const uint32_t x = exponent_of_word<DT>(exponent_word<DT>(t.in + uint64_t(k) * kBlockElems * kElemBytes, tid));
-                red_add_one(work + Shape::kHistAt + lane * 4 + (x & (Shape::kRows - 1)) * HistShape<DT>::kRowBytes);
+                if (HIST) red_add_one(work + Shape::kHistAt + lane * 4 + (x & (Shape::kRows - 1)) * HistShape<DT>::kRowBytes);
                 bad = (((uint32_t(t.b - int(x)) + (1u << (t.n - 1))) & ((1u << E) - 1)) >> t.n) != 0;
             }
             if (__syncthreads_or(bad)) {
-                if (tid == 0) end_pass();
-                recount_block<DT>(ctl, k);
+                if (CHECK && tid == 0) say_lossy();
+                if (HIST && tid == 0) end_pass();
+                if (HIST) recount_block<DT>(ctl, k);
             }
         }
     }
@@ -1300,7 +1320,7 @@ __device__ __noinline__ uint32_t pack_pass(FusedControl* ctl, uint32_t pass, int
     if (pend_block != 0xFFFFFFFFu) place_waiting(false);
     if (ends_short) {
         __syncthreads();
-        pack_short_block<DT>(k, status);
+        pack_short_block<DT, CHECK>(k, status);
     }
     return mine;
 }
@@ -1318,7 +1338,7 @@ enec_fused_kernel(const FusedJob job, int* status) {
     FusedControl* const ctl = job.ctl;
     const uint32_t nblocks = uint32_t((job.count + kBlockElems - 1) / kBlockElems);
     pdl_launch_dependents();
-    if (gridDim.x == 1)
+    if (gridDim.x == 1 && !job.given)
         for (uint32_t i = tid; i < uint32_t(HistShape<DT>::kBytes / 16); i += kFusedThreads) sts128(work + 16 * i, make_uint4(0, 0, 0, 0));
     if (tid == 0) {
         t.in = job.in; t.out = job.out; t.count = job.count; t.out_size = job.out_size;
@@ -1336,7 +1356,11 @@ enec_fused_kernel(const FusedJob job, int* status) {
     // ---- sample stage ----
     uint32_t word = 0;                              // the parameters
     bool exact = job.sample == nblocks;             // they are the whole tensor's
-    if (gridDim.x == 1) {  // one block: nothing to hand out, nobody to tell
+    if (job.given) {
+        word = job.given;
+        exact = true;
+        if (tid == 0) sh.next = nblocks == 1 ? 0u : atomicAdd(&ctl->pack_ticket[0].value, 1u);
+    } else if (gridDim.x == 1) {  // one block: nothing to hand out, nobody to tell
         count_block<DT>(job.in, t.tail_real, work + lane * 4, tid);
         __syncthreads();
         uint32_t* counts = reinterpret_cast<uint32_t*>(smem + Shape::kPendAt);
@@ -1374,6 +1398,13 @@ enec_fused_kernel(const FusedJob job, int* status) {
             for (uint32_t i = tid; i < Shape::kHistBytes / 16; i += kFusedThreads) sts128(work + Shape::kHistAt + 16 * i, make_uint4(0, 0, 0, 0));
         }
         __syncthreads();
+        if (job.given) {
+            if (tid == 0) t.lossy = &ctl->lossy;
+            __syncthreads();
+            if (t.plain || DT == ENEC_FP16) pack_pass<DT, true, false, true>(ctl, 0, status);
+            else pack_pass<DT, false, false, true>(ctl, 0, status);
+            return;
+        }
         const uint32_t left = !exact                       ? pack_pass<DT, true, true>(ctl, pass, status)
                               : t.plain || DT == ENEC_FP16 ? pack_pass<DT, true, false>(ctl, pass, status)
                                                            : pack_pass<DT, false, false>(ctl, pass, status);

@@ -143,6 +143,33 @@ def test_decompress_last_blocks(oracle, dt, count, wide):
 
 
 @pytest.mark.parametrize("dt", [0, 1, 2])
+@pytest.mark.parametrize("blocks", [0, 1, 2, 129, 445, 889])
+@pytest.mark.parametrize("tail", [0, 37, 5003])
+def test_compress_with_given_parameters(dt, blocks, tail):
+    """The search's parameters given back lead to the search's stream (checked against the oracle elsewhere); parameters that
+    lose a value, wherever it is, lead to an error and no stream length."""
+    import paper_2604_03298_b200 as enec
+    n = blocks * 16384 + tail
+    if n == 0:
+        return
+    t = _weights(n, dt, blocks + tail)
+    want = enec.compress_tensor(t)
+    b, nn, m = want[20:23].tolist()
+    assert torch.equal(enec.compress_tensor(t, params=(b, nn, m)), want)
+    size, status = torch.full((1,), -1, dtype=torch.int64, device="cuda"), status_tensor()
+    buf = torch.zeros(enec.enec_max_compressed_size(dt, n), dtype=torch.uint8, device="cuda")
+    for at in {0, n // 2, n - 1}:
+        bad = t.clone()
+        bad[at] = 3.0e4                      # an exponent far above the others
+        status.zero_()
+        assert enec.enec_compress_with_params(bad, dt, n, b, 4, min(m, 4), buf, buf.numel(), size, status) == 0
+        assert int(status.item()) == -5 and int(size.item()) == -1
+    wide = (b, 8 if dt != 1 else 5, m)       # any exponent survives the full width; the groups' form differs
+    back = enec.decompress_tensor(enec.compress_tensor(t, params=wide), t.dtype, t.shape)
+    assert torch.equal(back.view(BITS[dt]), t.view(BITS[dt]))
+
+
+@pytest.mark.parametrize("dt", [0, 1, 2])
 @pytest.mark.parametrize("blocks", [443, 444, 445, 887, 888, 889, 1331])
 @pytest.mark.parametrize("tail", [0, 1, 5003])
 def test_decompress_last_block_apart(dt, blocks, tail):
