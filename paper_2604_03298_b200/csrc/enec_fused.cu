@@ -16,8 +16,9 @@ static enec_status launch_fused_dt(FusedJob job, uint32_t nblocks, int sms, bool
     if (grid > kMaxFusedGrid) grid = kMaxFusedGrid;
     if (grid > nblocks) grid = nblocks;
     // Up to 44 MB the sample is the whole tensor: its second reading comes from L2, and the parameters need no check. Beyond,
-    // one block per SM is sampled. bf16, sampled against whole: 740 blocks 24.8 / 23.1 us, 1024 28.0 / 28.8, 1500 33.9 /
-    // 34.9, 2048 40.7 / 44.3; a few exact zeros in 1024 blocks, which a sample misses, 53 / 29 us.
+    // one block per SM is sampled. bf16, sampled against whole: 1024 blocks 24.6 / 25.1 us, 1400 29.0 / 30.8, 1600 30.3 / 33.5, 2000
+    // 35.0 / 40.1; the line lies above the crossing because the whole count spares tensors with outliers the wasted sample, and
+    // those with a few exact zeros, which a sample misses, the second pass (1024 blocks 53 / 29 us).
     job.sample = uint64_t(nblocks) * kBlockElems * elem_bytes(DT) <= (uint64_t(44) << 20) ? nblocks : uint32_t(sms);
     if (launch_pdl(enec_fused_kernel<DT>, grid, kFusedThreads, Shape::kBytes, stream, job, d_status) != cudaSuccess) return ENEC_ERR_CUDA;
     g_launches.fetch_add(1, std::memory_order_relaxed);
