@@ -19,7 +19,7 @@
 namespace enec {
 
 constexpr uint32_t kHistBlocks = 4;
-constexpr uint64_t kWaveBytes = uint64_t(40) << 20;
+constexpr uint64_t kWaveBytes = uint64_t(40) << 20;   // 8 experts and 32 vectors: 12 MB 106 us, 24 MB 97, 40 MB 91
 
 struct alignas(16) FusedItemControl {
     unsigned long long hist[256];
