@@ -490,7 +490,8 @@ static enec_status decompress_one(const void* d_in, size_t in_size, enec_dtype d
     batch.jobs = nullptr;
     batch.prefix = nullptr;
     batch.n_jobs = 1;
-    batch.option = blockwise ? 1 : 0;
+    batch.blockwise = blockwise ? 1 : 0;
+    batch.chunk_blocks = 0;
     batch.total_blocks = make_geometry(count).nblocks;
     batch.inline_jobs[0] = DecodeJob{static_cast<const uint8_t*>(d_in), static_cast<uint16_t*>(d_out), uint64_t(count),
                                      uint64_t(in_size)};
@@ -568,7 +569,8 @@ enec_status enec_decompress_batched(const enec_batch_item* h_items, int n_items,
             part.jobs = nullptr;
             part.prefix = nullptr;
             part.n_jobs = uint32_t(n);
-            part.option = 0;
+            part.blockwise = 0;
+            part.chunk_blocks = 0;
             part.total_blocks = prefix[first + n] - prefix[first];
             for (int i = 0; i < n; ++i) part.inline_jobs[i] = jobs[first + i];
             for (int i = 0; i <= n; ++i) part.inline_prefix[i] = prefix[first + i] - prefix[first];
@@ -579,7 +581,8 @@ enec_status enec_decompress_batched(const enec_batch_item* h_items, int n_items,
     }
     DecodeBatch batch;
     batch.n_jobs = uint32_t(n_items);
-    batch.option = 0;
+    batch.blockwise = 0;
+    batch.chunk_blocks = 0;
     batch.total_blocks = uint32_t(total);
     bool ticketed = false;
     // A short list travels in the launch parameters: no copy, no scratch. Unless it has so many blocks that the
@@ -595,7 +598,7 @@ enec_status enec_decompress_batched(const enec_batch_item* h_items, int n_items,
         // first block travel with the descriptors
         const size_t ticket_at = host.size();
         const uint32_t chunk = batched_chunk_blocks(total);
-        batch.option = chunk;
+        batch.chunk_blocks = chunk;
         const size_t n_chunks = size_t((total + chunk - 1) / chunk);
         host.resize(ticket_at + 16 + n_chunks * sizeof(uint32_t), 0);
         {

@@ -696,7 +696,8 @@ struct DecodeBatch {
     const uint32_t* prefix;   // device array [n_jobs + 1]: blocks before each tensor (null with jobs)
     uint32_t n_jobs;
     uint32_t total_blocks;
-    uint32_t option;          // one tensor: 1 = its stream is of the block-wise variant; TICKET = 1: blocks per chunk
+    uint32_t blockwise;       // 1 = the stream is of the block-wise variant (one tensor only)
+    uint32_t chunk_blocks;    // TICKET = 1: blocks per chunk
     uint32_t apart;           // fixed shares: 1 = the last CTA has the last block and no other (see launch_decode)
     DecodeJob inline_jobs[kInlineJobs];          // used when jobs is null (one tensor, or a short list)
     uint32_t inline_prefix[kInlineJobs + 1];
@@ -802,7 +803,7 @@ enec_decode_kernel(const __grid_constant__ DecodeBatch batch, int* status) {
         for (uint32_t q = threadIdx.x; q < batch.n_jobs; q += blockDim.x) {
             if (all_jobs[q].count == 0) {
                 JobCtx jc;
-                const int err = load_job<DT, MAPPED>(all_jobs[q], jc, TICKET != 1 && batch.option != 0);
+                const int err = load_job<DT, MAPPED>(all_jobs[q], jc, TICKET != 1 && batch.blockwise != 0);
                 if (err) report(status, err);
             }
         }
@@ -824,7 +825,7 @@ enec_decode_kernel(const __grid_constant__ DecodeBatch batch, int* status) {
         // and the blocks of the chunk in hand that are issued
         [[maybe_unused]] uint32_t chunk = 0, next_chunk = 0, in_chunk = 0;
         [[maybe_unused]] uint32_t next_j = 0, next_first = 0, next_end = 0;  // the next chunk's tensor and its range of blocks
-        const uint32_t kChunk = TICKET == 2 ? kSingleTicketChunk : batch.option;
+        const uint32_t kChunk = TICKET == 2 ? kSingleTicketChunk : batch.chunk_blocks;
         [[maybe_unused]] const uint32_t n_chunks = TICKET ? (batch.total_blocks + kChunk - 1) / kChunk : 0;
         [[maybe_unused]] uint32_t* const ticket =
             TICKET == 1 ? reinterpret_cast<uint32_t*>(reinterpret_cast<uintptr_t>(batch.prefix) + ticket_offset_behind_prefix(batch.n_jobs))
@@ -917,7 +918,7 @@ enec_decode_kernel(const __grid_constant__ DecodeBatch batch, int* status) {
                     e0 = tb[k];
                     e1 = tb[k + 1];
                 }
-                const int err = early ? load_job<DT, MAPPED>(job, jc, TICKET != 1 && batch.option != 0) : ENEC_ERR_BAD_STREAM;
+                const int err = early ? load_job<DT, MAPPED>(job, jc, TICKET != 1 && batch.blockwise != 0) : ENEC_ERR_BAD_STREAM;
                 if (err) {
                     *abort_flag = 1;
                     report(status, err);
