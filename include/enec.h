@@ -82,7 +82,8 @@ enec_status enec_compress(const void* d_in, enec_dtype dt, size_t count, void* d
  * As enec_compress, with the caller's (b, n, m) instead of the search of Sec. 5.5 (the paper's offline
  * tuned mode, Sec. 6 "Compression Configurations"). 0 <= b < 2^E, 1 <= m <= n <= E (E = 8 for bf16,
  * 5 for fp16). If some exponent of the tensor does not survive (b, n) the device reports
- * ENEC_ERR_PARAMS_NOT_LOSSLESS in *d_status and writes no stream.
+ * ENEC_ERR_PARAMS_NOT_LOSSLESS in *d_status and writes no stream: d_out has no valid header then, whatever it held before,
+ * and *d_out_size is 0.
  */
 enec_status enec_compress_with_params(const void* d_in, enec_dtype dt, size_t count, int b, int n, int m,
                                       void* d_out, size_t out_capacity, size_t* d_out_size, int* d_status,

@@ -670,6 +670,13 @@ __device__ __forceinline__ void copy_halves(uint8_t* dst, uint32_t src, uint32_t
     if (tid == 32 && halves > odd && ((halves - odd) & 1)) *reinterpret_cast<uint16_t*>(dst + 2 * (halves - 1)) = uint16_t(lds16(src + 2 * (halves - 1)));
 }
 
+// What a failed call leaves, as the other compressors do: a header that no decompressor accepts and the length 0. (The output may
+// hold an earlier stream, whose header would go with this call's sections.) One thread; any number of threads may say it.
+__device__ __forceinline__ void leave_no_stream(const FusedTensor& t) {
+    reinterpret_cast<Header*>(t.out)->magic = 0;
+    if (t.out_size) *t.out_size = 0;
+}
+
 // The end of a block, by a warp that knows its offset: table entry; for the last block also the header, the end of
 // the table, the padding behind the records and the stream length.
 // CHECK (given parameters): nothing of that, when some block lost a value. Its CTA has said so before it published its count.
@@ -1208,6 +1215,7 @@ __device__ __noinline__ uint32_t pack_pass(FusedControl* ctl, uint32_t pass, int
     };
     auto say_lossy = [&]() {   // one thread, before the block's count is published
         report(status, ENEC_ERR_PARAMS_NOT_LOSSLESS);
+        leave_no_stream(t);   // nobody writes a header: see finish_block
         atomicOr(&ctl->lossy, 1u);
         __threadfence();
     };

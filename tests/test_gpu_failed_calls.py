@@ -30,3 +30,32 @@ def test_batched_decompress_of_a_list_without_elements(dt, tensors):
     streams[-1][0] = 0x58   # the magic
     assert enec.enec_decompress_batched([(s, s.numel(), out, 0) for s in streams], dt, status) == 0
     assert int(status.item()) == -4
+
+
+@pytest.mark.parametrize("dt", [0, 1, 2])
+@pytest.mark.parametrize("count", [100, 5000, 16384 * 3, 16384 * 60 + 77, 16384 * 500 + 5003])
+def test_given_parameters_that_lose_a_value_leave_no_stream(dt, count):
+    """The output held a valid stream of the same size, the length word something else: neither may stand for the failed
+    call's result. With and without a status word, the lost value in the first, a middle and the last block."""
+    import paper_2604_03298_b200 as enec
+    t = _weights(count, dt, count)
+    least = 2e-3 if dt == 1 else 1e-6   # a range of exponents that does not need all bits: there are some to lose
+    t = torch.where(t.abs() < least, torch.full_like(t, least), t)
+    before = enec.compress_tensor(t)
+    b, n, m = before[20:23].tolist()
+    assert n < (5 if dt == 1 else 8)
+    cap = enec.enec_max_compressed_size(dt, count)
+    buf = torch.zeros(cap, dtype=torch.uint8, device="cuda")
+    out = torch.empty_like(t)
+    for at in {0, count // 2, count - 1}:
+        for status in (status_tensor(), None):
+            buf[:before.numel()] = before
+            bad = t.clone()
+            bad[at] = 3.0e4 if dt == 1 else 1.0e12   # the only value that (b, n) loses
+            size, decoded = torch.full((1,), 77, dtype=torch.int64, device="cuda"), status_tensor()
+            assert enec.enec_compress_with_params(bad, dt, count, b, n, m, buf, cap, size, status) == 0
+            assert int(size.item()) == 0
+            assert status is None or int(status.item()) == -5
+            assert buf[:4].tolist() == [0, 0, 0, 0]
+            assert enec.enec_decompress(buf, cap, dt, count, out, decoded) == 0
+            assert int(decoded.item()) == -4
