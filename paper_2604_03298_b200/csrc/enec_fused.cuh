@@ -954,7 +954,8 @@ __device__ __forceinline__ void count_block(const uint8_t* in, uint32_t real, ui
         red_add_one(column + exponent_of_word<DT>(exponent_word<DT>(in, e)) * HistShape<DT>::kRowBytes);
 }
 
-// publish: with all that the thread (and, before a barrier, its CTA) has written; publish_word: the word stands for itself.
+// publish: with all that the thread (and, before a barrier, its CTA) has written or has seen written; publish_word: the word stands
+// for itself, whoever reads it relies on no other store.
 __device__ __forceinline__ void publish(uint32_t* where, uint32_t word) {
     asm volatile("st.release.gpu.global.u32 [%0], %1;" ::"l"(where), "r"(word) : "memory");
 }
@@ -1006,7 +1007,12 @@ __device__ __forceinline__ void count_done(FusedControl* ctl, uint32_t which, ui
     if (sh.word && tid < 32) {
         const uint32_t found = search_global<DT>(ctl->hist[which], which == 1 ? ctl->pack_hist : nullptr,
                                                  reinterpret_cast<unsigned long long*>(fused_smem())) | kParamsValid;
-        if (tid == 0) publish_word(&ctl->params[which], found);
+        if (tid == 0) {
+            // hist[1]'s parameters may begin a second pass, which writes where the first one has written: what the CTAs counted
+            // by hist_done wrote before is ordered before it
+            if (which == 0) publish_word(&ctl->params[0], found);
+            else publish(&ctl->params[1], found);
+        }
     }
 }
 

@@ -1,0 +1,26 @@
+"""Memory-ordering rules of the one-kernel compressors, checked on their source text (no GPU run can show that an order is
+guaranteed): every word that other CTAs wait for is published with release where the readers rely on other stores."""
+import os
+import re
+
+CSRC = os.path.join(os.path.dirname(os.path.dirname(os.path.abspath(__file__))), "paper_2604_03298_b200", "csrc")
+
+# words whose readers use nothing but the word (the parameters of the sample, a count of blocks, and the parameters of the whole
+# tensor as long as nothing is written on the strength of them: a second pass waits for all_left)
+STANDS_FOR_ITSELF = {"ctl->params[0]", "ctl->pack_target", "ctl->verdict"}
+
+
+def _source(name):
+    text = open(os.path.join(CSRC, name)).read()
+    return re.sub(r"//[^\n]*", "", text)
+
+
+def test_words_that_order_stores_are_published_with_release():
+    text = _source("enec_fused.cuh") + _source("enec_fused_list.cuh")
+    awaited = set(re.findall(r"await_published\(&([\w>\[\].-]+)", text))
+    assert awaited == {"ctl->params[which]", "ctl->pack_target", "ctl->verdict", "ctl->all_left", "ctl.ready"}
+    relaxed = set(re.findall(r"publish_word\(&([\w>\[\].-]+)", text))
+    released = set(re.findall(r"\bpublish\(&([\w>\[\].-]+)", text))
+    assert relaxed <= STANDS_FOR_ITSELF, relaxed - STANDS_FOR_ITSELF
+    assert {"ctl->params[1]", "ctl->all_left", "ctl.ready"} <= released
+    assert "st.release.gpu" in re.search(r"void publish\(.*?\n}", text, re.S).group(0)
