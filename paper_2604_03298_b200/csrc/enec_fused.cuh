@@ -1164,6 +1164,7 @@ template <int DT>
 __device__ __noinline__ void first_pass_counted(FusedControl* ctl, uint32_t mine, uint32_t nblocks) {
     uint32_t last = 0;
     if ((threadIdx.x & 31) == 0) last = add_acq_rel(&ctl->pack_done.value, mine) + mine == nblocks;
+    __syncwarp();   // the other lanes read what the first one's count has made visible
     if (!__shfl_sync(0xFFFFFFFFu, last, 0)) return;
     const uint32_t found = search_global<DT>(ctl->pack_hist, ctl->hist[1],
                                              reinterpret_cast<unsigned long long*>(fused_smem() + FusedShape<DT>::kHistAt)) |

@@ -107,6 +107,7 @@ enec_fused_list_kernel(const FusedList list, int* status) {
         uint32_t ready = 0;
         if (lane == 0 && next_kind == kUnitPack)
             asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(ready) : "l"(&list.controls[next_item].ready) : "memory");
+        __syncwarp();   // the other lanes' reads come after the first lane's acquire, which a shuffle alone does not say
         brought_ready = __shfl_sync(0xFFFFFFFFu, ready, 0);
         if (brought_ready) {
             const uint32_t* from = reinterpret_cast<const uint32_t*>(&list.controls[__shfl_sync(0xFFFFFFFFu, next_item, 0)].tensor);

@@ -24,3 +24,12 @@ def test_words_that_order_stores_are_published_with_release():
     assert relaxed <= STANDS_FOR_ITSELF, relaxed - STANDS_FOR_ITSELF
     assert {"ctl->params[1]", "ctl->all_left", "ctl.ready"} <= released
     assert "st.release.gpu" in re.search(r"void publish\(.*?\n}", text, re.S).group(0)
+
+
+def test_other_lanes_read_behind_a_barrier_after_one_lane_acquires():
+    """A shuffle passes a value on, it orders no memory access: between one lane's acquire and the others' reads stands a
+    __syncwarp()."""
+    scout = re.search(r"auto scout_middle = .*?\n    };", _source("enec_fused_list.cuh"), re.S).group(0)
+    counted = re.search(r"void first_pass_counted\(.*?\n}", _source("enec_fused.cuh"), re.S).group(0)
+    assert scout.index("ld.acquire") < scout.index("__syncwarp()") < scout.index("ld_relaxed_u32(from")
+    assert counted.index("add_acq_rel(") < counted.index("__syncwarp()") < counted.index("search_global")
