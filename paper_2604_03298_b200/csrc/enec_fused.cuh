@@ -679,16 +679,20 @@ __device__ __forceinline__ void leave_no_stream(const FusedTensor& t) {
 
 // The end of a block, by a warp that knows its offset: table entry; for the last block also the header, the end of
 // the table, the padding behind the records and the stream length.
-// CHECK (given parameters): nothing of that, when some block lost a value. Its CTA has said so before it published its count.
+// CHECK (given parameters): nothing of that, when some block lost a value. Its CTA has said so before it published its count, and
+// the last block's offset is looked up by the warp that comes here (no block follows it in its CTA).
 template <int DT, bool CHECK = false>
 __device__ __forceinline__ void finish_block(const FusedTensor& t, uint32_t k, uint32_t before, uint32_t wide) {
+    if constexpr (CHECK) {
+        if (k + 1 == t.nblocks) {   // every lane has read counts: what was written before them is there for all lanes
+            __threadfence();
+            __syncwarp();
+        }
+    }
     if ((threadIdx.x & 31) != 0) return;
     t.table[k] = before;
     if (k + 1 != t.nblocks) return;
-    if constexpr (CHECK) {
-        __threadfence();
-        if (ld_relaxed_u32(t.lossy)) return;
-    }
+    if (CHECK && ld_relaxed_u32(t.lossy)) return;
     const uint32_t a_total = before + wide;
     const uint64_t high_bytes = uint64_t(a_total) * 2 * uint32_t(t.hbits);
     const uint64_t total = uint64_t(t.high - t.out) + align16(high_bytes);

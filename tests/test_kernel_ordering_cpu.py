@@ -33,3 +33,14 @@ def test_other_lanes_read_behind_a_barrier_after_one_lane_acquires():
     counted = re.search(r"void first_pass_counted\(.*?\n}", _source("enec_fused.cuh"), re.S).group(0)
     assert scout.index("ld.acquire") < scout.index("__syncwarp()") < scout.index("ld_relaxed_u32(from")
     assert counted.index("add_acq_rel(") < counted.index("__syncwarp()") < counted.index("search_global")
+
+
+def test_the_loss_flag_is_read_behind_a_fence_of_every_lane():
+    """The lanes that look up the last block's offset read other CTAs' counts; the flag that those CTAs set before is read after a
+    fence by each of these lanes and a barrier, and before the header is written."""
+    text = _source("enec_fused.cuh")
+    finish = re.search(r"void finish_block\(.*?\n}", text, re.S).group(0)
+    order = [finish.index(s) for s in ("__threadfence()", "__syncwarp()", "(threadIdx.x & 31) != 0", "t.lossy", "Header hd;")]
+    assert order == sorted(order)
+    say = re.search(r"auto say_lossy = .*?\n    };", text, re.S).group(0)
+    assert say.index("leave_no_stream(t)") < say.index("&ctl->lossy") < say.index("__threadfence()")
