@@ -770,6 +770,7 @@ enec_status enec_compress_batched(const enec_batch_item* h_items, int n_items, e
     list.chunk_item = reinterpret_cast<const uint32_t*>(scratch + off_chunks);
     list.segments = reinterpret_cast<const FusedListSegment*>(scratch + off_segments);
     list.n_segments = uint32_t(segments.size() - 1);
+    list.n_items = uint32_t(items.size());
     list.n_multi = n_multi;
     list.multi_blocks = multi_blocks;
     list.ticket = reinterpret_cast<uint32_t*>(scratch);

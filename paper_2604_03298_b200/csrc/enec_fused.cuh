@@ -676,6 +676,15 @@ __device__ __forceinline__ void leave_no_stream(const FusedTensor& t) {
     reinterpret_cast<Header*>(t.out)->magic = 0;
     if (t.out_size) *t.out_size = 0;
 }
+// The counts before block k did not come in time (or its CTA gives up for another reason): its records are not placed, so no later
+// block finds its offset either, and the last one's header is not written. One thread; the tensor has two blocks or more.
+__device__ __forceinline__ void give_up(const FusedTensor& t, uint32_t k, int* status) {
+    report(status, ENEC_ERR_TIMEOUT);
+    st_relaxed_u64(&t.state[k], 0ull);                            // no call's epoch
+    atomicAdd(&t.super[k / kSuperBlocks], 1ull << 32);            // one block too many
+    if (t.nblocks > kSuperBlocks * kHyperSupers) atomicAdd(&t.hyper[k / (kSuperBlocks * kHyperSupers)], 1ull << 32);
+    leave_no_stream(t);
+}
 
 // The end of a block, by a warp that knows its offset: table entry; for the last block also the header, the end of
 // the table, the padding behind the records and the stream length.
@@ -921,7 +930,7 @@ __device__ __noinline__ void pack_short_block(uint32_t k, int* status, uint32_t 
             if (tid < wide * hbits) out_rec[tid] = reinterpret_cast<const uint16_t*>(s_rec)[tid];   // at most 28
             finish_block<DT, CHECK>(t, k, before, wide);
         } else if (tid == 0) {
-            report(status, ENEC_ERR_TIMEOUT);
+            give_up(t, k, status);
         }
     }
     __syncthreads();
@@ -1209,7 +1218,7 @@ __device__ __noinline__ uint32_t pack_pass(FusedControl* ctl, uint32_t pass, int
                 if (lane == 0) {
                     sh.before = before;
                     sh.ok = ok;
-                    if (!ok) report(status, ENEC_ERR_TIMEOUT);
+                    if (!ok) give_up(t, pend_block, status);
                 }
             }
             __syncthreads();
@@ -1280,7 +1289,7 @@ __device__ __noinline__ uint32_t pack_pass(FusedControl* ctl, uint32_t pass, int
                 uint32_t before = 0;
                 const bool ok = groups_before(t, k, before);
                 if (ok) finish_block<DT, CHECK>(t, k, before, wide);
-                else if (lane == 0) report(status, ENEC_ERR_TIMEOUT);
+                else if (lane == 0) give_up(t, k, status);
                 if (lane == 0) { sh.before = before; sh.ok = ok; }
             }
             __syncthreads();
@@ -1402,7 +1411,10 @@ enec_fused_kernel(const FusedJob job, int* status) {
     // ---- pack stage ----
     for (uint32_t pass = 0;; ++pass) {
         if (word == 0) {
-            if (tid == 0) report(status, ENEC_ERR_TIMEOUT);
+            if (tid == 0) {   // if the CTA has a ticket for a block, that one stays unpacked and nobody writes a header
+                report(status, ENEC_ERR_TIMEOUT);
+                leave_no_stream(t);
+            }
             return;
         }
         __syncthreads();

@@ -50,7 +50,7 @@ struct FusedList {
     FusedItemControl* controls;          // per tensor of two blocks or more; zero when the call starts
     const uint32_t* chunk_item;          // the tensor of every kHistBlocks blocks
     const FusedListSegment* segments;    // [n_segments + 1], the last with the number of tickets
-    uint32_t n_segments, n_multi;        // n_multi: tensors of two blocks or more
+    uint32_t n_segments, n_items, n_multi;   // n_multi: tensors of two blocks or more
     uint32_t multi_blocks;               // index of the first block of the tensors of one block
     uint32_t* ticket;                    // zero when the call starts
 };
@@ -152,7 +152,7 @@ enec_fused_list_kernel(const FusedList list, int* status) {
                 if (lane == 0) {
                     sh.before = before;
                     sh.ok = ok;
-                    if (!ok) report(status, ENEC_ERR_TIMEOUT);
+                    if (!ok) give_up(t, pend_block, status);
                 }
             }
             __syncthreads();
@@ -238,8 +238,8 @@ enec_fused_list_kernel(const FusedList list, int* status) {
                     if (tid == 0) sh.word = await_published(&ctl.ready);
                     __syncthreads();
                     if (!sh.word) {
-                        if (tid == 0) report(status, ENEC_ERR_TIMEOUT);
-                        return;
+                        stop = true;
+                        break;
                     }
                     if (tid < sizeof(FusedTensor) / 4)
                         reinterpret_cast<uint32_t*>(&fused_tensor<DT>(slot))[tid] = ld_relaxed_u32(reinterpret_cast<const uint32_t*>(&ctl.tensor) + tid);
@@ -283,7 +283,7 @@ enec_fused_list_kernel(const FusedList list, int* status) {
                         uint32_t before = 0;
                         const bool ok = groups_before(t, k, before);
                         if (ok) finish_block<DT>(t, k, before, wide);
-                        else if (lane == 0) report(status, ENEC_ERR_TIMEOUT);
+                        else if (lane == 0) give_up(t, k, status);
                         if (lane == 0) { sh.before = before; sh.ok = ok; }
                     }
                     __syncthreads();
@@ -318,6 +318,18 @@ enec_fused_list_kernel(const FusedList list, int* status) {
     }
     __syncthreads();   // sh.before has been read by everybody
     if (pend_block != 0xFFFFFFFFu && !stop) place_waiting(false);
+    if (stop) {
+        // A wait ran out. The CTA's waiting block is not placed and the unit that it has a ticket for is not done; whose tensor
+        // that is, and which tensors wait for it, is not followed up: no tensor of the list keeps a header from before.
+        if (tid == 0) {
+            if (pend_block != 0xFFFFFFFFu) give_up(fused_tensor<DT>(pend_slot), pend_block, status);
+            else report(status, ENEC_ERR_TIMEOUT);
+        }
+        for (uint32_t i = tid; i < list.n_items; i += kFusedThreads) {
+            reinterpret_cast<Header*>(list.items[i].out)->magic = 0;
+            if (list.items[i].out_size) *list.items[i].out_size = 0;
+        }
+    }
 }
 
 }  // namespace enec

@@ -44,3 +44,23 @@ def test_the_loss_flag_is_read_behind_a_fence_of_every_lane():
     assert order == sorted(order)
     say = re.search(r"auto say_lossy = .*?\n    };", text, re.S).group(0)
     assert say.index("leave_no_stream(t)") < say.index("&ctl->lossy") < say.index("__threadfence()")
+
+
+def test_a_wait_that_ran_out_leaves_no_stream():
+    """No run makes these bounded waits end early, so their error paths are read here: wherever one reports ENEC_ERR_TIMEOUT, the
+    header's magic and the length are zeroed too (the output may hold an earlier stream), and a block whose records were
+    not placed takes its count back, so that the last block's CTA does not write a header."""
+    text = _source("enec_fused.cuh")
+    give_up = re.search(r"void give_up\(.*?\n}", text, re.S).group(0)
+    for part in ("report(status, ENEC_ERR_TIMEOUT)", "t.state[k], 0ull", "&t.super[k / kSuperBlocks]", "leave_no_stream(t)"):
+        assert part in give_up
+    rest = text.replace(give_up, "")
+    assert len(re.findall(r"give_up\(t, ", rest)) == 3      # waiting block, block without room to wait, short block
+    for report in re.finditer(r"report\(status, ENEC_ERR_TIMEOUT\);", rest):
+        assert re.match(r"\s*leave_no_stream\(t\);", rest[report.end():])
+    text = _source("enec_fused_list.cuh")
+    assert len(re.findall(r"give_up\(", text)) == 3
+    end = text[text.index("if (stop) {"):]
+    assert text.count("report(status, ENEC_ERR_TIMEOUT)") == end.count("report(status, ENEC_ERR_TIMEOUT)") == 1
+    assert "i < list.n_items" in end and "->magic = 0" in end and "out_size = 0" in end
+    assert not re.search(r"\breturn;", text[text.index("enec_fused_list_kernel("):text.index("if (stop) {")].split("for (uint32_t iter = 0;;")[1])
