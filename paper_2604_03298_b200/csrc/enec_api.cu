@@ -598,7 +598,7 @@ enec_status enec_decompress_batched(const enec_batch_item* h_items, int n_items,
         // first block travel with the descriptors
         const size_t ticket_at = host.size();
         const uint32_t chunk = batched_chunk_blocks(total);
-        batch.chunk_blocks = chunk;
+        batch.chunk_blocks = uint16_t(chunk);
         const size_t n_chunks = size_t((total + chunk - 1) / chunk);
         host.resize(ticket_at + 16 + n_chunks * sizeof(uint32_t), 0);
         {

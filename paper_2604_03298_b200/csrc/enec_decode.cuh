@@ -696,8 +696,8 @@ struct DecodeBatch {
     const uint32_t* prefix;   // device array [n_jobs + 1]: blocks before each tensor (null with jobs)
     uint32_t n_jobs;
     uint32_t total_blocks;
-    uint32_t blockwise;       // 1 = the stream is of the block-wise variant (one tensor only)
-    uint32_t chunk_blocks;    // TICKET = 1: blocks per chunk
+    uint16_t blockwise;       // 1 = the stream is of the block-wise variant (one tensor only)
+    uint16_t chunk_blocks;    // TICKET = 1: blocks per chunk
     uint32_t apart;           // fixed shares: 1 = the last CTA has the last block and no other (see launch_decode)
     DecodeJob inline_jobs[kInlineJobs];          // used when jobs is null (one tensor, or a short list)
     uint32_t inline_prefix[kInlineJobs + 1];
