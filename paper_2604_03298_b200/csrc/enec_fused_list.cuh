@@ -137,7 +137,8 @@ enec_fused_list_kernel(const FusedList list, int* status) {
     }
     uint32_t pend_block = 0xFFFFFFFFu, pend_wide = 0, pend_at = 0, pend_slot = 1;   // the block whose records wait in shared memory
     uint32_t slot = 0;                                                             // of this unit's tensor
-    bool stop = false;
+    bool stop = false;                                                             // a wait ran out
+    uint32_t lost = 0;                                                             // slot << 28 | block: not placed (0: none is known)
     auto place_waiting = [&](bool asked_for) {   // see pack_pass
         const FusedTensor& t = fused_tensor<DT>(pend_slot);
         uint32_t before = 0;
@@ -152,12 +153,11 @@ enec_fused_list_kernel(const FusedList list, int* status) {
                 if (lane == 0) {
                     sh.before = before;
                     sh.ok = ok;
-                    if (!ok) give_up(t, pend_block, status);
                 }
             }
             __syncthreads();
             before = sh.before;
-            if (!sh.ok) { stop = true; return; }
+            if (!sh.ok) { stop = true; lost = pend_slot << 28 | pend_block; return; }
         }
         copy_halves(t.high + uint64_t(before) * 2 * uint32_t(t.hbits), pend_at, pend_wide * uint32_t(t.hbits), tid);
         if (warp == 0) finish_block<DT>(t, pend_block, before, pend_wide);
@@ -239,6 +239,7 @@ enec_fused_list_kernel(const FusedList list, int* status) {
                     __syncthreads();
                     if (!sh.word) {
                         stop = true;
+                        if (pend_block != 0xFFFFFFFFu) lost = pend_slot << 28 | pend_block;
                         break;
                     }
                     if (tid < sizeof(FusedTensor) / 4)
@@ -283,11 +284,10 @@ enec_fused_list_kernel(const FusedList list, int* status) {
                         uint32_t before = 0;
                         const bool ok = groups_before(t, k, before);
                         if (ok) finish_block<DT>(t, k, before, wide);
-                        else if (lane == 0) give_up(t, k, status);
                         if (lane == 0) { sh.before = before; sh.ok = ok; }
                     }
                     __syncthreads();
-                    if (!sh.ok) stop = true;
+                    if (!sh.ok) { stop = true; lost = slot << 28 | k; }
                 }
                 if (!stop)
                     pack_records_any<DT>(int(hbits), work + Shape::kValuesAt, work + Shape::kListAt + warp * 128, wide_of_warp, mask_word, excl,
@@ -322,7 +322,7 @@ enec_fused_list_kernel(const FusedList list, int* status) {
         // A wait ran out. The CTA's waiting block is not placed and the unit that it has a ticket for is not done; whose tensor
         // that is, and which tensors wait for it, is not followed up: no tensor of the list keeps a header from before.
         if (tid == 0) {
-            if (pend_block != 0xFFFFFFFFu) give_up(fused_tensor<DT>(pend_slot), pend_block, status);
+            if (lost) give_up(fused_tensor<DT>(lost >> 28), lost & 0x0FFFFFFFu, status);   // a tensor has at most 2^22 blocks
             else report(status, ENEC_ERR_TIMEOUT);
         }
         for (uint32_t i = tid; i < list.n_items; i += kFusedThreads) {
