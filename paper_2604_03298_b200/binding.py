@@ -176,11 +176,13 @@ class _Answer:
     """Where a checked call's kernels leave stream length and status: 16 bytes of pinned host memory, which the GPU writes
     itself, so that the call neither clears nor copies device memory and waits for its stream only once."""
 
-    def __init__(self):
-        self.memory = torch.zeros(2, dtype=torch.int64).pin_memory()
-        self.address = self.memory.data_ptr()
-        self.size = C.c_int64.from_address(self.address)
-        self.status = C.c_int32.from_address(self.address + 8)
+    def __init__(self, for_kernels=True):
+        memory = torch.zeros(2, dtype=torch.int64)
+        self.memory = memory.pin_memory() if for_kernels else memory
+        address = self.memory.data_ptr()
+        self.size = C.c_int64.from_address(address)
+        self.status = C.c_int32.from_address(address + 8)
+        self.size_at, self.status_at = (address, address + 8) if for_kernels else (None, None)   # what the call is given
         self.where = None      # (device, stream handle) of the last call, and the stream as an object
         self.stream = None
         self.pending = False   # kernels may still write here: a call that failed half way leaves it set
@@ -193,7 +195,10 @@ def _answer():
     """This thread's answer memory, cleared, and the current stream's handle. (One per thread is enough: a checked call ends
     after its stream's work has. Asking torch for the stream object on every call took 3 us.)"""
     a = getattr(_local, "answer", None)
-    if a is None:
+    if (a is None or a.pending) and torch.cuda.is_current_stream_capturing():
+        # Pinning memory or waiting would end the capture, before the call itself has said whether it can be recorded.
+        a = _Answer(for_kernels=False)
+    elif a is None:
         a = _local.answer = _Answer()
     elif a.pending:
         a.stream.synchronize()
@@ -211,6 +216,7 @@ def _finish(a, st, where):
     """Waits for the call's stream and raises on an error of the call (st) or of its kernels. (Cleared and copied device memory,
     as before, cost 15 us more for each call: 4 M values there and back took 97 us, 62 us now.)"""
     if st != 0:
+        a.pending = st == -7   # a call that was refused has enqueued nothing; after a CUDA error part of it may run
         raise EnecError(st, where)
     a.stream.synchronize()
     a.pending = False
@@ -228,9 +234,9 @@ def compress_tensor(t: torch.Tensor, params=None) -> torch.Tensor:
     out = torch.empty(cap, dtype=torch.uint8, device=t.device)
     a, stream_handle = _answer()
     if params is None:
-        st = lib().enec_compress(t.data_ptr(), dt, count, out.data_ptr(), cap, a.address, a.address + 8, stream_handle)
+        st = lib().enec_compress(t.data_ptr(), dt, count, out.data_ptr(), cap, a.size_at, a.status_at, stream_handle)
     else:
-        st = lib().enec_compress_with_params(t.data_ptr(), dt, count, *params, out.data_ptr(), cap, a.address, a.address + 8, stream_handle)
+        st = lib().enec_compress_with_params(t.data_ptr(), dt, count, *params, out.data_ptr(), cap, a.size_at, a.status_at, stream_handle)
     _finish(a, st, "enec_compress")
     return out[:a.size.value]
 
@@ -239,6 +245,6 @@ def decompress_tensor(stream: torch.Tensor, dtype: torch.dtype, shape) -> torch.
     dt = _DT[dtype]
     out = torch.empty(shape, dtype=dtype, device=stream.device)
     a, stream_handle = _answer()
-    st = lib().enec_decompress(stream.data_ptr(), stream.numel(), dt, out.numel(), out.data_ptr(), a.address + 8, stream_handle)
+    st = lib().enec_decompress(stream.data_ptr(), stream.numel(), dt, out.numel(), out.data_ptr(), a.status_at, stream_handle)
     _finish(a, st, "enec_decompress")
     return out

@@ -59,3 +59,40 @@ def test_given_parameters_that_lose_a_value_leave_no_stream(dt, count):
             assert buf[:4].tolist() == [0, 0, 0, 0]
             assert enec.enec_decompress(buf, cap, dt, count, out, decoded) == 0
             assert int(decoded.item()) == -4
+
+
+def test_checked_calls_while_the_stream_is_captured():
+    """A checked compress call cannot be recorded: it is refused each time it is made and leaves the capture as it is, in a thread that
+    has made checked calls before and in one that makes its first, after a call that failed and after one that did not."""
+    import threading
+    import paper_2604_03298_b200 as enec
+    t = _weights(50000, 0, 3)
+    stream = enec.compress_tensor(t)
+
+    def work(said):
+        x = torch.ones(8, device="cuda")
+        for _ in range(2):
+            graph, side = torch.cuda.CUDAGraph(), torch.cuda.Stream()
+            side.wait_stream(torch.cuda.current_stream())
+            with torch.cuda.graph(graph, stream=side):
+                for _ in range(3):
+                    with pytest.raises(enec.EnecError) as err:
+                        enec.compress_tensor(t)
+                    said.append(err.value.status)
+                y = x + 1
+            graph.replay()
+            torch.cuda.synchronize()
+            said.append(bool((y == 2).all()))
+            said.append(torch.equal(enec.compress_tensor(t), stream))   # and outside it works
+            with pytest.raises(enec.EnecError):
+                enec.compress_tensor(t, params=(100, 1, 1))               # loses exponents
+
+    for place in ("here", "thread"):
+        said = []
+        if place == "here":
+            work(said)
+        else:
+            th = threading.Thread(target=work, args=(said,))
+            th.start()
+            th.join()
+        assert said == [-1, -1, -1, True, True] * 2, place
