@@ -157,27 +157,21 @@ static void place_job(EncodeJob& job, uint8_t* scratch, uint32_t epoch) {
     job.epoch = epoch;
 }
 
-// enec_compress takes the one-kernel form (enec_fused.cuh) for every tensor. With ENEC_SPLIT_MIN_BLOCKS in the environment
-// (read once; for measurements and tests) it takes the forms before that: tensors of split_min_blocks() ..
-// split_max_blocks() - 1 blocks the split form (histogram, pack kernel, then the kernel that places the records), others
-// histogram and look-back kernel. One kernel against those: 4096 values 8.4 against 11.0 us, 256 blocks 14.3 / 22.5,
-// 1024 blocks 28.5 / 35.1, 3584 blocks 58 / 87, 27000 blocks 325 / 520 (bf16, in a stream).
+// enec_compress takes the one-kernel form (enec_fused.cuh) for every size: none is known where the split form (histogram, pack
+// kernel, then the kernel that places the records) is the faster one. That one is kept to measure and test against: for tensors of
+// ENEC_SPLIT_MIN_BLOCKS .. ENEC_SPLIT_MAX_BLOCKS - 1 blocks, both from the environment and read once; without the first there is
+// no such size. Given parameters always take the one-kernel form. One kernel against histogram and look-back kernel (up to 1024
+// blocks) and split form (beyond): 4096 values 8.5 against 11.0 us, 256 blocks 13.0 / 22.5, 1024 blocks 25.1 / 35.1, 3584 blocks
+// 53 / 83, 32064 blocks 354 / 594 (bf16, in a stream). Where its sample misleads the one-kernel form it can be the slower one:
+// see enec_fused.cu.
 static uint32_t env_blocks(const char* name, uint32_t fallback) {
     const char* e = getenv(name);
     return e && *e ? uint32_t(strtoul(e, nullptr, 10)) : fallback;
 }
-static uint32_t split_min_blocks() {
-    static const uint32_t value = env_blocks("ENEC_SPLIT_MIN_BLOCKS", 2048u);
-    return value;
-}
-static uint32_t split_max_blocks() {
-    static const uint32_t value = env_blocks("ENEC_SPLIT_MAX_BLOCKS", 0xFFFFFFFFu);
-    return value;
-}
-
-static bool earlier_forms() {
-    static const bool value = getenv("ENEC_SPLIT_MIN_BLOCKS") != nullptr;
-    return value;
+static bool in_split_range(uint32_t nblocks) {
+    static const uint32_t min_blocks = env_blocks("ENEC_SPLIT_MIN_BLOCKS", 0xFFFFFFFFu);
+    static const uint32_t max_blocks = env_blocks("ENEC_SPLIT_MAX_BLOCKS", 0xFFFFFFFFu);
+    return nblocks >= min_blocks && nblocks < max_blocks;
 }
 
 template <int DT>
@@ -206,31 +200,29 @@ static enec_status launch_split(const EncodeJob& job, uint32_t nblocks, int* d_s
 }
 
 template <int DT>
-static enec_status launch_encode(const EncodeJob& job, uint32_t nblocks, bool search, int* d_status, DeviceInfo& info,
-                                 cudaStream_t stream, bool may_split = false) {
-    if (search) {
-        const uint32_t smem = HistShape<DT>::kBytes;
-        if (!info.hist_attr_set[DT]) {
-            if (cudaFuncSetAttribute(enec_histogram_kernel<DT, false>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                     int(smem)) != cudaSuccess ||
-                cudaFuncSetAttribute(enec_histogram_kernel<DT, true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                     int(smem)) != cudaSuccess)
-                return ENEC_ERR_CUDA;
-            info.hist_attr_set[DT] = true;
-        }
-        const uint64_t chunks = (job.count * uint64_t(elem_bytes(DT))) >> 4;  // 16-byte loads
-        uint64_t grid = (chunks + kHistThreads - 1) / kHistThreads;
-        if (grid > uint64_t(info.sms) * 3) grid = uint64_t(info.sms) * 3;
-        if (grid == 0) grid = 1;
-        const cudaError_t herr =
-            job.ranked ? launch_pdl(enec_histogram_kernel<DT, true>, uint32_t(grid), kHistThreads, smem, stream, job.in,
-                                    job.count, job.ctl)
-                       : launch_pdl(enec_histogram_kernel<DT, false>, uint32_t(grid), kHistThreads, smem, stream, job.in,
-                                    job.count, job.ctl);
-        if (herr != cudaSuccess) return ENEC_ERR_CUDA;
-        g_launches.fetch_add(1, std::memory_order_relaxed);
-        if (may_split && !job.ranked && nblocks >= split_min_blocks() && nblocks < split_max_blocks()) return launch_split<DT>(job, nblocks, d_status, info, stream);
+static enec_status launch_encode(const EncodeJob& job, uint32_t nblocks, int* d_status, DeviceInfo& info, cudaStream_t stream,
+                                 bool split = false) {
+    const uint32_t smem = HistShape<DT>::kBytes;
+    if (!info.hist_attr_set[DT]) {
+        if (cudaFuncSetAttribute(enec_histogram_kernel<DT, false>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                 int(smem)) != cudaSuccess ||
+            cudaFuncSetAttribute(enec_histogram_kernel<DT, true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                 int(smem)) != cudaSuccess)
+            return ENEC_ERR_CUDA;
+        info.hist_attr_set[DT] = true;
     }
+    const uint64_t chunks = (job.count * uint64_t(elem_bytes(DT))) >> 4;  // 16-byte loads
+    uint64_t hist_grid = (chunks + kHistThreads - 1) / kHistThreads;
+    if (hist_grid > uint64_t(info.sms) * 3) hist_grid = uint64_t(info.sms) * 3;
+    if (hist_grid == 0) hist_grid = 1;
+    const cudaError_t herr =
+        job.ranked ? launch_pdl(enec_histogram_kernel<DT, true>, uint32_t(hist_grid), kHistThreads, smem, stream, job.in,
+                                job.count, job.ctl)
+                   : launch_pdl(enec_histogram_kernel<DT, false>, uint32_t(hist_grid), kHistThreads, smem, stream, job.in,
+                                job.count, job.ctl);
+    if (herr != cudaSuccess) return ENEC_ERR_CUDA;
+    g_launches.fetch_add(1, std::memory_order_relaxed);
+    if (split) return launch_split<DT>(job, nblocks, d_status, info, stream);
     if (!info.encode_attr_set[DT]) {
         if (cudaFuncSetAttribute(enec_encode_kernel<DT, false>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                  int(EncodeSmem<DT>::kBytes)) != cudaSuccess ||
@@ -281,7 +273,8 @@ static enec_status compress_common(const void* d_in, enec_dtype dt, size_t count
     cudaStreamCaptureStatus capturing = cudaStreamCaptureStatusNone;
     if (cudaStreamIsCapturing(stream, &capturing) != cudaSuccess) return ENEC_ERR_CUDA;
     if (capturing != cudaStreamCaptureStatusNone) return ENEC_ERR_INVALID_ARG;
-    if (!ranked && !earlier_forms()) {
+    const bool split = !ranked && !with_params && in_split_range(g.nblocks);
+    if (!ranked && !split) {
         FusedJob fused;
         enec_status fst = lease_fused_scratch(dev, stream, g.nblocks, fused);
         if (fst != ENEC_OK) return fst;
@@ -304,13 +297,10 @@ static enec_status compress_common(const void* d_in, enec_dtype dt, size_t count
     job.count = count;
     place_job(job, scratch, epoch);
     job.out_size = out_size;
-    job.b = b; job.n = n; job.m = m;
-    job.from_search = with_params ? 0 : 1;
-    job.check = with_params ? 1 : 0;
     job.ranked = ranked ? 1 : 0;
-    st = dt == ENEC_BF16   ? launch_encode<ENEC_BF16>(job, g.nblocks, !with_params, d_status, info, stream, true)
-         : dt == ENEC_FP16 ? launch_encode<ENEC_FP16>(job, g.nblocks, !with_params, d_status, info, stream, true)
-                           : launch_encode<ENEC_FP32>(job, g.nblocks, !with_params, d_status, info, stream, true);
+    st = dt == ENEC_BF16   ? launch_encode<ENEC_BF16>(job, g.nblocks, d_status, info, stream, split)
+         : dt == ENEC_FP16 ? launch_encode<ENEC_FP16>(job, g.nblocks, d_status, info, stream, split)
+                           : launch_encode<ENEC_FP32>(job, g.nblocks, d_status, info, stream, split);
     if (st != ENEC_OK) mark_compress_scratch_unclean(dev, stream);  // a kernel of the call may not have run
     return st;
 }
@@ -809,13 +799,10 @@ enec_status enec_compress_noalloc(const void* d_in, enec_dtype dt, size_t count,
     job.count = count;
     place_job(job, scratch, 1);  // everything was just cleared, so every call is call number 1
     job.out_size = out_size;
-    job.b = 0; job.n = 0; job.m = 0;
-    job.from_search = 1;
-    job.check = 0;
     job.ranked = 0;
-    return dt == ENEC_BF16   ? launch_encode<ENEC_BF16>(job, g.nblocks, true, d_status, info, stream)
-           : dt == ENEC_FP16 ? launch_encode<ENEC_FP16>(job, g.nblocks, true, d_status, info, stream)
-                             : launch_encode<ENEC_FP32>(job, g.nblocks, true, d_status, info, stream);
+    return dt == ENEC_BF16   ? launch_encode<ENEC_BF16>(job, g.nblocks, d_status, info, stream)
+           : dt == ENEC_FP16 ? launch_encode<ENEC_FP16>(job, g.nblocks, d_status, info, stream)
+                             : launch_encode<ENEC_FP32>(job, g.nblocks, d_status, info, stream);
 }
 
 uint64_t enec_launch_count(void) { return g_launches.load(std::memory_order_relaxed); }

@@ -219,7 +219,7 @@ enec_block_params_kernel(const BlockwiseJob job, int* status) {
             tid < uint32_t(1 << E) ? fold_hist_row<true>(smem_u32(smem) + tid * HistShape<DT>::kRowBytes, tid) : 0u;
         int b, n, m;
         parameter_search_counts<DT>(mine, b, n, m);
-        const TransformCtx tc = make_transform_ctx(E, b, n);
+        const TransformCtx tc = make_transform_ctx(b, n);
         uint32_t wide;
         if (full) {
             wide = count_wide_full<DT>(raw, tc, m);

@@ -37,13 +37,11 @@ struct alignas(16) EncodeControl {
 };
 static_assert(sizeof(EncodeControl) <= kControlSlotBytes, "a control set fits its slot");
 
-// state word: bits 63..62 = kind, bit 61 = this block or one summed into the value saw parameters that lose
-// exponents, bits 60..32 = epoch of the writing call, bits 31..0 = value. Failure travels inside the words, so
-// no fence is needed around them.
+// state word: bits 63..62 = kind, bits 60..32 = epoch of the writing call, bits 31..0 = value. Failure travels inside the
+// words, so no fence is needed around them.
 constexpr unsigned long long kStateAggregate = 1ull << 62;  // value = wide groups in the block
 constexpr unsigned long long kStatePrefix = 2ull << 62;     // value = wide groups up to and including the block
 constexpr unsigned long long kStatePoison = 3ull << 62;     // a predecessor failed
-constexpr unsigned long long kStateTaint = 1ull << 61;
 constexpr uint32_t kEpochMax = (1u << 29) - 1;
 __host__ __device__ constexpr unsigned long long epoch_bits(uint32_t epoch) { return (unsigned long long)epoch << 32; }
 // The word as this call sees it: words of other calls are empty.
@@ -60,9 +58,6 @@ struct EncodeJob {
     unsigned long long* state;
     uint32_t epoch;                // number of this call on the scratch area
     unsigned long long* out_size;  // device, may be null
-    int b, n, m;                   // used when from_search == 0
-    int from_search;               // take (b, n, m) from ctl
-    int check;                     // verify that (b, n) keeps every exponent
     int ranked;                    // frequency-rank variant: stored value = ctl->lut[exponent]
 };
 
@@ -557,8 +552,6 @@ struct TransformCtx {
     uint32_t b4;        // rep4(b)
     uint32_t nmask4;    // rep4(2^n - 1)
     uint32_t s4;        // rep4(2^(n-1))
-    uint32_t emask4;    // rep4(2^E - 1)
-    int n, E;
     uint32_t lut;       // frequency-rank variant: shared address of the exponent -> rank table, else 0
 };
 
@@ -574,14 +567,6 @@ __device__ __forceinline__ uint32_t bytewise_b_minus(const TransformCtx& t, uint
     return (t.b4_or_h - (x & 0x7F7F7F7Fu)) ^ ((t.b4 ^ ~x) & 0x80808080u);
 }
 
-// Bytes whose exponent is not reproduced by (b, n): x != (b - sext_n(y)) mod 2^E. Non-zero = some byte fails.
-__device__ __forceinline__ uint32_t lossy_bytes(const TransformCtx& t, uint32_t d, uint32_t y) {
-    if (t.n == t.E) return 0;
-    // sext_n(y) = (y ^ s) - s per byte; (y ^ s) < 128 because n < 8
-    const uint32_t sext = (((y ^ t.s4) | 0x80808080u) - t.s4) ^ 0x80808080u;
-    return (sext ^ d) & t.emask4;
-}
-
 // ---------------------------------------------------------------------------------------------------
 struct EncodeShared {
     uint32_t mask[32];     // the block's group mask, bit g = group g is wide
@@ -589,7 +574,6 @@ struct EncodeShared {
     uint32_t next[2];      // tickets of the CTA's current and next block, by iteration parity
     uint32_t before;       // P_k
     uint32_t poisoned;
-    uint32_t tainted;      // the block or a predecessor saw parameters that lose exponents
 };
 
 // fp32: the eight values at `p` (32 bytes, 16-byte aligned) as their high halves, which have bf16's layout; the
@@ -614,7 +598,7 @@ __device__ __forceinline__ uint4 load_fp32_run(const uint8_t* __restrict__ p, ui
 // Phase 1 of a full block (16384 real elements), all 256 threads: loads, split, transform, sign/mantissa
 // stores and group widths with immediate offsets and no bounds logic. Lanes l and l + 16 share a group, so
 // the two halves of a ballot OR into the mask of the warp's sixteen groups of run c.
-// SIMPLE (n < 8 and no loss check): only the low seven bits of b - x matter, so the exponent is taken
+// SIMPLE (n < 8): only the low seven bits of b - x matter, so the exponent is taken
 // without its top bit and a guard bit absorbs the borrow: y = ((b & 127 | 128) - (x & 127)) & (2^n - 1).
 // Returns the wide flags of the thread's eight runs (bit c).
 // With DT = ENEC_FP32 the values are 32-bit words: their high halves take bf16's path, their low halves are
@@ -622,7 +606,7 @@ __device__ __forceinline__ uint4 load_fp32_run(const uint8_t* __restrict__ p, ui
 template <int DT, bool SIMPLE, bool RANKED = false>
 __device__ __forceinline__ uint32_t encode_full_runs(const uint8_t* in_thread, uint8_t* sm_thread, uint8_t* lo_thread,
                                                      const TransformCtx& tc, int m, uint32_t warp, uint32_t lane,
-                                                     uint32_t* mask_words, uint2 (&y)[8], uint2 (&hs)[8], int& bad) {
+                                                     uint32_t* mask_words, uint2 (&y)[8], uint2 (&hs)[8]) {
     constexpr uint32_t kRunStride = kBlockElems / 8;  // elements between a thread's runs
     uint4 raw[8];
 #pragma unroll
@@ -663,7 +647,6 @@ __device__ __forceinline__ uint32_t encode_full_runs(const uint8_t* in_thread, u
             } else {
                 const uint32_t d0 = bytewise_b_minus(tc, s0.x), d1 = bytewise_b_minus(tc, s1.x);
                 y[c] = make_uint2(d0 & tc.nmask4, d1 & tc.nmask4);
-                bad |= (lossy_bytes(tc, d0, y[c].x) | lossy_bytes(tc, d1, y[c].y)) != 0;
             }
             hs[c] = make_uint2(s0.hs, s1.hs);
             sm0 = s0.sm;
@@ -681,8 +664,8 @@ __device__ __forceinline__ uint32_t encode_full_runs(const uint8_t* in_thread, u
 
 // Blocks shorter than 128 elements (16, 32 or 64): one element per thread, bits placed one by one.
 template <int DT>
-__device__ __noinline__ int encode_short_block(const uint16_t* in, uint32_t N, uint32_t real, const TransformCtx& tc,
-                                               int b, int n, int m, int check, uint8_t* out_sm, uint8_t* out_low,
+__device__ __noinline__ void encode_short_block(const uint16_t* in, uint32_t N, uint32_t real, const TransformCtx& tc,
+                                               int b, int n, int m, uint8_t* out_sm, uint8_t* out_low,
                                                uint8_t* out_smhi, uint8_t* out_mask, uint8_t* out_smlo, EncodeShared* sh,
                                                uint32_t* s_low, uint32_t* s_hi3, uint32_t* s_rec) {
     const uint32_t tid = threadIdx.x;
@@ -692,7 +675,6 @@ __device__ __noinline__ int encode_short_block(const uint16_t* in, uint32_t N, u
     if (tid < 16) { s_low[tid] = 0; s_rec[tid] = 0; }
     if (tid < 8) s_hi3[tid] = 0;
     __syncthreads();
-    int bad = 0;
     uint32_t y = 0;
     if (tid < N) {
         uint32_t w = 0;
@@ -709,10 +691,6 @@ __device__ __noinline__ int encode_short_block(const uint16_t* in, uint32_t N, u
         else { x = (w >> 10) & 0x1F; sm = w & 0xFF; hs = ((w >> 13) & 4) | ((w >> 8) & 3); }
         if (tid < real) {
             y = tc.lut ? lds8(tc.lut + x) : uint32_t(b - int(x)) & ((1u << n) - 1);
-            if (check && n < tc.E && !tc.lut) {
-                const int v = (y >> (n - 1)) ? int(y) - (1 << n) : int(y);
-                bad = (uint32_t(b - v) & ((1u << tc.E) - 1)) != x;
-            }
             out_sm[tid] = uint8_t(sm);
         } else if (tid < uint32_t(align16(real))) {
             out_sm[tid] = 0;
@@ -755,7 +733,6 @@ __device__ __noinline__ int encode_short_block(const uint16_t* in, uint32_t N, u
         const uint32_t hi_words = uint32_t(align16(N * 3 / 8)) / 4;
         if (tid < hi_words) reinterpret_cast<uint32_t*>(out_smhi)[tid] = s_hi3[tid];
     }
-    return bad;
 }
 
 // Dynamic shared memory of the encode kernel.
@@ -780,11 +757,10 @@ struct EncodeTensor {
 // warp 0, up to 256 words per round trip, down to the nearest block that already knows its prefix.
 template <int DT, bool RANKED = false>
 __device__ __forceinline__ void resolve_block(const EncodeJob& job, const EncodeTensor& t, uint32_t k, uint32_t wide_count,
-                                              bool own_taint, const uint8_t* rec, EncodeShared& sh, int* status) {
+                                              const uint8_t* rec, EncodeShared& sh, int* status) {
     const uint32_t tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     if (warp == 0 && k > 0) {
         uint32_t before = 0;
-        uint32_t tainted = own_taint ? 1u : 0u;
         int64_t pos = int64_t(k) - 1;
         int outcome = 0;  // 1 = done, 2 = poisoned, 3 = gave up
         uint32_t polls = 0;
@@ -813,10 +789,7 @@ __device__ __forceinline__ void resolve_block(const EncodeJob& job, const Encode
                     } else if (empty_lanes & needed) {
                         blocked = true;  // a nearer block has not published yet
                     } else {
-                        if ((needed >> lane) & 1) {
-                            mine += uint32_t(st[i]);
-                            tainted |= uint32_t(st[i] >> 61) & 1u;
-                        }
+                        if ((needed >> lane) & 1) mine += uint32_t(st[i]);
                         if (first < 32) outcome = 1;
                         else ++advanced;
                     }
@@ -832,26 +805,21 @@ __device__ __forceinline__ void resolve_block(const EncodeJob& job, const Encode
                 __nanosleep(polls > 2 ? 400 : 100);
             }
         }
-        tainted = __any_sync(0xFFFFFFFFu, tainted != 0);
         if (lane == 0) {
             if (outcome == 1) {
                 sh.before = before;
                 sh.poisoned = 0;
-                sh.tainted = tainted;
-                st_relaxed_u64(&job.state[k], kStatePrefix | (tainted ? kStateTaint : 0ull) | epoch_bits(job.epoch) |
-                                                  (unsigned long long)(before + wide_count));
+                st_relaxed_u64(&job.state[k], kStatePrefix | epoch_bits(job.epoch) | (unsigned long long)(before + wide_count));
             } else {
                 if (outcome == 3) report(status, ENEC_ERR_TIMEOUT);
                 st_relaxed_u64(&job.state[k], kStatePoison | epoch_bits(job.epoch));
                 sh.poisoned = 1;
-                sh.tainted = 1;
                 sh.before = 0;
             }
         }
     } else if (tid == 0 && k == 0) {
         sh.before = 0;
         sh.poisoned = 0;
-        sh.tainted = own_taint ? 1u : 0u;
     }
     __syncthreads();
     const uint32_t before = sh.before;
@@ -872,9 +840,8 @@ __device__ __forceinline__ void resolve_block(const EncodeJob& job, const Encode
         const uint32_t a_total = before + wide_count;
         const uint64_t high_bytes = uint64_t(a_total) * 2 * hbits;
         const uint64_t total = t.sec.high + align16(high_bytes);
-        const bool failed = poisoned || sh.tainted != 0;
         Header hd;
-        hd.magic = failed ? 0 : kMagic;
+        hd.magic = poisoned ? 0 : kMagic;
         hd.version = kVersion;
         hd.dtype = DT;
         hd.variant = RANKED ? 1 : 0;
@@ -894,15 +861,13 @@ __device__ __forceinline__ void resolve_block(const EncodeJob& job, const Encode
             for (uint64_t p = high_bytes; p < align16(high_bytes); p += 2)
                 *reinterpret_cast<uint16_t*>(job.out + t.sec.high + p) = 0;
         }
-        if (job.out_size) *job.out_size = failed ? 0ull : total;
+        if (job.out_size) *job.out_size = poisoned ? 0ull : total;
     }
 }
 
 template <int DT, bool RANKED = false>
 __device__ __forceinline__ void fill_tensor_ctx(const EncodeJob& job, EncodeTensor& tensor, TransformCtx& tc) {
-    constexpr int E = DT == ENEC_FP16 ? 5 : 8;
-    int b = job.b, n = job.n, m = job.m;
-    if (job.from_search) { b = job.ctl->b; n = job.ctl->n; m = job.ctl->m; }
+    const int b = job.ctl->b, n = job.ctl->n, m = job.ctl->m;
     tensor.g = make_geometry(job.count);
     tensor.sec = make_sections(DT, job.count, tensor.g, n, m, 0, RANKED);
     tensor.b = b; tensor.n = n; tensor.m = m; tensor.hbits = n - m;
@@ -910,9 +875,6 @@ __device__ __forceinline__ void fill_tensor_ctx(const EncodeJob& job, EncodeTens
     tc.b4_or_h = tc.b4 | 0x80808080u;
     tc.nmask4 = rep4((1u << n) - 1);
     tc.s4 = rep4(1u << (n - 1));
-    tc.emask4 = rep4((1u << E) - 1);
-    tc.n = n;
-    tc.E = E;
     tc.lut = 0;
 }
 
@@ -954,7 +916,6 @@ enec_encode_kernel(const EncodeJob job, int* status) {
     // before its CTA waits for anything, and a wait only concerns blocks with smaller indices, so all
     // waits end.
     uint32_t pending_block = 0xFFFFFFFFu, pending_wide = 0, cur = 0;
-    bool pending_bad = false;
     if (tid == 0) sh.next[0] = atomicAdd(ticket, 1u);
     uint32_t iter = 0;
     for (;; ++iter) {
@@ -976,7 +937,6 @@ enec_encode_kernel(const EncodeJob job, int* status) {
     uint8_t* out_smhi = job.out + sec.smhi + uint64_t(k) * (kBlockElems / 8) * 3;
     uint8_t* out_mask = job.out + sec.mask + uint64_t(k) * (kGroupsPerBlock / 8);
 
-    int bad = 0;
     uint2 y[8];
     uint32_t wide_bits = 0;  // bit c: the group of run c is wide
     const bool fast = N == kBlockElems && real == kBlockElems;
@@ -990,10 +950,10 @@ enec_encode_kernel(const EncodeJob job, int* status) {
 
     uint2 hs[8];
     if (fast) {
-        if (!RANKED && !job.check && n < 8)
-            wide_bits = encode_full_runs<DT, true>(in_bytes + j * kElemBytes, out_sm + j, out_smlo + j * 2, tc, m, warp, lane, sh.mask, y, hs, bad);
+        if (!RANKED && n < 8)
+            wide_bits = encode_full_runs<DT, true>(in_bytes + j * kElemBytes, out_sm + j, out_smlo + j * 2, tc, m, warp, lane, sh.mask, y, hs);
         else
-            wide_bits = encode_full_runs<DT, false, RANKED>(in_bytes + j * kElemBytes, out_sm + j, out_smlo + j * 2, tc, m, warp, lane, sh.mask, y, hs, bad);
+            wide_bits = encode_full_runs<DT, false, RANKED>(in_bytes + j * kElemBytes, out_sm + j, out_smlo + j * 2, tc, m, warp, lane, sh.mask, y, hs);
         uint2 ylow[8];
         const uint32_t lowmask4 = rep4((1u << m) - 1);
 #pragma unroll
@@ -1039,14 +999,10 @@ enec_encode_kernel(const EncodeJob job, int* status) {
             const uint32_t e0 = c * n8 + j;
             const Split4 s0 = split4<DT>(raw[c].x, raw[c].y);
             const Split4 s1 = split4<DT>(raw[c].z, raw[c].w);
-            uint32_t d0 = 0, d1 = 0;
-            if constexpr (RANKED) {  // frequency-rank variant (never with job.check)
+            if constexpr (RANKED)  // frequency-rank variant
                 y[c] = make_uint2(lut4(tc.lut, s0.x), lut4(tc.lut, s1.x));
-            } else {
-                d0 = bytewise_b_minus(tc, s0.x);
-                d1 = bytewise_b_minus(tc, s1.x);
-                y[c] = make_uint2(d0 & tc.nmask4, d1 & tc.nmask4);
-            }
+            else
+                y[c] = make_uint2(bytewise_b_minus(tc, s0.x) & tc.nmask4, bytewise_b_minus(tc, s1.x) & tc.nmask4);
             hs[c] = make_uint2(s0.hs, s1.hs);
             if (active && e0 + 8 > real) {  // padding elements carry y = 0
                 const uint32_t valid = e0 < real ? real - e0 : 0;
@@ -1056,14 +1012,6 @@ enec_encode_kernel(const EncodeJob job, int* status) {
                 y[c].y &= k1;
             }
             if (!active) y[c] = make_uint2(0, 0);
-            if (job.check && active && e0 + 8 <= real)
-                bad |= (lossy_bytes(tc, d0, y[c].x) | lossy_bytes(tc, d1, y[c].y)) != 0;
-            else if (job.check && active && e0 < real) {
-                const uint32_t valid = real - e0;
-                const uint32_t k0 = valid >= 4 ? 0xFFFFFFFFu : (1u << (8 * valid)) - 1;
-                const uint32_t k1 = valid > 4 ? (1u << (8 * (valid - 4))) - 1 : 0;
-                bad |= ((lossy_bytes(tc, d0, y[c].x) & k0) | (lossy_bytes(tc, d1, y[c].y) & k1)) != 0;
-            }
             if (active && e0 < uint32_t(align16(real)))
                 __stcs(reinterpret_cast<uint2*>(out_sm + e0), make_uint2(s0.sm, s1.sm));
             uint32_t o = y[c].x | y[c].y;
@@ -1089,11 +1037,11 @@ enec_encode_kernel(const EncodeJob job, int* status) {
             if (DT == ENEC_FP16) pack_plane<3>(smem_u32(s_hi3), j, N, hs);
         }
     } else {
-        bad = encode_short_block<DT>(in, N, real, tc, b, n, m, job.check, out_sm, out_low, out_smhi, out_mask, out_smlo, &sh,
-                                     reinterpret_cast<uint32_t*>(s_low), reinterpret_cast<uint32_t*>(s_hi3),
-                                     reinterpret_cast<uint32_t*>(s_rec));
+        encode_short_block<DT>(in, N, real, tc, b, n, m, out_sm, out_low, out_smhi, out_mask, out_smlo, &sh,
+                               reinterpret_cast<uint32_t*>(s_low), reinterpret_cast<uint32_t*>(s_hi3),
+                               reinterpret_cast<uint32_t*>(s_rec));
     }
-    const int any_bad = __syncthreads_or(bad);
+    __syncthreads();
     {
         // the CTA's next block is known by now: pull its 32 KB towards L2 (one 128-byte line per thread, two for fp32)
         // so that the loads of the next iteration do not wait for DRAM
@@ -1121,10 +1069,8 @@ enec_encode_kernel(const EncodeJob job, int* status) {
     const uint32_t mask_excl = mask_incl - __popc(mask_word);
     const uint32_t wide_count = __shfl_sync(0xFFFFFFFFu, mask_incl, 31);
     if (tid == 31) {
-        if (any_bad) report(status, ENEC_ERR_PARAMS_NOT_LOSSLESS);
         // publish this block's count at once; block 0 knows its prefix already
-        st_relaxed_u64(&job.state[k], (k == 0 ? kStatePrefix : kStateAggregate) | (any_bad ? kStateTaint : 0ull) |
-                                          epoch_bits(job.epoch) | wide_count);
+        st_relaxed_u64(&job.state[k], (k == 0 ? kStatePrefix : kStateAggregate) | epoch_bits(job.epoch) | wide_count);
     }
     if (N >= 128) {
         fold_plane_out(smem_u32(s_low), N * uint32_t(m) / 8, out_low, tid);
@@ -1166,16 +1112,15 @@ enec_encode_kernel(const EncodeJob job, int* status) {
 
     // the previous block of this CTA, whose records wait in the other buffer
     if (pending_block != 0xFFFFFFFFu) {
-        resolve_block<DT, RANKED>(job, tensor, pending_block, pending_wide, pending_bad,
+        resolve_block<DT, RANKED>(job, tensor, pending_block, pending_wide,
                           s_rec_base + (cur ^ 1) * EncodeSmem<DT>::kRecBytes, sh, status);
     }
     pending_block = k;
     pending_wide = wide_count;
-    pending_bad = any_bad != 0;
     cur ^= 1;
     }
     if (pending_block != 0xFFFFFFFFu) {
-        resolve_block<DT, RANKED>(job, tensor, pending_block, pending_wide, pending_bad,
+        resolve_block<DT, RANKED>(job, tensor, pending_block, pending_wide,
                           s_rec_base + (cur ^ 1) * EncodeSmem<DT>::kRecBytes, sh, status);
     }
 }

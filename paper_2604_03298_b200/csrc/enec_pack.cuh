@@ -19,15 +19,12 @@ namespace enec {
 
 constexpr int kPackThreads = 256;
 
-__device__ __forceinline__ TransformCtx make_transform_ctx(int dt_exp_bits, int b, int n) {
+__device__ __forceinline__ TransformCtx make_transform_ctx(int b, int n) {
     TransformCtx tc;
     tc.b4 = rep4(uint32_t(b));
     tc.b4_or_h = tc.b4 | 0x80808080u;
     tc.nmask4 = rep4((1u << n) - 1);
     tc.s4 = rep4(1u << (n - 1));
-    tc.emask4 = rep4((1u << dt_exp_bits) - 1);
-    tc.n = n;
-    tc.E = dt_exp_bits;
     tc.lut = 0;
     return tc;
 }
@@ -150,7 +147,6 @@ __device__ __forceinline__ uint32_t pack_full_block(const uint8_t* in_bytes, int
     constexpr uint32_t N = kBlockElems;
     constexpr uint32_t kSpare = kGroupsPerBlock * 16;
     constexpr uint32_t kElemBytes = DT == ENEC_FP32 ? 4 : 2;
-    constexpr int E = HistShape<DT>::E;
     uint8_t* s_low = pack_smem;
     uint8_t* s_hi3 = pack_smem + 10240;  // fp16 only (m <= 5, so the low plane ends below)
     const uint32_t s_exp = smem_u32(pack_smem) + kBlockElems;
@@ -160,14 +156,13 @@ __device__ __forceinline__ uint32_t pack_full_block(const uint8_t* in_bytes, int
     const uint32_t perm = warp * 32 + 2 * (lane & 15) + (lane >> 4);
     const uint32_t j = 8 * perm;
     const uint32_t lower = (1u << ((j >> 4) & 31)) - 1;  // groups below this thread's in its mask word
-    const TransformCtx tc = make_transform_ctx(E, b, n);
+    const TransformCtx tc = make_transform_ctx(b, n);
     uint2 y[8], hs[8];
-    int bad = 0;
     uint32_t wide_bits;
     if (n < 8)
-        wide_bits = encode_full_runs<DT, true>(in_bytes + j * kElemBytes, out_sm + j, out_smlo + j * 2, tc, m, warp, lane, s_mask, y, hs, bad);
+        wide_bits = encode_full_runs<DT, true>(in_bytes + j * kElemBytes, out_sm + j, out_smlo + j * 2, tc, m, warp, lane, s_mask, y, hs);
     else
-        wide_bits = encode_full_runs<DT, false>(in_bytes + j * kElemBytes, out_sm + j, out_smlo + j * 2, tc, m, warp, lane, s_mask, y, hs, bad);
+        wide_bits = encode_full_runs<DT, false>(in_bytes + j * kElemBytes, out_sm + j, out_smlo + j * 2, tc, m, warp, lane, s_mask, y, hs);
     {
         uint2 ylow[8];
         const uint32_t lowmask4 = rep4((1u << m) - 1);

@@ -215,3 +215,33 @@ def test_checked_calls_report_errors_and_recover():
     for th in threads:
         th.join()
     assert ok == {i: True for i in range(4)}
+
+
+@pytest.mark.parametrize("low, high", [("100", ""), ("100", "150"), ("", "150")])
+def test_the_environment_moves_the_split_forms_bounds(low, high):
+    """ENEC_SPLIT_MIN_BLOCKS and ENEC_SPLIT_MAX_BLOCKS say for which sizes enec_compress takes three kernels; all other sizes, and
+    given parameters of any size, take one. (Read once per process, hence the child.)"""
+    import os
+    import subprocess
+    import sys
+    root = os.path.dirname(os.path.dirname(os.path.abspath(__file__)))
+    child = f"""
+import sys
+sys.path.insert(0, {root!r})
+import torch
+import paper_2604_03298_b200 as enec
+for blocks in (1, 99, 100, 149, 150, 300):
+    t = (torch.randn(blocks * 16384, device="cuda", generator=torch.Generator(device="cuda").manual_seed(blocks)) * 0.02).bfloat16()
+    before = enec.enec_launch_count()
+    stream = enec.compress_tensor(t)
+    searched = enec.enec_launch_count() - before
+    assert torch.equal(enec.compress_tensor(t, params=stream[20:23].tolist()), stream)
+    given = enec.enec_launch_count() - before - searched
+    print(blocks, searched, given)
+"""
+    env = {k: v for k, v in os.environ.items() if not k.startswith("ENEC_")}
+    env.update({k: v for k, v in (("ENEC_SPLIT_MIN_BLOCKS", low), ("ENEC_SPLIT_MAX_BLOCKS", high)) if v})
+    res = subprocess.run([sys.executable, "-c", child], env=env, capture_output=True, text=True, timeout=300)
+    assert res.returncode == 0, res.stderr[-2000:]
+    want = {b: 3 if low and b >= 100 and (not high or b < 150) else 1 for b in (1, 99, 100, 149, 150, 300)}
+    assert res.stdout.split("\n")[:-1] == [f"{b} {n} 1" for b, n in want.items()]
