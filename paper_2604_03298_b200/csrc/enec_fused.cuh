@@ -680,7 +680,9 @@ __device__ __forceinline__ void leave_no_stream(const FusedTensor& t) {
 // its offset and nobody completes the header. One thread. (Out of line and behind the pack loop: it moves the loop's code, and
 // with it at the two waits in there 1024 blocks of bf16 took 23.5 us instead of 22.0, nine tensors of a layer up to 277
 // instead of 270; as it is 21.9 and 272.)
-[[maybe_unused]] static __device__ __noinline__ void give_up(const FusedTensor& t, uint32_t k, int* status) {
+template <int DT>
+__device__ __noinline__ void give_up(uint32_t k, int* status, uint32_t slot = 0) {
+    const FusedTensor& t = fused_tensor<DT>(slot);
     report(status, ENEC_ERR_TIMEOUT);
     st_relaxed_u64(&t.state[k], 0ull);                            // no call's epoch
     atomicAdd(&t.super[k / kSuperBlocks], 1ull << 32);            // one block too many
@@ -1351,7 +1353,7 @@ __device__ __noinline__ uint32_t pack_pass(FusedControl* ctl, uint32_t pass, int
         __syncthreads();
         pack_short_block<DT, CHECK>(k, status);
     }
-    if (lost && tid == 0) give_up(t, lost, status);
+    if (lost && tid == 0) give_up<DT>(lost, status);
     return mine;
 }
 

@@ -322,7 +322,7 @@ enec_fused_list_kernel(const FusedList list, int* status) {
         // A wait ran out. The CTA's waiting block is not placed and the unit that it has a ticket for is not done; whose tensor
         // that is, and which tensors wait for it, is not followed up: no tensor of the list keeps a header from before.
         if (tid == 0) {
-            if (lost) give_up(fused_tensor<DT>(lost >> 28), lost & 0x0FFFFFFFu, status);   // a tensor has at most 2^22 blocks
+            if (lost) give_up<DT>(lost & 0x0FFFFFFFu, status, lost >> 28);   // a tensor has at most 2^22 blocks
             else report(status, ENEC_ERR_TIMEOUT);
         }
         for (uint32_t i = tid; i < list.n_items; i += kFusedThreads) {

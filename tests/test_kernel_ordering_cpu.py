@@ -56,12 +56,12 @@ def test_a_wait_that_ran_out_leaves_no_stream():
         assert part in give_up
     rest = text.replace(give_up, "")
     assert len(re.findall(r"if \(!sh\.ok\) (?:{ )?lost = ", rest)) == 2     # waiting block, block without room to wait
-    assert rest.count("if (lost && tid == 0) give_up(t, lost, status);") == 1
+    assert rest.count("if (lost && tid == 0) give_up<DT>(lost, status);") == 1
     for report in re.finditer(r"report\(status, ENEC_ERR_TIMEOUT\);", rest):
         assert re.match(r"\s*leave_no_stream\(t\);", rest[report.end():])
     text = _source("enec_fused_list.cuh")
     assert len(re.findall(r"lost = (?:pend_)?slot << 28", text)) == 3       # those two, and a CTA that waits for parameters
     end = text[text.index("if (stop) {"):]
     assert text.count("report(status, ENEC_ERR_TIMEOUT)") == end.count("report(status, ENEC_ERR_TIMEOUT)") == 1
-    assert "give_up(" in end and "i < list.n_items" in end and "->magic = 0" in end and "out_size = 0" in end
+    assert "give_up<DT>(" in end and "i < list.n_items" in end and "->magic = 0" in end and "out_size = 0" in end
     assert not re.search(r"\breturn;", text[text.index("enec_fused_list_kernel("):text.index("if (stop) {")].split("for (uint32_t iter = 0;;")[1])
