@@ -518,9 +518,9 @@ enec_status enec_decompress_ranked(const void* d_in, size_t in_size, enec_dtype 
 
 // Blocks per chunk of a ticketed list (see DecodeBatch): two, or one when that leaves CTAs (three per SM) without a
 // second chunk.
-static uint32_t batched_chunk_blocks(uint64_t total_blocks) {
-    constexpr uint64_t kCtasOfALaunch = 148 * 3;
-    return total_blocks < 4 * kCtasOfALaunch ? 1u : 2u;
+static uint32_t batched_chunk_blocks(uint64_t total_blocks, int sms) {
+    const uint64_t ctas_of_a_launch = uint64_t(sms) * 3;
+    return total_blocks < 4 * ctas_of_a_launch ? 1u : 2u;
 }
 
 enec_status enec_decompress_batched(const enec_batch_item* h_items, int n_items, enec_dtype dt, int* d_status,
@@ -587,7 +587,11 @@ enec_status enec_decompress_batched(const enec_batch_item* h_items, int n_items,
         // the blocks of a long list are handed out in chunks: a zeroed ticket word and the tensor of every chunk's
         // first block travel with the descriptors
         const size_t ticket_at = host.size();
-        const uint32_t chunk = batched_chunk_blocks(total);
+        int dev = 0;
+        if (cudaGetDevice(&dev) != cudaSuccess) return ENEC_ERR_CUDA;
+        const DeviceInfo* info = device_info(dev);
+        if (!info) return ENEC_ERR_CUDA;
+        const uint32_t chunk = batched_chunk_blocks(total, info->sms);
         batch.chunk_blocks = uint16_t(chunk);
         const size_t n_chunks = size_t((total + chunk - 1) / chunk);
         host.resize(ticket_at + 16 + n_chunks * sizeof(uint32_t), 0);
@@ -601,8 +605,6 @@ enec_status enec_decompress_batched(const enec_batch_item* h_items, int n_items,
                 chunk_job[c] = j;
             }
         }
-        int dev = 0;
-        if (cudaGetDevice(&dev) != cudaSuccess) return ENEC_ERR_CUDA;
         uint8_t* scratch = nullptr;
         const enec_status st = get_scratch(dev, stream, kScratchBatch, host.size(), &scratch);
         if (st != ENEC_OK) return st;

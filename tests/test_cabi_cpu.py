@@ -60,6 +60,15 @@ def test_binding_has_the_same_names():
         assert hasattr(enec, name), name
 
 
+def test_launch_rules_take_the_number_of_sms_from_the_device():
+    """No rule of a launch or dispatch spells out the 148 SMs of one part; figures in comments may."""
+    csrc = os.path.join(ROOT, "paper_2604_03298_b200", "csrc")
+    for name in sorted(os.listdir(csrc)):
+        if name.endswith((".cu", ".cuh")):
+            code = re.sub(r"//[^\n]*", "", open(os.path.join(csrc, name)).read())
+            assert not re.search(r"\b148\b", code), name
+
+
 def test_missing_library_fails_loudly(monkeypatch, tmp_path):
     from paper_2604_03298_b200 import binding
     monkeypatch.setattr(binding, "_LIB", None)
