@@ -245,3 +245,38 @@ for blocks in (1, 99, 100, 149, 150, 300):
     assert res.returncode == 0, res.stderr[-2000:]
     want = {b: 3 if low and b >= 100 and (not high or b < 150) else 1 for b in (1, 99, 100, 149, 150, 300)}
     assert res.stdout.split("\n")[:-1] == [f"{b} {n} 1" for b, n in want.items()]
+
+
+def _mislead(t, blocks, what):
+    """Changes values of blocks that the sample (every (blocks // 148)-th, from the first on) does not hold."""
+    step = blocks // 148
+    body = t[:blocks * 16384].view(blocks, 16384)
+    at = {"early": 1, "middle": blocks // 2 // step * step + 1, "late": (blocks - 2) // step * step + 1}
+    if what in at:
+        body[at[what], 77] = 0            # the pass ends there, the rest is counted, everything packed again
+    else:
+        for k in range(1, step):          # no value is lost, but the whole tensor has another (b, m)
+            body[k::step] *= 3.0
+    return t
+
+
+@pytest.mark.parametrize("dt, blocks", [(0, 1409), (1, 1409), (2, 705)])
+@pytest.mark.parametrize("tail", [0, 37, 5003])
+@pytest.mark.parametrize("what", ["early", "middle", "late", "other parameters"])
+def test_misled_samples_just_above_the_bound(oracle, dt, blocks, tail, what):
+    """The smallest sizes of which a sample is taken."""
+    import paper_2604_03298_b200 as enec
+    least = 2e-3 if dt == 1 else 1e-6
+    t = _weights(blocks * 16384 + tail, dt, 11)
+    t = _mislead(torch.where(t.abs() < least, torch.full_like(t, least), t), blocks, what)
+    assert np.array_equal(_compress_twice(enec, t, dt), oracle.compress(_words(t, dt), dt))
+
+
+@pytest.mark.parametrize("what", ["early", "late", "other parameters"])
+def test_misled_samples_with_second_level_sums(oracle, what):
+    """More than 16384 blocks: the second pass has second-level sums of its own."""
+    import paper_2604_03298_b200 as enec
+    blocks = 16384 + 300
+    t = _weights(blocks * 16384 + 100, 0, 12)
+    t = _mislead(torch.where(t.abs() < 1e-6, torch.full_like(t, 1e-6), t), blocks, what)
+    assert np.array_equal(_compress_twice(enec, t, 0), oracle.compress(_words(t, 0), 0))
