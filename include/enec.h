@@ -18,6 +18,7 @@
  * are returned at once. Errors only the device can see (damaged stream, parameters that are not
  * lossless, a wait that ran out) are written to *d_status if d_status is not NULL: the first error wins,
  * the value is one of enec_status, and it stays 0 when the call succeeded. The caller zeroes *d_status.
+ * A compress call that fails on the device leaves no stream: the header's magic and the length are 0.
  * A kernel that finds an error stops touching the output; it never reads or writes out of range.
  *
  * The library keeps one small device scratch area per (device, stream) for the compressor (histogram

@@ -10,7 +10,7 @@
 //      CTAs pack the tensor again; a value that the sampled parameters cannot represent ends the pack stage at once, and the blocks
 //      not packed yet are counted first.
 // Parameters given by the caller: stage 2 alone, without the histogram, from the first block on; a value that they lose ends
-// the call without a stream. (With a look-back kernel, or two kernels from 2048 blocks up, 3584 blocks of bf16 took 54 us, now 38.7;
+// the call without a stream. (With a look-back kernel, or two kernels from 2048 blocks up, 3584 blocks of bf16 took 54 us, now 37.3;
 // 1024 blocks 23.2 -> 15.1, fp16 4096 blocks 63.8 -> 47.5, fp32 8192 blocks 192 -> 168.)
 // A tensor whose sample needs n > 6 exponent bits (bf16, fp32) takes the histogram of the whole tensor before it packs:
 // the table kept beside the packing has 64 rows, and rare outliers of such a tensor are what a sample misses.

@@ -7,11 +7,12 @@
 //   pack    one block with its tensor's parameters (as in enec_fused_kernel, always with the whole tensor's parameters)
 //   whole   a tensor of one block: count, search and pack, by one CTA
 // The order is: count the first wave of tensors, the tensors of one block, then in turn count the wave after the next and
-// pack a wave. A wave has about kWaveBytes, so that its second reading comes from L2, and the wave counted in between gives
-// the searches time. A unit waits only for units with smaller tickets.
+// pack a wave. A wave ends with the tensor that brings it to kWaveBytes, so that its second reading comes from L2 unless one of its
+// tensors is too large for that; the wave counted in between gives the searches time. A unit waits only for units with
+// smaller tickets.
 //
 // Against the two launches before (histograms of all tensors, then a look-back kernel over all blocks): 56 tensors of 139 MB
-// bf16 121 -> 103 us, a Llama-3-8B-shaped layer 308 -> 272 us.
+// bf16 120 -> 87 us, a Llama-3-8B-shaped layer 308 -> 241 us.
 #pragma once
 
 #include "enec_fused.cuh"

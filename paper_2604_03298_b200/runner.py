@@ -166,7 +166,7 @@ class CodecSet:
         return self.batches
 
     def compress_batched(self) -> None:
-        """One enec_compress_batched call per dtype of the set (two launches each) on the current stream."""
+        """One enec_compress_batched call per dtype of the set (one launch each) on the current stream."""
         for dt, comp, _, sizes, where in self._batches():
             st = enec.enec_compress_batched(comp, dt, sizes, self.status)
             if st != 0:
