@@ -90,7 +90,7 @@ struct FusedShape {
     static constexpr uint32_t kRows = DT == ENEC_FP16 ? 32 : 64;       // rows of the pack stage's histogram
     static constexpr uint32_t kHistAt = kWork;
     static constexpr uint32_t kHistBytes = kRows * HistShape<DT>::kRowBytes;
-    static constexpr uint32_t kListAt = kHistAt + kHistBytes;          // the wide groups' numbers, a byte each, by warp
+    static constexpr uint32_t kListAt = kHistAt + kHistBytes;          // the wide groups' numbers, a byte each, by mask word
     static constexpr uint32_t kPend = 4096;                            // a block's packed records waiting for their offset
     static constexpr uint32_t kPendAt = kListAt + 1024;
     static constexpr uint32_t kTensorAt = kPendAt + 2 * kPend;         // FusedTensor (lists: of the block, the waiting block, the next)
@@ -545,21 +545,31 @@ __device__ __forceinline__ void record_words(const uint4& v, uint32_t s4, int m,
     }
 }
 
-// The calling warp's wide groups (the block's values at shared address `values`, the groups' numbers at `list`): records to
-// shared memory at `pend`, or, when they do not fit there, straight to `out` (2-byte aligned). mask_word, excl: see scan_mask.
+// The wide groups of a block, shared out over the CTA's threads in the order of their ranks: thread t packs those of rank t,
+// t + 256, .. (the block's values at shared address `values`; the numbers of mask word w's wide groups, a byte each, at
+// list + 32 w; lane w of every warp: wide groups before word w in `excl`). Records go to shared memory at `pend`, or, when they
+// do not fit there, straight to `out` (2-byte aligned). A weight's block has about 250 wide groups: one round for the CTA. (Every
+// warp packing the wide groups of its own runs takes two as a rule, since they are rarely 32 at most: 32064 blocks of bf16 363.5 us,
+// now 356; 4096 blocks of fp32 100.3, now 97.3; 1024 heavy-tailed ones of bf16 23.1, now 22.6.)
 template <int H>
-__device__ __forceinline__ void pack_records(uint32_t values, uint32_t list, uint32_t count, uint32_t mask_word, uint32_t excl,
-                                             uint32_t s4, int m, uint32_t pend, uint8_t* out) {
-    const uint32_t lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    for (uint32_t base = 0; base < count; base += 32) {
-        const uint32_t i = base + lane;
-        const uint32_t number = lds8(list + (i < count ? i : 0));
-        const uint32_t word = (number >> 5) * kFusedWarps + warp;
-        const uint32_t rank = __shfl_sync(0xFFFFFFFFu, excl, word) +
-                              __popc(__shfl_sync(0xFFFFFFFFu, mask_word, word) & ((1u << (number & 31)) - 1));
-        if (i < count) {
+__device__ __forceinline__ void pack_records(uint32_t values, uint32_t list, uint32_t wide, uint32_t excl, uint32_t s4, int m, uint32_t pend,
+                                             uint8_t* out) {
+    const uint32_t lane = threadIdx.x & 31;
+    for (uint32_t base = threadIdx.x & ~31u; base < wide; base += kFusedThreads) {
+        const uint32_t rank = base + lane;
+        uint32_t word = 0, first = 0;   // the last word with at most `rank` wide groups before it
+#pragma unroll
+        for (uint32_t step = 16; step; step >>= 1) {
+            const uint32_t before = __shfl_sync(0xFFFFFFFFu, excl, word + step);
+            if (before <= rank) {
+                word += step;
+                first = before;
+            }
+        }
+        if (rank < wide) {
+            const uint32_t number = lds8(list + word * 32 + (rank - first));
             uint32_t q[H];
-            record_words<H>(lds128(values + ((number >> 5) * kFusedThreads + warp * 32 + (number & 31)) * 16), s4, m, q);
+            record_words<H>(lds128(values + (word * 32 + number) * 16), s4, m, q);
             if (out == nullptr) {
 #pragma unroll
                 for (int k = 0; k < H; ++k) sts16(pend + (rank * H + k) * 2, q[k]);
@@ -572,17 +582,17 @@ __device__ __forceinline__ void pack_records(uint32_t values, uint32_t list, uin
 }
 
 template <int DT>
-__device__ __forceinline__ void pack_records_any(int h, uint32_t values, uint32_t list, uint32_t count, uint32_t mask_word, uint32_t excl,
-                                                 uint32_t s4, int m, uint32_t pend, uint8_t* out) {
+__device__ __forceinline__ void pack_records_any(int h, uint32_t values, uint32_t list, uint32_t wide, uint32_t excl, uint32_t s4, int m,
+                                                 uint32_t pend, uint8_t* out) {
     switch (h) {
         case 0: break;
-        case 1: pack_records<1>(values, list, count, mask_word, excl, s4, m, pend, out); break;
-        case 2: pack_records<2>(values, list, count, mask_word, excl, s4, m, pend, out); break;
-        case 3: pack_records<3>(values, list, count, mask_word, excl, s4, m, pend, out); break;
-        case 4: pack_records<4>(values, list, count, mask_word, excl, s4, m, pend, out); break;
-        case 5: if constexpr (DT != ENEC_FP16) pack_records<5>(values, list, count, mask_word, excl, s4, m, pend, out); break;
-        case 6: if constexpr (DT != ENEC_FP16) pack_records<6>(values, list, count, mask_word, excl, s4, m, pend, out); break;
-        default: if constexpr (DT != ENEC_FP16) pack_records<7>(values, list, count, mask_word, excl, s4, m, pend, out); break;
+        case 1: pack_records<1>(values, list, wide, excl, s4, m, pend, out); break;
+        case 2: pack_records<2>(values, list, wide, excl, s4, m, pend, out); break;
+        case 3: pack_records<3>(values, list, wide, excl, s4, m, pend, out); break;
+        case 4: pack_records<4>(values, list, wide, excl, s4, m, pend, out); break;
+        case 5: if constexpr (DT != ENEC_FP16) pack_records<5>(values, list, wide, excl, s4, m, pend, out); break;
+        case 6: if constexpr (DT != ENEC_FP16) pack_records<6>(values, list, wide, excl, s4, m, pend, out); break;
+        default: if constexpr (DT != ENEC_FP16) pack_records<7>(values, list, wide, excl, s4, m, pend, out); break;
     }
 }
 // Number of wide groups before block k, by one warp; false when the blocks before were not counted in time.
@@ -736,12 +746,12 @@ __device__ __forceinline__ Run load32_any(const uint8_t* p, bool wide) {
     return load32<false>(p);
 }
 // One run of sixteen values of a block, group `g` of it: sign/mantissa plane, histogram, values (16 bytes per group; fp16:
-// the bits of the fp16 plane in bits 7..5 of each byte), votes for the group mask and the numbers of the warp's wide
-// groups. number: 32 x (which of the thread's groups) + lane. Returns the OR of all values.
+// the bits of the fp16 plane in bits 7..5 of each byte), votes for the group mask and the lanes of the wide groups among the
+// warp's, at `list`. Returns the OR of all values.
 template <int DT, bool PLAIN, bool HIST, bool CHECK = false>
 __device__ __forceinline__ uint32_t pack_run(const Run& r, uint32_t minuend, uint32_t nmask4, uint32_t s4, uint32_t wide4, uint32_t hist,
-                                             uint32_t lane, uint32_t value_at, uint32_t number, uint32_t list, uint32_t& wide,
-                                             uint32_t* mask_word, bool store, uint8_t* sm_out) {
+                                             uint32_t lane, uint32_t value_at, uint32_t list, uint32_t* mask_word, bool store,
+                                             uint8_t* sm_out) {
     uint4 v, hs, sm;
     transform_run<DT, PLAIN, HIST, CHECK>(r, minuend, nmask4, hist, lane * 4, v, hs, sm);
     if (store) __stcs(reinterpret_cast<uint4*>(sm_out), sm);
@@ -753,18 +763,16 @@ __device__ __forceinline__ uint32_t pack_run(const Run& r, uint32_t minuend, uin
     sts128(value_at, v);
     const uint32_t votes = __ballot_sync(0xFFFFFFFFu, is_wide);
     if (lane == 0) *mask_word = votes;
-    if (is_wide) sts8(list + wide + __popc(votes & ((1u << lane) - 1)), number);
-    wide += __popc(votes);
+    if (is_wide) sts8(list + __popc(votes & ((1u << lane) - 1)), lane);
     return all;
 }
 
 // First phase of a full block, all threads: thread t takes the groups t, t + 256, .. of the block through pack_run.
-// Returns whether some value is not representable (HIST only); `wide_of_warp`: the warp's wide groups.
+// Returns whether some value is not representable (HIST only).
 // All loads of a thread's four runs are in flight together (3584 blocks of bf16: 56.2 us; two runs, in a rolled loop, 59.6) and
 // take no room in L1, of which the shared memory of three CTAs leaves little.
 template <int DT, bool PLAIN, bool HIST, bool CHECK = false>
-__device__ __forceinline__ bool pack_front_full(const FusedTensor& t, uint32_t k, uint32_t work, uint32_t* s_mask, uint32_t tid,
-                                                uint32_t& wide_of_warp) {
+__device__ __forceinline__ bool pack_front_full(const FusedTensor& t, uint32_t k, uint32_t work, uint32_t* s_mask, uint32_t tid) {
     using Shape = FusedShape<DT>;
     constexpr uint32_t kElemBytes = DT == ENEC_FP32 ? 4 : 2;
     constexpr uint32_t kStep = 16 * kFusedThreads;   // elements between a thread's runs
@@ -774,12 +782,12 @@ __device__ __forceinline__ bool pack_front_full(const FusedTensor& t, uint32_t k
     uint8_t* sm_out = t.sm + (uint64_t(k) * kBlockElems + 16 * tid);
     uint8_t* lo_out = t.lo + (uint64_t(k) * kBlockElems + 16 * tid) * 2;
     const uint32_t minuend = t.c, nmask4 = t.nmask4, s4 = t.s4, wide4 = t.wide4, wide_ok = t.wide_ok;
-    const uint32_t values = work + Shape::kValuesAt + tid * 16, list = work + Shape::kListAt + warp * 128;
-    uint32_t all = 0, wide = 0;
+    const uint32_t values = work + Shape::kValuesAt + tid * 16, list = work + Shape::kListAt + warp * 32;
+    uint32_t all = 0;
     const bool wide_in = (wide_ok & 1) != 0;
     auto run = [&](const Run& r, uint32_t i) {
-        all |= pack_run<DT, PLAIN, HIST, CHECK>(r, minuend, nmask4, s4, wide4, work + Shape::kHistAt, lane, values + i * kStep, i * 32 + lane, list,
-                                         wide, &s_mask[i * kFusedWarps + warp], true, sm_out + i * kStep);
+        all |= pack_run<DT, PLAIN, HIST, CHECK>(r, minuend, nmask4, s4, wide4, work + Shape::kHistAt, lane, values + i * kStep,
+                                                list + i * kFusedThreads, &s_mask[i * kFusedWarps + warp], true, sm_out + i * kStep);
     };
     if constexpr (DT == ENEC_FP32) {   // one run's 64 bytes in flight (two runs', unrolled: 1024 blocks 45.3 -> 49.6 us)
         Run a = load32_any(in, wide_in), b = load32_any(in + 32, wide_in);
@@ -798,13 +806,12 @@ __device__ __forceinline__ bool pack_front_full(const FusedTensor& t, uint32_t k
         run(c, 2);
         run(d, 3);
     }
-    wide_of_warp = wide;
     return (HIST || CHECK) && (DT == ENEC_FP16 ? all & rep4(0x1F) & ~nmask4 : all & ~nmask4) != 0;
 }
 
 // The same for the tensor's last block when it is not full and has at least 128 padded elements.
 template <int DT, bool PLAIN, bool HIST, bool CHECK = false>
-__device__ __noinline__ bool pack_front_tail(uint32_t k, uint32_t* wide_of_warp, uint32_t slot = 0) {
+__device__ __noinline__ bool pack_front_tail(uint32_t k, uint32_t slot = 0) {
     using Shape = FusedShape<DT>;
     const FusedTensor& t = fused_tensor<DT>(slot);
     FusedShared& sh = fused_shared<DT>();
@@ -820,7 +827,7 @@ __device__ __noinline__ bool pack_front_tail(uint32_t k, uint32_t* wide_of_warp,
         red_add_one(work + Shape::kHistAt + lane * 4 + (x & (Shape::kRows - 1)) * HistShape<DT>::kRowBytes);
     }
     __syncthreads();
-    uint32_t wide = 0, all = 0;
+    uint32_t all = 0;
     // (one run at a time: with more registers the full blocks' loop, which shares its frame with the call, loses 6 %)
 #pragma unroll 1
     for (uint32_t i = 0; i < kBlockElems / (16 * kFusedThreads); ++i) {
@@ -843,18 +850,17 @@ __device__ __noinline__ bool pack_front_tail(uint32_t k, uint32_t* wide_of_warp,
                                   int(align16(2 * uint64_t(real)) / 2) - int(e0), t.pad);
         }
         // the padding's sign/mantissa bytes are zero
-        all |= pack_run<DT, PLAIN, false, CHECK>(r, t.c, t.nmask4, t.s4, t.wide4, 0, lane, work + Shape::kValuesAt + g * 16, i * 32 + lane,
-                                          work + Shape::kListAt + warp * 128, wide, &sh.mask[i * kFusedWarps + warp], left > 0,
-                                          t.sm + uint64_t(k) * kBlockElems + e0);
+        all |= pack_run<DT, PLAIN, false, CHECK>(r, t.c, t.nmask4, t.s4, t.wide4, 0, lane, work + Shape::kValuesAt + g * 16,
+                                                 work + Shape::kListAt + first, &sh.mask[i * kFusedWarps + warp], left > 0,
+                                                 t.sm + uint64_t(k) * kBlockElems + e0);
     }
     const bool bad = (HIST || CHECK) && (DT == ENEC_FP16 ? all & rep4(0x1F) & ~t.nmask4 : all & ~t.nmask4) != 0;
-    *wide_of_warp = wide;
     return bad;
 }
 
-// Every warp: the block's mask words (lane l: word l) and the wide groups before each; returns the block's wide groups.
-__device__ __forceinline__ uint32_t scan_mask(const uint32_t* s_mask, uint32_t lane, uint32_t& word, uint32_t& before) {
-    word = s_mask[lane];
+// Every warp: the wide groups before each of the block's mask words (lane l: word l); returns the block's wide groups.
+__device__ __forceinline__ uint32_t scan_mask(const uint32_t* s_mask, uint32_t lane, uint32_t& before) {
+    const uint32_t word = s_mask[lane];
     uint32_t incl = __popc(word);
 #pragma unroll
     for (int d = 1; d < 32; d <<= 1) {
@@ -1252,12 +1258,11 @@ __device__ __noinline__ uint32_t pack_pass(FusedControl* ctl, uint32_t pass, int
         ++mine;
         const bool last = k + 1 == t.nblocks && t.tail_real != kBlockElems;   // the tensor's last block, not full
         const uint32_t N = last ? t.tail_padded : kBlockElems;
-        uint32_t wide_of_warp = 0;
         bool bad = false;
         if (!last) {
-            bad = pack_front_full<DT, PLAIN, HIST, CHECK>(t, k, work, sh.mask, tid, wide_of_warp);
+            bad = pack_front_full<DT, PLAIN, HIST, CHECK>(t, k, work, sh.mask, tid);
         } else {
-            bad = pack_front_tail<DT, PLAIN, HIST, CHECK>(k, &wide_of_warp);
+            bad = pack_front_tail<DT, PLAIN, HIST, CHECK>(k);
         }
         if (tid == 0) {
             sh.next = asked;
@@ -1269,8 +1274,8 @@ __device__ __noinline__ uint32_t pack_pass(FusedControl* ctl, uint32_t pass, int
         const bool waiting = pend_block != 0xFFFFFFFFu;
         unsigned long long answer = 0;
         if (waiting) answer = ask_before(t, pend_block, tid);   // it comes while the block is packed
-        uint32_t mask_word, excl;
-        const uint32_t wide = scan_mask(sh.mask, lane, mask_word, excl);
+        uint32_t excl;
+        const uint32_t wide = scan_mask(sh.mask, lane, excl);
         if (tid == 0 && t.nblocks != 1) {
             st_relaxed_u64(&t.state[k], ((unsigned long long)t.epoch << 32) | wide);
             atomicAdd(&t.super[k / kSuperBlocks], (1ull << 32) | wide);
@@ -1299,7 +1304,7 @@ __device__ __noinline__ uint32_t pack_pass(FusedControl* ctl, uint32_t pass, int
             if (!sh.ok) lost = k;
         }
         if (!direct || sh.ok)
-            pack_records_any<DT>(int(hbits), work + Shape::kValuesAt, work + Shape::kListAt + warp * 128, wide_of_warp, mask_word, excl, t.s4, int(m),
+            pack_records_any<DT>(int(hbits), work + Shape::kValuesAt, work + Shape::kListAt, wide, excl, t.s4, int(m),
                                  work + Shape::kPendAt + (iter & 1) * Shape::kPend,
                                  direct ? t.high + uint64_t(sh.before) * 2 * hbits : nullptr);
         if (waiting) {

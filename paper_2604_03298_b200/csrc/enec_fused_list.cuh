@@ -252,14 +252,13 @@ enec_fused_list_kernel(const FusedList list, int* status) {
             }
             const bool last = k + 1 == t.nblocks && t.tail_real != kBlockElems;
             const uint32_t N = last ? t.tail_padded : kBlockElems;
-            uint32_t wide_of_warp = 0;
             if (!present) {
             } else if (!last) {
-                if (t.plain || DT == ENEC_FP16) pack_front_full<DT, true, false>(t, k, work, sh.mask, tid, wide_of_warp);
-                else pack_front_full<DT, false, false>(t, k, work, sh.mask, tid, wide_of_warp);
+                if (t.plain || DT == ENEC_FP16) pack_front_full<DT, true, false>(t, k, work, sh.mask, tid);
+                else pack_front_full<DT, false, false>(t, k, work, sh.mask, tid);
             } else if (N >= 128) {
-                if (t.plain || DT == ENEC_FP16) pack_front_tail<DT, true, false>(k, &wide_of_warp, slot);
-                else pack_front_tail<DT, false, false>(k, &wide_of_warp, slot);
+                if (t.plain || DT == ENEC_FP16) pack_front_tail<DT, true, false>(k, slot);
+                else pack_front_tail<DT, false, false>(k, slot);
             }
             __syncthreads();                                      // barrier A
             if (waiting) answer = ask_before(fused_tensor<DT>(pend_slot), pend_block, tid);
@@ -267,8 +266,8 @@ enec_fused_list_kernel(const FusedList list, int* status) {
             if (present && N < 128) {
                 pack_short_block<DT>(k, status, slot);            // its records go straight to their place
             } else if (present) {
-                uint32_t mask_word, excl;
-                wide = scan_mask(sh.mask, lane, mask_word, excl);
+                uint32_t excl;
+                wide = scan_mask(sh.mask, lane, excl);
                 if (tid == 0 && t.nblocks != 1) {
                     st_relaxed_u64(&t.state[k], ((unsigned long long)t.epoch << 32) | wide);
                     atomicAdd(&t.super[k / kSuperBlocks], (1ull << 32) | wide);
@@ -291,7 +290,7 @@ enec_fused_list_kernel(const FusedList list, int* status) {
                     if (!sh.ok) { stop = true; lost = slot << 28 | k; }
                 }
                 if (!stop)
-                    pack_records_any<DT>(int(hbits), work + Shape::kValuesAt, work + Shape::kListAt + warp * 128, wide_of_warp, mask_word, excl,
+                    pack_records_any<DT>(int(hbits), work + Shape::kValuesAt, work + Shape::kListAt, wide, excl,
                                          t.s4, int(m), work + Shape::kPendAt + (iter & 1) * Shape::kPend,
                                          direct ? t.high + uint64_t(sh.before) * 2 * hbits : nullptr);
                 leaves_records = !direct;
