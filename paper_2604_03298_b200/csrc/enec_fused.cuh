@@ -137,7 +137,7 @@ struct FusedShared {
     uint32_t before;
     uint32_t ok;
     uint32_t unit[2][3];          // lists: what the CTA does now and next (see enec_fused_list_kernel)
-    uint32_t part[kFusedWarps];   // each warp's share of the wide groups before the waiting block; kNotReady: some are not counted yet
+    alignas(16) uint32_t part[4];   // the last four warps' shares of the wide groups before the waiting block; kNotReady: some are not counted yet
 };
 constexpr uint32_t kNotReady = 0xFFFFFFFFu;   // a tensor has at most 2^32 - 2^10 groups of 16 counted before a block
 static_assert(sizeof(FusedTensor) <= 256 && sizeof(FusedShared) <= 256, "they fit their places");
@@ -351,6 +351,13 @@ __device__ __forceinline__ Run load_run_tail(const uint8_t* in, uint8_t* lo, int
     return r;
 }
 
+// The bits of a where the mask has ones, those of b elsewhere: one instruction (written with two masks it takes two).
+__device__ __forceinline__ uint32_t select_bits(uint32_t mask, uint32_t a, uint32_t b) {
+    uint32_t d;
+    asm("lop3.b32 %0, %1, %2, %3, 0xCA;" : "=r"(d) : "r"(mask), "r"(a), "r"(b));
+    return d;
+}
+
 // ---- one run: transform, sign/mantissa, histogram -------------------------------------------------------
 // hist: the pack stage's table; lane4: four times the lane, the lane's column.
 template <int DT>
@@ -364,6 +371,13 @@ __device__ __forceinline__ void count_halves(uint32_t hist, uint32_t lane4, uint
     }
 }
 
+// a - 2 w as one multiply-add.
+__device__ __forceinline__ uint32_t minus_twice(uint32_t a, uint32_t w) {
+    uint32_t d;
+    asm("mad.lo.u32 %0, %1, 0xFFFFFFFE, %2;" : "=r"(d) : "r"(w), "r"(a));
+    return d;
+}
+
 template <int DT, bool PLAIN, bool HIST, bool CHECK>
 __device__ __forceinline__ void transform_run(const Run& r, uint32_t minuend, uint32_t nmask4, uint32_t hist, uint32_t lane4, uint4& v,
                                               uint4& hs, uint4& sm) {
@@ -375,12 +389,12 @@ __device__ __forceinline__ void transform_run(const Run& r, uint32_t minuend, ui
         if constexpr (DT == ENEC_FP16) {
             vv[q] = minuend - ((hi >> 2) & 0x1F1F1F1Fu);
             ss[q] = lo;
-            hh[q] = (hi & 0x03030303u) | ((hi >> 5) & 0x04040404u);
+            hh[q] = select_bits(0x03030303u, hi, (hi >> 5) & 0x04040404u);
         } else {
-            ss[q] = (hi & 0x80808080u) | (lo & 0x7F7F7F7Fu);
+            ss[q] = select_bits(0x80808080u, hi, lo);
             hh[q] = 0;
             if constexpr (PLAIN) {
-                vv[q] = prmt(minuend - 2 * w0, minuend - 2 * w1, 0x7531u);
+                vv[q] = prmt(minus_twice(minuend, w0), minus_twice(minuend, w1), 0x7531u);
             } else {
                 const uint32_t x = prmt(2 * w0, 2 * w1, 0x7531u);
                 vv[q] = ((minuend | 0x80808080u) - (x & 0x7F7F7F7Fu)) ^ ((minuend ^ ~x) & 0x80808080u);
@@ -409,14 +423,14 @@ __device__ __forceinline__ void insert_field(uint32_t& lo, uint32_t& hi, uint32_
     constexpr uint32_t kField = (1u << W) - 1;
     if (s + W <= 8) {
         const uint32_t mask = rep4(kField << s);
-        lo = (lo & ~mask) | ((v << s) & mask);
+        lo = select_bits(mask, v << s, lo);
     } else if (s >= 8) {
         const uint32_t mask = rep4(kField << (s - 8));
-        hi = (hi & ~mask) | ((v << (s - 8)) & mask);
+        hi = select_bits(mask, v << (s - 8), hi);
     } else {
         const uint32_t mask_lo = rep4(0xFFu << s), mask_hi = rep4(kField >> (8 - s));
-        lo = (lo & ~mask_lo) | ((v << s) & mask_lo);
-        hi = (hi & ~mask_hi) | ((v >> (8 - s)) & mask_hi);
+        lo = select_bits(mask_lo, v << s, lo);
+        hi = select_bits(mask_hi, v >> (8 - s), hi);
     }
 }
 
@@ -482,17 +496,21 @@ __device__ __forceinline__ void pack_planes(const FusedTensor& t, uint32_t work,
     }
 }
 
-// The final fold (see fold_plane_out), all threads.
+// The final fold (see fold_plane_out), all threads. (Not unrolled: a thread has one or two rounds for m = 3, and the code around an
+// unrolled loop costs more.)
 __device__ __forceinline__ void fold_out(uint32_t S, uint32_t T, uint8_t* dst, uint32_t tid) {
-    const uint32_t thalf = T >> 1;
-    for (uint32_t u = tid; u < (thalf >> 3); u += kFusedThreads) {
-        const uint2 lo = lds64(S + 8 * u), hi = lds64(S + thalf + 8 * u);
+    const uint32_t thalf = T >> 1, end = S + thalf;
+    uint32_t at = S + 8 * tid;
+    dst += 16 * tid;
+#pragma unroll 1
+    for (; at < end; at += 8 * kFusedThreads, dst += 16 * kFusedThreads) {
+        const uint2 lo = lds64(at), hi = lds64(at + thalf);
         uint4 w;
         w.x = prmt(lo.x, hi.x, 0x5140u);
         w.y = prmt(lo.x, hi.x, 0x7362u);
         w.z = prmt(lo.y, hi.y, 0x5140u);
         w.w = prmt(lo.y, hi.y, 0x7362u);
-        __stcs(reinterpret_cast<uint4*>(dst + 16 * u), w);
+        __stcs(reinterpret_cast<uint4*>(dst), w);
     }
 }
 
@@ -639,24 +657,27 @@ __device__ __forceinline__ bool groups_before(const FusedTensor& t, uint32_t k, 
     return false;
 }
 
-// The same question put by the warps of a CTA together, without waiting: the first four ask for the state words, the others
-// for the first-level sums ...
-static_assert(kSuperBlocks == 128 && kHyperSupers == 128 && kFusedThreads == 256, "a thread asks for one word");
-__device__ __forceinline__ unsigned long long ask_before(const FusedTensor& t, uint32_t k, uint32_t tid) {
-    const uint32_t sb = k / kSuperBlocks;
-    if (tid < 128) {
-        const uint32_t at = sb * kSuperBlocks + tid;
-        return at < k ? ld_relaxed_u64(&t.state[at]) : (unsigned long long)t.epoch << 32;
-    }
-    const uint32_t at = sb / kHyperSupers * kHyperSupers + tid - 128;
-    return at < sb ? ld_relaxed_u64(&t.super[at]) : (unsigned long long)kSuperBlocks << 32;
+// The last four warps of a CTA look up a waiting block's offset and copy its records (for m = 3 the first four have one
+// more round of the final fold).
+constexpr uint32_t kPlaceThread0 = 128, kPlaceWarp0 = 4;
+
+// The same question put by those warps together, without waiting: a thread asks for one state word and one first-level sum ...
+static_assert(kSuperBlocks == 128 && kHyperSupers == 128 && kFusedThreads == 256, "a thread asks for two words");
+struct Asked { unsigned long long state, super; };
+__device__ __forceinline__ Asked ask_before(const FusedTensor& t, uint32_t k, uint32_t tid) {
+    const uint32_t sb = k / kSuperBlocks, u = tid - kPlaceThread0;
+    const uint32_t at = sb * kSuperBlocks + u, at_super = sb / kHyperSupers * kHyperSupers + u;
+    Asked a;
+    a.state = at < k ? ld_relaxed_u64(&t.state[at]) : (unsigned long long)t.epoch << 32;
+    a.super = at_super < sb ? ld_relaxed_u64(&t.super[at_super]) : (unsigned long long)kSuperBlocks << 32;
+    return a;
 }
-// ... and later each warp sums up its answers: its share, or kNotReady (the same in every lane).
-__device__ __forceinline__ uint32_t share_before(const FusedTensor& t, unsigned long long answer, uint32_t k, uint32_t tid) {
-    bool ready = uint32_t(answer >> 32) == (tid < 128 ? t.epoch : kSuperBlocks);
-    uint32_t sum = uint32_t(answer);
-    if (tid < 32) {
-        for (uint32_t i = tid; i < k / (kSuperBlocks * kHyperSupers); i += 32) {   // tensors of more than 2^28 values
+// ... and later each of the warps sums up its answers: its share, or kNotReady (the same in every lane).
+__device__ __forceinline__ uint32_t share_before(const FusedTensor& t, const Asked& a, uint32_t k, uint32_t tid) {
+    bool ready = uint32_t(a.state >> 32) == t.epoch && uint32_t(a.super >> 32) == kSuperBlocks;
+    uint32_t sum = uint32_t(a.state) + uint32_t(a.super);
+    if (tid < kPlaceThread0 + 32) {
+        for (uint32_t i = tid - kPlaceThread0; i < k / (kSuperBlocks * kHyperSupers); i += 32) {   // tensors of more than 2^28 values
             const unsigned long long w = ld_relaxed_u64(&t.hyper[i]);
             ready = ready && uint32_t(w >> 32) == kSuperBlocks * kHyperSupers;
             sum += uint32_t(w);
@@ -665,19 +686,38 @@ __device__ __forceinline__ uint32_t share_before(const FusedTensor& t, unsigned 
     sum = __reduce_add_sync(0xFFFFFFFFu, sum);
     return __all_sync(0xFFFFFFFFu, ready) ? sum : kNotReady;
 }
+// All threads: the sum of the shares; false where one of them is missing.
+__device__ __forceinline__ bool sum_shares(const uint32_t* part, uint32_t& before) {
+    const uint4 p = lds128(smem_u32(part));
+    before = p.x + p.y + p.z + p.w;
+    return max(max(p.x, p.y), max(p.z, p.w)) != kNotReady;
+}
 
-// All threads: `halves` 16-bit words from shared memory (4-byte aligned) to global memory (2-byte aligned).
+// The last four warps: `halves` 16-bit words from shared memory (4-byte aligned) to global memory (2-byte aligned), in aligned
+// pieces of 16 bytes and single halves before and behind them.
 __device__ __forceinline__ void copy_halves(uint8_t* dst, uint32_t src, uint32_t halves, uint32_t tid) {
-    const uint32_t odd = uint32_t(reinterpret_cast<uintptr_t>(dst) >> 1) & 1;   // a leading half before the first aligned word
-    const uint32_t words = halves > odd ? (halves - odd) / 2 : 0;
-    uint32_t* d32 = reinterpret_cast<uint32_t*>(dst + 2 * odd);
-    if (odd) {
-        for (uint32_t i = tid; i < words; i += kFusedThreads) d32[i] = prmt(lds32(src + 4 * i), lds32(src + 4 * i + 4), 0x5432u);
-    } else {
-        for (uint32_t i = tid; i < words; i += kFusedThreads) d32[i] = lds32(src + 4 * i);
+    const uint32_t u = tid - kPlaceThread0;
+    const uint32_t to_aligned = (0u - (uint32_t(reinterpret_cast<uintptr_t>(dst)) >> 1)) & 7;
+    const uint32_t head = min(to_aligned, halves);
+    const uint32_t pieces = (halves - head) >> 3;
+#pragma unroll 1
+    for (uint32_t p = u; p < pieces; p += kFusedThreads - kPlaceThread0) {
+        const uint32_t at = src + ((2 * head) & ~3u) + 16 * p;
+        uint32_t w[5];
+#pragma unroll
+        for (int i = 0; i < 4; ++i) w[i] = lds32(at + 4 * i);
+        if (head & 1) {
+            w[4] = lds32(at + 16);
+#pragma unroll
+            for (int i = 0; i < 4; ++i) w[i] = prmt(w[i], w[i + 1], 0x5432u);
+        }
+        *reinterpret_cast<uint4*>(dst + 2 * head + 16 * p) = make_uint4(w[0], w[1], w[2], w[3]);
     }
-    if (tid == 0 && odd && halves > 0) *reinterpret_cast<uint16_t*>(dst) = uint16_t(lds16(src));
-    if (tid == 32 && halves > odd && ((halves - odd) & 1)) *reinterpret_cast<uint16_t*>(dst + 2 * (halves - 1)) = uint16_t(lds16(src + 2 * (halves - 1)));
+    if (u < 16) {
+        const uint32_t behind = head + 8 * pieces;
+        const uint32_t h = u < 8 ? u : behind + u - 8;
+        if (u < 8 ? h < head : h < halves) reinterpret_cast<uint16_t*>(dst)[h] = uint16_t(lds16(src + 2 * h));
+    }
 }
 
 // What a failed call leaves, as the other compressors do: a header that no decompressor accepts and the length 0. (The output may
@@ -745,12 +785,19 @@ __device__ __forceinline__ Run load32_any(const uint8_t* p, bool wide) {
     if (wide) return load32<true>(p);
     return load32<false>(p);
 }
+// Stores of some lanes, predicated (an if around them becomes a branch).
+__device__ __forceinline__ void sts32_if(bool p, uint32_t a, uint32_t v) {
+    asm volatile("{\n\t.reg .pred p;\n\tsetp.ne.u32 p, %0, 0;\n\t@p st.shared.u32 [%1], %2;\n\t}" ::"r"(uint32_t(p)), "r"(a), "r"(v) : "memory");
+}
+__device__ __forceinline__ void sts8_if(bool p, uint32_t a, uint32_t v) {
+    asm volatile("{\n\t.reg .pred p;\n\tsetp.ne.u32 p, %0, 0;\n\t@p st.shared.u8 [%1], %2;\n\t}" ::"r"(uint32_t(p)), "r"(a), "r"(v) : "memory");
+}
 // One run of sixteen values of a block, group `g` of it: sign/mantissa plane, histogram, values (16 bytes per group; fp16:
 // the bits of the fp16 plane in bits 7..5 of each byte), votes for the group mask and the lanes of the wide groups among the
 // warp's, at `list`. Returns the OR of all values.
 template <int DT, bool PLAIN, bool HIST, bool CHECK = false>
 __device__ __forceinline__ uint32_t pack_run(const Run& r, uint32_t minuend, uint32_t nmask4, uint32_t s4, uint32_t wide4, uint32_t hist,
-                                             uint32_t lane, uint32_t value_at, uint32_t list, uint32_t* mask_word, bool store,
+                                             uint32_t lane, uint32_t below, uint32_t value_at, uint32_t list, uint32_t mask_word, bool store,
                                              uint8_t* sm_out) {
     uint4 v, hs, sm;
     transform_run<DT, PLAIN, HIST, CHECK>(r, minuend, nmask4, hist, lane * 4, v, hs, sm);
@@ -762,8 +809,8 @@ __device__ __forceinline__ uint32_t pack_run(const Run& r, uint32_t minuend, uin
                        (v.w & 0x1F1F1F1Fu) | (hs.w << 5));
     sts128(value_at, v);
     const uint32_t votes = __ballot_sync(0xFFFFFFFFu, is_wide);
-    if (lane == 0) *mask_word = votes;
-    if (is_wide) sts8(list + __popc(votes & ((1u << lane) - 1)), lane);
+    sts32_if(lane == 0, mask_word, votes);
+    sts8_if(is_wide, list + __popc(votes & below), lane);
     return all;
 }
 
@@ -771,8 +818,8 @@ __device__ __forceinline__ uint32_t pack_run(const Run& r, uint32_t minuend, uin
 // Returns whether some value is not representable (HIST only).
 // All loads of a thread's four runs are in flight together (3584 blocks of bf16: 56.2 us; two runs, in a rolled loop, 59.6) and
 // take no room in L1, of which the shared memory of three CTAs leaves little.
-template <int DT, bool PLAIN, bool HIST, bool CHECK = false>
-__device__ __forceinline__ bool pack_front_full(const FusedTensor& t, uint32_t k, uint32_t work, uint32_t* s_mask, uint32_t tid) {
+template <int DT, bool PLAIN, bool HIST, bool CHECK, bool WIDE>
+__device__ __forceinline__ bool pack_front_runs(const FusedTensor& t, uint32_t k, uint32_t work, uint32_t* s_mask, uint32_t tid) {
     using Shape = FusedShape<DT>;
     constexpr uint32_t kElemBytes = DT == ENEC_FP32 ? 4 : 2;
     constexpr uint32_t kStep = 16 * kFusedThreads;   // elements between a thread's runs
@@ -782,14 +829,15 @@ __device__ __forceinline__ bool pack_front_full(const FusedTensor& t, uint32_t k
     uint8_t* sm_out = t.sm + (uint64_t(k) * kBlockElems + 16 * tid);
     uint8_t* lo_out = t.lo + (uint64_t(k) * kBlockElems + 16 * tid) * 2;
     const uint32_t minuend = t.c, nmask4 = t.nmask4, s4 = t.s4, wide4 = t.wide4, wide_ok = t.wide_ok;
-    const uint32_t values = work + Shape::kValuesAt + tid * 16, list = work + Shape::kListAt + warp * 32;
+    const uint32_t values = work + Shape::kValuesAt + tid * 16, list = work + Shape::kListAt + warp * 32,
+                   masks = smem_u32(&s_mask[warp]), below = (1u << lane) - 1;
     uint32_t all = 0;
-    const bool wide_in = (wide_ok & 1) != 0;
     auto run = [&](const Run& r, uint32_t i) {
-        all |= pack_run<DT, PLAIN, HIST, CHECK>(r, minuend, nmask4, s4, wide4, work + Shape::kHistAt, lane, values + i * kStep,
-                                                list + i * kFusedThreads, &s_mask[i * kFusedWarps + warp], true, sm_out + i * kStep);
+        all |= pack_run<DT, PLAIN, HIST, CHECK>(r, minuend, nmask4, s4, wide4, work + Shape::kHistAt, lane, below, values + i * kStep,
+                                                list + i * kFusedThreads, masks + i * (kFusedWarps * 4), true, sm_out + i * kStep);
     };
     if constexpr (DT == ENEC_FP32) {   // one run's 64 bytes in flight (two runs', unrolled: 1024 blocks 45.3 -> 49.6 us)
+        const bool wide_in = (wide_ok & 1) != 0;
         Run a = load32_any(in, wide_in), b = load32_any(in + 32, wide_in);
 #pragma unroll 1
         for (uint32_t i = 0; i < 4; ++i) {
@@ -799,14 +847,22 @@ __device__ __forceinline__ bool pack_front_full(const FusedTensor& t, uint32_t k
             run(r, i);
         }
     } else {                           // all of the thread's runs
-        const Run a = load32_any(in, wide_in), b = load32_any(in + kStep * kElemBytes, wide_in),
-                  c = load32_any(in + 2 * kStep * kElemBytes, wide_in), d = load32_any(in + 3 * kStep * kElemBytes, wide_in);
+        const Run a = load32<WIDE>(in), b = load32<WIDE>(in + kStep * kElemBytes), c = load32<WIDE>(in + 2 * kStep * kElemBytes),
+                  d = load32<WIDE>(in + 3 * kStep * kElemBytes);
         run(a, 0);
         run(b, 1);
         run(c, 2);
         run(d, 3);
     }
     return (HIST || CHECK) && (DT == ENEC_FP16 ? all & rep4(0x1F) & ~nmask4 : all & ~nmask4) != 0;
+}
+
+// Two bodies for 16-bit types, since one with both kinds of loads moves what was loaded to the registers of the other kind (31
+// instructions per thread and block); fp32, with one run in flight, has one.
+template <int DT, bool PLAIN, bool HIST, bool CHECK = false>
+__device__ __forceinline__ bool pack_front_full(const FusedTensor& t, uint32_t k, uint32_t work, uint32_t* s_mask, uint32_t tid) {
+    if (DT == ENEC_FP32 || (t.wide_ok & 1)) return pack_front_runs<DT, PLAIN, HIST, CHECK, true>(t, k, work, s_mask, tid);
+    return pack_front_runs<DT, PLAIN, HIST, CHECK, false>(t, k, work, s_mask, tid);
 }
 
 // The same for the tensor's last block when it is not full and has at least 128 padded elements.
@@ -850,8 +906,8 @@ __device__ __noinline__ bool pack_front_tail(uint32_t k, uint32_t slot = 0) {
                                   int(align16(2 * uint64_t(real)) / 2) - int(e0), t.pad);
         }
         // the padding's sign/mantissa bytes are zero
-        all |= pack_run<DT, PLAIN, false, CHECK>(r, t.c, t.nmask4, t.s4, t.wide4, 0, lane, work + Shape::kValuesAt + g * 16,
-                                                 work + Shape::kListAt + first, &sh.mask[i * kFusedWarps + warp], left > 0,
+        all |= pack_run<DT, PLAIN, false, CHECK>(r, t.c, t.nmask4, t.s4, t.wide4, 0, lane, (1u << lane) - 1, work + Shape::kValuesAt + g * 16,
+                                                 work + Shape::kListAt + first, smem_u32(&sh.mask[i * kFusedWarps + warp]), left > 0,
                                                  t.sm + uint64_t(k) * kBlockElems + e0);
     }
     const bool bad = (HIST || CHECK) && (DT == ENEC_FP16 ? all & rep4(0x1F) & ~t.nmask4 : all & ~t.nmask4) != 0;
@@ -1215,16 +1271,11 @@ __device__ __noinline__ uint32_t pack_pass(FusedControl* ctl, uint32_t pass, int
     uint32_t iter = 0, mine = 0;
     uint32_t lost = 0;       // a block whose offset did not come in time (0: none; block 0 waits for nobody)
     // All threads: the waiting block's records to their place. Its offset is in sh.part, if the look-up begun during the
-    // block after it (`asked_for`) found all blocks before it counted; else the first warp waits for them.
+    // block after it (`asked_for`) found all blocks before it counted; else one of the last warps waits for them.
     auto place_waiting = [&](bool asked_for) {
         uint32_t before = 0;
-        bool ready = asked_for;
-        for (uint32_t w = 0; w < kFusedWarps; ++w) {
-            ready = ready && sh.part[w] != kNotReady;
-            before += sh.part[w];
-        }
-        if (!ready) {
-            if (warp == 0) {
+        if (!sum_shares(sh.part, before) || !asked_for) {
+            if (warp == kPlaceWarp0) {
                 const bool ok = groups_before(t, pend_block, before);
                 if (lane == 0) {
                     sh.before = before;
@@ -1235,8 +1286,9 @@ __device__ __noinline__ uint32_t pack_pass(FusedControl* ctl, uint32_t pass, int
             before = sh.before;
             if (!sh.ok) { lost = pend_block; return; }
         }
+        if (warp < kPlaceWarp0) return;
         copy_halves(t.high + uint64_t(before) * 2 * uint32_t(t.hbits), pend_at, pend_wide * uint32_t(t.hbits), tid);
-        if (warp == 0) finish_block<DT, CHECK>(t, pend_block, before, pend_wide);
+        if (warp == kPlaceWarp0) finish_block<DT, CHECK>(t, pend_block, before, pend_wide);
     };
     // one thread: no further block is handed out; those handed out already are packed, so that nobody waits for them in vain
     auto end_pass = [&]() {
@@ -1272,8 +1324,8 @@ __device__ __noinline__ uint32_t pack_pass(FusedControl* ctl, uint32_t pass, int
         if (CHECK && lossy && tid == 0) say_lossy();
         if ((lossy || lost) && tid == 0) end_pass();
         const bool waiting = pend_block != 0xFFFFFFFFu;
-        unsigned long long answer = 0;
-        if (waiting) answer = ask_before(t, pend_block, tid);   // it comes while the block is packed
+        Asked answer{0, 0};
+        if (waiting && warp >= kPlaceWarp0) answer = ask_before(t, pend_block, tid);   // it comes while the block is packed
         uint32_t excl;
         const uint32_t wide = scan_mask(sh.mask, lane, excl);
         if (tid == 0 && t.nblocks != 1) {
@@ -1307,13 +1359,13 @@ __device__ __noinline__ uint32_t pack_pass(FusedControl* ctl, uint32_t pass, int
             pack_records_any<DT>(int(hbits), work + Shape::kValuesAt, work + Shape::kListAt, wide, excl, t.s4, int(m),
                                  work + Shape::kPendAt + (iter & 1) * Shape::kPend,
                                  direct ? t.high + uint64_t(sh.before) * 2 * hbits : nullptr);
-        if (waiting) {
+        if (waiting && warp >= kPlaceWarp0) {
             const uint32_t share = share_before(t, answer, pend_block, tid);
-            if (lane == 0) sh.part[warp] = share;
+            if (lane == 0) sh.part[warp - kPlaceWarp0] = share;
         }
         const uint32_t next = sh.next;
         __syncthreads();                                      // barrier B
-        fold_out(work, N * m / 8, t.low + uint64_t(k) * (kBlockElems / 8) * m, tid);   // N >= 128: whole pieces of 16 bytes
+        fold_out(work, N * m / 8, t.low + uint64_t(k * m) * (kBlockElems / 8), tid);   // N >= 128: whole pieces of 16 bytes
         if (DT == ENEC_FP16) fold_out(work + Shape::kSmhiAt, N * 3 / 8, t.smhi + uint64_t(k) * (kBlockElems / 8) * 3, tid);
         if (waiting) place_waiting(true);
         pend_block = direct ? 0xFFFFFFFFu : k;
@@ -1340,8 +1392,8 @@ __device__ __noinline__ uint32_t pack_pass(FusedControl* ctl, uint32_t pass, int
             }
         }
     }
-    if (HIST && mine && warp == kFusedWarps - 1) {
-        // The CTA's counts go out, and the search on the whole tensor's is run, while the first warp looks up the last block's offset.
+    if (HIST && mine && warp == 0) {
+        // The CTA's counts go out, and the search on the whole tensor's is run, while the last four warps look up the last block's offset.
         // Row r of the table holds the exponent x of that remainder that the parameters can represent.
         for (uint32_t row = lane; row < Shape::kRows; row += 32) {
             const uint32_t n = fold_hist_row<false>(work + Shape::kHistAt + row * HistShape<DT>::kRowBytes, row);
