@@ -84,19 +84,26 @@ template <int DT>
 struct FusedShape {
     static constexpr int E = HistShape<DT>::E;
     static constexpr int kCtasPerSm = 3;
-    // low plane | fp16 plane | the block's values: at the same places for every m, since a list's next block may have another
-    static constexpr uint32_t kSmhiAt = kBlockElems * 5 / 8, kValuesAt = kBlockElems, kWork = 2 * kBlockElems;
-    static_assert(kSmhiAt + kBlockElems * 3 / 8 <= kValuesAt, "the planes end before the values");
-    static constexpr uint32_t kRows = DT == ENEC_FP16 ? 32 : 64;       // rows of the pack stage's histogram
-    static constexpr uint32_t kHistAt = kWork;
-    static constexpr uint32_t kHistBytes = kRows * HistShape<DT>::kRowBytes;
-    static constexpr uint32_t kListAt = kHistAt + kHistBytes;          // the wide groups' numbers, a byte each, by mask word
-    static constexpr uint32_t kPend = 4096;                            // a block's packed records waiting for their offset
-    static constexpr uint32_t kPendAt = kListAt + 1024;
-    static constexpr uint32_t kTensorAt = kPendAt + 2 * kPend;         // FusedTensor (lists: of the block, the waiting block, the next)
+    static constexpr uint32_t kListAt = 0;                             // the wide groups' numbers, a byte each, by mask word
+    static constexpr uint32_t kTensorAt = 1024;                        // FusedTensor (lists: of the block, the waiting block, the next)
     static constexpr uint32_t kSharedAt = kTensorAt + 3 * 256;         // FusedShared
-    static constexpr uint32_t kBytes = kSharedAt + 256;
-    static_assert(HistShape<DT>::kBytes <= int(kHistAt + kHistBytes), "the sample stage's table fits");
+    static constexpr uint32_t kPend = 4096;                            // a block's packed records waiting for their offset: two places
+    static constexpr uint32_t kPendAt = kSharedAt + 256;
+    // The pack stage's histogram lies on a multiple of its size (a CTA's shared memory begins with 1 KB of the system's), so that the
+    // address of a value's counter is an AND-OR of the value's word: see histogram_in_place.
+    static constexpr uint32_t kRows = DT == ENEC_FP16 ? 32 : 64;
+    static constexpr uint32_t kHistAt = 7168;
+    static constexpr uint32_t kHistBytes = kRows * HistShape<DT>::kRowBytes;
+    static_assert(kPendAt + kPend <= kHistAt && (kHistAt + 1024) % kHistBytes == 0, "the histogram's place");
+    // low plane | fp16 plane | the block's values: at the same places for every m, since a list's next block may have another
+    static constexpr uint32_t kPlanesAt = kHistAt + kHistBytes;
+    static constexpr uint32_t kSmhiAt = kPlanesAt + kBlockElems * 5 / 8, kValuesAt = kPlanesAt + kBlockElems;
+    static_assert(kSmhiAt + kBlockElems * 3 / 8 <= kValuesAt, "the planes end before the values");
+    static constexpr uint32_t kPend2At = kValuesAt + kBlockElems;
+    static constexpr uint32_t kTableAt = kHistAt;                      // the table of the stages that count, and a search's
+    static_assert(kTableAt + HistShape<DT>::kBytes <= kPend2At, "the table ends before the waiting records");
+    static constexpr uint32_t kBytes = kPend2At + kPend;
+    __device__ static uint32_t pend_at(uint32_t iter) { return iter & 1 ? kPend2At : kPendAt; }
     static_assert(kCtasPerSm * (kBytes + 1024) <= 228 * 1024, "the CTAs of an SM fit its shared memory");
 };
 
@@ -156,6 +163,11 @@ __device__ __forceinline__ FusedShared& fused_shared() { return *reinterpret_cas
 template <int DT>
 __device__ __forceinline__ bool plain_form(int b, int n) {
     return DT == ENEC_FP16 || (b + (1 << (n - 1)) <= 255 && (1 << n) <= b + (1 << (n - 1)));
+}
+// Whether the pack stage's histogram lies on a multiple of its size. (It does; a kernel where it did not would count whole tensors first.)
+template <int DT>
+__device__ __forceinline__ bool histogram_in_place() {
+    return ((smem_u32(fused_smem()) + FusedShape<DT>::kHistAt) & (FusedShape<DT>::kHistBytes - 1)) == 0;
 }
 // Whether the pack stage can keep the histogram: representable exponents are told apart by their low six bits.
 template <int DT>
@@ -359,15 +371,16 @@ __device__ __forceinline__ uint32_t select_bits(uint32_t mask, uint32_t a, uint3
 }
 
 // ---- one run: transform, sign/mantissa, histogram -------------------------------------------------------
-// hist: the pack stage's table; lane4: four times the lane, the lane's column.
+// column: the lane's in the pack stage's table, whose address is a multiple of its size. (Adding the row to any other address is one
+// instruction more per value: 32064 blocks of bf16 314.7 us, now 311.3, 4096 of fp16 59.7 and 58.9.)
 template <int DT>
-__device__ __forceinline__ void count_halves(uint32_t hist, uint32_t lane4, uint32_t w) {
+__device__ __forceinline__ void count_halves(uint32_t column, uint32_t w) {
     if constexpr (DT == ENEC_FP16) {
-        red_add_one(hist + (((w >> 3) & 0xF80u) | lane4));
-        red_add_one(hist + (((w >> 19) & 0xF80u) | lane4));
+        red_add_one(((w >> 3) & 0xF80u) | column);
+        red_add_one(((w >> 19) & 0xF80u) | column);
     } else {
-        red_add_one(hist + ((w & 0x1F80u) | lane4));
-        red_add_one(hist + (((w >> 16) & 0x1F80u) | lane4));
+        red_add_one((w & 0x1F80u) | column);
+        red_add_one(((w >> 16) & 0x1F80u) | column);
     }
 }
 
@@ -379,7 +392,7 @@ __device__ __forceinline__ uint32_t minus_twice(uint32_t a, uint32_t w) {
 }
 
 template <int DT, bool PLAIN, bool HIST, bool CHECK>
-__device__ __forceinline__ void transform_run(const Run& r, uint32_t minuend, uint32_t nmask4, uint32_t hist, uint32_t lane4, uint4& v,
+__device__ __forceinline__ void transform_run(const Run& r, uint32_t minuend, uint32_t nmask4, uint32_t column, uint4& v,
                                               uint4& hs, uint4& sm) {
     uint32_t vv[4], ss[4], hh[4];
 #pragma unroll
@@ -402,8 +415,8 @@ __device__ __forceinline__ void transform_run(const Run& r, uint32_t minuend, ui
             }
         }
         if constexpr (HIST) {
-            count_halves<DT>(hist, lane4, w0);
-            count_halves<DT>(hist, lane4, w1);
+            count_halves<DT>(column, w0);
+            count_halves<DT>(column, w1);
         }
     }
     v = make_uint4(vv[0], vv[1], vv[2], vv[3]);
@@ -480,7 +493,7 @@ __device__ __forceinline__ void pack_planes(const FusedTensor& t, uint32_t work,
     using Shape = FusedShape<DT>;
     const uint32_t j = 8 * tid, n8 = N >> 3;
     if (j >= n8) return;
-    const uint32_t values = work + Shape::kValuesAt, s4 = t.s4;
+    const uint32_t values = work + Shape::kValuesAt, planes = work + Shape::kPlanesAt, s4 = t.s4;
     uint2 v[8];
 #pragma unroll
     for (int c = 0; c < 8; ++c) v[c] = lds64(values + c * n8 + j);
@@ -488,7 +501,7 @@ __device__ __forceinline__ void pack_planes(const FusedTensor& t, uint32_t work,
 #pragma unroll
         for (int c = 0; c < 8; ++c) v[c] = make_uint2(v[c].x ^ s4, v[c].y ^ s4);
     }
-    pack_lanes_any<DT>(t.m, work, j, n8, v);
+    pack_lanes_any<DT>(t.m, planes, j, n8, v);
     if constexpr (DT == ENEC_FP16) {
 #pragma unroll
         for (int c = 0; c < 8; ++c) v[c] = make_uint2(v[c].x >> 5, v[c].y >> 5);
@@ -796,11 +809,11 @@ __device__ __forceinline__ void sts8_if(bool p, uint32_t a, uint32_t v) {
 // the bits of the fp16 plane in bits 7..5 of each byte), votes for the group mask and the lanes of the wide groups among the
 // warp's, at `list`. Returns the OR of all values.
 template <int DT, bool PLAIN, bool HIST, bool CHECK = false>
-__device__ __forceinline__ uint32_t pack_run(const Run& r, uint32_t minuend, uint32_t nmask4, uint32_t s4, uint32_t wide4, uint32_t hist,
+__device__ __forceinline__ uint32_t pack_run(const Run& r, uint32_t minuend, uint32_t nmask4, uint32_t s4, uint32_t wide4, uint32_t column,
                                              uint32_t lane, uint32_t below, uint32_t value_at, uint32_t list, uint32_t mask_word, bool store,
                                              uint8_t* sm_out) {
     uint4 v, hs, sm;
-    transform_run<DT, PLAIN, HIST, CHECK>(r, minuend, nmask4, hist, lane * 4, v, hs, sm);
+    transform_run<DT, PLAIN, HIST, CHECK>(r, minuend, nmask4, column, v, hs, sm);
     if (store) __stcs(reinterpret_cast<uint4*>(sm_out), sm);
     const uint32_t all = v.x | v.y | v.z | v.w;
     const bool is_wide = (or_flipped(v, s4) & wide4) != 0;
@@ -833,7 +846,7 @@ __device__ __forceinline__ bool pack_front_runs(const FusedTensor& t, uint32_t k
                    masks = smem_u32(&s_mask[warp]), below = (1u << lane) - 1;
     uint32_t all = 0;
     auto run = [&](const Run& r, uint32_t i) {
-        all |= pack_run<DT, PLAIN, HIST, CHECK>(r, minuend, nmask4, s4, wide4, work + Shape::kHistAt, lane, below, values + i * kStep,
+        all |= pack_run<DT, PLAIN, HIST, CHECK>(r, minuend, nmask4, s4, wide4, work + Shape::kHistAt + lane * 4, lane, below, values + i * kStep,
                                                 list + i * kFusedThreads, masks + i * (kFusedWarps * 4), true, sm_out + i * kStep);
     };
     if constexpr (DT == ENEC_FP32) {   // one run's 64 bytes in flight (two runs', unrolled: 1024 blocks 45.3 -> 49.6 us)
@@ -899,7 +912,7 @@ __device__ __noinline__ bool pack_front_tail(uint32_t k, uint32_t slot = 0) {
                 r = load32<false>(in + uint64_t(e0) * 2);
             if (HIST) {
 #pragma unroll
-                for (int q = 0; q < 8; ++q) count_halves<DT>(work + Shape::kHistAt, lane * 4, r.w[q]);
+                for (int q = 0; q < 8; ++q) count_halves<DT>(work + Shape::kHistAt + lane * 4, r.w[q]);
             }
         } else {
             r = load_run_tail<DT>(in + uint64_t(e0) * kElemBytes, out_lo + uint64_t(e0) * 2, left,
@@ -939,7 +952,7 @@ __device__ __noinline__ void pack_short_block(uint32_t k, int* status, uint32_t 
     uint8_t* out_sm = t.sm + uint64_t(k) * kBlockElems;
     uint8_t* out_lo = t.lo + uint64_t(k) * kBlockElems * 2;  // fp32 only
     const uint32_t hbits = uint32_t(t.hbits);
-    uint32_t* s_low = reinterpret_cast<uint32_t*>(fused_smem());   // 64 bytes
+    uint32_t* s_low = reinterpret_cast<uint32_t*>(fused_smem() + FusedShape<DT>::kPlanesAt);   // 64 bytes
     uint32_t* s_hi3 = s_low + 16;                                  // 32 bytes
     uint32_t* s_rec = s_hi3 + 16;                                  // 4 records of up to 14 bytes
     uint32_t* s_or = s_rec + 16;                                   // OR of y per group
@@ -1086,7 +1099,7 @@ __device__ __forceinline__ void count_done(FusedControl* ctl, uint32_t which, ui
     __syncthreads();
     if (sh.word && tid < 32) {
         const uint32_t found = search_global<DT>(ctl->hist[which], which == 1 ? ctl->pack_hist : nullptr,
-                                                 reinterpret_cast<unsigned long long*>(fused_smem())) | kParamsValid;
+                                                 reinterpret_cast<unsigned long long*>(fused_smem() + FusedShape<DT>::kTableAt)) | kParamsValid;
         if (tid == 0) {
             // hist[1]'s parameters may begin a second pass, which writes where the first one has written: what the CTAs counted
             // by hist_done wrote before is ordered before it
@@ -1109,7 +1122,7 @@ __device__ __noinline__ uint32_t histogram_stage(FusedControl* ctl, uint32_t whi
     FusedShared& sh = fused_shared<DT>();
     constexpr uint32_t kElemBytes = DT == ENEC_FP32 ? 4 : 2;
     const uint32_t tid = threadIdx.x, lane = tid & 31;
-    const uint32_t work = smem_u32(fused_smem());
+    const uint32_t table = smem_u32(fused_smem()) + FusedShape<DT>::kTableAt;
     uint32_t* const ticket = &ctl->hist_ticket[which].value;
     const uint32_t claimed = which != 0 ? 0 : total < gridDim.x ? total : gridDim.x;   // blocks that are claimed
     auto claim = [&](uint32_t i) { return (atomicOr(&ctl->claims[i / 32].value, 1u << (i & 31)) >> (i & 31) & 1) == 0; };
@@ -1120,7 +1133,7 @@ __device__ __noinline__ uint32_t histogram_stage(FusedControl* ctl, uint32_t whi
     uint32_t word;
     for (bool first = true;; first = false) {
         __syncthreads();
-        for (uint32_t i = tid; i < uint32_t(HistShape<DT>::kBytes / 16); i += kFusedThreads) sts128(work + 16 * i, make_uint4(0, 0, 0, 0));
+        for (uint32_t i = tid; i < uint32_t(HistShape<DT>::kBytes / 16); i += kFusedThreads) sts128(table + 16 * i, make_uint4(0, 0, 0, 0));
         const bool own = first && blockIdx.x < claimed;
         uint32_t taken = 0;   // thread 0: not zero when somebody else counts the block of this CTA's number
         uint32_t i = blockIdx.x;
@@ -1152,7 +1165,7 @@ __device__ __noinline__ uint32_t histogram_stage(FusedControl* ctl, uint32_t whi
             if (tid == 0 && claimed < total) asked = atomicAdd(ticket, 1u);
             const uint32_t k = base + i * stride;
             const uint32_t real = k + 1 == t.nblocks ? t.tail_real : kBlockElems;
-            count_block<DT>(t.in + uint64_t(k) * kBlockElems * kElemBytes, real, work + lane * 4, tid);
+            count_block<DT>(t.in + uint64_t(k) * kBlockElems * kElemBytes, real, table + lane * 4, tid);
             __syncthreads();
             if (tid == 0) {
                 sh.word = claimed < total ? claimed + asked : total;
@@ -1164,13 +1177,13 @@ __device__ __noinline__ uint32_t histogram_stage(FusedControl* ctl, uint32_t whi
             if (sh.ok) {
                 ++mine;
             } else {
-                for (uint32_t j = tid; j < uint32_t(HistShape<DT>::kBytes / 16); j += kFusedThreads) sts128(work + 16 * j, make_uint4(0, 0, 0, 0));
+                for (uint32_t j = tid; j < uint32_t(HistShape<DT>::kBytes / 16); j += kFusedThreads) sts128(table + 16 * j, make_uint4(0, 0, 0, 0));
                 __syncthreads();
             }
         }
         if (mine) {
             if (tid < uint32_t(HistShape<DT>::kBins)) {
-                const uint32_t n = fold_hist_row<false>(work + tid * HistShape<DT>::kRowBytes, tid);
+                const uint32_t n = fold_hist_row<false>(table + tid * HistShape<DT>::kRowBytes, tid);
                 if (n) atomicAdd(&ctl->hist[which][tid], (unsigned long long)n);
             }
             count_done<DT>(ctl, which, mine, complete);
@@ -1210,13 +1223,13 @@ __device__ __noinline__ void recount_block(FusedControl* ctl, uint32_t k) {
     const uint8_t* in = t.in + uint64_t(k) * kBlockElems * kElemBytes;
     const uint32_t real = k + 1 == t.nblocks ? t.tail_real : kBlockElems;
     __syncthreads();
-    for (uint32_t i = tid; i < kBins * kColumns / 4; i += kFusedThreads) sts128(work + 16 * i, make_uint4(0, 0, 0, 0));
+    for (uint32_t i = tid; i < kBins * kColumns / 4; i += kFusedThreads) sts128(work + Shape::kPlanesAt + 16 * i, make_uint4(0, 0, 0, 0));
     __syncthreads();
     auto move = [&](uint32_t w) {   // one value's 16-bit word
         const uint32_t x = exponent_of_word<DT>(w);
         asm volatile("red.shared.add.u32 [%0], %1;" ::"r"(work + Shape::kHistAt + lane * 4 + (x & (Shape::kRows - 1)) * HistShape<DT>::kRowBytes), "r"(~0u)
                      : "memory");
-        red_add_one(work + (x * kColumns + (lane & (kColumns - 1))) * 4);
+        red_add_one(work + Shape::kPlanesAt + (x * kColumns + (lane & (kColumns - 1))) * 4);
     };
     constexpr uint32_t kPer = HistShape<DT>::kPerLoad;
     for (uint32_t i = tid; i < real / kPer; i += kFusedThreads) {
@@ -1232,7 +1245,7 @@ __device__ __noinline__ void recount_block(FusedControl* ctl, uint32_t k) {
     __syncthreads();
     if (tid < kBins) {
         uint32_t n = 0;
-        for (uint32_t c = 0; c < kColumns; ++c) n += lds32(work + (tid * kColumns + c) * 4);
+        for (uint32_t c = 0; c < kColumns; ++c) n += lds32(work + Shape::kPlanesAt + (tid * kColumns + c) * 4);
         if (n) atomicAdd(&ctl->hist[1][tid], (unsigned long long)n);
     }
     __syncthreads();
@@ -1357,7 +1370,7 @@ __device__ __noinline__ uint32_t pack_pass(FusedControl* ctl, uint32_t pass, int
         }
         if (!direct || sh.ok)
             pack_records_any<DT>(int(hbits), work + Shape::kValuesAt, work + Shape::kListAt, wide, excl, t.s4, int(m),
-                                 work + Shape::kPendAt + (iter & 1) * Shape::kPend,
+                                 work + Shape::pend_at(iter),
                                  direct ? t.high + uint64_t(sh.before) * 2 * hbits : nullptr);
         if (waiting && warp >= kPlaceWarp0) {
             const uint32_t share = share_before(t, answer, pend_block, tid);
@@ -1365,12 +1378,12 @@ __device__ __noinline__ uint32_t pack_pass(FusedControl* ctl, uint32_t pass, int
         }
         const uint32_t next = sh.next;
         __syncthreads();                                      // barrier B
-        fold_out(work, N * m / 8, t.low + uint64_t(k * m) * (kBlockElems / 8), tid);   // N >= 128: whole pieces of 16 bytes
+        fold_out(work + Shape::kPlanesAt, N * m / 8, t.low + uint64_t(k * m) * (kBlockElems / 8), tid);   // N >= 128: whole pieces of 16 bytes
         if (DT == ENEC_FP16) fold_out(work + Shape::kSmhiAt, N * 3 / 8, t.smhi + uint64_t(k) * (kBlockElems / 8) * 3, tid);
         if (waiting) place_waiting(true);
         pend_block = direct ? 0xFFFFFFFFu : k;
         pend_wide = wide;
-        pend_at = work + Shape::kPendAt + (iter & 1) * Shape::kPend;
+        pend_at = work + Shape::pend_at(iter);
         if (HIST && lossy) recount_block<DT>(ctl, k);
         k = next;
     }
@@ -1423,12 +1436,13 @@ enec_fused_kernel(const FusedJob job, int* status) {
     using Shape = FusedShape<DT>;
     const uint32_t tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const uint32_t work = smem_u32(smem);
-    unsigned long long* const search_table = reinterpret_cast<unsigned long long*>(smem);
+    const uint32_t table = work + Shape::kTableAt;
+    unsigned long long* const search_table = reinterpret_cast<unsigned long long*>(smem + Shape::kTableAt);
     FusedControl* const ctl = job.ctl;
     const uint32_t nblocks = uint32_t((job.count + kBlockElems - 1) / kBlockElems);
     pdl_launch_dependents();
     if (gridDim.x == 1 && !job.given)
-        for (uint32_t i = tid; i < uint32_t(HistShape<DT>::kBytes / 16); i += kFusedThreads) sts128(work + 16 * i, make_uint4(0, 0, 0, 0));
+        for (uint32_t i = tid; i < uint32_t(HistShape<DT>::kBytes / 16); i += kFusedThreads) sts128(table + 16 * i, make_uint4(0, 0, 0, 0));
     if (tid == 0) {
         t.in = job.in; t.out = job.out; t.count = job.count; t.out_size = job.out_size;
         set_geometry<DT>(t);
@@ -1450,10 +1464,10 @@ enec_fused_kernel(const FusedJob job, int* status) {
         exact = true;
         if (tid == 0) sh.next = nblocks == 1 ? 0u : atomicAdd(&ctl->pack_ticket[0].value, 1u);
     } else if (gridDim.x == 1) {  // one block: nothing to hand out, nobody to tell
-        count_block<DT>(job.in, t.tail_real, work + lane * 4, tid);
+        count_block<DT>(job.in, t.tail_real, table + lane * 4, tid);
         __syncthreads();
         uint32_t* counts = reinterpret_cast<uint32_t*>(smem + Shape::kPendAt);
-        if (tid < uint32_t(HistShape<DT>::kBins)) counts[tid] = fold_hist_row<false>(work + tid * HistShape<DT>::kRowBytes, tid);
+        if (tid < uint32_t(HistShape<DT>::kBins)) counts[tid] = fold_hist_row<false>(table + tid * HistShape<DT>::kRowBytes, tid);
         __syncthreads();
         if (warp == 0) {
             const uint32_t found = search_by_warp<DT>([&](int x) { return (unsigned long long)counts[x]; }, search_table);
@@ -1463,7 +1477,7 @@ enec_fused_kernel(const FusedJob job, int* status) {
         word = sh.word;
     } else {
         word = histogram_stage<DT>(ctl, 0, 0, job.sample, nblocks / job.sample, job.sample);
-        if (!exact && word != 0 && !sample_will_do<DT>(word)) {
+        if (!exact && word != 0 && !(sample_will_do<DT>(word) && histogram_in_place<DT>())) {
             exact = true;
             word = histogram_stage<DT>(ctl, 1, 0, nblocks, 1, nblocks);
         }

@@ -76,7 +76,8 @@ enec_fused_list_kernel(const FusedList list, int* status) {
     FusedShared& sh = fused_shared<DT>();
     const uint32_t tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const uint32_t work = smem_u32(smem);
-    unsigned long long* const search_table = reinterpret_cast<unsigned long long*>(smem);
+    const uint32_t table = work + Shape::kTableAt;
+    unsigned long long* const search_table = reinterpret_cast<unsigned long long*>(smem + Shape::kTableAt);
     pdl_launch_dependents();
     pdl_wait();  // nothing above touches global memory
 
@@ -165,7 +166,7 @@ enec_fused_list_kernel(const FusedList list, int* status) {
         if (lane == 0) sh.part[warp - kPlaceWarp0] = share;
     };
     auto clear_table = [&]() {
-        for (uint32_t i = tid; i < uint32_t(HistShape<DT>::kBytes / 16); i += kFusedThreads) sts128(work + 16 * i, make_uint4(0, 0, 0, 0));
+        for (uint32_t i = tid; i < uint32_t(HistShape<DT>::kBytes / 16); i += kFusedThreads) sts128(table + 16 * i, make_uint4(0, 0, 0, 0));
     };
 
     __syncthreads();
@@ -195,12 +196,12 @@ enec_fused_list_kernel(const FusedList list, int* status) {
             clear_table();
             ask_waiting();
             __syncthreads();
-            count_block<DT>(in, left < n * kBlockElems ? uint32_t(left) : n * kBlockElems, work + lane * 4, tid);
+            count_block<DT>(in, left < n * kBlockElems ? uint32_t(left) : n * kBlockElems, table + lane * 4, tid);
             if (waiting) share_waiting(answer);
             scout_middle();
             __syncthreads();
             if (tid < uint32_t(HistShape<DT>::kBins)) {
-                const uint32_t c = fold_hist_row<false>(work + tid * HistShape<DT>::kRowBytes, tid);
+                const uint32_t c = fold_hist_row<false>(table + tid * HistShape<DT>::kRowBytes, tid);
                 if (c) atomicAdd(&ctl.hist[tid], (unsigned long long)c);
             }
             __syncthreads();
@@ -223,10 +224,10 @@ enec_fused_list_kernel(const FusedList list, int* status) {
                 __syncthreads();
                 clear_table();
                 __syncthreads();
-                count_block<DT>(item.in, uint32_t(item.count), work + lane * 4, tid);
+                count_block<DT>(item.in, uint32_t(item.count), table + lane * 4, tid);
                 __syncthreads();
                 uint32_t* counts = reinterpret_cast<uint32_t*>(smem + Shape::kListAt);   // 1 KB
-                if (tid < uint32_t(HistShape<DT>::kBins)) counts[tid] = fold_hist_row<false>(work + tid * HistShape<DT>::kRowBytes, tid);
+                if (tid < uint32_t(HistShape<DT>::kBins)) counts[tid] = fold_hist_row<false>(table + tid * HistShape<DT>::kRowBytes, tid);
                 __syncthreads();
                 if (warp == 0) {
                     const uint32_t found = search_by_warp<DT>([&](int x) { return (unsigned long long)counts[x]; }, search_table);
@@ -291,7 +292,7 @@ enec_fused_list_kernel(const FusedList list, int* status) {
                 }
                 if (!stop)
                     pack_records_any<DT>(int(hbits), work + Shape::kValuesAt, work + Shape::kListAt, wide, excl,
-                                         t.s4, int(m), work + Shape::kPendAt + (iter & 1) * Shape::kPend,
+                                         t.s4, int(m), work + Shape::pend_at(iter),
                                          direct ? t.high + uint64_t(sh.before) * 2 * hbits : nullptr);
                 leaves_records = !direct;
             }
@@ -303,7 +304,7 @@ enec_fused_list_kernel(const FusedList list, int* status) {
             __syncthreads();                                      // barrier B
             if (present && N >= 128) {
                 const uint32_t m = uint32_t(t.m);
-                fold_out(work, N * m / 8, t.low + uint64_t(k * m) * (kBlockElems / 8), tid);
+                fold_out(work + Shape::kPlanesAt, N * m / 8, t.low + uint64_t(k * m) * (kBlockElems / 8), tid);
                 if (DT == ENEC_FP16) fold_out(work + Shape::kSmhiAt, N * 3 / 8, t.smhi + uint64_t(k) * (kBlockElems / 8) * 3, tid);
             }
         }
@@ -314,7 +315,7 @@ enec_fused_list_kernel(const FusedList list, int* status) {
         if (leaves_records) {
             pend_block = k;
             pend_wide = wide;
-            pend_at = work + Shape::kPendAt + (iter & 1) * Shape::kPend;
+            pend_at = work + Shape::pend_at(iter);
             pend_slot = slot;
         }
         slot = next_slot;
