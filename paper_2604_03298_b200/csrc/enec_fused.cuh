@@ -1436,6 +1436,18 @@ enec_fused_kernel(const FusedJob job, int* status) {
     pdl_launch_dependents();
     if (gridDim.x == 1 && !job.given)
         for (uint32_t i = tid; i < uint32_t(HistShape<DT>::kBytes / 16); i += kFusedThreads) sts128(table + 16 * i, make_uint4(0, 0, 0, 0));
+    if (tid == 32) {
+        // The block that the CTA most likely begins with is asked for while the kernel before still runs: L2 is coherent, so a line that
+        // is written until then is simply updated, and nothing is read here (1024 blocks of bf16 23.7 us, now 22.8, 3584 blocks 48.9 and
+        // 48.2, with given parameters 14.6 and 14.0, 36.2 and 35.3).
+        const uint32_t stride = job.given ? 1 : nblocks / job.sample, k = blockIdx.x * stride;
+        if (job.given || blockIdx.x < job.sample) {
+            constexpr uint32_t kElemBytes = DT == ENEC_FP32 ? 4 : 2;
+            const uint64_t from = uint64_t(k) * kBlockElems, left = job.count - from;
+            const uint32_t bytes = ((left < kBlockElems ? uint32_t(left) : kBlockElems) * kElemBytes) & ~15u;
+            if (bytes) bulk_prefetch_l2(job.in + from * kElemBytes, bytes);
+        }
+    }
     if (tid == 0) {
         t.in = job.in; t.out = job.out; t.count = job.count; t.out_size = job.out_size;
         set_geometry<DT>(t);
