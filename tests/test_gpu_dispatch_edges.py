@@ -280,3 +280,40 @@ def test_misled_samples_with_second_level_sums(oracle, what):
     t = _weights(blocks * 16384 + 100, 0, 12)
     t = _mislead(torch.where(t.abs() < 1e-6, torch.full_like(t, 1e-6), t), blocks, what)
     assert np.array_equal(_compress_twice(enec, t, 0), oracle.compress(_words(t, 0), 0))
+
+
+def _sixteen_behind(t):
+    """A copy of the tensor that starts 16 bytes behind a 32-byte boundary (torch's allocator never gives such an address)."""
+    ahead = 16 // t.element_size()
+    holder = torch.zeros(t.numel() + ahead, dtype=t.dtype, device="cuda")
+    assert holder.data_ptr() % 32 == 0
+    holder[ahead:].copy_(t)
+    return holder[ahead:]
+
+
+@pytest.mark.parametrize("dt", [0, 1, 2])
+@pytest.mark.parametrize("full_width", [False, True])
+@pytest.mark.parametrize("count", [16384, 8192 + 300, 16384 * 5, 16384 * 5 + 300, 16384 * 3 + 37, 16384 * 1409, 16384 * 1409 + 300])
+def test_compress_inputs_sixteen_bytes_behind_a_32_byte_boundary(oracle, dt, full_width, count):
+    """Such inputs take 16-byte loads, for bf16 and fp16 in a body of its own: with a search on the whole tensor and on a sample, with
+    given parameters, and in a list beside inputs on a 32-byte boundary. full_width: an exact zero, so that n = E (for bf16 and fp32
+    the form in which b + 2^(n-1) does not fit a byte)."""
+    import paper_2604_03298_b200 as enec
+    t = _weights(count, dt, count)
+    t = torch.where(t.abs() < 2e-3, torch.full_like(t, 2e-3), t)
+    if full_width:
+        t[count // 2] = 0
+    want = oracle.compress(_words(t, dt), dt)
+    odd = _sixteen_behind(t)
+    assert odd.data_ptr() % 32 == 16
+    assert np.array_equal(_compress_twice(enec, odd, dt), want)
+    assert np.array_equal(enec.compress_tensor(odd, params=want[20:23].tolist()).cpu().numpy(), want)
+    srcs = [odd, t, odd]
+    cap = enec.enec_max_compressed_size(dt, count)
+    bufs = [torch.full((cap + 16,), 0xA5, dtype=torch.uint8, device="cuda") for _ in srcs]
+    sizes, status = torch.zeros(len(srcs), dtype=torch.int64, device="cuda"), status_tensor()
+    assert enec.enec_compress_batched([(s, b, count, cap) for s, b in zip(srcs, bufs)], dt, sizes, status) == 0
+    assert int(status.item()) == 0
+    for b, n in zip(bufs, sizes.tolist()):
+        assert bool((b[cap:] == 0xA5).all())
+        assert np.array_equal(b[:n].cpu().numpy(), want)
