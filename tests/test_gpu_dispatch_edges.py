@@ -317,3 +317,39 @@ def test_compress_inputs_sixteen_bytes_behind_a_32_byte_boundary(oracle, dt, ful
     for b, n in zip(bufs, sizes.tolist()):
         assert bool((b[cap:] == 0xA5).all())
         assert np.array_equal(b[:n].cpu().numpy(), want)
+
+
+@pytest.mark.parametrize("dt, b, n, m", [(0, 120, 5, 3), (0, 120, 6, 3), (0, 120, 7, 3), (0, 127, 8, 3), (0, 127, 8, 1), (0, 120, 4, 3),
+                                         (1, 14, 5, 4), (1, 14, 5, 3), (1, 14, 5, 2), (1, 14, 5, 1), (2, 120, 6, 3), (2, 127, 8, 1)])
+def test_waiting_records_are_copied_to_any_offset(oracle, dt, b, n, m):
+    """A block's packed records wait in 4096 bytes of shared memory and go to their offset in pieces of 16 bytes, with single halves
+    (16 bits) before and behind them: blocks with no, few, many and all groups wide, with records that fill the 4096 bytes, fall just
+    short of them or exceed them (those go straight to their place), at offsets of every remainder. Enough blocks that a CTA
+    packs several and uses both of its places."""
+    import paper_2604_03298_b200 as enec
+    blocks, h = 1400, n - m
+    rng = np.random.default_rng(100 * n + m + dt)
+    fit = 2048 // h   # wide groups whose records fit
+    wide = rng.choice([c for c in (0, 1, 2, 3, 4, 5, 6, 7, 8, 9, 15, 250, fit - 1, fit, fit + 1, 1024) if c <= 1024], blocks)
+    start = (np.cumsum(wide) - wide) * h   # in halves, from an address that is a multiple of 16 bytes
+    waits = (wide <= fit) & (wide > 0)
+    assert set((start[waits] % 8).tolist()) == (set(range(8)) if h % 8 % 2 else set(range(0, 8, 2 if h % 4 else 4)))
+    assert h in (4, 7) or ((wide * h < (-start) % 8) & waits).any()   # records that end before the first aligned piece
+    # every group holds b (stored as 0); a wide one also b + 1 (stored as 2^n - 1) and any below b
+    is_wide = np.argsort(rng.random((blocks, 1024)), 1) < wide[:, None]
+    x = np.full((blocks, 1024, 16), b, dtype=np.uint32)
+    x[..., 5] += is_wide
+    x[..., 11] = np.where(is_wide, b - rng.integers(0, 1 << (n - 1), is_wide.shape), b)
+    x = x.reshape(-1)
+    other = rng.integers(0, 1 << 32, x.size, dtype=np.uint32)   # sign and mantissa
+    if dt == 2:
+        w = x << 23 | (other & 0x807FFFFF)
+    else:
+        mant = 7 if dt == 0 else 10
+        w = (x << mant | (other & (0x8000 | ((1 << mant) - 1)))).astype(np.uint16)
+    t = torch.from_numpy(w.view(np.int32 if dt == 2 else np.int16)).cuda().view(DTYPES[dt])
+    want = oracle.compress(w, dt, (b, n, m))
+    assert want[32:36].view(np.uint32)[0] == wide.sum()   # the header's count of wide groups
+    for _ in range(2):
+        got = enec.compress_tensor(t, params=(b, n, m))
+        assert np.array_equal(got.cpu().numpy(), want)
