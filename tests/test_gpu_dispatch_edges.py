@@ -353,3 +353,31 @@ def test_waiting_records_are_copied_to_any_offset(oracle, dt, b, n, m):
     for _ in range(2):
         got = enec.compress_tensor(t, params=(b, n, m))
         assert np.array_equal(got.cpu().numpy(), want)
+
+
+def test_where_a_ctas_shared_memory_begins():
+    """The pack stage addresses its histogram by an AND-OR, which wants it on a multiple of its size; where it is not, sampled tensors
+    are counted whole first (a waste that no stream shows). The kernels have no static shared memory, and dynamic shared memory
+    begins where the layout in enec_fused.cuh takes it to begin."""
+    import ctypes
+    import os
+    import re
+    import paper_2604_03298_b200 as enec
+
+    lib, runtime = enec.lib(), ctypes.CDLL("libcudart.so.12")
+    for dt in range(3):
+        for kernel, job in (("17enec_fused_kernel", "8FusedJob"), ("22enec_fused_list_kernel", "9FusedList")):
+            attributes = (ctypes.c_size_t * 64)()   # cudaFuncAttributes begins with sharedSizeBytes
+            stub = ctypes.cast(getattr(lib, f"_ZN4enec{kernel}ILi{dt}EEEvNS_{job}EPi"), ctypes.c_void_p)
+            assert runtime.cudaFuncGetAttributes(attributes, stub) == 0
+            assert attributes[0] == 0
+    probe = torch.cuda._compile_kernel("""extern "C" __global__ void base(unsigned* out) {
+        extern __shared__ __align__(128) unsigned char s[];
+        if (threadIdx.x == 0) *out = (unsigned)__cvta_generic_to_shared(s);
+    }""", "base")
+    out = torch.zeros(1, dtype=torch.int32, device="cuda")
+    probe(grid=(1, 1, 1), block=(32, 1, 1), args=[out], shared_mem=1024)
+    text = open(os.path.join(os.path.dirname(enec.__file__), "csrc", "enec_fused.cuh")).read()
+    place = int(re.search(r"kHistAt = (\d+);", text).group(1))
+    for rows in (32, 64):   # of 32 counters
+        assert (int(out.item()) + place) % (rows * 128) == 0
