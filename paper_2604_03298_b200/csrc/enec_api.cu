@@ -160,10 +160,10 @@ static void place_job(EncodeJob& job, uint8_t* scratch, uint32_t epoch) {
 // enec_compress takes the one-kernel form (enec_fused.cuh) for every size: none is known where the split form (histogram, pack
 // kernel, then the kernel that places the records) is the faster one. That one is kept to measure and test against: for tensors of
 // ENEC_SPLIT_MIN_BLOCKS .. ENEC_SPLIT_MAX_BLOCKS - 1 blocks, both from the environment and read once; without the first there is
-// no such size. Given parameters always take the one-kernel form. One kernel against histogram and look-back kernel (up to 1024
-// blocks) and split form (beyond): 4096 values 8.5 against 11.0 us, 256 blocks 13.0 / 22.5, 1024 blocks 25.1 / 35.1, 3584 blocks
-// 53 / 83, 32064 blocks 354 / 594 (bf16, in a stream). Where its sample misleads the one-kernel form it can be the slower one:
-// see enec_fused.cu.
+// no such size. Given parameters always take the one-kernel form. One kernel against histogram and look-back
+// kernel (as enec_compress_noalloc runs them, behind a memset) and against the split form: 4096 values 5.6 us against 12.9 and 27.4,
+// 256 blocks 12.6 / 20.4 / 21.2, 1024 blocks 21.2 / 31.1 / 31.2, 3584 blocks 48.9 / 79.1 / 84.8, 32064 blocks 313 / 559 / 603 (bf16, in
+// a stream). Where its sample misleads the one-kernel form it can be the slower one: see enec_fused.cu.
 static uint32_t env_blocks(const char* name, uint32_t fallback) {
     const char* e = getenv(name);
     return e && *e ? uint32_t(strtoul(e, nullptr, 10)) : fallback;

@@ -10,15 +10,15 @@
 //      CTAs pack the tensor again; a value that the sampled parameters cannot represent ends the pack stage at once, and the blocks
 //      not packed yet are counted first.
 // Parameters given by the caller: stage 2 alone, without the histogram, from the first block on; a value that they lose ends
-// the call without a stream. (With a look-back kernel, or two kernels from 2048 blocks up, 3584 blocks of bf16 took 54 us, now 37.3;
-// 1024 blocks 23.2 -> 15.1, fp16 4096 blocks 63.8 -> 47.5, fp32 8192 blocks 192 -> 168.)
+// the call without a stream. (With a look-back kernel, or two kernels from 2048 blocks up, 3584 blocks of bf16 took 54 us, now 35.1;
+// 1024 blocks 23.2 -> 13.9, fp16 4096 blocks 63.8 -> 43.8, fp32 8192 blocks 192 -> 158.)
 // A tensor whose sample needs n > 6 exponent bits (bf16, fp32) takes the histogram of the whole tensor before it packs:
 // the table kept beside the packing has 64 rows, and rare outliers of such a tensor are what a sample misses.
 //
 // Block offsets (the prefix sum of Sec. 5.1 / 5.4): every block's count of wide groups goes to a state word and is added
 // to a sum per 128 blocks and a sum per 16384 blocks. A CTA keeps a block's packed records in shared memory while it
-// packs its next block; by then all blocks handed out before have been counted as a rule, so one warp finds the block's
-// offset with one round of loads and copies the records to their place.
+// packs its next block; by then all blocks handed out before have been counted as a rule, so its last four warps find the block's
+// offset with one round of loads and copy the records to their place (if some block is not counted yet, one of them waits for it).
 //
 // A wait concerns only work whose tickets were handed out before, hence running CTAs, and in the pack stage only blocks
 // with smaller numbers: the CTA with the smallest block that is not counted yet waits for nobody. Every wait is bounded
@@ -573,8 +573,10 @@ __device__ __forceinline__ void record_words(const uint4& v, uint32_t s4, int m,
 // t + 256, .. (the block's values at shared address `values`; the numbers of mask word w's wide groups, a byte each, at
 // list + 32 w; lane w of every warp: wide groups before word w in `excl`). Records go to shared memory at `pend`, or, when they
 // do not fit there, straight to `out` (2-byte aligned). A weight's block has about 250 wide groups: one round for the CTA. (Every
-// warp packing the wide groups of its own runs takes two as a rule, since they are rarely 32 at most: 32064 blocks of bf16 363.5 us,
-// now 356; 4096 blocks of fp32 100.3, now 97.3; 1024 heavy-tailed ones of bf16 23.1, now 22.6.)
+// warp packing the wide groups of its own runs takes two as a rule, since they are rarely 32 at most: nine tensors of a layer
+// 277.2 us, now 271.0; 32064 blocks of bf16 366.5, now 358.9. Blocks whose groups are all wide, of random exponents, gain nothing
+// and pay for the look-up of the words: 3584 blocks of bf16 82.5 -> 83.4, a list of 56 tensors 96.4 -> 98.7. Leaving it out
+// for them brings 3584 blocks to 79.9, but costs the list compressor registers: a layer of ordinary weights 243.3 -> 247.6.)
 template <int H>
 __device__ __forceinline__ void pack_records(uint32_t values, uint32_t list, uint32_t wide, uint32_t excl, uint32_t s4, int m, uint32_t pend,
                                              uint8_t* out) {
@@ -1453,7 +1455,7 @@ enec_fused_kernel(const FusedJob job, int* status) {
         set_geometry<DT>(t);
     }
     __syncthreads();
-    pdl_wait();  // nothing above touches global memory
+    pdl_wait();  // above, lines of the input are asked for; nothing is read or written
     {
         // the next call on this scratch area finds its control set and sums zeroed
         const uint32_t at = blockIdx.x * kFusedThreads + tid, all = gridDim.x * kFusedThreads;

@@ -12,7 +12,7 @@
 // smaller tickets.
 //
 // Against the two launches before (histograms of all tensors, then a look-back kernel over all blocks): 56 tensors of 139 MB
-// bf16 120 -> 87 us, a Llama-3-8B-shaped layer 308 -> 241 us.
+// bf16 120 -> 86 us, a Llama-3-8B-shaped layer 308 -> 242 us.
 #pragma once
 
 #include "enec_fused.cuh"
@@ -279,7 +279,9 @@ enec_fused_list_kernel(const FusedList list, int* status) {
                 if (tid < uint32_t(align16(((N >> 4) + 7) / 8)) / 16)
                     reinterpret_cast<uint4*>(t.mask + uint64_t(k) * (kGroupsPerBlock / 8))[tid] = reinterpret_cast<const uint4*>(sh.mask)[tid];
                 pack_planes<DT>(t, work, N, tid);
-                ask_waiting();   // (before the planes, the fp32 kernel keeps 100 bytes more of a thread in local memory: 88 -> 94 us)
+                // (asked for right behind barrier A, the answers are held over the scan and the planes, for which there are no registers:
+                // 56 tensors of fp32 152.2 -> 154.9 us, of bf16 86.8 -> 87.4, heavy-tailed 89.4 -> 91.9)
+                ask_waiting();
                 if (direct) {
                     if (warp == 0) {
                         uint32_t before = 0;
